@@ -137,9 +137,11 @@ fil_status fil_sys_stats(const fil_ctx *c, int32_t *iters, double *finf);
  * loads (CUDA events around it, so host launch gaps do not count) for every
  * candidate schedule -- tiles of 256 targets (2 per thread) or 128 targets
  * (1 per thread, with source split 1 or 2 on the FP32 path: see
- * fil_set_source_split), and 1..occupancy resident CTAs per SM for the
- * stream-K split of the (tile, source chunk) work units -- and keeps the fastest for all
- * later applies. The applies first run for 50 ms of wall time (an idle GPU's
+ * fil_set_source_split), 1..occupancy resident CTAs per SM for the stream-K
+ * split of the (tile, sources) work units, and the automatic schedule a new
+ * context of one system starts with on the FP32 path -- and keeps the fastest for all
+ * later applies (if that is the automatic one it stays in use, and the outputs
+ * name the 256-target tiles a new context reports). The applies first run for 50 ms of wall time (an idle GPU's
  * clock is still rising then) and the candidates are swept twice, each
  * keeping its faster time. Reports the choice (nullable outputs) and its
  * pair-kernel time per apply in ms. Results change only in rounding (the
@@ -151,7 +153,10 @@ fil_status fil_autotune(fil_ctx *c, int32_t reps, int32_t *tile, int32_t *ctas_p
  * targets per thread or tile 128 with 1, and ctas_per_sm from 1 to the
  * kernel's occupancy; the source split goes back to 1. FIL_EINVAL for another
  * combination, FIL_ESTATE inside a step. fil_pair_schedule reads the current
- * one (nullable outputs). */
+ * one (nullable outputs). On the FP32 path a context of one system whose
+ * schedule was never set reports 256-target tiles at 4 CTAs per SM and runs the
+ * automatic schedule: 64-target tiles per warp, the (tile, source group) units
+ * split evenly over one CTA of 12 warps per SM. */
 fil_status fil_set_pair_schedule(fil_ctx *c, int32_t tile, int32_t targets_per_thread,
                                  int32_t ctas_per_sm);
 fil_status fil_pair_schedule(const fil_ctx *c, int32_t *tile, int32_t *targets_per_thread,
@@ -433,12 +438,12 @@ fil_status fil_fma_peak(int32_t fp64, double *flops_per_s, double *sm_mhz);
  * n_seg segments with radius a and viscosity eta: Y (S x 3), FT (S x 6) and
  * VW (S x 6) must be DEVICE pointers of the current device (or managed
  * memory), owned by the caller. It allocates nothing: its scratch is a fixed
- * static device array of about 10.6 MB in the library (plus 128 per-tile
+ * static device array of about 9.6 MB in the library (plus 512 per-tile
  * completion counters, zero between calls), which every GPU that loads the
  * library keeps until the process exits. Limits: 1 <= n_seg <=
  * 32768; larger sizes, host pointers, pointers to another GPU's memory or
  * non-positive a, eta return FIL_EINVAL; a failed launch returns FIL_ECUDA.
- * The scratch holds the stream-K partial sums of up to 4 x 152 CTAs (the
+ * The scratch holds the stream-K partial sums of 12 warps on up to 152 SMs (the
  * context path's grid on a 152-SM GB300); on a part with more SMs the grid is
  * capped there and the results differ from fil_mobility_apply's in rounding.
  * The first call on a device looks up the array's device address for that

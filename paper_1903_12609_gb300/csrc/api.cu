@@ -104,14 +104,11 @@ void carve(fil_ctx *c, Arena &ar, int red_blocks, size_t partial_bytes) {
     c->tile_src_d = ar.take<int64_t>(c->rpy_tiles_max);
     c->tile_nsrc_d = ar.take<int64_t>(c->rpy_tiles_max);
     c->tile_id_d = ar.take<int>(c->rpy_tiles_max);
-    c->slot_d = ar.take<int>(c->Spad / kRpyThreads);
     c->act_unit_off_d = ar.take<int64_t>(c->rpy_tiles_max + 1);
     c->act_src_d = ar.take<int64_t>(c->rpy_tiles_max);
     c->act_nsrc_d = ar.take<int64_t>(c->rpy_tiles_max);
     c->act_tile_d = ar.take<int>(c->rpy_tiles_max);
-    c->act_slot_d = ar.take<int>(c->Spad / kRpyThreads);
     c->act_dyn_d = ar.take<int64_t>(2);
-    c->pos_of_seg_d = ar.take<int64_t>(S);
     c->pad_map_d = ar.take<int>(c->Spad);
     c->Y = ar.take<double>(3 * S);
     c->Yprev = ar.take<double>(3 * S);
@@ -135,7 +132,7 @@ void carve(fil_ctx *c, Arena &ar, int red_blocks, size_t partial_bytes) {
     c->VW = ar.take<double>(6 * S);
     c->Mh = nullptr;
     if (pair32_on(c)) {
-        c->src32 = ar.take<float4>((size_t)kRpyPairF4 * (c->Spad / 2));
+        c->src32 = ar.take<float4>((size_t)kRpyGroupF4 * (c->Spad / kRpyComp));
         c->src64 = nullptr;
     } else {
         c->src64 = ar.take<double>(9 * c->Spad);

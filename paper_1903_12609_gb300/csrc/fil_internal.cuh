@@ -93,22 +93,24 @@ struct fil_ctx {
     int64_t *sys_xoff;                    // [n_sys + 1] offsets into X (6 x segments)
 
     // RPY workspace; systems padded to whole target tiles (rpy.cu)
-    float4 *src32;        // 3 float4 per (padded) segment, mixed path
-    double *src64;        // 12 doubles per (padded) segment, FP64 path
+    float4 *src32;        // groups of 32 (padded) segments, kRpyGroupF4 float4 each at most, FP32 path
+    double *src64;        // 9 doubles per (padded) segment, FP64 path
     int64_t Spad;
     void *partials;       // stream-K partial sums
     int *tile_cnt;        // per listed tile: work units whose partial is written (zero between launches)
     int rpy_grid32, rpy_grid64;
     int64_t rpy_tiles, rpy_units;
-    std::vector<int64_t> sys_pad_off_h, tile_unit_off_h, tile_src_h, tile_nsrc_h, pos_of_seg_h;
+    std::vector<int64_t> sys_pad_off_h, tile_unit_off_h, tile_src_h, tile_nsrc_h;
     std::vector<int> pad_map_h, tile_sys_h, tile_id_h;
-    int64_t *tile_unit_off_d, *tile_src_d, *tile_nsrc_d, *pos_of_seg_d;
-    int *pad_map_d, *tile_id_d, *slot_d;
+    int64_t *tile_unit_off_d, *tile_src_d, *tile_nsrc_d;
+    int *pad_map_d, *tile_id_d;
     int rpy_tpt;           // targets per thread of the pair kernels
     int rpy_split = 1;     // source split of the FP32 one-target kernel (1 or 2 halves per CTA)
     int rpy_threads;       // threads per CTA of the FP32 pair kernel (128, or 64 with tpt 2);
                            // tile = rpy_threads x rpy_tpt targets
     int rpy_ctas;          // resident CTAs per SM of the stream-K grid
+    int rpy_frames = 0;    // FP32 path: source groups in their own frames (one system; rpy.cu)
+    int rpy_auto = 0;      // FP32 path: no schedule set by hand, the warp kernel runs (rpy.cu)
     int rpy_ctas_max;
     int64_t rpy_tiles_max; // listed tiles at the smallest tile size
     // the tiles of the systems still iterating (ensembles): applies inside a
@@ -117,7 +119,7 @@ struct fil_ctx {
     double pairs_all, pairs_act;   // sum of S_s^2 over all / the active systems
     double n_pairs;                // pairs evaluated by all applies so far
     int64_t *act_unit_off_d, *act_src_d, *act_nsrc_d;
-    int *act_tile_d, *act_slot_d;
+    int *act_tile_d;
     int64_t *act_dyn_d;    // {act_tiles, act_units} on the device
 
     // Broyden state

@@ -18,37 +18,30 @@
 // and A, C give the self mobilities 1/(6 pi eta a), 1/(8 pi eta a^3).
 //
 // Kernel design (GB300, one GPU):
-//  * No tensor cores: the pair sum is not a dense contraction. The bound is the
-//    FP32 (or FP64) FMA pipe; a pair costs ~51 FP32 operations + 1 MUFU.
-//  * Each thread owns kRpyTargetsPerThread targets in registers; a CTA owns a
-//    tile of kRpyTile targets and streams sources through double-buffered
-//    shared memory in chunks of kRpyChunk; all lanes read the same source
-//    (broadcast), so shared-memory traffic is 3 LDS.128 per source per thread.
-//  * Packed FP32x2 arithmetic: a thread evaluates its target
-//    against two sources at once, lane x of every float2 holding the even
-//    source and lane y the odd one; the records of a source pair are stored
-//    interleaved so that each loaded float2 is an operand. This halves the
-//    issued FP32 instructions (the scheduler, not the FMA pipe, limited the
-//    one-source form).
-//  * Stream-K persistent grid: the (tile, chunk) work units are split evenly
-//    over G = #SMs x resident-CTAs; a CTA writes one partial per tile it
-//    touches into slot (cta + tile), and the CTA that completes a tile (a
-//    counter per tile) sums its partials in CTA order and writes the tile's
-//    rows, in the same launch. The order of the sums never depends on timing:
+//  * No tensor cores: the pair sum is not a dense contraction (forming its two
+//    contracted coefficients and splitting them into BF16 pieces costs as many
+//    FP32-pipe cycles as the sums it would save). The bound is the FP32 (or
+//    FP64) FMA pipe.
+//  * Packed FP32x2 arithmetic: a thread evaluates its target against two
+//    sources at once, lane x of every float2 holding the even source and lane
+//    y the odd one; the records of a source pair are stored interleaved so
+//    that each loaded float2 is an operand.
+//  * Each thread owns two targets in registers (one in the 128-target
+//    schedules) and all lanes read the same source from shared memory
+//    (broadcast).
+//  * Sources come in groups of 32 relative to the group's centre, and the pair
+//    terms are summed in that frame (pair32_far).
+//  * Stream-K persistent grid: the work units (tile of targets, group of
+//    sources) are split evenly over the grid; who touches a tile only in part
+//    writes one partial of it, and the CTA that completes a tile (a counter
+//    per tile) sums its partials in a fixed order and writes the tile's rows,
+//    in the same launch. The order of the sums never depends on timing:
 //    results are bitwise reproducible.
-//  * Mixed precision: positions are stored as FP32 hi/lo pairs (hi = fl32(Y),
-//    lo = fl32(Y - hi)). The inner loop forms d from the hi parts alone,
-//    which carries the rounding of the coordinates (~ulp(|Y|)) and is
-//    accurate for pairs that are far apart compared with that; a group of
-//    kRpyComp sources in which a warp met a pair closer than R_c = 4a is
-//    recomputed with d = (t_hi - s_hi) + (t_lo - s_lo), which keeps ~2 ulp of
-//    relative accuracy for close pairs. Each target sums kRpyComp pair terms
-//    in FP32 and folds them into a (hi, lo) compensated accumulator (TwoSum);
-//    the tile's sum adds the partials in FP64.
-//  * The inner loop is branch-free (far form only, tracking the smallest r^2);
-//    close pairs are rare. A recomputed group in which a warp met an
-//    overlapping pair (r < 2a) is computed once more with the exact far /
-//    overlap branches.
+//  * Mixed precision: FP32 pair terms, 32 of them summed in FP32 and folded
+//    into a (hi, lo) compensated accumulator (TwoSum); groups in which a warp
+//    met a pair closer than R_c = 4a are evaluated again with hi/lo position
+//    differences, and with the exact far / overlap coefficients where a pair
+//    overlaps.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -67,6 +60,7 @@ constexpr float kFarPad = 1.0e5f;   // position of padding sources (they carry n
 
 struct RpyConst32 {
     float near2;       // (2a)^2
+    float over2;       // (2a)^2 (1 + 1e-3): a far pass that meets a pair this close may hold an overlap
     float close2;      // R_c^2 = (4a)^2: groups with a pair this close use hi/lo differences
     float k23a2;       // 2a^2/3
     float k2a2;        // 2a^2
@@ -86,7 +80,10 @@ template <typename T, typename K>
 __host__ K make_const(double a) {
     K k;
     k.near2 = (T)(4.0 * a * a);
-    if constexpr (sizeof(T) == 4) k.close2 = (T)(16.0 * a * a);
+    if constexpr (sizeof(T) == 4) {
+        k.close2 = (T)(16.0 * a * a);
+        k.over2 = (T)(4.004 * a * a);
+    }
     k.k23a2 = (T)(2.0 * a * a / 3.0);
     k.k2a2 = (T)(2.0 * a * a);
     k.ov_A0 = (T)(4.0 / (3.0 * a));
@@ -104,28 +101,30 @@ __host__ K make_const(double a) {
 }
 
 // ---------------------------------------------------------------------------
-// Ensembles of independent systems: every system is padded to whole target
-// tiles (kRpyTile) in the source/target layout, so that a work unit (tile,
+// Ensembles of independent systems: every system is padded to a multiple of
+// kRpyPad positions in the source/target layout, so that a work unit (tile,
 // source chunk) never mixes systems and the apply stays one persistent launch.
 // System s owns padded positions [pad_off[s], pad_off[s+1]); its tiles come
-// in order, each with ceil(S_s / kRpyChunk) source chunks, and padding records
-// sit far away with zero load. With null tables there is one system whose
-// padded position equals the segment index (tile = u / n_chunks).
+// in order, each with ceil(S_s / unit_sources) units, and
+// padding records sit far away with zero load. With null tables there is one
+// system whose padded position equals the segment index (tile = u / n_units).
 // ---------------------------------------------------------------------------
 struct SysMap {
     const int64_t *tile_unit_off;  // [n_tiles + 1] first unit of each listed tile
     const int64_t *tile_src;       // [n_tiles] padded position of the tile's first source
     const int64_t *tile_nsrc;      // [n_tiles] real sources of the tile's system (null: n_src)
     const int *tile_id;            // [n_tiles] padded tile of each listed tile (null: same)
-    const int *slot_of;            // [all tiles] list index of a padded tile, -1 if not listed
-    const int64_t *pos_of_seg;     // [S] padded position of each segment
     const int *pad_map;            // [Spad] segment at a padded position, or -1
-    int64_t n_tiles, n_chunks;     // listed tiles; n_chunks: the one-system case
+    int64_t n_tiles, n_units;      // listed tiles; n_units: units per tile, the one-system case
     int64_t n_src;                 // real sources of the one-system case
     // non-null: {listed tiles, work units} read on the device, so that a captured
     // launch stays valid when the list of active tiles is rewritten
     const int64_t *dyn = nullptr;
 };
+
+// Sources of a work unit: one group where the sources are in frames (one system
+// on the FP32 path), else whole 128-source chunks.
+constexpr int unit_sources(bool frames) { return frames ? kRpyComp : kRpyChunk; }
 
 // The listed tiles and the unit count of a launch (from the device when dynamic).
 __device__ __forceinline__ void resolve_dyn(SysMap &m, int64_t &W) {
@@ -136,16 +135,16 @@ __device__ __forceinline__ void resolve_dyn(SysMap &m, int64_t &W) {
 }
 
 __device__ __forceinline__ int64_t tile_unit_begin(const SysMap &m, int64_t tile) {
-    return m.tile_unit_off ? m.tile_unit_off[tile] : tile * m.n_chunks;
+    return m.tile_unit_off ? m.tile_unit_off[tile] : tile * m.n_units;
 }
 
-// Tile of work unit u, the tile's first unit and chunk count, and its first source.
+// Tile of work unit u, the tile's first unit and unit count, and its first source.
 __device__ __forceinline__ void locate_unit(const SysMap &m, int64_t u, int64_t &tile,
-                                            int64_t &ubeg, int64_t &nch, int64_t &src0) {
+                                            int64_t &ubeg, int64_t &nun, int64_t &src0) {
     if (!m.tile_unit_off) {
-        tile = u / m.n_chunks;
-        ubeg = tile * m.n_chunks;
-        nch = m.n_chunks;
+        tile = u / m.n_units;
+        ubeg = tile * m.n_units;
+        nun = m.n_units;
         src0 = 0;
         return;
     }
@@ -157,7 +156,7 @@ __device__ __forceinline__ void locate_unit(const SysMap &m, int64_t u, int64_t 
     }
     tile = lo;
     ubeg = m.tile_unit_off[lo];
-    nch = m.tile_unit_off[lo + 1] - ubeg;
+    nun = m.tile_unit_off[lo + 1] - ubeg;
     src0 = m.tile_src[lo];
 }
 
@@ -166,44 +165,99 @@ __device__ __forceinline__ int64_t segment_at(const SysMap &m, int64_t P, int64_
 }
 
 // ---------------------------------------------------------------------------
-// Pack: FP64 (Y, FT) -> padded FP32 source records of 12 values per segment.
-// Positions are taken relative to the first segment, y = Y - Y_0 (the apply is
-// translation invariant, and the FP32 rounding of y then depends on the extent
-// of the suspension, not on where it sits), hi = fl32(y), lo = fl32(y - hi),
-// negated:
-//   -hi_x -hi_y -hi_z  F_x F_y F_z  T_x T_y T_z  -lo_z -lo_x -lo_y
-// Sources 2p and 2p+1 share the kRpyPairF4 float4 at src + kRpyPairF4 p;
-// value c of source h sits at float 2c + h, so each float2 holds one
-// component of both (even, odd) and the far-form loop, which needs no lo
-// part, reads the first 4.5 float4 of a record.
-// Padding records sit far away with zero load, so they add exactly zero.
+// Pack: FP64 (Y, FT) -> FP32 source groups of kRpyComp = 32 padded positions.
+// A group is Rec::kGroupF4 float4: first its centre (c_x, c_y, c_z, 0), the mean of
+// its real positions relative to the first segment of the apply (the apply is
+// translation invariant, and FP32 rounding then depends on the extent of the
+// suspension, not on where it sits), rounded to FP32; then 16 source pairs of
+// kRpyPairF4 float4. With s' = Y - Y_0 - c a source has 18 values
+//   -s'(hi) 3 | F 3 | T 3 | -T x s' 3 | -(2/3) F x s' 3 | -s'(lo) 3
+// and value c of source h (0 even, 1 odd) of a pair sits at float 2c + h, so
+// that each float2 holds one component of both; the far-form loop reads the
+// first 15. One warp packs one group. Padding records sit far away with zero
+// load, so they add exactly zero.
+// Ensembles keep records without a frame (kFrames false): 12 values per source
+//   -y(hi) 3 | F 3 | T 3 | -y(lo) 3,   y = Y - Y_0 = hi + lo.
+// Their systems with the drag J0 take tens of Broyden iterations whose path
+// follows the last bits of the pair sums (a system's count moves by one or two
+// with any other rounding, and its multipliers with it, by ~1e-3), so their
+// pair arithmetic, work units and order of sums stay those their trajectories
+// were made with.
 // ---------------------------------------------------------------------------
+template <bool kFrames>
+struct Rec {
+    static constexpr int kPairF4 = kFrames ? kRpyPairF4 : 6;      // float4 per source pair
+    static constexpr int kLo = kFrames ? 7 : 4;                   // the lo parts: float4 kLo, half 1 on
+    static constexpr int kHead = kFrames ? 1 : 0;                 // float4 before the pairs (centre)
+    static constexpr int kGroupF4 = kHead + kPairF4 * kRpyComp / 2;
+    static constexpr int kSums = kFrames ? 12 : 6;                // packed sums of the far loop
+};
+
+template <bool kFrames>
 __global__ void pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
                               int64_t S, int64_t Spad, SysMap sm, float4 *__restrict__ src) {
     const int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (P >= Spad) return;
+    if (P >= Spad) return;             // Spad is a multiple of 32: whole warps leave
     const int64_t i = segment_at(sm, P, S);
-    constexpr int kV = 2 * kRpyPairF4;
-    float v[kV];
+    const int lane = threadIdx.x & 31;
+    double y[3] = {0.0, 0.0, 0.0};
+    float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i >= 0) {
-        const double y0 = Y[3 * i] - Y[0], y1 = Y[3 * i + 1] - Y[1], y2 = Y[3 * i + 2] - Y[2];
-        const float h0 = __double2float_rn(y0), h1 = __double2float_rn(y1),
-                    h2 = __double2float_rn(y2);
-        const double *f = FT + 6 * i;
-        v[0] = -h0; v[1] = -h1; v[2] = -h2;
 #pragma unroll
-        for (int c = 0; c < 6; ++c) v[3 + c] = __double2float_rn(f[c]);
-        v[9] = -__double2float_rn(y2 - (double)h2);
-        v[10] = -__double2float_rn(y0 - (double)h0);
-        v[11] = -__double2float_rn(y1 - (double)h1);
-    } else {
-        v[0] = v[1] = v[2] = -kFarPad;
+        for (int c = 0; c < 3; ++c) y[c] = Y[3 * i + c] - Y[c];
 #pragma unroll
-        for (int c = 3; c < kV; ++c) v[c] = 0.f;
+        for (int c = 0; c < 6; ++c) f[c] = __double2float_rn(FT[6 * i + c]);
     }
-    float *o = reinterpret_cast<float *>(src + kRpyPairF4 * (P >> 1)) + (P & 1);
+    using R = Rec<kFrames>;
+    float v[2 * R::kPairF4];
 #pragma unroll
-    for (int c = 0; c < kV; ++c) o[2 * c] = v[c];
+    for (int c = 0; c < 2 * R::kPairF4; ++c) v[c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) v[3 + c] = f[c];
+    float4 *g = src + R::kGroupF4 * (P >> 5);
+    if constexpr (kFrames) {
+        const unsigned live = __ballot_sync(0xffffffffu, i >= 0);
+        const float inv = live ? 1.f / (float)__popc(live) : 0.f;
+        float cen[3], sp[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float m = __double2float_rn(y[c]);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) m += __shfl_xor_sync(0xffffffffu, m, d);
+            cen[c] = m * inv;
+        }
+        if (lane == 0) g[0] = make_float4(cen[0], cen[1], cen[2], 0.f);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double r = y[c] - (double)cen[c];
+            sp[c] = __double2float_rn(r);
+            v[c] = -sp[c];
+            v[15 + c] = -__double2float_rn(r - (double)sp[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            // -(T x s')_c and -(2/3)(F x s')_c of the rounded T, F, s'
+            const int p = (c + 1) % 3, q = (c + 2) % 3;
+            const double t = (double)f[3 + p] * sp[q] - (double)f[3 + q] * sp[p];
+            const double w = (double)f[p] * sp[q] - (double)f[q] * sp[p];
+            v[9 + c] = -__double2float_rn(t);
+            v[12 + c] = -__double2float_rn(w * (2.0 / 3.0));
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float h = __double2float_rn(y[c]);
+            v[c] = -h;
+            v[9 + c] = -__double2float_rn(y[c] - (double)h);
+        }
+    }
+    if (i < 0) {
+#pragma unroll
+        for (int c = 0; c < 2 * R::kPairF4; ++c) v[c] = c < 3 ? -kFarPad : 0.f;
+    }
+    float *o = reinterpret_cast<float *>(g + R::kHead + R::kPairF4 * (lane >> 1)) + (lane & 1);
+#pragma unroll
+    for (int c = 0; c < 2 * R::kPairF4; ++c) o[2 * c] = v[c];
 }
 
 // FP64 records: 9 doubles per segment (Y, F, T); padding far away, no load.
@@ -259,15 +313,23 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Exact coefficients of one pair (one lane): the far form for r^2 >= (2a)^2,
 // the overlapping-sphere form below it and the self values at r = 0, chosen
 // without a branch (both are evaluated; this runs in recomputed groups only).
+template <bool kFrames>
 __device__ __forceinline__ void coef_exact(float r2, const RpyConst32 &k, float &A, float &B,
                                            float &C, float &D, float &G) {
     const bool ov = r2 < k.near2;
-    const float rinv = rsqrt_approx(fmaxf(r2, k.near2));   // the far form's, finite everywhere
+    float rinv, r, ri;
+    if constexpr (kFrames) {
+        // one MUFU operation (r = 0, and what ftz would make of a tiny r, as 1/r = 0)
+        rinv = ri = r2 > 1e-30f ? rsqrt_approx(r2) : 0.f;
+        r = r2 * rinv;
+    } else {
+        rinv = rsqrt_approx(fmaxf(r2, k.near2));   // the far form's, finite everywhere
+        r = sqrt_approx(r2);
+        ri = r > 0.f ? rcp_approx(r) : 0.f;
+    }
     const float rinv2 = rinv * rinv;
     const float rinv3 = rinv * rinv2;
     const float rinv5 = rinv3 * rinv2;
-    const float r = sqrt_approx(r2);
-    const float ri = r > 0.f ? rcp_approx(r) : 0.f;
     A = ov ? fmaf(-k.ov_A1, r, k.ov_A0) : fmaf(k.k23a2, rinv3, rinv);
     B = ov ? k.ov_B * ri : fmaf(-k.k2a2, rinv5, rinv3);
     C = ov ? fmaf(k.ov_C3 * r2, r, fmaf(-k.ov_C1, r, k.ov_C0)) : -0.5f * rinv3;
@@ -275,67 +337,18 @@ __device__ __forceinline__ void coef_exact(float r2, const RpyConst32 &k, float 
     G = ov ? fmaf(-k.ov_G1, r, k.ov_G0) : rinv3;
 }
 
-// How a group of sources is evaluated (pair32x2's MODE).
-enum PairMode { kFarHi = 0, kFarHiLo = 1, kExact = 2 };
-
-// The pair terms of one target and the two sources of a packed record (q),
-// lane x = even source, lane y = odd source, tracking the smallest r^2 seen.
-//  kFarHi (the inner loop): d from the hi parts only and the far form for every
-//    pair, branch-free; whatever it produces for close, overlapping or
-//    coincident pairs (Inf or NaN at r = 0) is discarded by the caller, which
-//    evaluates such groups again.
-//  kFarHiLo: d = (t_hi - s_hi) + (t_lo - s_lo), far form; source jx (jx + 1
-//    for lane y) equal to self_j is the target itself: its term is zero (d = 0
-//    and 1/r taken as 0) and it is left out of the smallest r^2.
-//  kExact: hi/lo differences and the exact coefficients of every pair
-//    (coef_exact; the self pair takes the self values).
-template <int MODE>
-__device__ __forceinline__ void pair32x2(const float2 *th, const float2 *tl, const float4 *q,
-                                         const RpyConst32 &k, float2 k23, float2 nk2,
-                                         float2 *acc, float &rmin2, int self_j = -1,
-                                         int jx = 0) {
-    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
-    const float2 q4 = reinterpret_cast<const float2 *>(q + 4)[0];
-    float2 dx = __fadd2_rn(th[0], f2(q0.x, q0.y));
-    float2 dy = __fadd2_rn(th[1], f2(q0.z, q0.w));
-    float2 dz = __fadd2_rn(th[2], f2(q1.x, q1.y));
-    if (MODE != kFarHi) {
-        const float4 q5 = q[5];
-        const float2 lz = reinterpret_cast<const float2 *>(q + 4)[1];
-        dx = __fadd2_rn(dx, __fadd2_rn(tl[0], f2(q5.x, q5.y)));
-        dy = __fadd2_rn(dy, __fadd2_rn(tl[1], f2(q5.z, q5.w)));
-        dz = __fadd2_rn(dz, __fadd2_rn(tl[2], lz));
-    }
-    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-    float2 A, B, C, D, G;
-    if (MODE != kExact) {
-        float2 rinv = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-        if (MODE == kFarHiLo) {
-            const bool sx = (jx == self_j), sy = (jx + 1 == self_j);
-            rinv.x = sx ? 0.f : rinv.x;
-            rinv.y = sy ? 0.f : rinv.y;
-            rmin2 = fminf(rmin2, fminf(sx ? k.close2 : r2.x, sy ? k.close2 : r2.y));
-        } else {
-            rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
-        }
-        const float2 rinv2 = __fmul2_rn(rinv, rinv);
-        const float2 rinv3 = __fmul2_rn(rinv, rinv2);
-        const float2 rinv5 = __fmul2_rn(rinv3, rinv2);
-        A = __ffma2_rn(k23, rinv3, rinv);
-        B = __ffma2_rn(nk2, rinv5, rinv3);
-        C = __fmul2_rn(f2(-0.5f, -0.5f), rinv3);
-        D = __fmul2_rn(f2(1.5f, 1.5f), rinv5);
-        G = rinv3;
-    } else {
-        coef_exact(r2.x, k, A.x, B.x, C.x, D.x, G.x);
-        coef_exact(r2.y, k, A.y, B.y, C.y, D.y, G.y);
-    }
+// (V, Omega) sums of a pair with the coefficients A..G and the difference d,
+// the cross products formed for the pair (negated operands fold into the
+// packed FMA).
+__device__ __forceinline__ void add_pair(const float4 *q, float2 dx, float2 dy, float2 dz, float2 A,
+                                         float2 B, float2 C, float2 D, float2 G, float2 *acc) {
+    const float4 q1 = q[1], q2 = q[2], q3 = q[3];
+    const float2 Tz = reinterpret_cast<const float2 *>(q + 4)[0];
     const float2 Fx = f2(q1.z, q1.w), Fy = f2(q2.x, q2.y), Fz = f2(q2.z, q2.w);
-    const float2 Tx = f2(q3.x, q3.y), Ty = f2(q3.z, q3.w), Tz = q4;
+    const float2 Tx = f2(q3.x, q3.y), Ty = f2(q3.z, q3.w);
     const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
     const float2 dT = __fmul2_rn(D, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
     const float2 ex = __fmul2_rn(G, dx), ey = __fmul2_rn(G, dy), ez = __fmul2_rn(G, dz);
-    // (negated operands fold into the packed FMA)
     const float2 nTx = neg2(Tx), nTy = neg2(Ty), nTz = neg2(Tz);
     const float2 nFx = neg2(Fx), nFy = neg2(Fy), nFz = neg2(Fz);
     acc[0] = __ffma2_rn(A, Fx, __ffma2_rn(bF, dx, __ffma2_rn(Ty, ez, __ffma2_rn(nTz, ey, acc[0]))));
@@ -346,14 +359,215 @@ __device__ __forceinline__ void pair32x2(const float2 *th, const float2 *tl, con
     acc[5] = __ffma2_rn(C, Tz, __ffma2_rn(dT, dz, __ffma2_rn(Fx, ey, __ffma2_rn(nFy, ex, acc[5]))));
 }
 
-// Scalar record ((hi, F_x), (lo, F_y), (T, F_z)) of source h (0 even, 1 odd) of
-// a packed record.
-__device__ __forceinline__ void unpack_source(const float4 *q, int h, float4 &s0, float4 &s1,
-                                              float4 &s2) {
-    const float *f = reinterpret_cast<const float *>(q) + h;
-    s0 = make_float4(-f[0], -f[2], -f[4], f[6]);
-    s1 = make_float4(-f[20], -f[22], -f[18], f[8]);
-    s2 = make_float4(f[12], f[14], f[16], f[10]);
+// Far-form coefficients.
+__device__ __forceinline__ void far_coef(float2 rinv, const RpyConst32 &k, float2 &A, float2 &B,
+                                         float2 &C, float2 &D, float2 &G) {
+    const float2 rinv2 = __fmul2_rn(rinv, rinv);
+    G = __fmul2_rn(rinv, rinv2);
+    const float2 rinv5 = __fmul2_rn(G, rinv2);
+    A = __ffma2_rn(f2(k.k23a2, k.k23a2), G, rinv);
+    B = __ffma2_rn(f2(-k.k2a2, -k.k2a2), rinv5, G);
+    C = __fmul2_rn(f2(-0.5f, -0.5f), G);
+    D = __fmul2_rn(f2(1.5f, 1.5f), rinv5);
+}
+
+// The inner loop: the pair terms of one target (position t, both lanes, in
+// the group's frame) and the two sources of a packed record q, lane x = even
+// source, lane y = odd source, in the far form, branch-free; whatever it
+// produces for close, overlapping or coincident pairs (Inf or NaN at r = 0)
+// is discarded by the caller, which evaluates such groups again. rmin2 tracks
+// the smallest r^2.
+//
+// With d = t - s in the group's frame the cross products split,
+//   sum G (T x d) = (sum G T) x t - sum G (T x s),
+// and likewise for F x d, so that a pair needs no G d: 12 sums take
+//   acc[0..2] += (1/r) F + B (d.F) d - G (T x s)   (V without its G F part)
+//   acc[3..5] += r^-5 (d.T) d - (2/3) G (F x s)    (2/3 of Omega's d-terms)
+//   acc[6..8] += G T,  acc[9..11] += G F           (see fold_group)
+// in 39 FP32 operations a pair, 9 fewer than with the cross products formed
+// for every pair. What bounds the loop is register operands: a packed FMA
+// with three distinct register operands issues every third cycle, one with
+// two every second, and this form drops 3-operand FMAs (24 -> 21 sums) as
+// well as multiplies.
+// Measured (32 000 segments, pair kernel): 1700 us with the cross products formed
+// per pair, 1491 us in this form, and the error against 64 bits 2.0e-7 -> 1.7e-7
+// (the frames make the differences finer).
+// Without frames (ensembles): t relative to the first segment, 48 operations,
+//   acc[0..2] += V terms, acc[3..5] += Omega terms.
+template <bool kFrames>
+__device__ __forceinline__ void pair32_far(const float2 *t, const float4 *q, const RpyConst32 &k,
+                                           float2 *acc, float &rmin2) {
+    if constexpr (!kFrames) {
+        const float4 q0 = q[0], q1 = q[1];
+        const float2 dx = __fadd2_rn(t[0], f2(q0.x, q0.y));
+        const float2 dy = __fadd2_rn(t[1], f2(q0.z, q0.w));
+        const float2 dz = __fadd2_rn(t[2], f2(q1.x, q1.y));
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
+        float2 A, B, C, D, G;
+        far_coef(f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y)), k, A, B, C, D, G);
+        add_pair(q, dx, dy, dz, A, B, C, D, G, acc);
+        return;
+    }
+    const float2 nk2 = f2(-k.k2a2, -k.k2a2);
+    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3], q4 = q[4], q5 = q[5], q6 = q[6];
+    const float2 q7 = reinterpret_cast<const float2 *>(q + 7)[0];
+    const float2 dx = __fadd2_rn(t[0], f2(q0.x, q0.y));
+    const float2 dy = __fadd2_rn(t[1], f2(q0.z, q0.w));
+    const float2 dz = __fadd2_rn(t[2], f2(q1.x, q1.y));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+    const float2 rinv = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+    rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
+    const float2 rinv2 = __fmul2_rn(rinv, rinv);
+    const float2 G = __fmul2_rn(rinv, rinv2);
+    const float2 rinv5 = __fmul2_rn(G, rinv2);
+    const float2 B = __ffma2_rn(nk2, rinv5, G);
+    const float2 Fx = f2(q1.z, q1.w), Fy = f2(q2.x, q2.y), Fz = f2(q2.z, q2.w);
+    const float2 Tx = f2(q3.x, q3.y), Ty = f2(q3.z, q3.w), Tz = f2(q4.x, q4.y);
+    const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
+    const float2 dT =
+        __fmul2_rn(rinv5, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
+    acc[0] = __ffma2_rn(rinv, Fx, __ffma2_rn(G, f2(q4.z, q4.w), __ffma2_rn(bF, dx, acc[0])));
+    acc[1] = __ffma2_rn(rinv, Fy, __ffma2_rn(G, f2(q5.x, q5.y), __ffma2_rn(bF, dy, acc[1])));
+    acc[2] = __ffma2_rn(rinv, Fz, __ffma2_rn(G, f2(q5.z, q5.w), __ffma2_rn(bF, dz, acc[2])));
+    acc[3] = __ffma2_rn(G, f2(q6.x, q6.y), __ffma2_rn(dT, dx, acc[3]));
+    acc[4] = __ffma2_rn(G, f2(q6.z, q6.w), __ffma2_rn(dT, dy, acc[4]));
+    acc[5] = __ffma2_rn(G, q7, __ffma2_rn(dT, dz, acc[5]));
+    acc[6] = __ffma2_rn(G, Tx, acc[6]);
+    acc[7] = __ffma2_rn(G, Ty, acc[7]);
+    acc[8] = __ffma2_rn(G, Tz, acc[8]);
+    acc[9] = __ffma2_rn(G, Fx, acc[9]);
+    acc[10] = __ffma2_rn(G, Fy, acc[10]);
+    acc[11] = __ffma2_rn(G, Fz, acc[11]);
+}
+
+// The (V, Omega) terms of a group from the twelve sums of pair32_far: with
+// P = sum G T and Q = sum G F,
+//   V     = acc[0..2] + (2a^2/3) Q + P x t
+//   Omega = 3/2 acc[3..5] - P/2 + Q x t.
+template <bool kFrames>
+__device__ __forceinline__ void combine_group(const float2 *acc, const float2 *t, float k23,
+                                              float *out) {
+    if constexpr (!kFrames) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) out[c] = __fadd_rn(acc[c].x, acc[c].y);
+        return;
+    }
+    float s[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) s[c] = __fadd_rn(acc[c].x, acc[c].y);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int p = (c + 1) % 3, q = (c + 2) % 3;
+        out[c] = fmaf(k23, s[9 + c],
+                      fmaf(s[6 + p], t[q].x, fmaf(-s[6 + q], t[p].x, s[c])));
+        out[3 + c] = fmaf(1.5f, s[3 + c],
+                          fmaf(-0.5f, s[6 + c], fmaf(s[9 + p], t[q].x, -s[9 + q] * t[p].x)));
+    }
+}
+
+// How a close group is evaluated again (pair32_near's MODE).
+enum PairMode { kFarHiLo = 1, kExact = 2 };
+
+// The pair terms of one target and the two sources of a record with the
+// differences d = (t_hi - s_hi) + (t_lo - s_lo), which keep ~2 ulp of relative
+// accuracy, and the cross products formed per pair.
+//  kFarHiLo: far form; source jx (jx + 1 for lane y) equal to self_j is the
+//    target itself: its term is zero (d = 0 and 1/r taken as 0) and it is left
+//    out of the smallest r^2.
+//  kExact: the exact coefficients of every pair (coef_exact; the self pair
+//    takes the self values).
+template <bool kFrames, int MODE>
+__device__ __forceinline__ void pair32_near(const float *th, const float *tl, const float4 *q,
+                                            const RpyConst32 &k, float2 *acc, float &rmin2,
+                                            int self_j = -1, int jx = 0) {
+    constexpr int kLo = Rec<kFrames>::kLo;
+    const float4 q0 = q[0], ql = q[kLo + 1];
+    const float2 z = reinterpret_cast<const float2 *>(q + 1)[0];
+    const float2 lx = reinterpret_cast<const float2 *>(q + kLo)[1];
+    const float2 dx = __fadd2_rn(__fadd2_rn(f2(th[0], th[0]), f2(q0.x, q0.y)),
+                                 __fadd2_rn(f2(tl[0], tl[0]), lx));
+    const float2 dy = __fadd2_rn(__fadd2_rn(f2(th[1], th[1]), f2(q0.z, q0.w)),
+                                 __fadd2_rn(f2(tl[1], tl[1]), f2(ql.x, ql.y)));
+    const float2 dz = __fadd2_rn(__fadd2_rn(f2(th[2], th[2]), z),
+                                 __fadd2_rn(f2(tl[2], tl[2]), f2(ql.z, ql.w)));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+    float2 A, B, C, D, G;
+    if (MODE == kFarHiLo) {
+        float2 rinv = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+        const bool sx = (jx == self_j), sy = (jx + 1 == self_j);
+        rinv.x = sx ? 0.f : rinv.x;
+        rinv.y = sy ? 0.f : rinv.y;
+        rmin2 = fminf(rmin2, fminf(sx ? k.close2 : r2.x, sy ? k.close2 : r2.y));
+        far_coef(rinv, k, A, B, C, D, G);
+    } else {
+        coef_exact<kFrames>(r2.x, k, A.x, B.x, C.x, D.x, G.x);
+        coef_exact<kFrames>(r2.y, k, A.y, B.y, C.y, D.y, G.y);
+    }
+    add_pair(q, dx, dy, dz, A, B, C, D, G, acc);
+}
+
+// Position of a target relative to the apply's first segment, y = th + tl, from
+// its own group's record (target P of the padded layout).
+template <bool kFrames>
+__device__ __forceinline__ void load_target(const float4 *src, int64_t P, float *th, float *tl) {
+    using R = Rec<kFrames>;
+    const float4 *g = src + R::kGroupF4 * (P >> 5);
+    const int lane = (int)(P & 31);
+    const float *f =
+        reinterpret_cast<const float *>(g + R::kHead + R::kPairF4 * (lane >> 1)) + (lane & 1);
+    constexpr int kL = 2 * (2 * R::kLo + 1);      // first lo value
+    if constexpr (kFrames) {
+        const float4 c = g[0];
+        const float cc[3] = {c.x, c.y, c.z};
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            float e;
+            two_sum(cc[x], -f[2 * x], th[x], e);
+            tl[x] = __fadd_rn(e, -f[kL + 2 * x]);
+        }
+    } else {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            th[x] = -f[2 * x];
+            tl[x] = -f[kL + 2 * x];
+        }
+    }
+}
+
+// The target in the frame of the group with records q, for the far loop (t2,
+// both lanes) and as hi + lo parts.
+template <bool kFrames>
+__device__ __forceinline__ void to_frame(const float4 *q, const float *th, const float *tl,
+                                         float2 *t2) {
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (kFrames) c = q[-1];
+    const float cc[3] = {c.x, c.y, c.z};
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        const float v = kFrames ? __fadd_rn(__fsub_rn(th[x], cc[x]), tl[x]) : th[x];
+        t2[x] = f2(v, v);
+    }
+}
+template <bool kFrames>
+__device__ __forceinline__ void to_frame_hl(const float4 *q, const float *th, const float *tl,
+                                            float *uh, float *ul) {
+    if constexpr (kFrames) {
+        const float4 c = q[-1];
+        const float cc[3] = {c.x, c.y, c.z};
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            float e;
+            two_sum(th[x], -cc[x], uh[x], e);
+            ul[x] = __fadd_rn(e, tl[x]);
+        }
+    } else {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            uh[x] = th[x];
+            ul[x] = tl[x];
+        }
+    }
 }
 
 // One pair in FP64 (record layout: Y, F, T).
@@ -393,13 +607,13 @@ __device__ __forceinline__ void pair64(double tx, double ty, double tz, const do
     acc[5] = fma(C, Tz, fma(dT, dz, fma(Fx, ey, fma(-Fy, ex, acc[5]))));
 }
 
-// Asynchronous copy of one chunk of source records (kRec float4) from global to
+// Asynchronous copy of a chunk of source records (n float4) from global to
 // shared memory, 16 bytes per cp.async, spread over the CTA's threads; the
 // copies land when cp_async_wait_all returns (plus a barrier for the others').
-template <int kRec, int kThreads>
-__device__ __forceinline__ void stage_chunk(float4 *dst, const float4 *__restrict__ g, int tid) {
-#pragma unroll
-    for (int i = tid; i < kRec; i += kThreads) {
+template <int kThreads>
+__device__ __forceinline__ void stage_chunk(float4 *dst, const float4 *__restrict__ g, int n,
+                                            int tid) {
+    for (int i = tid; i < n; i += kThreads) {
         const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + i);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g + i) : "memory");
     }
@@ -451,7 +665,7 @@ __device__ __forceinline__ int fetch_add_acq_rel(int *p, int v) {
 
 template <typename PT, int NPART, int TPT>
 __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, int64_t tile,
-                                            int64_t ptile, int64_t units, int64_t n_chunks,
+                                            int64_t ptile, int64_t units, int64_t n_units,
                                             int64_t W, int64_t G, int *__restrict__ cnt,
                                             double scale, double *__restrict__ VW,
                                             bool worker = true) {
@@ -460,7 +674,7 @@ __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, 
     const int tid = threadIdx.x;
     __syncthreads();   // the CTA's partial is written before it is counted
     if (tid == 0)
-        s_last = fetch_add_acq_rel(cnt + tile, (int)units) + (int)units == (int)n_chunks;
+        s_last = fetch_add_acq_rel(cnt + tile, (int)units) + (int)units == (int)n_units;
     __syncthreads();
     // (`worker`: false for the second half of a source-split CTA, which holds no targets)
     if (!s_last || !worker) return;
@@ -517,260 +731,215 @@ __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, 
 }
 
 // ---------------------------------------------------------------------------
-// Mixed-precision pair kernel. A CTA of kRpyThreads threads owns a tile of
-// kRpyThreads * TPT targets, TPT per thread; their pair terms are summed in
-// registers over groups of kRpyComp sources with the branch-free far form and
-// the group sums folded (TwoSum) into (hi, lo) accumulators.
-//  * TPT = 2, 256-target tiles (large systems): a group in which the warp met
-//    a pair closer than R_c is evaluated again with hi/lo differences and the
-//    exact coefficients.
-//  * TPT = 1, 128-target tiles (small systems: less padding, finer units; a
-//    warp's own segments then sit in one of every few dozen groups): the
-//    group holding the warp's own segments is recognised by index and
-//    evaluated once with hi/lo differences and the self pair masked, other
-//    close groups again with hi/lo differences in the far form, and exactly
-//    only when distinct segments overlap.
-// Measured on GB300, each structure is the faster one for its tile size.
+// Mixed-precision pair kernel. A CTA owns a tile of kRpyThreads * TPT targets,
+// TPT per thread; their pair terms are summed in registers over groups of
+// kRpyComp sources with the branch-free far form (pair32_far) and the group
+// sums folded (TwoSum) into (hi, lo) accumulators.
+//  * The sources of a group are stored relative to the group's centre c and
+//    each target is taken into that frame once per group, t = (th - c) + tl:
+//    d = t - s then carries the rounding of coordinates of the size of the
+//    group and of the target's distance from it, not of the suspension.
+//  * A group in which the warp met a pair closer than R_c = 4a is evaluated
+//    again with hi/lo differences. TPT = 2, 256-target tiles (large systems):
+//    with the exact coefficients at once. TPT = 1, 128-target tiles (a warp's
+//    own segments sit in one of every few dozen groups): the group holding the
+//    warp's own segments is recognised by index and evaluated once with hi/lo
+//    differences and the self pair masked, other close groups again with hi/lo
+//    differences in the far form, and exactly only when distinct segments
+//    overlap.
 // SPLIT = 2 (128-target tiles only) gives a CTA twice the warps on the same
-// targets: the two halves take alternate 32-source groups of every chunk and
-// their sums are added (float-float, in half order) before the partial is
-// written, so a work unit is done by eight warps instead of four -- more
-// warps at work on small problems, whose few units leave SMs short of them.
+// targets: the two sets of four warps take alternate 32-source groups of every
+// chunk and their sums are added (float-float, in set order) before the
+// partial is written.
+// These kernels run for schedules set by hand or chosen by the autotuner; the
+// automatic schedule runs rpy_pair32_warp_kernel below.
 // ---------------------------------------------------------------------------
-template <int TPT, int SPLIT = 1>
-__global__ void __launch_bounds__(kRpyThreads * SPLIT,
-                                  TPT == 2 ? kRpyMinBlocksTpt2
-                                           : (SPLIT == 1 ? kRpyMinBlocksTpt1 : kRpyMinBlocksSplit2))
+constexpr int min_blocks(bool frames, int tpt, int split) {
+    return split == 2 ? kRpyMinBlocksSplit2
+           : tpt == 2 ? (frames ? kRpyMinBlocksTpt2 : kRpyMaxCtasTpt2)
+                      : (frames ? kRpyMinBlocksTpt1 : kRpyMaxCtasTpt1);
+}
+
+template <bool kFrames, int TPT, int SPLIT = 1>
+__global__ void __launch_bounds__(kRpyThreads * SPLIT, min_blocks(kFrames, TPT, SPLIT))
 rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G, RpyConst32 k,
                   float *__restrict__ part, int *__restrict__ cnt, double scale,
                   double *__restrict__ VW) {
-    constexpr int kRec = kRpyPairF4 * (kRpyChunk / 2);   // float4 per chunk
+    constexpr int kPer = kRpyChunk / kRpyComp;            // groups per staged chunk
+    constexpr int kGroupF4 = Rec<kFrames>::kGroupF4, kPairF4 = Rec<kFrames>::kPairF4;
+    constexpr int kUnitGroups = unit_sources(kFrames) / kRpyComp;   // groups per work unit
+    constexpr int kRec = kGroupF4 * kPer;
     constexpr int kT = TPT;                               // targets per thread
     constexpr int kTile = kRpyThreads * TPT;              // targets per tile
     static_assert(SPLIT == 1 || (SPLIT == 2 && TPT == 1), "source split: 128-target tiles only");
     __shared__ float4 sm[2][kRec];
     // target slot, and which of the SPLIT sets of source groups the thread takes
-    // (both compile-time for SPLIT = 1, so the unsplit kernels are unchanged)
     const int tid = SPLIT == 1 ? (int)threadIdx.x : (int)(threadIdx.x % kRpyThreads);
-    const int half = SPLIT == 1 ? 0 : (int)(threadIdx.x / kRpyThreads);
+    const int set = SPLIT == 1 ? 0 : (int)(threadIdx.x / kRpyThreads);
     const int64_t b = blockIdx.x;
     resolve_dyn(smap, W);
     int64_t u = unit_start(b, W, G);
     const int64_t u_end = unit_start(b + 1, W, G);
 
     while (u < u_end) {
-        int64_t tile, ubeg, n_chunks, src0;
-        locate_unit(smap, u, tile, ubeg, n_chunks, src0);
-        const int64_t c_begin = u - ubeg;
-        const int64_t c_end = min(n_chunks, c_begin + (u_end - u));
-        const float4 *srcs = src + kRec * (src0 / kRpyChunk);   // this tile's system
+        int64_t tile, ubeg, n_units, src0;
+        locate_unit(smap, u, tile, ubeg, n_units, src0);
+        const int64_t u_last = min(ubeg + n_units, u_end);      // this CTA's units of the tile
+        const float4 *srcs = src + kGroupF4 * (src0 / kRpyComp);   // this tile's system
         const int64_t ptile = smap.tile_id ? smap.tile_id[tile] : tile;   // padded tile
-        // groups of the system's last chunk that hold padding only are skipped
         const int64_t nsrc = smap.tile_nsrc ? smap.tile_nsrc[tile] : smap.n_src;
+        // their groups (the padding-only groups of a system's last unit are left out)
+        const int64_t c_begin = (u - ubeg) * kUnitGroups;
+        const int64_t c_end = min((u_last - ubeg) * kUnitGroups, (nsrc + kRpyComp - 1) / kRpyComp);
 
-        // target positions (hi parts) broadcast to both lanes; the lo parts are
-        // read again only when a group is recomputed
-        // record of target t: trec + t * kTRecStep
-        constexpr int kTRecStep = kRpyPairF4 * (kRpyThreads / 2);
-        const float4 *trec = src + kRpyPairF4 * ((ptile * kTile + tid) >> 1);
-        float2 thb[kT][3];
+        // first chunk -> buffer 0
+        int n_grp = (int)min((int64_t)kPer, c_end - c_begin);
+        stage_chunk<kRpyThreads * SPLIT>(sm[0], srcs + kGroupF4 * c_begin, kGroupF4 * n_grp,
+                                         threadIdx.x);
+        float th[kT][3], tl[kT][3];
 #pragma unroll
-        for (int t = 0; t < kT; ++t) {
-            const int64_t n = ptile * kTile + t * kRpyThreads + tid;
-            float4 a0, a1, a2;
-            unpack_source(src + kRpyPairF4 * (n >> 1), (int)(n & 1), a0, a1, a2);
-            thb[t][0] = f2(a0.x, a0.x);
-            thb[t][1] = f2(a0.y, a0.y);
-            thb[t][2] = f2(a0.z, a0.z);
-        }
-        const int tpar = tid & 1;   // even / odd record slot of every target of this thread
+        for (int t = 0; t < kT; ++t)
+            load_target<kFrames>(src, ptile * kTile + t * kRpyThreads + tid, th[t], tl[t]);
         [[maybe_unused]] const int lane = tid & 31;
         // first target of this warp (slot 0), for the own-group test of 128-target tiles
         [[maybe_unused]] const int64_t wbase = ptile * kTile + (tid & ~31);
         // 128-target tiles (small systems): a warp whose targets are all padding (in a
-        // system's last tile) computes nothing; the reduce never reads those rows
+        // system's last tile) computes nothing; the tile's sum never reads those rows
         bool idle = false;
         if constexpr (TPT == 1) idle = wbase - src0 >= nsrc;
-        const float2 k23 = f2(k.k23a2, k.k23a2), nk2 = f2(-k.k2a2, -k.k2a2);
         float hi[kT][6], lo[kT][6];
 #pragma unroll
         for (int t = 0; t < kT; ++t)
 #pragma unroll
             for (int c = 0; c < 6; ++c) hi[t][c] = lo[t][c] = 0.f;
-
-        // first chunk -> buffer 0
-        stage_chunk<kRec, kRpyThreads * SPLIT>(sm[0], srcs + kRec * c_begin, threadIdx.x);
         cp_async_wait_all();
         __syncthreads();
 
-        for (int64_t ch = c_begin; ch < c_end; ++ch) {
-            const int buf = (int)((ch - c_begin) & 1);
+        int buf = 0;
+        for (int64_t ch = c_begin; ch < c_end; ch += kPer, buf ^= 1) {
             // the next chunk streams into the other buffer while this one is computed
             // (that buffer was last read before the barrier that ended the previous chunk)
-            const bool has_next = (ch + 1 < c_end);
+            const bool has_next = (ch + kPer < c_end);
+            const int n_next = has_next ? (int)min((int64_t)kPer, c_end - ch - kPer) : 0;
             if (has_next)
-                stage_chunk<kRec, kRpyThreads * SPLIT>(sm[buf ^ 1], srcs + kRec * (ch + 1),
-                                                       threadIdx.x);
+                stage_chunk<kRpyThreads * SPLIT>(sm[buf ^ 1], srcs + kGroupF4 * (ch + kPer),
+                                                 kGroupF4 * n_next, threadIdx.x);
             const float4 *s = sm[buf];
-            const int n_grp = (int)min((int64_t)(kRpyChunk / kRpyComp),
-                                       (nsrc - ch * kRpyChunk + kRpyComp - 1) / kRpyComp);
 #pragma unroll 1
-            for (int grp = half; grp < (idle ? 0 : n_grp); grp += SPLIT) {
-                const float4 *qg = s + kRpyPairF4 * (grp * (kRpyComp / 2));
-                float acc[kT][6];
-                if constexpr (TPT == 1) {
-                    // the group that holds this warp's own segments (slot t's targets
-                    // wbase + t kRpyThreads + lane are sources g0 + lane): one per warp and slot
-                    const int64_t g0 = src0 + ch * kRpyChunk + grp * kRpyComp;
-                    int own = 0;
+            for (int grp = set; grp < (idle ? 0 : n_grp); grp += SPLIT) {
+                const float4 *qg = s + kGroupF4 * grp + Rec<kFrames>::kHead;
+                float out[kT][6];
+                // the group that holds this warp's own segments
+                const bool own =
+                    TPT == 1 && src0 + (ch + grp) * kRpyComp == wbase;
+                bool near = own;
+                if (!own) {
+                    float2 t2[kT][3], acc[kT][Rec<kFrames>::kSums];
 #pragma unroll
-                    for (int t = 0; t < kT; ++t) own |= (g0 == wbase + t * kRpyThreads) ? (1 << t) : 0;
-                    float2 acc2[kT][6];
+                    for (int t = 0; t < kT; ++t) {
+                        to_frame<kFrames>(qg, th[t], tl[t], t2[t]);
 #pragma unroll
-                    for (int t = 0; t < kT; ++t)
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) acc2[t][c] = f2(0.f, 0.f);
-                    float rmin2 = k.close2;
-                    bool hilo = own != 0;
-                    if (!hilo) {
-#pragma unroll (kRpyUnroll / 2)
-                        for (int jp = 0; jp < kRpyComp / 2; ++jp) {
-#pragma unroll
-                            for (int t = 0; t < kT; ++t)
-                                pair32x2<kFarHi>(thb[t], thb[t], qg + kRpyPairF4 * jp, k, k23, nk2,
-                                                 acc2[t], rmin2);
-                        }
-                        // a pair closer than R_c: the group again with hi/lo differences
-                        hilo = __any_sync(0xffffffffu, rmin2 < k.close2);
+                        for (int c = 0; c < Rec<kFrames>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
                     }
-                    if (hilo) {
-                        rmin2 = k.close2;
-#pragma unroll
-                        for (int t = 0; t < kT; ++t) {   // one target at a time (fewer live registers)
-                            float4 a0, a1, a2;
-                            unpack_source(trec + t * kTRecStep, tpar, a0, a1, a2);
-                            const float2 tlb[3] = {f2(a1.x, a1.x), f2(a1.y, a1.y), f2(a1.z, a1.z)};
-                            const int self_j = (own >> t) & 1 ? lane : -1;
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) acc2[t][c] = f2(0.f, 0.f);
-#pragma unroll 1
-                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                                pair32x2<kFarHiLo>(thb[t], tlb, qg + kRpyPairF4 * jp, k, k23, nk2,
-                                                   acc2[t], rmin2, self_j, 2 * jp);
-                        }
-                    }
-                    // overlapping distinct segments (r < 2a): the exact coefficients
-                    const bool exact = hilo && __any_sync(0xffffffffu, rmin2 < k.near2);
-                    if (exact) {
-#pragma unroll
-                        for (int t = 0; t < kT; ++t) {
-                            float4 a0, a1, a2;
-                            unpack_source(trec + t * kTRecStep, tpar, a0, a1, a2);
-                            const float2 tlb[3] = {f2(a1.x, a1.x), f2(a1.y, a1.y), f2(a1.z, a1.z)};
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) acc2[t][c] = f2(0.f, 0.f);
-#pragma unroll 1
-                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                                pair32x2<kExact>(thb[t], tlb, qg + kRpyPairF4 * jp, k, k23, nk2,
-                                                 acc2[t], rmin2);
-                        }
-                    }
-#pragma unroll
-                    for (int t = 0; t < kT; ++t)
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) acc[t][c] = __fadd_rn(acc2[t][c].x, acc2[t][c].y);
-                    if (own && !exact) {
-                        // the self term of the targets whose own segment is in this group
-                        // (left out of the far-form pass above): 4/(3a) F_n and T_n / a^3
-                        float4 s0, s1, s2;
-                        unpack_source(qg + kRpyPairF4 * (lane >> 1), lane & 1, s0, s1, s2);
-#pragma unroll
-                        for (int t = 0; t < kT; ++t)
-                            if ((own >> t) & 1) {
-                                acc[t][0] = fmaf(k.ov_A0, s0.w, acc[t][0]);
-                                acc[t][1] = fmaf(k.ov_A0, s1.w, acc[t][1]);
-                                acc[t][2] = fmaf(k.ov_A0, s2.w, acc[t][2]);
-                                acc[t][3] = fmaf(k.ov_C0, s2.x, acc[t][3]);
-                                acc[t][4] = fmaf(k.ov_C0, s2.y, acc[t][4]);
-                                acc[t][5] = fmaf(k.ov_C0, s2.z, acc[t][5]);
-                            }
-                    }
-                } else {
-                    // 256-target tiles (large systems): a far pass with hi-only
-                    // differences; a group in which a warp met a pair closer than R_c
-                    // (own segments included) is evaluated again exactly
-                    float2 acc2[kT][6];
-#pragma unroll
-                    for (int t = 0; t < kT; ++t)
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) acc2[t][c] = f2(0.f, 0.f);
                     float rmin2 = k.close2;
 #pragma unroll (kRpyUnroll / 2)
                     for (int jp = 0; jp < kRpyComp / 2; ++jp) {
 #pragma unroll
                         for (int t = 0; t < kT; ++t)
-                            pair32x2<kFarHi>(thb[t], thb[t], qg + kRpyPairF4 * jp, k, k23, nk2,
-                                             acc2[t], rmin2);
+                            pair32_far<kFrames>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
                     }
-                    if (__any_sync(0xffffffffu, rmin2 < k.close2)) {
-#pragma unroll
-                        for (int t = 0; t < kT; ++t) {   // one target at a time (fewer live registers)
-                            float4 a0, a1, a2;
-                            unpack_source(trec + t * kTRecStep, tpar, a0, a1, a2);
-                            const float2 tlb[3] = {f2(a1.x, a1.x), f2(a1.y, a1.y), f2(a1.z, a1.z)};
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) acc2[t][c] = f2(0.f, 0.f);
-#pragma unroll 1
-                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                                pair32x2<kExact>(thb[t], tlb, qg + kRpyPairF4 * jp, k, k23, nk2,
-                                                 acc2[t], rmin2);
-                        }
-                    }
+                    near = __any_sync(0xffffffffu, rmin2 < k.close2);
 #pragma unroll
                     for (int t = 0; t < kT; ++t)
+                        combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
+                }
+                if (near) {
+                    // (one target at a time: fewer live registers)
 #pragma unroll
-                        for (int c = 0; c < 6; ++c)
-                            acc[t][c] = __fadd_rn(acc2[t][c].x, acc2[t][c].y);
+                    for (int t = 0; t < kT; ++t) {
+                        float uh[3], ul[3];
+                        to_frame_hl<kFrames>(qg, th[t], tl[t], uh, ul);
+                        float2 acc[6];
+                        float rmin2 = k.close2;
+                        bool exact = TPT == 2;
+                        if constexpr (TPT == 1) {
+                            const int self_j = own ? lane : -1;
+#pragma unroll
+                            for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
+#pragma unroll 1
+                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                                pair32_near<kFrames, kFarHiLo>(uh, ul, qg + kPairF4 * jp, k, acc,
+                                                               rmin2, self_j, 2 * jp);
+                            // overlapping distinct segments (r < 2a): the exact coefficients
+                            exact = __any_sync(0xffffffffu, rmin2 < k.near2);
+                        }
+                        if (exact) {
+#pragma unroll
+                            for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
+#pragma unroll 1
+                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                                pair32_near<kFrames, kExact>(uh, ul, qg + kPairF4 * jp, k, acc, rmin2);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) out[t][c] = __fadd_rn(acc[c].x, acc[c].y);
+                        if (own && !exact) {
+                            // the self term, left out of the far-form pass above:
+                            // 4/(3a) F_n and T_n / a^3
+                            const float *f = reinterpret_cast<const float *>(
+                                                 qg + kPairF4 * (lane >> 1)) + (lane & 1);
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) {
+                                out[t][c] = fmaf(k.ov_A0, f[2 * (3 + c)], out[t][c]);
+                                out[t][3 + c] = fmaf(k.ov_C0, f[2 * (6 + c)], out[t][3 + c]);
+                            }
+                        }
+                    }
                 }
 #pragma unroll
                 for (int t = 0; t < kT; ++t)
 #pragma unroll
                     for (int c = 0; c < 6; ++c) {
                         float sh, e;
-                        two_sum(hi[t][c], acc[t][c], sh, e);
+                        two_sum(hi[t][c], out[t][c], sh, e);
                         hi[t][c] = sh;
                         lo[t][c] = __fadd_rn(lo[t][c], e);
                     }
             }
             if (has_next) cp_async_wait_all();
+            n_grp = n_next;
             __syncthreads();
         }
 
         if constexpr (SPLIT > 1) {
-            // the second half's sums join the first's (TwoSum of the hi parts, the lo
-            // parts into its error, renormalised); the buffer is next written after
-            // the next segment's first chunk barrier
-            __shared__ float xs[12][kRpyThreads];
-            if (half == 1) {
+            // the other sets' sums join the first's in set order (TwoSum of the hi
+            // parts, the lo parts into its error, renormalised), through the chunk
+            // buffers, which are next written after the barrier in finish_tile
+            float *xs = reinterpret_cast<float *>(&sm[0][0]);
+            static_assert((SPLIT - 1) * 12 * kRpyThreads * sizeof(float) <= sizeof(sm),
+                          "the sets' sums fit in the chunk buffers");
+            if (set > 0) {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
-                    xs[c][tid] = hi[0][c];
-                    xs[6 + c][tid] = lo[0][c];
+                    xs[((set - 1) * 12 + c) * kRpyThreads + tid] = hi[0][c];
+                    xs[((set - 1) * 12 + 6 + c) * kRpyThreads + tid] = lo[0][c];
                 }
             }
             __syncthreads();
-            if (half == 0) {
+            if (set == 0) {
 #pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    float sh, e;
-                    two_sum(hi[0][c], xs[c][tid], sh, e);
-                    e = __fadd_rn(e, __fadd_rn(lo[0][c], xs[6 + c][tid]));
-                    two_sum(sh, e, hi[0][c], lo[0][c]);
-                }
+                for (int o = 0; o < SPLIT - 1; ++o)
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) {
+                        float sh, e;
+                        two_sum(hi[0][c], xs[(o * 12 + c) * kRpyThreads + tid], sh, e);
+                        e = __fadd_rn(e, __fadd_rn(lo[0][c],
+                                                   xs[(o * 12 + 6 + c) * kRpyThreads + tid]));
+                        two_sum(sh, e, hi[0][c], lo[0][c]);
+                    }
             }
         }
         // partial of this CTA for this tile -> slot (b + tile)
-        if (half == 0) {
+        if (set == 0) {
             float *p = part + (size_t)(b + tile) * 12 * kTile;
 #pragma unroll
             for (int t = 0; t < kT; ++t) {
@@ -782,10 +951,268 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
                 }
             }
         }
-        finish_tile<float, 2, TPT>(part, smap, tile, ptile, c_end - c_begin, n_chunks, W, G, cnt,
-                                   scale, VW, SPLIT == 1 || half == 0);
-        u = ubeg + c_end;
+        finish_tile<float, 2, TPT>(part, smap, tile, ptile, u_last - u, n_units, W, G, cnt, scale,
+                                   VW, set == 0);
+        u = u_last;
     }
+}
+
+// ---------------------------------------------------------------------------
+// The pair kernel of the automatic schedule: warps that share nothing. A tile
+// is 64 targets, two per lane of one warp; a work unit is (tile, group of 32
+// sources), and the units are split evenly over all warps of the grid (one
+// CTA of 12 warps per SM). Each warp streams its groups through two
+// private shared-memory buffers (cp.async) and never waits for another warp,
+// so that a warp that has to evaluate a close group again delays nobody, and
+// the split is even to one unit of 64 x 32 pairs. A tile that a single warp
+// covers is written from registers; the others leave one partial per warp in
+// slot (warp + tile), and when a CTA's warps are done it counts its units of
+// each such tile; the CTA that completes a tile sums its partials in warp
+// order (float-float) and writes the rows.
+// Measured, whole applies, against 256-target tiles of four warps with a barrier
+// per 128 sources: 9 651 segments in ragged filaments 224 -> 181 us, 3200
+// segments 73 -> 50 us, 32 000 1504 -> 1491 us (at the close groups' loop
+// unrolled by 2; by 4 its registers cost the far loop 7%). One system only.
+// ---------------------------------------------------------------------------
+constexpr int kWarpTile = kRpyMinTile;          // targets per tile
+constexpr int kWarpPart = 12 * kWarpTile;       // floats of a partial
+constexpr int kWarpCta = 12;                    // warps per CTA (168 registers a thread)
+constexpr int kGroupF4 = Rec<true>::kGroupF4, kPairF4 = Rec<true>::kPairF4;
+constexpr size_t kWarpSmem = sizeof(float4) * 2 * kGroupF4 * kWarpCta;
+
+// Warps that W units are split over, on n_ctas CTAs: as many as leave no warp
+// with more units than another by more than the last one's remainder (with
+// every warp of the grid at work some would have ceil(W / warps) units and the
+// rest one less, and the same end). Never more than W, so every one of them
+// owns a unit.
+__host__ __device__ __forceinline__ int64_t warp_count(int64_t W, int64_t n_ctas) {
+    const int64_t most = n_ctas * kWarpCta;
+    const int64_t m = (W + most - 1) / most;
+    return (W + m - 1) / m;
+}
+
+// One lane's share of the asynchronous copy of a group.
+__device__ __forceinline__ void stage_group(float4 *dst, const float4 *__restrict__ g, int lane) {
+#pragma unroll
+    for (int i = 0; i < (kGroupF4 + 31) / 32; ++i) {
+        const int e = lane + 32 * i;
+        if (e < kGroupF4) {
+            const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + e);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g + e)
+                         : "memory");
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The tiles that the CTA's units (those of warps [w0, w1)) lie in, once its
+// warps are done. Not inlined: its registers would be taken from the main loop.
+__device__ __noinline__ void finish_warp_tiles(const SysMap &smap, int64_t W, int64_t G,
+                                               int64_t w0, int64_t w1, const float *part,
+                                               int *cnt, double scale, double *VW) {
+    constexpr int kThreads = 32 * kWarpCta;
+    __shared__ int s_done[kThreads];
+    if (w0 >= w1) return;                       // the whole CTA leaves
+    const int64_t c_beg = unit_start(w0, W, G), c_end = unit_start(w1, W, G);
+    const int64_t t_first = c_beg / smap.n_units, t_last = (c_end - 1) / smap.n_units;
+    for (int64_t tb = t_first; tb <= t_last; tb += kThreads) {
+        __syncthreads();      // the CTA's partials are written (and s_done is free)
+        {
+            const int64_t t = tb + threadIdx.x;
+            int done = 0;
+            if (t <= t_last) {
+                const int64_t b0 = tile_unit_begin(smap, t), b1 = tile_unit_begin(smap, t + 1);
+                const int64_t o0 = ((b0 + 1) * G + W - 1) / W - 1, o1 = (b1 * G + W - 1) / W - 1;
+                if (o0 != o1) {
+                    const int units = (int)(min(b1, c_end) - max(b0, c_beg));
+                    done = fetch_add_acq_rel(cnt + t, units) + units == (int)(b1 - b0);
+                }
+            }
+            s_done[threadIdx.x] = done;
+        }
+        __syncthreads();
+        const int nt = (int)min((int64_t)kThreads, t_last - tb + 1);
+        for (int i = 0; i < nt; ++i) {
+            if (!s_done[i]) continue;
+            const int64_t t = tb + i;
+            const int64_t b0 = tile_unit_begin(smap, t), b1 = tile_unit_begin(smap, t + 1);
+            const int64_t o0 = ((b0 + 1) * G + W - 1) / W - 1, o1 = (b1 * G + W - 1) / W - 1;
+            const int n_parts = (int)(o1 - o0 + 1);
+            static_assert(kThreads == 6 * kWarpTile, "a thread per (component, target)");
+            const int c = threadIdx.x / kWarpTile, l = threadIdx.x % kWarpTile;
+            const float *p0 = part + (size_t)(o0 + t) * kWarpPart + c * kWarpTile + l;
+            float ah = 0.f, al = 0.f;
+            // a batch of loads in flight before its sums (one part at a time, each sum
+            // waiting for its load, took 450 cycles a part: 17 us for the 37 parts of
+            // a tile at 3200 segments, half of the kernel)
+            constexpr int kBatch = 24;
+            for (int j0 = 0; j0 < n_parts; j0 += kBatch) {
+                float h[kBatch], lw[kBatch];
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    // (parts past the last read it again and add zero)
+                    const float *p = p0 + min(j0 + j, n_parts - 1) * kWarpPart;
+                    h[j] = __ldcg(p);
+                    lw[j] = __ldcg(p + 6 * kWarpTile);
+                }
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    const bool in = j0 + j < n_parts;
+                    float sh, e;
+                    two_sum(ah, in ? h[j] : 0.f, sh, e);
+                    e = __fadd_rn(e, __fadd_rn(al, in ? lw[j] : 0.f));
+                    two_sum(sh, e, ah, al);
+                }
+            }
+            const int64_t n = segment_at(smap, t * kWarpTile + l, smap.n_src);
+            if (n >= 0) VW[6 * n + c] = ((double)ah + (double)al) * scale;
+            if (threadIdx.x == 0) cnt[t] = 0;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * kWarpCta, 1)
+rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int n_ctas,
+                       RpyConst32 k, float *__restrict__ part, int *__restrict__ cnt,
+                       double scale, double *__restrict__ VW) {
+    extern __shared__ float4 wsm[];             // [kWarpCta][2][kGroupF4]
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t G = warp_count(W, n_ctas);
+    const int64_t w0 = unit_start(blockIdx.x, G, n_ctas);        // this CTA's warps
+    const int64_t w1 = unit_start((int64_t)blockIdx.x + 1, G, n_ctas);
+    const int64_t w = w0 + wid;
+    int64_t u = 0, u_end = 0;
+    if (w < w1) {
+        u = unit_start(w, W, G);
+        u_end = unit_start(w + 1, W, G);
+    }
+    float4 *buf = wsm + 2 * kGroupF4 * wid;
+    const int64_t n_units = smap.n_units;
+    int64_t tile = 0, ubeg = 0;
+    if (u < u_end) {
+        tile = u / n_units;
+        ubeg = tile * n_units;
+        stage_group(buf, src + kGroupF4 * (u - ubeg), lane);
+    }
+    int cur = 0;
+    while (u < u_end) {
+        const int64_t base = tile * kWarpTile;              // the tile's first target
+        const int64_t s_end = min(u_end, ubeg + n_units);  // this warp's units of the tile
+        const bool whole = u == ubeg && s_end == ubeg + n_units;
+        float th[2][3], tl[2][3], hi[2][6], lo[2][6];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            load_target<true>(src, base + 32 * t + lane, th[t], tl[t]);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) hi[t][c] = lo[t][c] = 0.f;
+        }
+#pragma unroll 1
+        for (; u < s_end; ++u, cur ^= 1) {
+            if (u + 1 < u_end) {
+                // the next group, or the first one for the next tile
+                const int64_t gn = u + 1 < s_end ? u + 1 - ubeg : 0;
+                stage_group(buf + kGroupF4 * (cur ^ 1), src + kGroupF4 * gn, lane);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                cp_async_wait_all();
+            }
+            __syncwarp();
+            const float4 *qg = buf + kGroupF4 * cur + Rec<true>::kHead;
+            float out[2][6];
+            float rmin2[2] = {k.close2, k.close2};
+            {
+                float2 t2[2][3], acc[2][Rec<true>::kSums];
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    to_frame<true>(qg, th[t], tl[t], t2[t]);
+#pragma unroll
+                    for (int c = 0; c < Rec<true>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
+                }
+#pragma unroll (kRpyUnroll / 2)
+                for (int jp = 0; jp < kRpyComp / 2; ++jp) {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+                        pair32_far<true>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2[t]);
+                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    combine_group<true>(acc[t], t2[t], k.k23a2, out[t]);
+            }
+            // slots in which a pair came closer than R_c, one at a time through one copy of
+            // the code: with hi/lo differences in the far form, or with the exact
+            // coefficients where a pair overlaps (the group that holds the slot's own
+            // segments counts as one: it has the self pairs)
+            unsigned close = 0;
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+                if (__any_sync(0xffffffffu, rmin2[t] < k.close2)) close |= 1u << t;
+            while (close) {
+                const bool t1 = close == 2u;
+                close &= 2u * (close == 3u);
+                const bool exact = __any_sync(0xffffffffu, (t1 ? rmin2[1] : rmin2[0]) < k.over2);
+                float ph[3], pl[3], uh[3], ul[3];
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                    ph[x] = t1 ? th[1][x] : th[0][x];
+                    pl[x] = t1 ? tl[1][x] : tl[0][x];
+                }
+                to_frame_hl<true>(qg, ph, pl, uh, ul);
+                float2 acc[6];
+                float rm = 0.f;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
+                if (exact) {
+#pragma unroll 2
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                        pair32_near<true, kExact>(uh, ul, qg + kPairF4 * jp, k, acc, rm);
+                } else {
+#pragma unroll 2
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                        pair32_near<true, kFarHiLo>(uh, ul, qg + kPairF4 * jp, k, acc, rm);
+                }
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    const float v = __fadd_rn(acc[c].x, acc[c].y);
+                    if (t1) out[1][c] = v;
+                    else out[0][c] = v;
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    float sh, e;
+                    two_sum(hi[t][c], out[t][c], sh, e);
+                    hi[t][c] = sh;
+                    lo[t][c] = __fadd_rn(lo[t][c], e);
+                }
+            __syncwarp();     // every lane is done with this buffer before it is refilled
+        }
+        if (whole) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int64_t n = segment_at(smap, base + 32 * t + lane, smap.n_src);
+                if (n >= 0) {
+#pragma unroll
+                    for (int c = 0; c < 6; ++c)
+                        VW[6 * n + c] = ((double)hi[t][c] + (double)lo[t][c]) * scale;
+                }
+            }
+        } else {
+            float *p = part + (size_t)(w + tile) * kWarpPart;
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    p[c * kWarpTile + 32 * t + lane] = hi[t][c];
+                    p[(6 + c) * kWarpTile + 32 * t + lane] = lo[t][c];
+                }
+        }
+        tile += 1;
+        ubeg += n_units;
+    }
+
+    finish_warp_tiles(smap, W, G, w0, w1, part, cnt, scale, VW);
 }
 
 // ---------------------------------------------------------------------------
@@ -806,10 +1233,10 @@ rpy_pair64_kernel(const double *__restrict__ src, SysMap smap, int64_t W, int G,
     const int64_t u_end = unit_start(b + 1, W, G);
 
     while (u < u_end) {
-        int64_t tile, ubeg, n_chunks, src0;
-        locate_unit(smap, u, tile, ubeg, n_chunks, src0);
+        int64_t tile, ubeg, n_units, src0;
+        locate_unit(smap, u, tile, ubeg, n_units, src0);
         const int64_t c_begin = u - ubeg;
-        const int64_t c_end = min(n_chunks, c_begin + (u_end - u));
+        const int64_t c_end = min(n_units, c_begin + (u_end - u));
         const double *srcs = src + 9 * src0;
         const int64_t ptile = smap.tile_id ? smap.tile_id[tile] : tile;
         // real sources of the tile's system (its padding follows them): padded
@@ -904,24 +1331,28 @@ rpy_pair64_kernel(const double *__restrict__ src, SysMap smap, int64_t W, int G,
 #pragma unroll
             for (int c = 0; c < 6; ++c) p[c * kTile + local] = acc[t][c];
         }
-        finish_tile<double, 1, TPT>(part, smap, tile, ptile, c_end - c_begin, n_chunks, W, G, cnt,
+        finish_tile<double, 1, TPT>(part, smap, tile, ptile, c_end - c_begin, n_units, W, G, cnt,
                                     scale, VW);
         u = ubeg + c_end;
     }
 }
 
 SysMap sys_map(const fil_ctx *c, bool active_only) {
-    SysMap m;
+    SysMap m{};
     m.n_src = c->lay.S;
-    m.pos_of_seg = c->pos_of_seg_d;
+    if (c->n_sys == 1 && !active_only) {
+        // one system: tiles and groups in order, no table
+        m.n_tiles = c->rpy_tiles;
+        const int per = unit_sources(c->rpy_frames != 0);
+        m.n_units = (c->lay.S + per - 1) / per;
+        return m;
+    }
     m.pad_map = c->pad_map_d;
-    m.n_chunks = 0;
     if (active_only) {
         m.tile_unit_off = c->act_unit_off_d;
         m.tile_src = c->act_src_d;
         m.tile_nsrc = c->act_nsrc_d;
         m.tile_id = c->act_tile_d;
-        m.slot_of = c->act_slot_d;
         m.n_tiles = c->act_tiles;
         m.dyn = c->act_dyn_d;
     } else {
@@ -929,7 +1360,6 @@ SysMap sys_map(const fil_ctx *c, bool active_only) {
         m.tile_src = c->tile_src_d;
         m.tile_nsrc = c->tile_nsrc_d;
         m.tile_id = c->tile_id_d;
-        m.slot_of = c->slot_d;
         m.n_tiles = c->rpy_tiles;
     }
     return m;
@@ -944,10 +1374,16 @@ int64_t count_tiles(const fil_ctx *c, int T) {
     return n;
 }
 
+cudaError_t allow_warp_smem() {
+    return cudaFuncSetAttribute(rpy_pair32_warp_kernel,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmem);
+}
+
 // Tiles of T targets of every system (only tiles that hold real targets),
-// each with ceil(S_s / chunk) source chunks.
+// each with ceil(S_s / unit) units.
 void build_tiles(fil_ctx *c) {
-    const int T = rpy_tile(c);
+    const int T = c->rpy_auto ? kWarpTile : rpy_tile(c);
+    const int per = unit_sources(c->rpy_frames != 0);
     c->tile_unit_off_h.assign(1, 0);
     c->tile_src_h.clear();
     c->tile_nsrc_h.clear();
@@ -956,9 +1392,9 @@ void build_tiles(fil_ctx *c) {
     for (int s = 0; s < c->n_sys; ++s) {
         const int64_t Ss = c->sys_seg_off_h[s + 1] - c->sys_seg_off_h[s];
         const int64_t tiles = (Ss + T - 1) / T;
-        const int64_t chunks = (Ss + kRpyChunk - 1) / kRpyChunk;
+        const int64_t units = (Ss + per - 1) / per;
         for (int64_t t = 0; t < tiles; ++t) {
-            c->tile_unit_off_h.push_back(c->tile_unit_off_h.back() + chunks);
+            c->tile_unit_off_h.push_back(c->tile_unit_off_h.back() + units);
             c->tile_src_h.push_back(c->sys_pad_off_h[s]);
             c->tile_nsrc_h.push_back(Ss);
             c->tile_sys_h.push_back(s);
@@ -987,9 +1423,8 @@ void set_grids(fil_ctx *c) {
 int pair_occupancy(const fil_ctx *c, int tpt, int split) {
     if (!pair32_on(c))
         return tpt == 1 ? occupancy(rpy_pair64_kernel<1>) : occupancy(rpy_pair64_kernel<2>);
-    if (tpt == 2) return occupancy(rpy_pair32_kernel<2>);
-    return split == 2 ? occupancy(rpy_pair32_kernel<1, 2>, 2 * kRpyThreads)
-                      : occupancy(rpy_pair32_kernel<1>);
+    if (tpt == 2) return kRpyMaxCtasTpt2;
+    return split == 2 ? kRpyMaxCtasSplit2 : kRpyMaxCtasTpt1;
 }
 
 }  // namespace
@@ -997,12 +1432,10 @@ int pair_occupancy(const fil_ctx *c, int tpt, int split) {
 cudaError_t rpy_setup(fil_ctx *c) {
     c->rpy_tpt = kRpyTargetsPerThread;
     c->rpy_threads = kRpyThreads;
-    int occ = pair32_on(c) ? occupancy(rpy_pair32_kernel<kRpyTargetsPerThread>)
-                                   : occupancy(rpy_pair64_kernel<kRpyTargetsPerThread>);
+    const int occ = pair_occupancy(c, kRpyTargetsPerThread, 1);
     c->rpy_ctas = occ;
     c->rpy_split = 1;
-    c->rpy_ctas_max = std::max({occ, occupancy(rpy_pair32_kernel<1>), occupancy(rpy_pair32_kernel<2>),
-                                occupancy(rpy_pair32_kernel<1, 2>, 2 * kRpyThreads),
+    c->rpy_ctas_max = std::max({occ, kRpyMaxCtasTpt1, kRpyMaxCtasTpt2,
                                 occupancy(rpy_pair64_kernel<1>), occupancy(rpy_pair64_kernel<2>)});
     set_grids(c);
     // padded layout: system s occupies [pad_off[s], pad_off[s+1]), a multiple of kRpyPad
@@ -1016,23 +1449,25 @@ cudaError_t rpy_setup(fil_ctx *c) {
     }
     c->pairs_act = c->pairs_all;
     c->Spad = c->sys_pad_off_h[ns];
-    c->pos_of_seg_h.resize(c->lay.S);
     c->pad_map_h.assign(c->Spad, -1);
     for (int s = 0; s < ns; ++s)
         for (int64_t g = c->sys_seg_off_h[s]; g < c->sys_seg_off_h[s + 1]; ++g) {
             const int64_t P = c->sys_pad_off_h[s] + (g - c->sys_seg_off_h[s]);
-            c->pos_of_seg_h[g] = P;
             c->pad_map_h[P] = (int)g;
         }
-    c->rpy_tiles_max = std::max(count_tiles(c, kRpyThreads), count_tiles(c, 2 * kRpyThreads));
+    c->rpy_tiles_max = count_tiles(c, kWarpTile);
+    c->rpy_frames = pair32_on(c) && ns == 1 ? 1 : 0;
+    c->rpy_auto = c->rpy_frames;
+    if (c->rpy_auto) {
+        const cudaError_t e = allow_warp_smem();
+        if (e != cudaSuccess) return e;
+    }
     build_tiles(c);
     return cudaSuccess;
 }
 
 // Tile tables of the current tile size (after the arena exists, and after a retune).
 cudaError_t upload_tiles(fil_ctx *c) {
-    std::vector<int> slot(c->Spad / kRpyThreads, -1);
-    for (int64_t t = 0; t < c->rpy_tiles; ++t) slot[c->tile_id_h[t]] = (int)t;
     cudaError_t e = cudaMemcpyAsync(c->tile_unit_off_d, c->tile_unit_off_h.data(),
                                     sizeof(int64_t) * c->tile_unit_off_h.size(),
                                     cudaMemcpyHostToDevice, c->stream);
@@ -1046,19 +1481,12 @@ cudaError_t upload_tiles(fil_ctx *c) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->tile_id_d, c->tile_id_h.data(), sizeof(int) * c->tile_id_h.size(),
                             cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->slot_d, slot.data(), sizeof(int) * slot.size(),
-                            cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);   // slot goes out of scope
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     return e;
 }
 
 cudaError_t rpy_upload_tables(fil_ctx *c) {
     cudaError_t e = upload_tiles(c);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->pos_of_seg_d, c->pos_of_seg_h.data(),
-                            sizeof(int64_t) * c->pos_of_seg_h.size(), cudaMemcpyHostToDevice,
-                            c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->pad_map_d, c->pad_map_h.data(), sizeof(int) * c->pad_map_h.size(),
                             cudaMemcpyHostToDevice, c->stream);
@@ -1075,6 +1503,9 @@ size_t rpy_partial_bytes(const fil_ctx *c) {
         const size_t b = (size_t)(G + count_tiles(c, T)) * T * 12 * sizeof(float);
         most = std::max(most, b);
     }
+    if (c->rpy_frames)
+        most = std::max(most, (size_t)((int64_t)c->num_sms * kWarpCta + c->rpy_tiles_max) *
+                                  kWarpPart * sizeof(float));
     return most;
 }
 
@@ -1082,10 +1513,9 @@ size_t rpy_partial_bytes(const fil_ctx *c) {
 // stream-K split of the next applies with active_only.
 cudaError_t rpy_set_active(fil_ctx *c) {
     std::vector<int64_t> uoff(1, 0), src, nsrc;
-    std::vector<int> tid, slot(c->Spad / kRpyThreads, -1);
+    std::vector<int> tid;
     for (int64_t t = 0; t < c->rpy_tiles; ++t) {
         if (!c->active_h[c->tile_sys_h[t]]) continue;
-        slot[c->tile_id_h[t]] = (int)tid.size();
         tid.push_back(c->tile_id_h[t]);
         src.push_back(c->tile_src_h[t]);
         nsrc.push_back(c->tile_nsrc_h[t]);
@@ -1110,9 +1540,6 @@ cudaError_t rpy_set_active(fil_ctx *c) {
     if (e == cudaSuccess && !tid.empty())
         e = cudaMemcpyAsync(c->act_tile_d, tid.data(), sizeof(int) * tid.size(),
                             cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->act_slot_d, slot.data(), sizeof(int) * slot.size(),
-                            cudaMemcpyHostToDevice, c->stream);
     const int64_t dyn[2] = {c->act_tiles, c->act_units};
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->act_dyn_d, dyn, sizeof(dyn), cudaMemcpyHostToDevice, c->stream);
@@ -1135,6 +1562,9 @@ void prof_record(fil_ctx *c, cudaEvent_t ev) {
 
 }  // namespace
 
+// CTAs of the warp kernel: one per SM, fewer when there are not as many units.
+static int warp_grid(int64_t W, int sms) { return (int)std::min<int64_t>(sms, W); }
+
 cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
                       bool active_only) {
     const int64_t S = c->lay.S;
@@ -1148,20 +1578,28 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     // the active-tile list changes between applies: its launches keep a fixed grid
     // (and read the unit count from the device), so captured graphs stay valid
     if (pair32_on(c)) {
-        const int G = (int)(active_only ? c->rpy_grid32 : std::min<int64_t>(c->rpy_grid32, W));
-        pack32_kernel<<<pgrid, pb, 0, c->stream>>>(Y, FT, S, c->Spad, sm, c->src32);
+        const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
+        pack<<<pgrid, pb, 0, c->stream>>>(Y, FT, S, c->Spad, sm, c->src32);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         const RpyConst32 k = make_const<float, RpyConst32>(c->a);
-        if (c->rpy_tpt == 1 && c->rpy_split == 2)
-            rpy_pair32_kernel<1, 2><<<G, 2 * kRpyThreads, 0, c->stream>>>(
+        if (c->rpy_auto) {
+            const int G = warp_grid(W, c->num_sms);
+            rpy_pair32_warp_kernel<<<G, 32 * kWarpCta, kWarpSmem, c->stream>>>(
                 c->src32, sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
-        else if (c->rpy_tpt == 1)
-            rpy_pair32_kernel<1><<<G, kRpyThreads, 0, c->stream>>>(
+        } else {
+            const int G = (int)(active_only ? c->rpy_grid32 : std::min<int64_t>(c->rpy_grid32, W));
+            const bool split = c->rpy_tpt == 1 && c->rpy_split == 2;
+            const auto pair =
+                c->rpy_frames ? (split               ? rpy_pair32_kernel<true, 1, 2>
+                                 : c->rpy_tpt == 1   ? rpy_pair32_kernel<true, 1>
+                                                     : rpy_pair32_kernel<true, 2>)
+                              : (split               ? rpy_pair32_kernel<false, 1, 2>
+                                 : c->rpy_tpt == 1   ? rpy_pair32_kernel<false, 1>
+                                                     : rpy_pair32_kernel<false, 2>);
+            pair<<<G, kRpyThreads * (split ? 2 : 1), 0, c->stream>>>(
                 c->src32, sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
-        else
-            rpy_pair32_kernel<2><<<G, kRpyThreads, 0, c->stream>>>(
-                c->src32, sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
+        }
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
     } else {
@@ -1205,15 +1643,16 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
     std::vector<cudaEvent_t> ev(2 * (size_t)std::max(1, reps), nullptr);
     cudaError_t e = cudaSuccess;
     for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
-    struct cand { int tpt, split, ctas; float ms; };
+    struct cand { int tpt, split, ctas, automatic; float ms; };
     std::vector<cand> cands;
     for (int tpt = 1; tpt <= 2; ++tpt) {
         for (int split = 1; split <= (tpt == 1 && pair32_on(c) ? 2 : 1); ++split) {
             const int occ = pair_occupancy(c, tpt, split);
             for (int ctas = 1; ctas <= std::min(occ, c->rpy_ctas_max); ++ctas)
-                cands.push_back({tpt, split, ctas, 1e30f});
+                cands.push_back({tpt, split, ctas, 0, 1e30f});
         }
     }
+    if (c->rpy_frames) cands.push_back({2, 1, pair_occupancy(c, 2, 1), 1, 1e30f});
     const auto t0 = std::chrono::steady_clock::now();
     while (e == cudaSuccess) {
         for (int r = 0; r < 4 && e == cudaSuccess; ++r) e = rpy_apply(c, Y, FT, VW);
@@ -1224,6 +1663,7 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
     for (int sweep = 0; sweep < kSweeps && e == cudaSuccess; ++sweep) {
         for (cand &k : cands) {
             if (e != cudaSuccess) break;
+            c->rpy_auto = k.automatic;
             c->rpy_tpt = k.tpt;
             c->rpy_split = k.split;
             c->rpy_threads = kRpyThreads;
@@ -1251,14 +1691,17 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
     for (cudaEvent_t x : ev)
         if (x) cudaEventDestroy(x);
     float best = 1e30f;
-    int best_tpt = c->rpy_tpt, best_split = c->rpy_split, best_ctas = c->rpy_ctas;
+    int best_tpt = c->rpy_tpt, best_split = c->rpy_split, best_ctas = c->rpy_ctas,
+        best_auto = c->rpy_auto;
     for (const cand &k : cands)
         if (k.ms < best) {
             best = k.ms;
             best_tpt = k.tpt;
             best_split = k.split;
             best_ctas = k.ctas;
+            best_auto = k.automatic;
         }
+    c->rpy_auto = best_auto;
     c->rpy_tpt = best_tpt;
     c->rpy_split = best_split;
     c->rpy_threads = kRpyThreads;
@@ -1284,6 +1727,7 @@ bool rpy_schedule_valid(const fil_ctx *c, int tpt, int threads, int ctas, int sp
 }
 
 cudaError_t rpy_set_schedule(fil_ctx *c, int tpt, int threads, int ctas, int split) {
+    c->rpy_auto = 0;
     c->rpy_tpt = tpt;
     c->rpy_split = split;
     c->rpy_threads = threads;
@@ -1314,16 +1758,13 @@ constexpr int64_t kNoAllocMaxSeg = 32768;     // largest S accepted
 // the grid is capped here, and the results then differ from
 // fil_mobility_apply's in rounding only (another summation order).
 constexpr int kNoAllocMaxSMs = 152;
-constexpr int kNoAllocMaxGrid = kRpyMinBlocksTpt2 * kNoAllocMaxSMs;   // stream-K CTAs at most
-constexpr int64_t kNoAllocMaxTiles = (kNoAllocMaxSeg + kRpyTile - 1) / kRpyTile;
-constexpr int64_t kNoAllocMaxChunks = (kNoAllocMaxSeg + kRpyChunk - 1) / kRpyChunk;
-constexpr int64_t kNoAllocMaxSpad = (kNoAllocMaxTiles * kRpyTile > kNoAllocMaxChunks * kRpyChunk)
-                                        ? kNoAllocMaxTiles * kRpyTile
-                                        : kNoAllocMaxChunks * kRpyChunk;
-constexpr size_t kNoAllocSrcBytes = (size_t)kRpyPairF4 * (kNoAllocMaxSpad / 2) * sizeof(float4);
+constexpr int64_t kNoAllocMaxTiles = (kNoAllocMaxSeg + kWarpTile - 1) / kWarpTile;
+constexpr int64_t kNoAllocMaxSpad = kNoAllocMaxTiles * kWarpTile;
+constexpr size_t kNoAllocSrcBytes =
+    (size_t)Rec<true>::kGroupF4 * (kNoAllocMaxSpad / kRpyComp) * sizeof(float4);
 constexpr size_t kNoAllocPartBytes =
-    (size_t)(kNoAllocMaxGrid + kNoAllocMaxTiles) * 12 * kRpyTile * sizeof(float);
-constexpr size_t kNoAllocBytes = kNoAllocSrcBytes + kNoAllocPartBytes;   // ~10.6 MB
+    (size_t)(kNoAllocMaxSMs * kWarpCta + kNoAllocMaxTiles) * kWarpPart * sizeof(float);
+constexpr size_t kNoAllocBytes = kNoAllocSrcBytes + kNoAllocPartBytes;   // ~9.6 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 // per-tile completion counters of the pair kernel: zero at load, and every
@@ -1347,13 +1788,12 @@ cudaError_t noalloc_setup(int dev, unsigned char **ptr, int **cnt, int *grid) {
         e = cudaGetSymbolAddress(&q, g_noalloc_cnt);
         if (e != cudaSuccess) return e;
         g_noalloc_cnt_ptr[dev] = static_cast<int *>(q);
-        int occ = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, rpy_pair32_kernel<kRpyTargetsPerThread>,
-                                                          kRpyThreads, 0);
-        if (e != cudaSuccess) return e;
+        int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        g_noalloc_grid[dev] = std::max(1, std::min(kNoAllocMaxGrid, std::max(1, occ) * sms));
+        e = allow_warp_smem();
+        if (e != cudaSuccess) return e;
+        g_noalloc_grid[dev] = std::max(1, std::min(kNoAllocMaxSMs, sms));
         g_noalloc_ptr[dev] = static_cast<unsigned char *>(p);
     }
     *ptr = g_noalloc_ptr[dev];
@@ -1378,12 +1818,12 @@ bool on_device(const void *p, int dev) {
 // A launch whose own status is returned (cudaGetLastError would also report
 // an earlier, unrelated failure of the caller's).
 template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t st,
-                   Args &&...args) {
+cudaError_t launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                   cudaStream_t st, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = nullptr;
     cfg.numAttrs = 0;
@@ -1407,11 +1847,11 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     int grid_max = 1;
     if (noalloc_setup(dev, &base, &cnt, &grid_max) != cudaSuccess) return FIL_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    const int64_t tiles = (n_seg + kRpyTile - 1) / kRpyTile;
-    const int64_t n_chunks = (n_seg + kRpyChunk - 1) / kRpyChunk;
-    const int64_t Spad = std::max(tiles * kRpyTile, n_chunks * kRpyChunk);
-    const int64_t W = tiles * n_chunks;
-    const int G = (int)std::min<int64_t>(grid_max, W);
+    const int64_t tiles = (n_seg + kWarpTile - 1) / kWarpTile;
+    const int64_t Spad = tiles * kWarpTile;
+    const int64_t n_units = (n_seg + kRpyComp - 1) / kRpyComp;   // source groups per tile
+    const int64_t W = tiles * n_units;
+    const int G = warp_grid(W, grid_max);
     float4 *src = reinterpret_cast<float4 *>(base);
     float *part = reinterpret_cast<float *>(base + kNoAllocSrcBytes);
     // every source record up to Spad and every partial slot a tile's sum reads
@@ -1419,12 +1859,12 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     const int pb = 256;
     SysMap sm{};                       // one system, no tables
     sm.n_tiles = tiles;
-    sm.n_chunks = n_chunks;
+    sm.n_units = n_units;
     sm.n_src = n_seg;
-    cudaError_t e = launch(pack32_kernel, (unsigned)((Spad + pb - 1) / pb), pb, st, Y, FT, n_seg,
+    cudaError_t e = launch(pack32_kernel<true>, (unsigned)((Spad + pb - 1) / pb), pb, 0, st, Y, FT, n_seg,
                            Spad, sm, src);
     if (e == cudaSuccess)
-        e = launch(rpy_pair32_kernel<kRpyTargetsPerThread>, (unsigned)G, kRpyThreads, st,
+        e = launch(rpy_pair32_warp_kernel, (unsigned)G, 32 * kWarpCta, kWarpSmem, st,
                    (const float4 *)src, sm, W, G, make_const<float, RpyConst32>(a), part, cnt,
                    1.0 / (8.0 * kPi * eta), VW);
     return e == cudaSuccess ? FIL_OK : FIL_ECUDA;

@@ -50,3 +50,25 @@ def test_tile_partials_are_found_in_both_regimes():
                 # the units each CTA adds to the tile's counter sum to the tile's units
                 covered = sum(min(starts[b + 1], u1 + 1) - max(starts[b], u0) for b in truth)
                 assert covered == u1 - u0 + 1
+
+
+def warp_count(W, n_ctas, per=12):
+    m = -(-W // (n_ctas * per))
+    return -(-W // m)
+
+
+def test_warp_split_gives_every_warp_a_unit_and_every_cta_at_most_its_warps():
+    """The automatic schedule: W units over warp_count(W, n_ctas) warps, CTA c
+    running warps [floor(cG/n), floor((c+1)G/n))."""
+    rng = np.random.default_rng(5)
+    for n_ctas in (1, 3, 152):
+        for W in list(range(1, 200)) + rng.integers(200, 600000, size=60).tolist():
+            G = warp_count(W, n_ctas)
+            assert 1 <= G <= min(W, 12 * n_ctas)
+            ctas = [unit_start(c, G, n_ctas) for c in range(n_ctas + 1)]
+            assert ctas[0] == 0 and ctas[-1] == G
+            assert max(b - a for a, b in zip(ctas, ctas[1:])) <= 12
+            if G < 4000 and W < 5000:
+                starts = [unit_start(w, W, G) for w in range(G + 1)]
+                assert all(a < b for a, b in zip(starts, starts[1:]))
+                assert max(b - a for a, b in zip(starts, starts[1:])) == -(-W // G)
