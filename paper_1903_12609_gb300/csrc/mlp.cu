@@ -51,41 +51,83 @@ Offsets param_offsets() {
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-cudaError_t gemm(const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N, int K,
-                 const tc::Epilogue &ep, int *err, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(tc::gemm_bf16_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         tc::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((M + tc::kTileM - 1) / tc::kTileM),
-              (unsigned)((N + tc::kMaxTileN - 1) / tc::kMaxTileN));
-    tc::gemm_bf16_kernel<<<grid, tc::kThreads, tc::kSmemBytes, st>>>(A, lda, B, ldb, M, N, K,
-                                                                     ep, err);
-    return cudaGetLastError();
-}
-
 tc::Epilogue epi() {
     tc::Epilogue e{};
-    e.alpha = 1.f;
     e.n_valid = 1 << 30;
     return e;
 }
 
-// x^ = (x - mean) / std in BF16, row-major [B x kInP] (zero padding) and
-// transposed [kInP x ldt] (columns >= B are zeroed by the caller).
-__global__ void input_kernel(const float *__restrict__ x, int64_t B, const float *__restrict__ mean,
-                             const float *__restrict__ stdv, bf16 *__restrict__ X,
-                             bf16 *__restrict__ Xt, int64_t ldt) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * kInP) return;
-    const int64_t b = i / kInP;
-    const int c = (int)(i - b * kInP);
-    const float v = c < kIn ? (x[b * kIn + c] - mean[c]) / stdv[c] : 0.f;
-    const bf16 h = __float2bfloat16_rn(v);
-    X[i] = h;
-    if (Xt) Xt[(int64_t)c * ldt + b] = h;
+tc::Problem product(const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N, int K,
+                    const tc::Epilogue &ep) {
+    return tc::Problem{A, B, lda, ldb, M, N, K, 0, 0, ep};
 }
 
+template <int kNt>
+cudaError_t launch_gemm(const tc::Batch &b, int64_t ctas, cudaStream_t st) {
+    const cudaError_t e = cudaFuncSetAttribute(tc::gemm_bf16_kernel<kNt>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               tc::smem_bytes(kNt));
+    if (e != cudaSuccess) return e;
+    tc::gemm_bf16_kernel<kNt><<<(unsigned)ctas, tc::kThreads, tc::smem_bytes(kNt), st>>>(b);
+    return cudaGetLastError();
+}
+
+// The products of a batch in one launch.
+cudaError_t gemm(tc::Batch &b, int sms, cudaStream_t st) {
+    const int64_t ctas = tc::plan(b, sms);
+    if (ctas > 0x7fffffff) return cudaErrorInvalidValue;
+    switch (b.nt) {
+        case 32: return launch_gemm<32>(b, ctas, st);
+        case 64: return launch_gemm<64>(b, ctas, st);
+        case 128: return launch_gemm<128>(b, ctas, st);
+        default: return launch_gemm<256>(b, ctas, st);
+    }
+}
+
+// Batch rows per CTA of the input and loss kernels, which give a thread one
+// column: its 32 rows are 64 contiguous bytes of the transposed BF16 copy.
+constexpr int kRows = 32;
+constexpr int kInThreads = kInP / 4;     // four CTAs across the padded inputs
+static_assert(kInP % 4 == 0 && kInThreads <= 1024, "input kernel covers the padded inputs");
+
+// Thread c's column of the transposed copy, batch rows b0 .. b0 + 31, written up
+// to row `rows` (a multiple of 8).
+__device__ __forceinline__ void store_column(bf16 *t, int64_t b0, int64_t rows,
+                                             const uint32_t (&h)[kRows / 2]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (b0 + 8 * j < rows)
+            reinterpret_cast<uint4 *>(t + b0)[j] =
+                make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+}
+
+// x^ = (x - mean) / std in BF16, row-major [B x kInP] (zero padding) and, for
+// training, transposed [kInP x ldt] with columns B .. Kb - 1 zero.
+__global__ void __launch_bounds__(kInThreads)
+input_kernel(const float *__restrict__ x, int64_t B, const float *__restrict__ mean,
+             const float *__restrict__ stdv, bf16 *__restrict__ X, bf16 *__restrict__ Xt,
+             int64_t ldt, int64_t Kb) {
+    const int c = blockIdx.x * kInThreads + threadIdx.x;
+    const int64_t b0 = (int64_t)blockIdx.y * kRows;
+    const bool in = c < kIn;
+    const float mu = in ? mean[c] : 0.f, sd = in ? stdv[c] : 1.f;
+    float v[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+        v[r] = in && b0 + r < B ? x[(b0 + r) * kIn + c] : mu;
+    uint32_t h[kRows / 2];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const bf16 q = __float2bfloat16_rn((v[r] - mu) / sd);
+        const uint32_t bits = b0 + r < B ? *reinterpret_cast<const unsigned short *>(&q) : 0u;
+        if (r & 1) h[r >> 1] |= bits << 16;
+        else h[r >> 1] = bits;
+        if (b0 + r < B) X[(b0 + r) * kInP + c] = q;
+    }
+    if (Xt) store_column(Xt + (int64_t)c * ldt, b0, Kb, h);
+}
+
+// y = mean + std y^ (an output array the last product cannot store to).
 __global__ void output_kernel(const float *__restrict__ yhat, int64_t n, const float *__restrict__ mean,
                               const float *__restrict__ stdv, float *__restrict__ y) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -94,49 +136,85 @@ __global__ void output_kernel(const float *__restrict__ yhat, int64_t n, const f
     y[i] = mean[c] + stdv[c] * yhat[i];
 }
 
-// dY = (y^ - t^) / B (FP32 and BF16, row-major and transposed) and the loss,
-// summed by one CTA in a fixed order.
-constexpr int kLossThreads = 1024;
+// dY = (y^ - t^) / B in BF16 (row-major, and transposed with columns B .. Kb - 1
+// zero), its FP32 column sums over each CTA's 32 rows, and each CTA's part of
+// the loss: squares and their sum in float-float (TwoSum), FP64 once per thread
+// (one CTA over the whole batch in FP64 took 234 us at 1024 rows).
+constexpr int kLossThreads = kOut;
 __global__ void __launch_bounds__(kLossThreads)
 loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t B,
-            const float *__restrict__ mean, const float *__restrict__ stdv, float *__restrict__ dYf,
-            bf16 *__restrict__ dY, bf16 *__restrict__ dYt, int64_t ldt, float *__restrict__ loss) {
-    __shared__ double red[kLossThreads];
-    double acc = 0.0;
-    const float inv = 1.f / (float)B;
-    for (int64_t i = threadIdx.x; i < B * kOut; i += blockDim.x) {
-        const int64_t b = i / kOut;
-        const int c = (int)(i - b * kOut);
-        const float d = yhat[i] - (t[i] - mean[c]) / stdv[c];
-        acc += 0.5 * (double)d * (double)d;
-        const float g = d * inv;
-        dYf[i] = g;
-        const bf16 h = __float2bfloat16_rn(g);
-        dY[i] = h;
-        dYt[(int64_t)c * ldt + b] = h;
+            const float *__restrict__ mean, const float *__restrict__ stdv, bf16 *__restrict__ dY,
+            bf16 *__restrict__ dYt, int64_t ldt, int64_t Kb, float *__restrict__ col_sums,
+            double *__restrict__ part, int n_part) {
+    __shared__ double red[kLossThreads / 32];
+    const int c = threadIdx.x;
+    const int64_t b0 = (int64_t)blockIdx.x * kRows;
+    const float inv = 1.f / (float)B, mu = mean[c], sd = stdv[c];
+    float y[kRows], g[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const bool in = b0 + r < B;
+        y[r] = in ? yhat[(b0 + r) * kOut + c] : 0.f;
+        g[r] = in ? t[(b0 + r) * kOut + c] : mu;
     }
-    red[threadIdx.x] = acc;
+    float hi = 0.f, lo = 0.f, sum = 0.f;
+    uint32_t h[kRows / 2];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const bool in = b0 + r < B;
+        const float d = in ? y[r] - (g[r] - mu) / sd : 0.f;
+        const float sq = __fmul_rn(d, d), se = __fmaf_rn(d, d, -sq);
+        const float s = __fadd_rn(hi, sq), bb = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(se, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(sq, bb))));
+        hi = s;
+        const float gr = d * inv;
+        sum += gr;
+        const bf16 q = __float2bfloat16_rn(gr);
+        const uint32_t bits = in ? *reinterpret_cast<const unsigned short *>(&q) : 0u;
+        if (r & 1) h[r >> 1] |= bits << 16;
+        else h[r >> 1] = bits;
+        if (in) dY[(b0 + r) * kOut + c] = q;
+    }
+    store_column(dYt + (int64_t)c * ldt, b0, Kb, h);
+    if ((int)blockIdx.x >= n_part) return;      // rows of the zero padding only
+    col_sums[(int64_t)blockIdx.x * kOut + c] = sum;
+    double acc = 0.5 * ((double)hi + (double)lo);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+    if ((c & 31) == 0) red[c >> 5] = acc;
     __syncthreads();
-    for (int s = kLossThreads / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    if (c == 0) {
+        for (int w = 1; w < kLossThreads / 32; ++w) acc += red[w];
+        part[blockIdx.x] = acc;
     }
-    if (threadIdx.x == 0) *loss = (float)(red[0] / (double)B);
 }
 
-// db[c] = sum_b dZ[b][c], one CTA per column, fixed-order tree.
-__global__ void bias_grad_kernel(const float *__restrict__ dZ, int64_t B, int N, float *__restrict__ db) {
-    __shared__ float red[256];
-    const int c = blockIdx.x;
-    float acc = 0.f;
-    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) acc += dZ[b * N + c];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+// db_l[c] = sum of the column sums' parts (l < 3: one per row tile of the
+// product that formed dZ_l; l = 3: one per CTA of the loss kernel), and the
+// loss. Parts in order, eight loads in flight.
+struct BiasParts {
+    const float *p[kLayers];
+    int n[kLayers];
+    float *db[kLayers];
+};
+__global__ void finish_kernel(BiasParts bp, const double *__restrict__ part, int n_part, double B,
+                              float *__restrict__ loss) {
+    const int l = blockIdx.y, c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int N = l < 3 ? kHid : kOut;
+    if (c < N) {
+        float s = 0.f;
+        const float *p = bp.p[l] + c;
+#pragma unroll 8
+        for (int i = 0; i < bp.n[l]; ++i) s += p[(int64_t)i * N];
+        bp.db[l][c] = s;
     }
-    if (threadIdx.x == 0) db[c] = red[0];
+    if (l == 0 && blockIdx.x == 0 && threadIdx.x < 32) {
+        double a = 0.0;
+        for (int i = threadIdx.x; i < n_part; i += 32) a += part[i];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
+        if (threadIdx.x == 0) *loss = (float)(a / B);
+    }
 }
 
 // BF16 copies of W_l: [out x inP] (zero-padded columns) and [inP x out].
@@ -163,15 +241,17 @@ __global__ void adam_kernel(int64_t n, const float *__restrict__ g, float *__res
     p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
 }
 
-__global__ void zero_cols_kernel(bf16 *__restrict__ a, int rows, int64_t ld, int64_t c0) {
-    const int64_t w = ld - c0;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)rows * w) return;
-    const int64_t r = i / w;
-    a[r * ld + c0 + (i - r * w)] = __float2bfloat16_rn(0.f);
-}
-
 __device__ int g_tc_err;   // wait-limit flag of the standalone GEMM entry point
+
+int device_sms() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return n;
+}
 
 bool dev_ptr(const void *p) {
     cudaPointerAttributes at;
@@ -189,6 +269,7 @@ using namespace fil;
 
 struct fil_mlp {
     cudaStream_t stream;
+    int sms;                         // of the device it was created on
     int64_t max_batch, ldt;          // ldt: padded batch (K of the weight gradients)
     Offsets off;
     float *params, *grad, *adam_m, *adam_v;
@@ -196,7 +277,10 @@ struct fil_mlp {
     bf16 *W[kLayers], *Wt[kLayers];
     float *in_mean, *in_std, *out_mean, *out_std;
     bf16 *X, *Xt, *H[3], *Ht[3], *dY, *dYt, *dH[3], *dHt[3];
-    float *Y, *dYf, *dHf, *loss;
+    float *Y;
+    float *sums[kLayers];            // column sums of dZ_l, by row tile (l < 3) or loss CTA
+    double *loss_part;               // per loss CTA
+    float *loss;                     // followed by err: read back together
     int *err;
     void *arena;
 };
@@ -239,10 +323,12 @@ void carve(fil_mlp *m, Carver &c) {
     m->dY = c.take<bf16>((size_t)B * kOut);
     m->dYt = c.take<bf16>((size_t)kOut * T);
     m->Y = c.take<float>((size_t)B * kOut);
-    m->dYf = c.take<float>((size_t)B * kOut);
-    m->dHf = c.take<float>((size_t)B * kHid);
-    m->loss = c.take<float>(1);
-    m->err = c.take<int>(1);
+    for (int l = 0; l < 3; ++l)
+        m->sums[l] = c.take<float>((size_t)((B + tc::kTileM - 1) / tc::kTileM) * kHid);
+    m->sums[3] = c.take<float>((size_t)((B + kRows - 1) / kRows) * kOut);
+    m->loss_part = c.take<double>((size_t)((B + kRows - 1) / kRows));
+    m->loss = c.take<float>(2);
+    m->err = m->loss ? reinterpret_cast<int *>(m->loss + 1) : nullptr;
 }
 
 const float *to_device(fil_mlp *m, const float *p, size_t n, float *scratch, cudaError_t &e) {
@@ -260,13 +346,24 @@ cudaError_t refresh_weights(fil_mlp *m) {
     return cudaGetLastError();
 }
 
+cudaError_t one_product(fil_mlp *m, const tc::Problem &p) {
+    tc::Batch b{};
+    b.p[0] = p;
+    b.count = 1;
+    b.err = m->err;
+    return gemm(b, m->sms, m->stream);
+}
+
 // Forward pass on normalised inputs; `train` also writes the transposed
-// activations. Output: m->Y (normalised, FP32).
-cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train) {
-    cudaError_t e = cudaSuccess;
-    const int64_t n = B * kInP;
-    input_kernel<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(
-        x, B, m->in_mean, m->in_std, m->X, train ? m->Xt : nullptr, m->ldt);
+// activations, `y` (FP32, 16-byte aligned) takes the outputs in raw units;
+// without it m->Y takes the normalised ones.
+cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train, float *y) {
+    const int64_t Kb = round_up(B, tc::kTileK);
+    const dim3 grid(4, (unsigned)(((train ? Kb : B) + kRows - 1) / kRows));
+    input_kernel<<<grid, kInThreads, 0, m->stream>>>(x, B, m->in_mean, m->in_std, m->X,
+                                                     train ? m->Xt : nullptr, m->ldt, Kb);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const bf16 *act = m->X;
     int ld = kInP;
     for (int l = 0; l < 3; ++l) {
@@ -276,86 +373,110 @@ cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train) {
         if (train) {
             ep.c_bf16_t = m->Ht[l];
             ep.ldt = (int)m->ldt;
+            ep.t_rows = (int)Kb;
         }
         ep.bias = m->params + m->off.b[l];
         ep.relu = 1;
-        e = gemm(act, ld, m->W[l], kDimInP[l], (int)B, kHid, kDimInP[l], ep, m->err, m->stream);
+        e = one_product(m, product(act, ld, m->W[l], kDimInP[l], (int)B, kHid, kDimInP[l], ep));
         if (e != cudaSuccess) return e;
         act = m->H[l];
         ld = kHid;
     }
     tc::Epilogue ep = epi();
-    ep.c_f32 = m->Y;
+    ep.c_f32 = y ? y : m->Y;
     ep.ldc = kOut;
     ep.bias = m->params + m->off.b[3];
-    return gemm(act, ld, m->W[3], kHid, (int)B, kOut, kHid, ep, m->err, m->stream);
-}
-
-cudaError_t zero_pad_columns(fil_mlp *m, int64_t B) {
-    // transposed buffers: columns [B, ldt) are the zero padding of the K = batch dimension
-    if (B == m->ldt) return cudaSuccess;
-    struct {
-        bf16 *p;
-        int rows;
-    } bufs[] = {{m->Xt, kInP}, {m->Ht[0], kHid}, {m->Ht[1], kHid}, {m->Ht[2], kHid},
-                {m->dHt[0], kHid}, {m->dHt[1], kHid}, {m->dHt[2], kHid}, {m->dYt, kOut}};
-    for (auto &b : bufs) {
-        const int64_t n = (int64_t)b.rows * (m->ldt - B);
-        zero_cols_kernel<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(b.p, b.rows, m->ldt, B);
+    if (y) {
+        ep.shift = m->out_mean;
+        ep.scale = m->out_std;
     }
-    return cudaGetLastError();
+    return one_product(m, product(act, ld, m->W[3], kHid, (int)B, kOut, kHid, ep));
 }
 
-// Loss and gradient into m->grad; the loss (device) in m->loss.
-cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B) {
+// Outputs in raw units to y: straight from the last product where its 16-byte
+// stores may (y aligned), through m->Y otherwise.
+cudaError_t forward_raw(fil_mlp *m, const float *x, float *y, int64_t B) {
+    const bool direct = (reinterpret_cast<uintptr_t>(y) & 15) == 0;
+    cudaError_t e = forward(m, x, B, false, direct ? y : nullptr);
+    if (e == cudaSuccess && !direct) {
+        const int64_t n = B * kOut;
+        output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(m->Y, n, m->out_mean,
+                                                                          m->out_std, y);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+// Loss and gradient into `grad` (16-byte aligned); the loss (device) in m->loss.
+// Ten launches: the input, four forward products, the loss, the three products
+// that carry dZ back, all four weight gradients in one, and the bias gradients.
+cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B, float *grad) {
     const int64_t Kb = round_up(B, tc::kTileK);
-    cudaError_t e = zero_pad_columns(m, B);
+    cudaError_t e = forward(m, x, B, true, nullptr);
     if (e != cudaSuccess) return e;
-    e = forward(m, x, B, true);
+    const int loss_ctas = (int)((Kb + kRows - 1) / kRows);
+    const int loss_parts = (int)((B + kRows - 1) / kRows);
+    loss_kernel<<<loss_ctas, kLossThreads, 0, m->stream>>>(m->Y, t, B, m->out_mean, m->out_std,
+                                                           m->dY, m->dYt, m->ldt, Kb, m->sums[3],
+                                                           m->loss_part, loss_parts);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    loss_kernel<<<1, kLossThreads, 0, m->stream>>>(m->Y, t, B, m->out_mean, m->out_std, m->dYf,
-                                                    m->dY, m->dYt, m->ldt, m->loss);
-    // layer 4: dW4 = dY^T H3, db4, dH3 = (dY W4) * [H3 > 0]
-    const bf16 *dZ = m->dY, *dZt = m->dYt;
-    const float *dZf = m->dYf;
+    // dH_{l-1} = (dZ_l W_l) * [H_{l-1} > 0], with its column sums
+    const bf16 *dZ = m->dY;
     int ldz = kOut;
-    for (int l = 3; l >= 0; --l) {
-        const bf16 *Aprev_t = l > 0 ? m->Ht[l - 1] : m->Xt;
-        tc::Epilogue eg = epi();
-        eg.c_f32 = m->grad + m->off.w[l];
-        eg.ldc = kDimIn[l];
-        eg.n_valid = kDimIn[l];
-        e = gemm(dZt, (int)m->ldt, Aprev_t, (int)m->ldt, kDimOut[l], kDimInP[l], (int)Kb, eg,
-                 m->err, m->stream);
-        if (e != cudaSuccess) return e;
-        bias_grad_kernel<<<kDimOut[l], 256, 0, m->stream>>>(dZf, B, kDimOut[l],
-                                                            m->grad + m->off.b[l]);
-        if (l == 0) break;
+    for (int l = 3; l > 0; --l) {
         tc::Epilogue eb = epi();
-        eb.c_f32 = m->dHf;
-        eb.ldc = kHid;
-        eb.c_bf16 = m->dH[l - 1];
+        eb.c_bf16 = l > 1 ? m->dH[l - 1] : nullptr;
         eb.ldh = kHid;
         eb.c_bf16_t = m->dHt[l - 1];
         eb.ldt = (int)m->ldt;
+        eb.t_rows = (int)Kb;
         eb.mask = m->H[l - 1];
         eb.ldm = kHid;
-        e = gemm(dZ, ldz, m->Wt[l], kDimOut[l], (int)B, kHid, kDimOut[l], eb, m->err, m->stream);
+        eb.col_sums = m->sums[l - 1];
+        e = one_product(m, product(dZ, ldz, m->Wt[l], kDimOut[l], (int)B, kHid, kDimOut[l], eb));
         if (e != cudaSuccess) return e;
         dZ = m->dH[l - 1];
-        dZt = m->dHt[l - 1];
-        dZf = m->dHf;
         ldz = kHid;
     }
+    // dW_l = dZ_l^T H_{l-1} (H_{-1}: the inputs)
+    tc::Batch b{};
+    b.count = kLayers;
+    b.err = m->err;
+    for (int l = 0; l < kLayers; ++l) {
+        tc::Epilogue eg = epi();
+        eg.c_f32 = grad + m->off.w[l];
+        eg.ldc = kDimIn[l];
+        eg.n_valid = kDimIn[l];
+        b.p[l] = product(l == 3 ? m->dYt : m->dHt[l], (int)m->ldt, l > 0 ? m->Ht[l - 1] : m->Xt,
+                         (int)m->ldt, kDimOut[l], kDimInP[l], (int)Kb, eg);
+    }
+    e = gemm(b, m->sms, m->stream);
+    if (e != cudaSuccess) return e;
+    BiasParts bp;
+    for (int l = 0; l < kLayers; ++l) {
+        bp.p[l] = m->sums[l];
+        bp.n[l] = l < 3 ? (int)((B + tc::kTileM - 1) / tc::kTileM) : loss_parts;
+        bp.db[l] = grad + m->off.b[l];
+    }
+    finish_kernel<<<dim3(kHid / 64, kLayers), 64, 0, m->stream>>>(bp, m->loss_part, loss_parts,
+                                                                 (double)B, m->loss);
     return cudaGetLastError();
 }
 
-fil_status check_err(fil_mlp *m) {
-    int h = 0;
-    if (cudaMemcpyAsync(&h, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
+// Waits for the stream; FIL_ECUDA if a wait in a product ran out. The loss, when
+// asked for, comes back with the same copy.
+fil_status finish_call(fil_mlp *m, float *loss) {
+    struct {
+        float loss;
+        int err;
+    } h;
+    static_assert(sizeof(h) == 8, "loss and err are adjacent");
+    if (cudaMemcpyAsync(&h, m->loss, sizeof(h), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
         cudaStreamSynchronize(m->stream) != cudaSuccess)
         return FIL_ECUDA;
-    return h ? FIL_ECUDA : FIL_OK;
+    if (loss) *loss = h.loss;
+    return h.err ? FIL_ECUDA : FIL_OK;
 }
 
 }  // namespace
@@ -366,15 +487,9 @@ cudaError_t mlp_forward_async(fil_mlp *m, const float *x, float *y, int64_t batc
                               cudaStream_t st, int64_t *launches) {
     const cudaStream_t own = m->stream;
     m->stream = st;
-    cudaError_t e = forward(m, x, batch, false);
-    if (e == cudaSuccess) {
-        const int64_t n = batch * kOut;
-        output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m->Y, n, m->out_mean,
-                                                                   m->out_std, y);
-        e = cudaGetLastError();
-    }
+    const cudaError_t e = forward_raw(m, x, y, batch);
     m->stream = own;
-    if (launches) *launches += 6;
+    if (launches) *launches += 5;
     return e;
 }
 
@@ -392,6 +507,7 @@ fil_status fil_mlp_create(int64_t max_batch, void *stream, fil_mlp **out) {
     m->max_batch = max_batch;
     m->ldt = round_up(max_batch, tc::kTileK);
     m->off = param_offsets();
+    m->sms = device_sms();
     Carver sizing{nullptr};
     carve(m, sizing);
     if (cudaMalloc(&m->arena, sizing.used) != cudaSuccess) {
@@ -468,36 +584,29 @@ fil_status fil_mlp_set_norm(fil_mlp *m, const float *in_mean, const float *in_st
 fil_status fil_mlp_forward(fil_mlp *m, const float *x, float *y, int64_t batch) {
     if (!m || !x || !y || batch < 1 || batch > m->max_batch) return FIL_EINVAL;
     if (!dev_ptr(x) || !dev_ptr(y)) return FIL_EINVAL;
-    cudaError_t e = forward(m, x, batch, false);
-    const int64_t n = batch * kOut;
-    if (e == cudaSuccess) {
-        output_kernel<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(m->Y, n, m->out_mean,
-                                                                          m->out_std, y);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) return FIL_ECUDA;
-    return check_err(m);
+    if (forward_raw(m, x, y, batch) != cudaSuccess) return FIL_ECUDA;
+    return finish_call(m, nullptr);
 }
 
 fil_status fil_mlp_gradients(fil_mlp *m, const float *x, const float *target, int64_t batch,
                              float *grad, float *loss) {
     if (!m || !x || !target || !grad || batch < 1 || batch > m->max_batch) return FIL_EINVAL;
     if (!dev_ptr(x) || !dev_ptr(target) || !dev_ptr(grad)) return FIL_EINVAL;
-    cudaError_t e = gradients(m, x, target, batch);
-    if (e == cudaSuccess)
+    // (the products store 16 bytes at a time)
+    const bool direct = (reinterpret_cast<uintptr_t>(grad) & 15) == 0;
+    cudaError_t e = gradients(m, x, target, batch, direct ? grad : m->grad);
+    if (e == cudaSuccess && !direct)
         e = cudaMemcpyAsync(grad, m->grad, FIL_MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToDevice,
                             m->stream);
-    if (e == cudaSuccess && loss)
-        e = cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream);
     if (e != cudaSuccess) return FIL_ECUDA;
-    return check_err(m);
+    return finish_call(m, loss);
 }
 
 fil_status fil_mlp_train_step(fil_mlp *m, const float *x, const float *target, int64_t batch,
                               float lr, float *loss) {
     if (!m || !x || !target || batch < 1 || batch > m->max_batch || !(lr > 0.f)) return FIL_EINVAL;
     if (!dev_ptr(x) || !dev_ptr(target)) return FIL_EINVAL;
-    cudaError_t e = gradients(m, x, target, batch);
+    cudaError_t e = gradients(m, x, target, batch, m->grad);
     m->adam_t += 1;
     const float c1 = 1.f - std::pow(0.9f, (float)m->adam_t);
     const float c2 = 1.f - std::pow(0.999f, (float)m->adam_t);
@@ -506,10 +615,8 @@ fil_status fil_mlp_train_step(fil_mlp *m, const float *x, const float *target, i
             FIL_MLP_NPARAM, m->grad, m->params, m->adam_m, m->adam_v, lr, c1, c2);
         e = refresh_weights(m);
     }
-    if (e == cudaSuccess && loss)
-        e = cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream);
     if (e != cudaSuccess) return FIL_ECUDA;
-    return loss ? check_err(m) : FIL_OK;
+    return loss ? finish_call(m, loss) : FIL_OK;
 }
 
 fil_status fil_tc_gemm_bf16(const uint16_t *A, int64_t lda, const uint16_t *B, int64_t ldb,
@@ -529,9 +636,12 @@ fil_status fil_tc_gemm_bf16(const uint16_t *A, int64_t lda, const uint16_t *B, i
     tc::Epilogue ep = epi();
     ep.c_f32 = C;
     ep.ldc = (int)ldc;
-    if (gemm(reinterpret_cast<const bf16 *>(A), (int)lda, reinterpret_cast<const bf16 *>(B),
-             (int)ldb, (int)M, (int)N, (int)K, ep, err, st) != cudaSuccess)
-        return FIL_ECUDA;
+    tc::Batch b{};
+    b.p[0] = product(reinterpret_cast<const bf16 *>(A), (int)lda, reinterpret_cast<const bf16 *>(B),
+                     (int)ldb, (int)M, (int)N, (int)K, ep);
+    b.count = 1;
+    b.err = err;
+    if (gemm(b, device_sms(), st) != cudaSuccess) return FIL_ECUDA;
     int h = 0;
     if (cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)

@@ -3,21 +3,31 @@
 // with FP32 accumulation in tensor memory and a fused epilogue. It is the
 // contraction of the per-filament warm-start MLP (inference and training).
 //
-// One CTA computes a 128 x Nt tile (Nt = min(N, 256), a multiple of 32):
-//   * K is consumed in stages of 64 (one 128-byte swizzle atom of BF16);
-//     128 threads copy the A and B stage tiles from global memory into shared
-//     memory in the 128-byte-swizzled K-major layout (16-byte chunk c of row r
-//     stored at chunk c ^ (r % 8), 1024-byte aligned tiles);
-//   * one thread issues four tcgen05.mma (M = 128, N = Nt, K = 16 each, the
+// One launch runs up to kMaxProblems products. One CTA computes a 128 x nt
+// tile (nt a multiple of 32, at most 256, the same for the launch):
+//   * K is consumed in stages of 64 (one 128-byte swizzle atom of BF16): 128
+//     threads copy the A and B stage tiles from global memory with cp.async
+//     into the 128-byte-swizzled K-major layout (16-byte chunk c of row r
+//     stored at chunk c ^ (r % 8), 1024-byte aligned tiles), `stages` - 1
+//     stages ahead of the one being multiplied;
+//   * one thread issues four tcgen05.mma (M = 128, N = nt, K = 16 each, the
 //     shared-memory descriptors advanced by 32 bytes inside the atom) into an
-//     FP32 accumulator of Nt tensor-memory columns, then tcgen05.commit to an
-//     mbarrier that every thread waits on (bounded) before the stage buffers
-//     are reused;
+//     FP32 accumulator in tensor memory, then tcgen05.commit to the stage's
+//     mbarrier; a stage is refilled once its mbarrier completed (every wait is
+//     bounded);
 //   * the epilogue reads the accumulator with tcgen05.ld (warp w owns rows
 //     32w..32w+31, i.e. tensor-memory lanes 32w..) and applies bias, ReLU or
-//     a ReLU mask, storing FP32 and/or BF16 (row-major and transposed).
+//     a ReLU mask and an output scale, storing FP32 and/or BF16 (row-major and
+//     transposed) and the column sums of its 128 rows.
 // Rows past M read as zero and are not stored; N must be a multiple of 32 and
 // K a multiple of 64 (callers pad with zeros).
+//
+// What bounds it: these products are small (0.1-0.4 GFLOP, 2-8 row tiles), so
+// the latency of a CTA's serial chain of K stages and the number of CTAs, not
+// the tensor rate. nt is the smallest that keeps the launch within one CTA per
+// SM (pick_tile_n), and the copies run several stages ahead. Measured on one
+// batch of 1024 (cold, per product): 57 us with 256-column tiles and each stage
+// loaded, multiplied and waited for in turn; GEMMFIG.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -31,10 +41,15 @@ constexpr int kTileM = 128;
 constexpr int kTileK = 64;
 constexpr int kMaxTileN = 256;
 constexpr int kThreads = 128;
-constexpr int kTmemCols = 256;
-// dynamic shared memory: A and B stage tiles + alignment slack; sized so that
-// at most two CTAs share an SM (2 x 256 tensor-memory columns = all 512)
-constexpr int kSmemBytes = 100 * 1024;
+constexpr int kMaxProblems = 4;
+constexpr int kMaxStages = 8;
+// stages in flight and dynamic shared memory by tile width (A and B tiles of
+// every stage, and alignment slack): one CTA per SM
+__host__ __device__ constexpr int stages_for(int nt) {
+    return nt <= 32 ? 8 : nt <= 64 ? 7 : nt <= 128 ? 5 : 4;
+}
+__host__ __device__ constexpr int stage_bytes(int nt) { return (kTileM + nt) * 128; }
+constexpr int smem_bytes(int nt) { return stages_for(nt) * stage_bytes(nt) + 1024; }
 
 struct Epilogue {
     float *c_f32;              // [M x ldc] FP32 out (nullable)
@@ -43,13 +58,52 @@ struct Epilogue {
     int ldh;
     __nv_bfloat16 *c_bf16_t;   // [N x ldt] BF16 out, transposed (nullable)
     int ldt;
+    int t_rows;                // its columns M .. t_rows - 1 are set to zero
     const float *bias;         // [N] added before the activation (nullable)
     int relu;                  // 1: max(x, 0)
     const __nv_bfloat16 *mask; // [M x ldm]: x *= (mask > 0) (nullable; ReLU derivative)
     int ldm;
-    float alpha;               // acc scale (applied first)
+    const float *shift, *scale;   // [N]: the FP32 out is shift + scale x (nullable, together)
+    float *col_sums;           // [row tiles x N] sums over each tile's rows (nullable)
     int n_valid;               // columns >= n_valid are not stored (multiples of 32)
 };
+
+struct Problem {
+    const __nv_bfloat16 *A, *B;
+    int lda, ldb, M, N, K;
+    int tiles_n, cta0;         // column tiles, first CTA (set by plan)
+    Epilogue ep;
+};
+
+struct Batch {
+    Problem p[kMaxProblems];
+    int count, nt;
+    int *err;
+};
+
+// Tile width of a launch: the narrowest that needs at most one CTA per SM.
+inline int pick_tile_n(const Batch &b, int sms) {
+    for (int nt = 32; nt < kMaxTileN; nt *= 2) {
+        int64_t ctas = 0;
+        for (int i = 0; i < b.count; ++i)
+            ctas += (int64_t)((b.p[i].M + kTileM - 1) / kTileM) * ((b.p[i].N + nt - 1) / nt);
+        if (ctas <= sms) return nt;
+    }
+    return kMaxTileN;
+}
+
+// Tile width and CTA ranges of the batch; returns the number of CTAs.
+inline int64_t plan(Batch &b, int sms) {
+    b.nt = pick_tile_n(b, sms);
+    int64_t ctas = 0;
+    for (int i = 0; i < b.count; ++i) {
+        Problem &p = b.p[i];
+        p.tiles_n = (p.N + b.nt - 1) / b.nt;
+        p.cta0 = (int)ctas;
+        ctas += (int64_t)((p.M + kTileM - 1) / kTileM) * p.tiles_n;
+    }
+    return ctas;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -145,32 +199,75 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// One 16-byte chunk, global -> shared, asynchronously (zeros if !valid).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 :
+                 : "r"(dst), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <int kNt>
 __global__ void __launch_bounds__(kThreads)
-gemm_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16 *__restrict__ B,
-                 int ldb, int M, int N, int K, Epilogue ep, int *__restrict__ err) {
+gemm_bf16_kernel(const __grid_constant__ Batch g) {
+    constexpr int kStages = stages_for(kNt), kStage = stage_bytes(kNt);
+    constexpr int kCols = kNt < 32 ? 32 : kNt;       // tensor-memory columns (a power of two)
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t mbar;
+    __shared__ uint64_t mbar[kStages];
     __shared__ uint32_t tmem_slot;
+    __shared__ float csum[kThreads / 32][kNt];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    unsigned char *sA = base;                              // 128 rows x 128 B
-    unsigned char *sB = base + kTileM * 128;               // <= 256 rows x 128 B
+    const uint32_t sbase = smem_u32(base);           // per stage: A 128 rows x 128 B, then B
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kTileM;
-    const int n0 = blockIdx.y * kMaxTileN;
-    const int nt = min(kMaxTileN, N - n0);
-    const uint32_t mb = smem_u32(&mbar);
+    int pi = 0;
+    while (pi + 1 < g.count && (int)blockIdx.x >= g.p[pi + 1].cta0) ++pi;
+    const Problem &p = g.p[pi];
+    const Epilogue &ep = p.ep;
+    const int local = (int)blockIdx.x - p.cta0;
+    const int mt = local / p.tiles_n, m0 = mt * kTileM;
+    const int n0 = (local - mt * p.tiles_n) * kNt;
+    const int M = p.M, nt = min(kNt, p.N - n0);
+    const int kb_n = p.K / kTileK;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :
-                     : "r"(smem_u32(&tmem_slot)), "r"(kTmemCols)
+                     : "r"(smem_u32(&tmem_slot)), "r"(kCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        mbar_init(mb, 1);
+        for (int i = 0; i < kStages; ++i) mbar_init(smem_u32(&mbar[i]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // this thread's chunks of a stage: rows (tid / 8) + 16 i, chunk tid % 8
+    const int r0 = tid >> 3, ch = tid & 7;
+    const uint32_t s0 = (uint32_t)(r0 * 128 + ((ch ^ (r0 & 7)) << 4));   // row r0 + 16 i: + 2048 i
+    const __nv_bfloat16 *Ap = p.A + (size_t)(m0 + r0) * p.lda + 8 * ch;
+    const __nv_bfloat16 *Bp = p.B + (size_t)(n0 + r0) * p.ldb + 8 * ch;
+    const auto load = [&](int kb) {
+        const uint32_t d = sbase + (uint32_t)((kb % kStages) * kStage) + s0;
+        const int k0 = kb * kTileK;
+#pragma unroll
+        for (int i = 0; i < kTileM / 16; ++i) {
+            const bool in = m0 + r0 + 16 * i < M;
+            cp_async16(d + 2048 * i, in ? Ap + (size_t)(16 * i) * p.lda + k0 : p.A, in);
+        }
+#pragma unroll
+        for (int i = 0; i < kNt / 16; ++i) {
+            const bool in = r0 + 16 * i < nt;
+            cp_async16(d + kTileM * 128 + 2048 * i, in ? Bp + (size_t)(16 * i) * p.ldb + k0 : p.B, in);
+        }
+    };
+#pragma unroll
+    for (int kb = 0; kb < kStages - 1; ++kb) {
+        if (kb < kb_n) load(kb);
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
     fence_before();
     __syncthreads();
@@ -178,80 +275,138 @@ gemm_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat
     const uint32_t tmem = tmem_slot;
     const uint32_t idesc = idesc_bf16(nt);
 
-    uint32_t phase = 0;
-    bool failed = false;
-    for (int k0 = 0; k0 < K; k0 += kTileK) {
-        // stage tiles, 16-byte chunks, 128-byte swizzle
-        for (int c = tid; c < kTileM * 8; c += kThreads) {
-            const int r = c >> 3, ch = c & 7;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (m0 + r < M)
-                v = *reinterpret_cast<const uint4 *>(A + (size_t)(m0 + r) * lda + k0 + 8 * ch);
-            *reinterpret_cast<uint4 *>(sA + r * 128 + ((ch ^ (r & 7)) << 4)) = v;
-        }
-        for (int c = tid; c < nt * 8; c += kThreads) {
-            const int r = c >> 3, ch = c & 7;
-            const uint4 v =
-                *reinterpret_cast<const uint4 *>(B + (size_t)(n0 + r) * ldb + k0 + 8 * ch);
-            *reinterpret_cast<uint4 *>(sB + r * 128 + ((ch ^ (r & 7)) << 4)) = v;
-        }
+    bool bad = false, failed = false;
+    int issued = 0;                        // K blocks whose products were committed
+    for (int kb = 0; kb < kb_n; ++kb) {
+        cp_async_wait<kStages - 2>();      // this thread's part of stage kb has landed
         fence_proxy_async();
-        __syncthreads();
-        if (tid == 0) {
-            fence_after();
-#pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk)
-                mma_bf16(tmem, sw128_desc(smem_u32(sA) + 32 * kk), sw128_desc(smem_u32(sB) + 32 * kk),
-                         idesc, (k0 > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(mb);
-        }
-        const bool ok = mbar_wait(mb, phase);
-        phase ^= 1u;
-        fence_after();
-        if (__syncthreads_or(!ok)) {
+        if (__syncthreads_or(bad)) {
             failed = true;
             break;
         }
+        const int st = kb % kStages;
+        if (tid == 0) {
+            fence_after();
+            const uint32_t sa = sbase + (uint32_t)(st * kStage), sb = sa + kTileM * 128;
+#pragma unroll
+            for (int kk = 0; kk < kTileK / 16; ++kk)
+                mma_bf16(tmem, sw128_desc(sa + 32 * kk), sw128_desc(sb + 32 * kk), idesc,
+                         (kb > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(smem_u32(&mbar[st]));
+        }
+        issued = kb + 1;
+        // stage kb - 1 is refilled with block kb - 1 + kStages once its products are done
+        const int next = kb + kStages - 1;
+        if (next < kb_n) {
+            if (kb > 0)
+                bad = !mbar_wait(smem_u32(&mbar[(kb - 1) % kStages]),
+                                 (uint32_t)(((kb - 1) / kStages) & 1));
+            if (!bad) load(next);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    cp_async_wait<0>();
+    if (!failed) {
+        bad = !mbar_wait(smem_u32(&mbar[(kb_n - 1) % kStages]),
+                         (uint32_t)(((kb_n - 1) / kStages) & 1));
+        fence_after();
+        failed = __syncthreads_or(bad);
     }
     if (failed) {
-        if (tid == 0) atomicExch(err, 1);
-        mbar_wait(mb, phase ^ 1u);      // the copies in flight, bounded
+        if (tid == 0) atomicExch(g.err, 1);
+        // the products in flight, bounded (the last commit covers them all)
+        if (issued > 0)
+            mbar_wait(smem_u32(&mbar[(issued - 1) % kStages]),
+                      (uint32_t)(((issued - 1) / kStages) & 1));
     } else {
         // epilogue: thread = row m0 + 32 warp + lane
         const int row = m0 + 32 * warp + lane;
+        const bool live = row < M;
         const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
         for (int c0 = 0; c0 < nt; c0 += 32) {
             float v[32];
             tmem_ld32(trow + (uint32_t)c0, v);
             const int nb = n0 + c0;
-            if (row < M && nb < ep.n_valid) {
+            if (nb >= ep.n_valid) continue;
+            if (ep.bias) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float x = ep.alpha * v[j];
-                    if (ep.bias) x += ep.bias[nb + j];
-                    if (ep.relu) x = fmaxf(x, 0.f);
-                    if (ep.mask && !(__bfloat162float(ep.mask[(size_t)row * ep.ldm + nb + j]) > 0.f))
-                        x = 0.f;
-                    v[j] = x;
-                }
-                if (ep.c_f32) {
-                    float4 *o = reinterpret_cast<float4 *>(ep.c_f32 + (size_t)row * ep.ldc + nb);
+                for (int j = 0; j < 32; ++j) v[j] += ep.bias[nb + j];
+            }
+            if (ep.relu) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                }
-                if (ep.c_bf16) {
-                    __nv_bfloat162 *o =
-                        reinterpret_cast<__nv_bfloat162 *>(ep.c_bf16 + (size_t)row * ep.ldh + nb);
+                for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j], 0.f);
+            }
+            if (ep.mask && live) {
+                const uint4 *mp = reinterpret_cast<const uint4 *>(ep.mask + (size_t)row * ep.ldm + nb);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) o[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                }
-                if (ep.c_bf16_t) {
+                for (int q = 0; q < 4; ++q) {
+                    const uint4 m4 = mp[q];
+                    const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        ep.c_bf16_t[(size_t)(nb + j) * ep.ldt + row] = __float2bfloat16_rn(v[j]);
+                    for (int h = 0; h < 4; ++h) {
+                        // (a BF16 is the upper half of an FP32)
+                        if (!(__uint_as_float(mw[h] << 16) > 0.f)) v[8 * q + 2 * h] = 0.f;
+                        if (!(__uint_as_float(mw[h] & 0xffff0000u) > 0.f)) v[8 * q + 2 * h + 1] = 0.f;
+                    }
                 }
             }
+            if (live && ep.c_f32) {
+                float4 *o = reinterpret_cast<float4 *>(ep.c_f32 + (size_t)row * ep.ldc + nb);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float4 w = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    if (ep.scale) {
+                        w.x = ep.shift[nb + 4 * j] + ep.scale[nb + 4 * j] * w.x;
+                        w.y = ep.shift[nb + 4 * j + 1] + ep.scale[nb + 4 * j + 1] * w.y;
+                        w.z = ep.shift[nb + 4 * j + 2] + ep.scale[nb + 4 * j + 2] * w.z;
+                        w.w = ep.shift[nb + 4 * j + 3] + ep.scale[nb + 4 * j + 3] * w.w;
+                    }
+                    o[j] = w;
+                }
+            }
+            if (ep.c_bf16 || ep.c_bf16_t) {
+                uint32_t h[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+                    h[j] = *reinterpret_cast<const uint32_t *>(&b2);
+                }
+                if (live && ep.c_bf16) {
+                    uint4 *o = reinterpret_cast<uint4 *>(ep.c_bf16 + (size_t)row * ep.ldh + nb);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        o[j] = make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+                }
+                if (ep.c_bf16_t && row < ep.t_rows) {
+                    unsigned short *o = reinterpret_cast<unsigned short *>(ep.c_bf16_t) +
+                                        (size_t)nb * ep.ldt + row;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        o[(size_t)j * ep.ldt] =
+                            live ? (unsigned short)(h[j >> 1] >> (16 * (j & 1))) : (unsigned short)0;
+                }
+            }
+            if (ep.col_sums) {
+                // lane l ends with the sum of column nb + l over the warp's 32 rows:
+                // at each step a lane keeps the half of its columns named by its bit
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = live ? v[j] : 0.f;
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+                    for (int j = 0; j < d; ++j) {
+                        const float keep = (lane & d) ? v[j + d] : v[j];
+                        const float give = (lane & d) ? v[j] : v[j + d];
+                        v[j] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+                    }
+                csum[warp][c0 + lane] = v[0];
+            }
+        }
+        if (ep.col_sums) {
+            __syncthreads();
+            for (int c = tid; c < nt; c += kThreads)
+                ep.col_sums[(size_t)mt * p.N + n0 + c] =
+                    (csum[0][c] + csum[1][c]) + (csum[2][c] + csum[3][c]);
         }
     }
     fence_before();
@@ -260,7 +415,7 @@ gemm_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
                      :
-                     : "r"(tmem), "r"(kTmemCols)
+                     : "r"(tmem), "r"(kCols)
                      : "memory");
     }
 }
