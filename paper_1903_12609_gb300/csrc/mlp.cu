@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
 #include <vector>
 
 #include "../../include/fil_mlp.h"
@@ -58,8 +59,27 @@ tc::Epilogue epi() {
 }
 
 tc::Problem product(const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N, int K,
-                    const tc::Epilogue &ep) {
-    return tc::Problem{A, B, lda, ldb, M, N, K, 0, 0, ep};
+                    const tc::Epilogue &ep, bool weights = false) {
+    return tc::Problem{A, B, lda, ldb, M, N, K, 0, 0, weights ? 1 : 0, ep};
+}
+
+// A launch whose prologue may overlap the kernel before it in the stream (both
+// call pdl_wait_previous / pdl_launch_next): the calls are chains of 5 and 10
+// kernels of a few microseconds, and each gap between two costs about as much.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
+                       cudaStream_t st, Args &&...args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 template <int kNt>
@@ -68,8 +88,8 @@ cudaError_t launch_gemm(const tc::Batch &b, int64_t ctas, cudaStream_t st) {
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                tc::smem_bytes(kNt));
     if (e != cudaSuccess) return e;
-    tc::gemm_bf16_kernel<kNt><<<(unsigned)ctas, tc::kThreads, tc::smem_bytes(kNt), st>>>(b);
-    return cudaGetLastError();
+    return launch_pdl(tc::gemm_bf16_kernel<kNt>, dim3((unsigned)ctas), tc::kThreads,
+                      tc::smem_bytes(kNt), st, b);
 }
 
 // The products of a batch in one launch.
@@ -107,6 +127,7 @@ __global__ void __launch_bounds__(kInThreads)
 input_kernel(const float *__restrict__ x, int64_t B, const float *__restrict__ mean,
              const float *__restrict__ stdv, bf16 *__restrict__ X, bf16 *__restrict__ Xt,
              int64_t ldt, int64_t Kb) {
+    tc::pdl_launch_next();
     const int c = blockIdx.x * kInThreads + threadIdx.x;
     const int64_t b0 = (int64_t)blockIdx.y * kRows;
     const bool in = c < kIn;
@@ -147,6 +168,8 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
             bf16 *__restrict__ dYt, int64_t ldt, int64_t Kb, float *__restrict__ col_sums,
             double *__restrict__ part, int n_part) {
     __shared__ double red[kLossThreads / 32];
+    tc::pdl_launch_next();
+    tc::pdl_wait_previous();
     const int c = threadIdx.x;
     const int64_t b0 = (int64_t)blockIdx.x * kRows;
     const float inv = 1.f / (float)B, mu = mean[c], sd = stdv[c];
@@ -199,6 +222,7 @@ struct BiasParts {
 };
 __global__ void finish_kernel(BiasParts bp, const double *__restrict__ part, int n_part, double B,
                               float *__restrict__ loss) {
+    tc::pdl_wait_previous();
     const int l = blockIdx.y, c = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = l < 3 ? kHid : kOut;
     if (c < N) {
@@ -377,7 +401,8 @@ cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train, float *y)
         }
         ep.bias = m->params + m->off.b[l];
         ep.relu = 1;
-        e = one_product(m, product(act, ld, m->W[l], kDimInP[l], (int)B, kHid, kDimInP[l], ep));
+        e = one_product(m, product(act, ld, m->W[l], kDimInP[l], (int)B, kHid, kDimInP[l], ep,
+                                   true));
         if (e != cudaSuccess) return e;
         act = m->H[l];
         ld = kHid;
@@ -390,7 +415,7 @@ cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train, float *y)
         ep.shift = m->out_mean;
         ep.scale = m->out_std;
     }
-    return one_product(m, product(act, ld, m->W[3], kHid, (int)B, kOut, kHid, ep));
+    return one_product(m, product(act, ld, m->W[3], kHid, (int)B, kOut, kHid, ep, true));
 }
 
 // Outputs in raw units to y: straight from the last product where its 16-byte
@@ -416,10 +441,9 @@ cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B, flo
     if (e != cudaSuccess) return e;
     const int loss_ctas = (int)((Kb + kRows - 1) / kRows);
     const int loss_parts = (int)((B + kRows - 1) / kRows);
-    loss_kernel<<<loss_ctas, kLossThreads, 0, m->stream>>>(m->Y, t, B, m->out_mean, m->out_std,
-                                                           m->dY, m->dYt, m->ldt, Kb, m->sums[3],
-                                                           m->loss_part, loss_parts);
-    e = cudaGetLastError();
+    e = launch_pdl(loss_kernel, dim3((unsigned)loss_ctas), kLossThreads, 0, m->stream,
+                   (const float *)m->Y, t, B, (const float *)m->out_mean, (const float *)m->out_std,
+                   m->dY, m->dYt, m->ldt, Kb, m->sums[3], m->loss_part, loss_parts);
     if (e != cudaSuccess) return e;
     // dH_{l-1} = (dZ_l W_l) * [H_{l-1} > 0], with its column sums
     const bf16 *dZ = m->dY;
@@ -434,7 +458,8 @@ cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B, flo
         eb.mask = m->H[l - 1];
         eb.ldm = kHid;
         eb.col_sums = m->sums[l - 1];
-        e = one_product(m, product(dZ, ldz, m->Wt[l], kDimOut[l], (int)B, kHid, kDimOut[l], eb));
+        e = one_product(m, product(dZ, ldz, m->Wt[l], kDimOut[l], (int)B, kHid, kDimOut[l], eb,
+                                   true));
         if (e != cudaSuccess) return e;
         dZ = m->dH[l - 1];
         ldz = kHid;
@@ -459,9 +484,8 @@ cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B, flo
         bp.n[l] = l < 3 ? (int)((B + tc::kTileM - 1) / tc::kTileM) : loss_parts;
         bp.db[l] = grad + m->off.b[l];
     }
-    finish_kernel<<<dim3(kHid / 64, kLayers), 64, 0, m->stream>>>(bp, m->loss_part, loss_parts,
-                                                                 (double)B, m->loss);
-    return cudaGetLastError();
+    return launch_pdl(finish_kernel, dim3(kHid / 64, kLayers), 64, 0, m->stream, bp,
+                      (const double *)m->loss_part, loss_parts, (double)B, m->loss);
 }
 
 // Waits for the stream; FIL_ECUDA if a wait in a product ran out. The loss, when

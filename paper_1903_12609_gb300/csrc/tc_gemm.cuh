@@ -72,6 +72,7 @@ struct Problem {
     const __nv_bfloat16 *A, *B;
     int lda, ldb, M, N, K;
     int tiles_n, cta0;         // column tiles, first CTA (set by plan)
+    int b_ready;               // B was complete before the launch's predecessor (weights)
     Epilogue ep;
 };
 
@@ -211,6 +212,16 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// Programmatic dependent launch: the next kernel of the stream may start its
+// prologue now / wait here until the previous kernel is complete and its writes
+// are visible. Nothing before the wait may read what that kernel writes.
+__device__ __forceinline__ void pdl_launch_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <int kNt>
 __global__ void __launch_bounds__(kThreads)
 gemm_bf16_kernel(const __grid_constant__ Batch g) {
@@ -250,7 +261,7 @@ gemm_bf16_kernel(const __grid_constant__ Batch g) {
     const uint32_t s0 = (uint32_t)(r0 * 128 + ((ch ^ (r0 & 7)) << 4));   // row r0 + 16 i: + 2048 i
     const __nv_bfloat16 *Ap = p.A + (size_t)(m0 + r0) * p.lda + 8 * ch;
     const __nv_bfloat16 *Bp = p.B + (size_t)(n0 + r0) * p.ldb + 8 * ch;
-    const auto load = [&](int kb) {
+    const auto load_a = [&](int kb) {
         const uint32_t d = sbase + (uint32_t)((kb % kStages) * kStage) + s0;
         const int k0 = kb * kTileK;
 #pragma unroll
@@ -258,15 +269,27 @@ gemm_bf16_kernel(const __grid_constant__ Batch g) {
             const bool in = m0 + r0 + 16 * i < M;
             cp_async16(d + 2048 * i, in ? Ap + (size_t)(16 * i) * p.lda + k0 : p.A, in);
         }
+    };
+    const auto load_b = [&](int kb) {
+        const uint32_t d = sbase + (uint32_t)((kb % kStages) * kStage) + s0 + kTileM * 128;
+        const int k0 = kb * kTileK;
 #pragma unroll
         for (int i = 0; i < kNt / 16; ++i) {
             const bool in = r0 + 16 * i < nt;
-            cp_async16(d + kTileM * 128 + 2048 * i, in ? Bp + (size_t)(16 * i) * p.ldb + k0 : p.B, in);
+            cp_async16(d + 2048 * i, in ? Bp + (size_t)(16 * i) * p.ldb + k0 : p.B, in);
         }
     };
+    // the first stages; weights are copied while the previous kernel still runs
+    pdl_launch_next();
+    if (p.b_ready)
+        for (int kb = 0; kb < min(kStages - 1, kb_n); ++kb) load_b(kb);
+    pdl_wait_previous();
 #pragma unroll
     for (int kb = 0; kb < kStages - 1; ++kb) {
-        if (kb < kb_n) load(kb);
+        if (kb < kb_n) {
+            load_a(kb);
+            if (!p.b_ready) load_b(kb);
+        }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     fence_before();
@@ -301,7 +324,10 @@ gemm_bf16_kernel(const __grid_constant__ Batch g) {
             if (kb > 0)
                 bad = !mbar_wait(smem_u32(&mbar[(kb - 1) % kStages]),
                                  (uint32_t)(((kb - 1) / kStages) & 1));
-            if (!bad) load(next);
+            if (!bad) {
+                load_a(next);
+                load_b(next);
+            }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
