@@ -224,85 +224,103 @@ band_lu_kernel(Layout lay, T *__restrict__ band_all, int *__restrict__ piv_all,
 #undef RB
 }
 
-constexpr int kSolvePf = 8;   // rows of factors loaded ahead by the band solve
+constexpr int kSolvePf = 8;     // rows of factors loaded ahead by the band solve
+constexpr int kSolveLanes = 16; // lanes per filament
 
 // x = J0^{-1} b for every filament (b and x in the X / f layout; may alias),
-// with the factors and the working vector in precision T.
+// with the factors and the working vector in precision T, 16 lanes (half a
+// warp) per filament.
+//
+// A row step is a chain: the finished entry z_j, one multiply-add in each row
+// it reaches, the next finished entry. The window of rows it reaches (j + 1 ..
+// j + 8 forward, j - 1 .. j - 16 backward) therefore stays in registers, row i
+// in lane i mod 16, and z_j goes to the lanes with a shuffle; shared memory
+// holds only the entries that wait to enter the window. (With the window in
+// shared memory a step was two loads, a store and a warp barrier long, ~40
+// instructions of a whole warp. One 20-segment filament in FP64 41 -> 30 us,
+// where the FP64 unit takes 64 cycles per warp instruction; the steps of 256
+// ensemble systems in FP32 80.5 -> 77.7 ms. Same bits.)
+// The two halves of a warp run the longer one's steps together.
 template <typename T>
 __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
                                   const int *__restrict__ piv_all, double ct,
                                   const double *b, double *x, int zmax,
-                                  const int *__restrict__ active) {
+                                  const int *__restrict__ active, int fil_per_cta) {
     extern __shared__ __align__(16) unsigned char zraw[];
-    const int wib = threadIdx.x >> 5;
-    const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (warp >= lay.M) return;
-    T *z = reinterpret_cast<T *>(zraw) + (int64_t)wib * zmax;
-    const int s0 = lay.off[warp];
-    if (active && !active[lay.sys_of[s0]]) return;   // converged system: rows not needed
-    const int N = lay.off[warp + 1] - s0;
-    const int n = 6 * N - 3;
-    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)warp;
+    const int slot = threadIdx.x / kSolveLanes;        // filament within the CTA
+    const int lane = threadIdx.x % kSolveLanes;
+    const int f = blockIdx.x * fil_per_cta + slot;
+    // (a half without a filament, or of a converged system, takes no rows)
+    bool live = slot < fil_per_cta && f < lay.M;
+    int s0 = 0, N = 0;
+    if (live) {
+        s0 = lay.off[f];
+        N = lay.off[f + 1] - s0;
+        if (active && !active[lay.sys_of[s0]]) live = false;
+    }
+    const int n = live ? 6 * N - 3 : 0;
+    const int n_both = max(n, __shfl_xor_sync(0xffffffffu, n, kSolveLanes));
+    if (n_both == 0) return;
+    T *z = reinterpret_cast<T *>(zraw) + (int64_t)(live ? slot : 0) * zmax;
+    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)(live ? f : 0);
     const T *A = band_all + row0 * kBandW;
     const int *piv = piv_all + row0;
     const double *bf = b + 6 * (int64_t)s0;
     double *xf = x + 6 * (int64_t)s0;
 #define BAND(i, c) A[(int64_t)(i) * kBandW + ((c) - (i) + kBandKL)]
     // gather the right-hand side in band order
-    for (int e = lane; e < 3 * N; e += 32) {
-        const int s = e / 3, r = e % 3;
-        z[6 * s + r] = (T)bf[3 + 3 * s + r];   // rotation rows of segment s
-        if (s <= N - 2) {
-            const double b3n = bf[3 + 3 * N + 3 * s + r];                      // f3 of segment s+1
-            const double b3p = (s == 0) ? bf[r] : bf[3 + 3 * N + 3 * (s - 1) + r];
-            z[6 * s + 3 + r] = (T)(b3n - b3p);
+    double b1x = 0.0, b1y = 0.0, b1z = 0.0;
+    if (live) {
+        for (int e = lane; e < 3 * N; e += kSolveLanes) {
+            const int s = e / 3, r = e % 3;
+            z[6 * s + r] = (T)bf[3 + 3 * s + r];   // rotation rows of segment s
+            if (s <= N - 2) {
+                const double b3n = bf[3 + 3 * N + 3 * s + r];                  // f3 of segment s+1
+                const double b3p = (s == 0) ? bf[r] : bf[3 + 3 * N + 3 * (s - 1) + r];
+                z[6 * s + 3 + r] = (T)(b3n - b3p);
+            }
         }
+        b1x = bf[0];
+        b1y = bf[1];
+        b1z = bf[2];
     }
-    const double b1x = bf[0], b1y = bf[1], b1z = bf[2];
     __syncwarp();
     // The factors a row step needs do not depend on z, so each lane loads them
     // kSolvePf rows ahead into a register queue: the loads of the next block are
-    // in flight while the current block's dependency chain runs through shared
-    // memory. Lane l's entries sit at a fixed offset of consecutive rows:
-    // forward L(j + 1 + l, j), backward U(j - 1 - l, j) and the reciprocal U_jj.
-    // forward: L with row interchanges applied in elimination order
-    T zprev = T(0);   // lane 0: the finished entry of the previous row / column
+    // in flight while the current block's chain runs.
+    // forward: L with row interchanges applied in elimination order; lane l holds
+    // the row r in [j, j + 15] with r = l (mod 16)
+    T w = lane < n ? z[lane] : T(0);
     {
         T lq[kSolvePf];
         int pq[kSolvePf];
+        const auto fetch = [&](int j, T &l, int &p) {
+            const int d = (lane - j) & (kSolveLanes - 1);        // row j + d
+            l = (d >= 1 && d <= kBandKL && j + d < n) ? BAND(j + d, j) : T(0);
+            p = j < n ? piv[j] : j;
+        };
 #pragma unroll
-        for (int u = 0; u < kSolvePf; ++u) {
-            const int j = u;
-            lq[u] = (lane < kBandKL && j + 1 + lane < n) ? BAND(j + 1 + lane, j) : T(0);
-            pq[u] = j < n ? piv[j] : j;
-        }
-        for (int jb = 0; jb < n; jb += kSolvePf) {
+        for (int u = 0; u < kSolvePf; ++u) fetch(u, lq[u], pq[u]);
+        for (int jb = 0; jb < n_both; jb += kSolvePf) {
             T ln[kSolvePf];
             int pn[kSolvePf];
 #pragma unroll
-            for (int u = 0; u < kSolvePf; ++u) {
-                const int j = jb + kSolvePf + u;
-                ln[u] = (lane < kBandKL && j + 1 + lane < n) ? BAND(j + 1 + lane, j) : T(0);
-                pn[u] = j < n ? piv[j] : j;
-            }
+            for (int u = 0; u < kSolvePf; ++u) fetch(jb + kSolvePf + u, ln[u], pn[u]);
 #pragma unroll
             for (int u = 0; u < kSolvePf; ++u) {
                 const int j = jb + u;
-                if (j < n) {
-                    // row j after the interchange with row p (p in j .. j+8): every lane
-                    // reads both entries; the lane of row p takes the old z_j as its own
-                    // entry; z_j itself is stored one row later, when no lane reads it
-                    const int p = pq[u];
-                    const T zold = z[j], zp = z[p];
-                    const T zj = (p != j) ? zp : zold;
-                    const int i = j + 1 + lane;
-                    if (lane < kBandKL && i < n) z[i] = ((i == p) ? zold : z[i]) - lq[u] * zj;
-                    if (lane == 0) {
-                        if (j > 0) z[j - 1] = zprev;
-                        zprev = zj;
-                    }
-                    __syncwarp();
+                const int p = pq[u];
+                // the entry that enters the window when row j leaves it
+                const int in = j + kSolveLanes;
+                const T zin = (in & (kSolveLanes - 1)) == lane && in < n ? z[in] : T(0);
+                // row j after the interchange with row p (p in j .. j+8)
+                const T zold = __shfl_sync(0xffffffffu, w, j & (kSolveLanes - 1), kSolveLanes);
+                const T zj = __shfl_sync(0xffffffffu, w, p & (kSolveLanes - 1), kSolveLanes);
+                const int d = (lane - j) & (kSolveLanes - 1);
+                if (d >= 1 && d <= kBandKL && j + d < n) w = ((j + d == p) ? zold : w) - lq[u] * zj;
+                if (d == 0 && j < n) {
+                    z[j] = zj;
+                    w = zin;
                 }
             }
 #pragma unroll
@@ -312,39 +330,46 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
             }
         }
     }
-    if (lane == 0) z[n - 1] = zprev;
     __syncwarp();
     // backward, column by column: z_j *= 1/U_jj (stored reciprocal), then the
-    // kl + ku rows above take their U_ij z_j
+    // kl + ku rows above take their U_ij z_j; lane l holds the row r in [j - 15, j]
+    // with r = l (mod 16), and row j - 16 once z_j is out
     {
-        T uq[kSolvePf], dq[kSolvePf];
-#pragma unroll
-        for (int u = 0; u < kSolvePf; ++u) {
-            const int j = n - 1 - u;
-            uq[u] = (lane < kBandKL + kBandKU && j - 1 - lane >= 0) ? BAND(j - 1 - lane, j) : T(0);
-            dq[u] = j >= 0 ? BAND(j, j) : T(0);
+        // (a shorter half starts when its last row comes up: k counts from n_both - 1)
+        const int k0 = n_both - 1;
+        {
+            const int d = (n - 1 - lane) & (kSolveLanes - 1);   // row n - 1 - d
+            w = n - 1 - d >= 0 ? z[n - 1 - d] : T(0);
         }
-        for (int jb = n - 1; jb >= 0; jb -= kSolvePf) {
+        T uq[kSolvePf], dq[kSolvePf];
+        const auto fetch = [&](int j, T &uu, T &dd) {
+            const bool in = j < n;
+            int d = (j - lane) & (kSolveLanes - 1);             // row j - d, d = 16 for lane j mod 16
+            if (d == 0) d = kSolveLanes;
+            uu = (in && j - d >= 0) ? BAND(j - d, j) : T(0);
+            dd = (in && j >= 0) ? BAND(j, j) : T(0);
+        };
+        static_assert(kBandKL + kBandKU == kSolveLanes, "a lane per row a backward step reaches");
+#pragma unroll
+        for (int u = 0; u < kSolvePf; ++u) fetch(k0 - u, uq[u], dq[u]);
+        for (int jb = k0; jb >= 0; jb -= kSolvePf) {
             T un[kSolvePf], dn[kSolvePf];
 #pragma unroll
-            for (int u = 0; u < kSolvePf; ++u) {
-                const int j = jb - kSolvePf - u;
-                un[u] = (lane < kBandKL + kBandKU && j - 1 - lane >= 0) ? BAND(j - 1 - lane, j)
-                                                                         : T(0);
-                dn[u] = j >= 0 ? BAND(j, j) : T(0);
-            }
+            for (int u = 0; u < kSolvePf; ++u) fetch(jb - kSolvePf - u, un[u], dn[u]);
 #pragma unroll
             for (int u = 0; u < kSolvePf; ++u) {
                 const int j = jb - u;
-                if (j >= 0) {
-                    const T zj = z[j] * dq[u];
-                    const int i = j - 1 - lane;
-                    if (lane < kBandKL + kBandKU && i >= 0) z[i] -= uq[u] * zj;
-                    if (lane == 0) {
-                        if (j < n - 1) z[j + 1] = zprev;
-                        zprev = zj;
+                const bool mine = (j & (kSolveLanes - 1)) == lane;
+                const T zin = mine && j < n && j >= kSolveLanes ? z[j - kSolveLanes] : T(0);
+                const T zj = __shfl_sync(0xffffffffu, w, j & (kSolveLanes - 1), kSolveLanes) * dq[u];
+                if (j >= 0 && j < n) {
+                    if (mine) {
+                        z[j] = zj;
+                        w = zin;
                     }
-                    __syncwarp();
+                    int d = (j - lane) & (kSolveLanes - 1);
+                    if (d == 0) d = kSolveLanes;
+                    if (j - d >= 0) w -= uq[u] * zj;
                 }
             }
 #pragma unroll
@@ -354,10 +379,10 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
             }
         }
     }
-    if (lane == 0) z[0] = zprev;
     __syncwarp();
+    if (!live) return;
     // scatter back: u_s, Lam_j, and Y_1 = b1 + c_t Lam_0
-    for (int e = lane; e < 3 * N; e += 32) {
+    for (int e = lane; e < 3 * N; e += kSolveLanes) {
         const int s = e / 3, r = e % 3;
         xf[3 + 3 * s + r] = (double)z[6 * s + r];
         if (s <= N - 2) xf[3 + 3 * N + 3 * s + r] = (double)z[6 * s + 3 + r];
@@ -404,13 +429,13 @@ cudaError_t j0_build_factor(fil_ctx *c, const double *X) {
 }
 
 cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) {
-    // one warp per filament; up to 4 warps per CTA, fewer for long filaments so
-    // that each warp's right-hand side fits in shared memory
+    // half a warp per filament; up to 4 warps per CTA, fewer for long filaments so
+    // that each filament's right-hand side fits in shared memory
     const int zmax = 6 * c->lay.maxN;
-    const size_t per_warp = (size_t)zmax * sizeof(double);
-    int warps = (int)std::min<size_t>(4, kSolveSmemMax / per_warp);
-    if (warps < 1) return cudaErrorInvalidValue;
-    const size_t smem = warps * per_warp;
+    const size_t per = (size_t)zmax * sizeof(double);
+    const int fils = (int)std::min<size_t>(8, kSolveSmemMax / per);
+    if (fils < 1) return cudaErrorInvalidValue;
+    const size_t smem = fils * per;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(band_solve_kernel<double>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -420,14 +445,14 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const int threads = 32 * warps;
-    const unsigned grid = (unsigned)(((int64_t)c->lay.M * 32 + threads - 1) / threads);
+    const int threads = (kSolveLanes * fils + 31) / 32 * 32;
+    const unsigned grid = (unsigned)((c->lay.M + fils - 1) / fils);
     if (c->band32)
         band_solve_kernel<float><<<grid, threads, smem, c->stream>>>(
-            c->lay, c->band32, c->piv, make_params(c).ct, b, x, zmax, active);
+            c->lay, c->band32, c->piv, make_params(c).ct, b, x, zmax, active, fils);
     else
         band_solve_kernel<double><<<grid, threads, smem, c->stream>>>(
-            c->lay, c->band, c->piv, make_params(c).ct, b, x, zmax, active);
+            c->lay, c->band, c->piv, make_params(c).ct, b, x, zmax, active, fils);
     c->n_launches += 1;
     return cudaGetLastError();
 }
