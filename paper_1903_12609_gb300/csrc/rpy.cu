@@ -1337,6 +1337,237 @@ rpy_pair64_kernel(const double *__restrict__ src, SysMap smap, int64_t W, int G,
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP64 applies of one system without packed records: two kernels that read the
+// caller's arrays. The FP64 unit is the bound (2 lanes per clock and SM: a warp
+// instruction takes 64 cycles of its sub-partition, whatever its lanes do), so
+// shuffles, shared memory and integer work cost nothing beside it, and what
+// counts is the FP64 instructions per pair and how evenly they are spread.
+// ---------------------------------------------------------------------------
+
+// 1/sqrt(x) for normal x > 0: the hardware's approximation (PTX
+// rsqrt.approx.ftz.f64, ~20 bits) and one step of the third-order iteration
+//   y <- y + y e (1/2 + 3/8 e),  e = 1 - x y^2
+// (the series of (1 - e)^{-1/2}), whose next term, 5/16 e^3, is below 2^-57.
+__device__ __forceinline__ double rsqrt_iter(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(fma(0.375, e, 0.5), y * e, y);
+}
+
+// Coefficients of a pair at r^2. The comparisons are on the bits (r^2 >= 0), so
+// they take no FP64 instruction; the overlapping form runs only in warps that
+// hold such a pair, from the same 1/r.
+__device__ __forceinline__ void coef64(double r2, const RpyConst64 &k, double &A, double &B,
+                                       double &C, double &D, double &G) {
+    const long long bits = __double_as_longlong(r2);
+    const bool none = bits < __double_as_longlong(1e-290);    // r = 0: 1/r taken as 0
+    const double rinv = none ? 0.0 : rsqrt_iter(r2);
+    const double rinv2 = rinv * rinv;
+    G = rinv * rinv2;
+    const double rinv5 = G * rinv2;
+    A = fma(k.k23a2, G, rinv);
+    B = fma(-k.k2a2, rinv5, G);
+    C = -0.5 * G;
+    D = 1.5 * rinv5;
+    if (bits < __double_as_longlong(k.near2)) {
+        const double r = r2 * rinv;
+        A = fma(-k.ov_A1, r, k.ov_A0);
+        B = k.ov_B * rinv;
+        C = fma(k.ov_C3 * r2, r, fma(-k.ov_C1, r, k.ov_C0));
+        D = fma(k.ov_D0, rinv, -k.ov_D1 * r);
+        G = fma(-k.ov_G1, r, k.ov_G0);
+    }
+}
+
+// acc += the (V, Omega) terms of loads (F, T) = f at difference d, with e = sg G d
+// (sg = -1 for the source of the pair: its difference is -d).
+__device__ __forceinline__ void add64(const double *f, const double *d, const double *e, double A,
+                                      double B, double C, double D, double *acc) {
+    const double bF = B * fma(d[0], f[0], fma(d[1], f[1], d[2] * f[2]));
+    const double dT = D * fma(d[0], f[3], fma(d[1], f[4], d[2] * f[5]));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int p = (c + 1) % 3, q = (c + 2) % 3;
+        acc[c] = fma(A, f[c], fma(bF, d[c], fma(f[3 + p], e[q], fma(-f[3 + q], e[p], acc[c]))));
+        acc[3 + c] = fma(C, f[3 + c], fma(dT, d[c], fma(f[p], e[q], fma(-f[q], e[p], acc[3 + c]))));
+    }
+}
+
+// Small systems: a warp per target, its lanes over the sources, one warp per
+// CTA, so that the few hundred pairs of a single filament spread over the SMs.
+// The lane sums are combined by halving: at each step a lane keeps some of its
+// components and gives the others away, 8 FP64 adds instead of 30.
+// Measured (apply on the device, packed kernel -> this): 20 segments 25 -> 9 us,
+// 256 segments 523 -> 22 us, 1024 segments 525 -> 109 us (the packed kernel gives a
+// small system's few 256 x 128 units to as few SMs).
+__global__ void __launch_bounds__(32)
+rpy_direct64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, int S,
+                    RpyConst64 k, double scale, double *__restrict__ VW) {
+    const int n = blockIdx.x, lane = threadIdx.x;
+    const double t0 = Y[3 * (int64_t)n], t1 = Y[3 * (int64_t)n + 1], t2 = Y[3 * (int64_t)n + 2];
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int m = lane; m < S; m += 32) {
+        const double *y = Y + 3 * (int64_t)m, *f = FT + 6 * (int64_t)m;
+        const double d[3] = {t0 - y[0], t1 - y[1], t2 - y[2]};
+        const double ft[6] = {f[0], f[1], f[2], f[3], f[4], f[5]};
+        double A, B, C, D, G;
+        coef64(fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2])), k, A, B, C, D, G);
+        const double e[3] = {G * d[0], G * d[1], G * d[2]};
+        add64(ft, d, e, A, B, C, D, v);
+    }
+    const unsigned all = 0xffffffffu;
+    double w[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {          // V in lanes 0-15, Omega in lanes 16-31
+        const double keep = lane & 16 ? v[3 + c] : v[c], give = lane & 16 ? v[c] : v[3 + c];
+        w[c] = keep + __shfl_xor_sync(all, give, 16);
+    }
+    // components 0, 1 where lane bit 3 is clear, component 2 where it is set
+    const double g0 = __shfl_xor_sync(all, lane & 8 ? w[0] : w[2], 8);
+    const double g1 = __shfl_xor_sync(all, w[1], 8);
+    double a = (lane & 8 ? w[2] : w[0]) + g0;
+    const double b = w[1] + g1;
+    // lane bit 2 splits components 0 and 1; component 2 is summed by both halves
+    const double g = __shfl_xor_sync(all, lane & 8 ? a : (lane & 4 ? a : b), 4);
+    a = (lane & 8 ? a : (lane & 4 ? b : a)) + g;
+    a += __shfl_xor_sync(all, a, 2);
+    a += __shfl_xor_sync(all, a, 1);
+    const int c = (lane & 16 ? 3 : 0) + (lane & 8 ? 2 : (lane & 4 ? 1 : 0));
+    if ((lane & 3) == 0 && (lane & 12) != 12) VW[6 * (int64_t)n + c] = a * scale;
+}
+
+// Medium systems: every unordered pair once. A CTA of four warps takes a pair of
+// 64-segment tiles (I <= J), a warp one 32 x 32 block: a lane keeps one segment
+// of the row block; the segments of the column block go round the lanes, their
+// sums travelling with them by shuffles, so that after 32 steps both sides of
+// every pair were added. 85 FP64 instructions for the two ordered pairs instead
+// of 106 (the difference, 1/r and the coefficients are shared). A block on the
+// diagonal takes its pairs at distance 1 .. 16 round the block, and the self
+// terms. The CTA's sums go to the rows of its two tiles in slots named by the
+// other tile, and sum64_kernel adds a row's slots in order. The CTAs are handed
+// out by the hardware as SMs come free (the cost of a block depends on its
+// overlapping pairs), the diagonal ones last.
+// Measured: 3200 segments 1476 -> 827 us (a warp per target: 1012), 4000 1976 ->
+// 1258; at 1024 both small forms take 108 us. Error against 64 bits 7e-16 -> 5e-16.
+constexpr int kSymTile = 64;
+constexpr int kSymThreads = 128;
+constexpr int64_t kSymMaxSeg = 8192;          // slots: (S / 64) x 6 S doubles
+constexpr int64_t kDirectMaxSeg = 1024;       // up to here a warp per target is faster
+
+__global__ void __launch_bounds__(kSymThreads)
+rpy_sym64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, int S, int tiles,
+                 RpyConst64 k, double *__restrict__ slots) {
+    __shared__ double sf[2][9][kSymTile];     // positions and loads of the two tiles
+    __shared__ double sums[2][2][6][kSymTile];   // [side][which of the two blocks added][...]
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // CTA -> (I, J): off-diagonal pairs row by row, then the diagonal tiles
+    const int off = tiles * (tiles - 1) / 2;
+    int I, J;
+    if ((int)blockIdx.x >= off) {
+        I = J = (int)blockIdx.x - off;
+    } else {
+        // pairs of row J (I < J) start at J (J - 1) / 2
+        J = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)blockIdx.x)) * 0.5f);
+        while (J * (J - 1) / 2 > (int)blockIdx.x) --J;
+        while ((J + 1) * J / 2 <= (int)blockIdx.x) ++J;
+        I = (int)blockIdx.x - J * (J - 1) / 2;
+    }
+    {
+        const int side = threadIdx.x >> 6, l = threadIdx.x & 63;
+        const int n = (side ? J : I) * kSymTile + l;
+        const bool in = n < S;
+        // (past the end: no load, and a place of its own far away)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            sf[side][c][l] = in ? Y[3 * (int64_t)n + c] : (double)kFarPad * (double)(2 + l + 64 * side);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) sf[side][3 + c][l] = in ? FT[6 * (int64_t)n + c] : 0.0;
+    }
+    __syncthreads();
+    const int a = wid >> 1, b = wid & 1;      // blocks of I and J
+    const bool diag = I == J;
+    const bool self = diag && a == b;
+    double vt[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, vs[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (!(diag && a > b)) {
+        double t[9];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) t[c] = sf[0][c][32 * a + lane];
+        if (self) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                vt[c] = k.ov_A0 * t[3 + c];
+                vt[3 + c] = k.ov_C0 * t[6 + c];
+            }
+        }
+        const int first = self ? 1 : 0, last = self ? 16 : 31;
+        for (int st = first; st <= last; ++st) {
+            if (st > 0) {                     // the sums of segment (lane + st) mod 32 arrive
+#pragma unroll
+                for (int c = 0; c < 6; ++c)
+                    vs[c] = __shfl_sync(0xffffffffu, vs[c], (lane + 1) & 31);
+            }
+            const int j = 32 * b + ((lane + st) & 31);
+            double f[6];
+            const double d[3] = {t[0] - sf[1][0][j], t[1] - sf[1][1][j], t[2] - sf[1][2][j]};
+#pragma unroll
+            for (int c = 0; c < 6; ++c) f[c] = sf[1][3 + c][j];
+            // (at distance 16 in a diagonal block each pair comes up twice)
+            if (!(self && st == 16 && lane >= 16)) {
+                double A, B, C, D, G;
+                coef64(fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2])), k, A, B, C, D, G);
+                const double e[3] = {G * d[0], G * d[1], G * d[2]};
+                const double ne[3] = {-e[0], -e[1], -e[2]};
+                add64(f, d, e, A, B, C, D, vt);
+                add64(t + 3, d, ne, A, B, C, D, vs);
+            }
+        }
+        // home: after `last` steps the sums of segment (lane + last) mod 32 are here
+#pragma unroll
+        for (int c = 0; c < 6; ++c) vs[c] = __shfl_sync(0xffffffffu, vs[c], (lane - last) & 31);
+    }
+    // rows of I: blocks (a, 0) and (a, 1); rows of J: blocks (0, b) and (1, b)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        sums[0][b][c][32 * a + lane] = vt[c];
+        sums[1][a][c][32 * b + lane] = vs[c];
+    }
+    __syncthreads();
+    const int64_t rows = (int64_t)tiles * kSymTile;
+    for (int i = threadIdx.x; i < 6 * kSymTile; i += kSymThreads) {
+        const int c = i / kSymTile, l = i % kSymTile;
+        const double x = sums[0][0][c][l] + sums[0][1][c][l];
+        const double y = sums[1][0][c][l] + sums[1][1][c][l];
+        if (diag) {
+            slots[((int64_t)I * 6 + c) * rows + I * kSymTile + l] = x + y;
+        } else {
+            slots[((int64_t)J * 6 + c) * rows + I * kSymTile + l] = x;
+            slots[((int64_t)I * 6 + c) * rows + J * kSymTile + l] = y;
+        }
+    }
+}
+
+// Row sums over the slots, in order.
+__global__ void __launch_bounds__(64)
+sum64_kernel(const double *__restrict__ slots, int S, int tiles, double scale,
+             double *__restrict__ VW) {
+    const int n = blockIdx.x * 64 + threadIdx.x, c = blockIdx.y;
+    if (n >= S) return;
+    const int64_t rows = (int64_t)tiles * kSymTile;
+    const double *p = slots + c * rows + n;
+    double a = 0.0;
+#pragma unroll 16
+    for (int t = 0; t < tiles; ++t) a += p[(int64_t)t * 6 * rows];
+    VW[6 * (int64_t)n + c] = a * scale;
+}
+
+// Bytes of [p, p + n) and [q, q + m) overlap.
+bool overlaps(const double *p, int64_t n, const double *q, int64_t m) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+    return a < b + 8 * (uintptr_t)m && b < a + 8 * (uintptr_t)n;
+}
+
 SysMap sys_map(const fil_ctx *c, bool active_only) {
     SysMap m{};
     m.n_src = c->lay.S;
@@ -1382,7 +1613,7 @@ cudaError_t allow_warp_smem() {
 // Tiles of T targets of every system (only tiles that hold real targets),
 // each with ceil(S_s / unit) units.
 void build_tiles(fil_ctx *c) {
-    const int T = c->rpy_auto ? kWarpTile : rpy_tile(c);
+    const int T = c->rpy_auto && c->rpy_frames ? kWarpTile : rpy_tile(c);
     const int per = unit_sources(c->rpy_frames != 0);
     c->tile_unit_off_h.assign(1, 0);
     c->tile_src_h.clear();
@@ -1457,8 +1688,8 @@ cudaError_t rpy_setup(fil_ctx *c) {
         }
     c->rpy_tiles_max = count_tiles(c, kWarpTile);
     c->rpy_frames = pair32_on(c) && ns == 1 ? 1 : 0;
-    c->rpy_auto = c->rpy_frames;
-    if (c->rpy_auto) {
+    c->rpy_auto = ns == 1 ? 1 : 0;
+    if (c->rpy_frames) {
         const cudaError_t e = allow_warp_smem();
         if (e != cudaSuccess) return e;
     }
@@ -1506,6 +1737,10 @@ size_t rpy_partial_bytes(const fil_ctx *c) {
     if (c->rpy_frames)
         most = std::max(most, (size_t)((int64_t)c->num_sms * kWarpCta + c->rpy_tiles_max) *
                                   kWarpPart * sizeof(float));
+    else if (c->n_sys == 1 && c->lay.S > kDirectMaxSeg && c->lay.S <= kSymMaxSeg) {
+        const size_t tiles = (size_t)(c->lay.S + kSymTile - 1) / kSymTile;
+        most = std::max(most, tiles * 6 * tiles * kSymTile * sizeof(double));
+    }
     return most;
 }
 
@@ -1603,11 +1838,35 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
     } else {
+        const RpyConst64 k = make_const<double, RpyConst64>(c->a);
+        // one system on the automatic schedule: straight from the caller's arrays, unless
+        // the result overwrites them (or is too large for the slots)
+        if (c->rpy_auto && S <= kSymMaxSeg && !overlaps(VW, 6 * S, Y, 3 * S) &&
+            !overlaps(VW, 6 * S, FT, 6 * S)) {
+            if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
+            if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
+            if (S <= kDirectMaxSeg) {
+                rpy_direct64_kernel<<<(unsigned)S, 32, 0, c->stream>>>(Y, FT, (int)S, k, scale, VW);
+                c->n_launches += 1;
+            } else {
+                const int tiles = (int)((S + kSymTile - 1) / kSymTile);
+                rpy_sym64_kernel<<<(unsigned)(tiles * (tiles + 1) / 2), kSymThreads, 0, c->stream>>>(
+                    Y, FT, (int)S, tiles, k, (double *)c->partials);
+                sum64_kernel<<<dim3((unsigned)((S + 63) / 64), 6), 64, 0, c->stream>>>(
+                    (const double *)c->partials, (int)S, tiles, scale, VW);
+                c->n_launches += 2;
+            }
+            if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
+            if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
+            if (timed) c->prof_n += 1;
+            c->n_applies += 1;
+            c->n_pairs += c->pairs_all;
+            return cudaGetLastError();
+        }
         const int G = (int)(active_only ? c->rpy_grid64 : std::min<int64_t>(c->rpy_grid64, W));
         pack64_kernel<<<pgrid, pb, 0, c->stream>>>(Y, FT, S, c->Spad, sm, c->src64);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
-        const RpyConst64 k = make_const<double, RpyConst64>(c->a);
         if (c->rpy_tpt == 1)
             rpy_pair64_kernel<1><<<G, kRpyThreads, 0, c->stream>>>(
                 c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
@@ -1652,7 +1911,7 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
                 cands.push_back({tpt, split, ctas, 0, 1e30f});
         }
     }
-    if (c->rpy_frames) cands.push_back({2, 1, pair_occupancy(c, 2, 1), 1, 1e30f});
+    if (c->n_sys == 1) cands.push_back({2, 1, pair_occupancy(c, 2, 1), 1, 1e30f});
     const auto t0 = std::chrono::steady_clock::now();
     while (e == cudaSuccess) {
         for (int r = 0; r < 4 && e == cudaSuccess; ++r) e = rpy_apply(c, Y, FT, VW);
