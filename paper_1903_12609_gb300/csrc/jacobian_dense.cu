@@ -424,7 +424,7 @@ j0_assemble32_kernel(Layout lay, const int64_t *__restrict__ jofs,
     }
 }
 
-constexpr int kMfLanes = 16;   // lanes per target in the matrix-free pair sums
+constexpr int kMfLanes = 8;    // lanes per target in the matrix-free pair sums
 
 // r = b - J0 x for the filament of this CTA, matrix-free in FP64 from the
 // aux block (every thread of the CTA calls it; it ends with a barrier):
@@ -449,7 +449,9 @@ __device__ void residual_mf_cta(const AuxView &g, int N, const DenseParams &dp,
         st3(Ys + 3 * m, ld3(g.Y + 3 * m));
     }
     __syncthreads();
-    // pair sums: kMfLanes lanes per target, reduced with shuffles in fixed order
+    // pair sums: kMfLanes lanes per target; the lane sums are combined in a fixed
+    // order by halving (a lane keeps some components and gives the others away:
+    // 6 FP64 adds instead of 18 for 8 lanes)
     const int lane = threadIdx.x & 31;
     for (int base = 0; base < N; base += (int)blockDim.x / kMfLanes) {
         const int n = base + (int)threadIdx.x / kMfLanes;
@@ -459,27 +461,35 @@ __device__ void residual_mf_cta(const AuxView &g, int N, const DenseParams &dp,
             const V3 Yn = ld3(Ys + 3 * n);
             for (int m = sub; m < N; m += kMfLanes) {
                 const double *pc = g.pc + 5 * ((int64_t)n * N + m);
-                const PairCoef k{pc[0], pc[1], pc[2], pc[3], pc[4]};
-                apply_pair(k, Yn - ld3(Ys + 3 * m), ld3(FT + 6 * m), ld3(FT + 6 * m + 3), V, W);
+                const double A = pc[0], B = pc[1], C = pc[2], D = pc[3];
+                const V3 d = Yn - ld3(Ys + 3 * m);
+                const V3 e = pc[4] * d;                       // G d: both cross products
+                const V3 F = ld3(FT + 6 * m), T = ld3(FT + 6 * m + 3);
+                const double bF = B * dot(d, F), dT = D * dot(d, T);
+                V.x = fma(A, F.x, fma(bF, d.x, fma(T.y, e.z, fma(-T.z, e.y, V.x))));
+                V.y = fma(A, F.y, fma(bF, d.y, fma(T.z, e.x, fma(-T.x, e.z, V.y))));
+                V.z = fma(A, F.z, fma(bF, d.z, fma(T.x, e.y, fma(-T.y, e.x, V.z))));
+                W.x = fma(C, T.x, fma(dT, d.x, fma(F.y, e.z, fma(-F.z, e.y, W.x))));
+                W.y = fma(C, T.y, fma(dT, d.y, fma(F.z, e.x, fma(-F.x, e.z, W.y))));
+                W.z = fma(C, T.z, fma(dT, d.z, fma(F.x, e.y, fma(-F.y, e.x, W.z))));
             }
         }
-#pragma unroll
-        for (int d = kMfLanes / 2; d > 0; d >>= 1) {
-            V.x += __shfl_xor_sync(0xffffffffu, V.x, d);
-            V.y += __shfl_xor_sync(0xffffffffu, V.y, d);
-            V.z += __shfl_xor_sync(0xffffffffu, V.z, d);
-            W.x += __shfl_xor_sync(0xffffffffu, W.x, d);
-            W.y += __shfl_xor_sync(0xffffffffu, W.y, d);
-            W.z += __shfl_xor_sync(0xffffffffu, W.z, d);
-        }
-        if (n < N && sub == 0) {
-            st3(VW + 6 * n, dp.inv8pieta * V);
-            st3(VW + 6 * n + 3, dp.inv8pieta * W);
-        }
+        static_assert(kMfLanes == 8, "the halving below");
+        const bool om = sub & 4, c2 = sub & 2, c1 = sub & 1;
+        const unsigned all = 0xffffffffu;
+        const double w0 = (om ? W.x : V.x) + __shfl_xor_sync(all, om ? V.x : W.x, 4);
+        const double w1 = (om ? W.y : V.y) + __shfl_xor_sync(all, om ? V.y : W.y, 4);
+        const double w2 = (om ? W.z : V.z) + __shfl_xor_sync(all, om ? V.z : W.z, 4);
+        double a = (c2 ? w2 : w0) + __shfl_xor_sync(all, c2 ? w0 : w2, 2);
+        const double b1 = w1 + __shfl_xor_sync(all, w1, 2);
+        a = (c2 ? a : (c1 ? b1 : a)) + __shfl_xor_sync(all, c2 ? a : (c1 ? a : b1), 1);
+        if (n < N && !(c2 && c1))
+            VW[6 * n + (om ? 3 : 0) + (c2 ? 2 : (c1 ? 1 : 0))] = dp.inv8pieta * a;
     }
     __syncthreads();
-    // rotation rows
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
+    // rotation rows, by the warps after the first (whose sub-partitions' FP64 units
+    // are free while it forms the position rows)
+    for (int n = (int)threadIdx.x - 32; n >= 0 && n < N; n += (int)blockDim.x - 32) {
         const V3 un = ld3(xu + 3 * n);
         const V3 rot = un - dp.bdt * (mv(ld33(g.A + 9 * n), ld3(VW + 6 * n + 3)) +
                                       mv(ld33(g.Du + 9 * n), un));
@@ -525,33 +535,36 @@ __device__ void residual_mf_cta(const AuxView &g, int N, const DenseParams &dp,
     __syncthreads();
 }
 
-// x (+)= Inv r for one filament, Inv (n x n, row-major) and r in shared
-// memory: warp per row, lanes stride the columns (conflict-free).
-// Each warp takes kGemvRows rows at a time, so that a lane has the loads of
-// several rows in flight; every row is summed in the same order as one row
-// at a time (lane-strided FMAs, then a butterfly over the lanes).
-template <int ROWS = kGemvRows>
-__device__ __forceinline__ void inv_gemv_cta(const float *Inv, const float *r, double *x, int n,
-                                             bool accumulate) {
+// y = Inv r for one filament, Inv (n x n, row-major) in global memory, r and y
+// in shared memory: warp per row, lanes stride the columns. Each warp takes
+// kGemvRows = 4 rows at a time, so that a lane has the loads of several rows in
+// flight; a row is summed by lane-strided FMAs and a butterfly over the lanes,
+// of which each lane does only the part whose rows it keeps. y stays FP32: the
+// conversion to FP64 is done afterwards with full warps (one row per warp
+// instruction, it was a quarter of the solve's FP64 work).
+__device__ __forceinline__ void inv_gemv_cta(const float *Inv, const float *r, float *y, int n) {
+    static_assert(kGemvRows == 4, "the halving below");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i0 = wid * ROWS; i0 < n; i0 += nw * ROWS) {
-        float t[ROWS];
+    const unsigned all = 0xffffffffu;
+    for (int i0 = wid * kGemvRows; i0 < n; i0 += nw * kGemvRows) {
+        float t[kGemvRows];
 #pragma unroll
-        for (int u = 0; u < ROWS; ++u) t[u] = 0.f;
-#pragma unroll 2
+        for (int u = 0; u < kGemvRows; ++u) t[u] = 0.f;
+#pragma unroll 6
         for (int c = lane; c < n; c += 32) {
             const float rc = r[c];
 #pragma unroll
-            for (int u = 0; u < ROWS; ++u)
+            for (int u = 0; u < kGemvRows; ++u)
                 if (i0 + u < n) t[u] = fmaf(Inv[(int64_t)(i0 + u) * n + c], rc, t[u]);
         }
+        const bool hi = lane & 16, odd = lane & 8;
+        const float p = (hi ? t[2] : t[0]) + __shfl_xor_sync(all, hi ? t[0] : t[2], 16);
+        const float q = (hi ? t[3] : t[1]) + __shfl_xor_sync(all, hi ? t[1] : t[3], 16);
+        float v = (odd ? q : p) + __shfl_xor_sync(all, odd ? p : q, 8);
 #pragma unroll
-        for (int u = 0; u < ROWS; ++u) {
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) t[u] += __shfl_xor_sync(0xffffffffu, t[u], d);
-            if (lane == 0 && i0 + u < n) x[i0 + u] = accumulate ? x[i0 + u] + (double)t[u]
-                                                               : (double)t[u];
-        }
+        for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(all, v, d);
+        const int row = i0 + (hi ? 2 : 0) + (odd ? 1 : 0);
+        if ((lane & 7) == 0 && row < n) y[row] = v;
     }
 }
 
@@ -564,7 +577,7 @@ __global__ void __launch_bounds__(kApplyThreads)
 j0_apply_inverse_kernel(Layout lay, const int64_t *__restrict__ jofs,
                         const float *__restrict__ inv_all, const double *b, double *x,
                         const int *__restrict__ active) {
-    __shared__ float rs[6 * kMaxDenseSeg];
+    __shared__ float rs[6 * kMaxDenseSeg], ys[6 * kMaxDenseSeg];
     const int f = blockIdx.x;
     const int s0 = lay.off[f];
     if (active && !active[lay.sys_of[s0]]) return;   // converged system: rows not needed
@@ -572,7 +585,10 @@ j0_apply_inverse_kernel(Layout lay, const int64_t *__restrict__ jofs,
     const double *bg = b + 6 * (int64_t)s0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) rs[i] = (float)bg[i];
     __syncthreads();
-    inv_gemv_cta<kGemvRows>(inv_all + jofs[f], rs, x + 6 * (int64_t)s0, n, false);
+    inv_gemv_cta(inv_all + jofs[f], rs, ys, n);
+    __syncthreads();
+    double *xg = x + 6 * (int64_t)s0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) xg[i] = (double)ys[i];
 }
 
 // J0 solve, one CTA per filament:  x = Inv b;  `refine` times { r = b - J0 x
@@ -582,9 +598,15 @@ j0_apply_inverse_kernel(Layout lay, const int64_t *__restrict__ jofs,
 // run per SM, and the FP64 residual of one filament overlaps the inverse
 // products of others (staging the 147 KB inverse of a 32-segment filament
 // allowed one CTA per SM and serialised the two). b and x may alias.
+// What bounds it: the FP64 unit (a warp instruction takes 16 cycles of the SM
+// whatever its lanes do), behind enough CTAs to overlap one's reads and
+// barriers with another's FP64 work: 64 registers, 4 CTAs per SM (at 110
+// registers, 2 CTAs: 168 us; 5 spill: 132). Measured, 1000 filaments of 32:
+// 188 us with 16 lanes per target, each row of a product converted and added
+// by one lane, and two columns of a row in flight; 111 us in this form.
 constexpr int kSolveThreads = 256;
 
-__global__ void __launch_bounds__(kSolveThreads)
+__global__ void __launch_bounds__(kSolveThreads, 4)
 j0_solve_fused_kernel(Layout lay, const int64_t *__restrict__ jofs,
                       const int64_t *__restrict__ auxofs, DenseParams dp,
                       const double *__restrict__ aux_all, const float *__restrict__ inv_all,
@@ -599,7 +621,7 @@ j0_solve_fused_kernel(Layout lay, const int64_t *__restrict__ jofs,
     const float *Inv = inv_all + jofs[f];
     double *bs = reinterpret_cast<double *>(smraw);
     double *xs = bs + n, *FT = xs + n, *VW = FT + 6 * N, *Ys = VW + 6 * N;
-    float *rs = reinterpret_cast<float *>(Ys + 3 * N);
+    float *rs = reinterpret_cast<float *>(Ys + 3 * N), *ys = rs + n;
     const AuxView g = aux_view(const_cast<double *>(aux_all) + auxofs[f], N);
     const double *bg = b + 6 * (int64_t)s0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -608,11 +630,15 @@ j0_solve_fused_kernel(Layout lay, const int64_t *__restrict__ jofs,
         rs[i] = (float)v;
     }
     __syncthreads();
-    inv_gemv_cta(Inv, rs, xs, n, false);
+    inv_gemv_cta(Inv, rs, ys, n);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = (double)ys[i];
     __syncthreads();
     for (int it = 0; it < refine; ++it) {
         residual_mf_cta(g, N, dp, xs, bs, rs, FT, VW, Ys);
-        inv_gemv_cta(Inv, rs, xs, n, true);
+        inv_gemv_cta(Inv, rs, ys, n);
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] += (double)ys[i];
         __syncthreads();
     }
     double *xg = x + 6 * (int64_t)s0;
@@ -1000,7 +1026,7 @@ cudaError_t j0_dense_build_factor(fil_ctx *c, const double *X) {
 
 size_t j0_solve_smem(int maxN) {
     const size_t n = 6 * (size_t)maxN;
-    return (2 * n + 15 * (size_t)maxN) * sizeof(double) + n * sizeof(float);
+    return (2 * n + 15 * (size_t)maxN) * sizeof(double) + 2 * n * sizeof(float);
 }
 
 cudaError_t j0_dense_solve(fil_ctx *c, const double *b, double *x, const int *active) {
