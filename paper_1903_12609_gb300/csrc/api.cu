@@ -28,6 +28,7 @@ struct StatusBlock {
     double fmax;    // max over the systems still iterating (all systems outside a step)
 };
 constexpr int kRedChunk = 2048;   // X entries per Broyden reduction block
+constexpr int64_t kAheadMaxSeg = 2048;   // segments up to which an iteration runs ahead of its test
 
 fil_status set_err(fil_ctx *c, fil_status s, const std::string &msg) {
     if (c) c->err = msg;
@@ -195,10 +196,20 @@ void carve(fil_ctx *c, Arena &ar, int red_blocks, size_t partial_bytes) {
 
 // Flags and the per-system norms (into c->finf_h); fmax over the systems still
 // iterating when `active_only`, else over all.
-fil_status read_status(fil_ctx *c, StatusBlock *hs, bool active_only = false) {
-    const size_t bytes = 16 + 8 * (size_t)c->n_sys;
-    CK(cudaMemcpyAsync(c->h_pinned, c->d_flags, bytes, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+cudaError_t copy_status(fil_ctx *c) {
+    return cudaMemcpyAsync(c->h_pinned, c->d_flags, 16 + 8 * (size_t)c->n_sys,
+                           cudaMemcpyDeviceToHost, c->stream);
+}
+
+// copied: copy_status was enqueued and status_ev recorded after it.
+fil_status read_status(fil_ctx *c, StatusBlock *hs, bool active_only = false,
+                       bool copied = false) {
+    if (copied) {
+        CK(cudaEventSynchronize(c->status_ev));
+    } else {
+        CK(copy_status(c));
+        CK(cudaStreamSynchronize(c->stream));
+    }
     const char *h = reinterpret_cast<const char *>(c->h_pinned);
     std::memcpy(hs->flags, h, 16);
     if (hs->flags[2]) {
@@ -231,16 +242,22 @@ double finf_of(const StatusBlock &s) { return s.fmax; }
 // Unpack of X and the loads of the mobility problem: with tethered filaments
 // the unpack runs on X with the prescribed values in the slots (c->txr, also
 // returned in *Xu) and the multipliers join the loads; then the steric barrier.
+// step: X (c->Xn) is first set to Xk - w.
 cudaError_t unpack_all(fil_ctx *c, const double *X, int with_forces, bool act,
-                       const double **Xu) {
+                       const double **Xu, bool step = false) {
     *Xu = X;
     cudaError_t e;
     if (c->tether_on) {
+        if (step) {
+            e = broyden_axpy_step(c);
+            if (e != cudaSuccess) return e;
+            step = false;
+        }
         e = tether_resolve(c, X, c->txr);
         if (e != cudaSuccess) return e;
         *Xu = c->txr;
     }
-    e = unpack_forces(c, *Xu, with_forces, act);
+    e = unpack_forces(c, *Xu, with_forces, act, true, step);
     if (e != cudaSuccess) return e;
     if (c->tether_on) {
         e = tether_loads(c, X, act);
@@ -249,11 +266,12 @@ cudaError_t unpack_all(fil_ctx *c, const double *X, int with_forces, bool act,
     return steric_forces(c, act);
 }
 
+// step: the evaluation of a Broyden iteration, X = c->Xn = Xk - w formed on the way.
 cudaError_t eval_residual(fil_ctx *c, const double *X, double *f, int with_forces,
-                          const double *fprev = nullptr) {
+                          const double *fprev = nullptr, bool step = false) {
     const bool act = fprev != nullptr;
     const double *Xu = X;
-    cudaError_t e = unpack_all(c, X, with_forces, act, &Xu);
+    cudaError_t e = unpack_all(c, X, with_forces, act, &Xu, step);
     if (e != cudaSuccess) return e;
     e = rpy_apply(c, c->Yc, c->FT, c->VW, act);
     if (e != cudaSuccess) return e;
@@ -472,6 +490,7 @@ void fil_destroy(fil_ctx *c) {
     if (c->steric_bucket) cudaFree(c->steric_bucket);
     if (c->bmem_mem) cudaFree(c->bmem_mem);
     if (c->h_pinned) cudaFreeHost(c->h_pinned);
+    if (c->status_ev) cudaEventDestroy(c->status_ev);
     if (c->prof_ev) {
         for (int i = 0; i < 2 * kProfMax; ++i) cudaEventDestroy(c->prof_ev[i]);
         delete[] c->prof_ev;
@@ -715,8 +734,7 @@ void drop_graphs(fil_ctx *c) {
 // (wasted once per step; for systems that have just converged, w is masked
 // afterwards).
 cudaError_t iteration_body(fil_ctx *c) {
-    cudaError_t e = broyden_axpy_step(c);
-    if (e == cudaSuccess) e = eval_residual(c, c->Xn, c->fn, 1, c->n_sys > 1 ? c->fk : nullptr);
+    cudaError_t e = eval_residual(c, c->Xn, c->fn, 1, c->n_sys > 1 ? c->fk : nullptr, true);
     if (e == cudaSuccess) e = broyden_dots(c);
     if (e == cudaSuccess) e = j0_apply(c, c->fn, c->g, true);
     if (e == cudaSuccess) e = broyden_update(c);
@@ -888,10 +906,23 @@ fil_status fil_broyden_step(fil_ctx *c, int32_t *converged, double *finf) {
         if (converged) *converged = 0;
         return FIL_OK;
     }
-    CK(broyden_axpy_step(c));
-    CK(eval_residual(c, c->Xn, c->fn, 1, c->n_sys > 1 ? c->fk : nullptr));
+    CK(eval_residual(c, c->Xn, c->fn, 1, c->n_sys > 1 ? c->fk : nullptr, true));
+    // One small system: the rest of the iteration is enqueued behind the status copy
+    // and the host waits for the copy alone, so that the GPU works while the host
+    // decides. What the last iteration of a step enqueued in vain (it touches the step
+    // w and history slots that no pair counts) is cheaper there than a round trip of
+    // ~20 us in every iteration; for large systems it is not.
+    const bool ahead = c->n_sys == 1 && c->lay.S <= kAheadMaxSeg;
+    if (ahead) {
+        if (!c->status_ev) CK(cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming));
+        CK(copy_status(c));
+        CK(cudaEventRecord(c->status_ev, c->stream));
+        CK(broyden_dots(c));
+        CK(j0_apply(c, c->fn, c->g, true));
+        CK(broyden_update(c));
+    }
     StatusBlock sb;
-    fil_status s = read_status(c, &sb);
+    fil_status s = read_status(c, &sb, false, ahead);
     if (s != FIL_OK) return s;
     if (sb.flags[0]) return set_err(c, FIL_ESTALL, "Broyden: ||df|| = 0 (stalled)");
     const double fv = finf_of(sb);
@@ -910,9 +941,11 @@ fil_status fil_broyden_step(fil_ctx *c, int32_t *converged, double *finf) {
         CK(upload_active(c));
         CK(rpy_set_active(c));
     }
-    CK(broyden_dots(c));
-    CK(j0_apply(c, c->fn, c->g, true));
-    CK(broyden_update(c));
+    if (!ahead) {
+        CK(broyden_dots(c));
+        CK(j0_apply(c, c->fn, c->g, true));
+        CK(broyden_update(c));
+    }
     std::swap(c->Xk, c->Xn);
     std::swap(c->fk, c->fn);
     c->k += 1;

@@ -33,9 +33,25 @@ __global__ void axpy_neg_kernel(int64_t n, const double *__restrict__ x,
 
 // Sums of G per-thread values over the block, written to part[o_j * nb + b]
 // (fixed order: warp shuffles, then the warps in order).
+// (direct: every system is one block, whose sums are the results; see Direct)
+struct Direct {
+    double *out;       // null: partials are written and dots_final_kernel adds them
+    float *out32;
+    int sstride;
+};
+
+// One result of a system: output o, and where it is |df|^2 (o = k) also 1/|df| in
+// slot k + 2 (free until the next iteration), so that the update multiplies
+// instead of dividing in every entry.
+__device__ __forceinline__ void write_result(const Direct &r, int sy, int o, int k, double s) {
+    r.out[(int64_t)sy * r.sstride + o] = s;
+    if (r.out32) r.out32[(int64_t)sy * r.sstride + o] = (float)s;   // for the FP32 history sums
+    if (o == k) r.out[(int64_t)sy * r.sstride + o + 2] = s > 0.0 ? 1.0 / sqrt(s) : 0.0;
+}
+
 template <int G>
 __device__ __forceinline__ void block_reduce_write(double (&acc)[G], double *sh, const int *o,
-                                                   int nb, double *part) {
+                                                   int nb, double *part, const Direct &dir, int k) {
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
 #pragma unroll
     for (int j = 0; j < G; ++j) {
@@ -48,7 +64,8 @@ __device__ __forceinline__ void block_reduce_write(double (&acc)[G], double *sh,
     if ((int)threadIdx.x < G) {
         double s = 0.0;
         for (int w = 0; w < nw; ++w) s += sh[threadIdx.x * 32 + w];
-        part[(int64_t)o[threadIdx.x] * nb + blockIdx.x] = s;
+        if (dir.out) write_result(dir, blockIdx.x, o[threadIdx.x], k, s);
+        else part[(int64_t)o[threadIdx.x] * nb + blockIdx.x] = s;
     }
     __syncthreads();
 }
@@ -59,7 +76,8 @@ __device__ __forceinline__ void block_reduce_write(double (&acc)[G], double *sh,
 template <int G, typename H>
 __device__ __forceinline__ void dots_group(const H *__restrict__ D, int64_t n, int o0,
                                            const double *__restrict__ fn, int64_t i0, int64_t i1,
-                                           double *sh, int nb, double *part) {
+                                           double *sh, int nb, double *part, const Direct &dir,
+                                           int k) {
     H acc[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) acc[j] = H(0);
@@ -75,7 +93,7 @@ __device__ __forceinline__ void dots_group(const H *__restrict__ D, int64_t n, i
         accd[j] = (double)acc[j];
         o[j] = o0 + j;
     }
-    block_reduce_write<G>(accd, sh, o, nb, part);
+    block_reduce_write<G>(accd, sh, o, nb, part, dir, k);
 }
 
 // Outputs o = 0..k-1: d_o . fn;  o = k: |fn - fk|^2;  o = k+1: (fn - fk) . fn,
@@ -89,8 +107,10 @@ __global__ void dots_partial_kernel(int64_t n, const double *__restrict__ fn,
                                     const double *__restrict__ fk, const H *__restrict__ D,
                                     const int *__restrict__ dk, const int64_t *__restrict__ blk_beg,
                                     const int *__restrict__ blk_sys,
-                                    const int *__restrict__ active, double *__restrict__ part) {
+                                    const int *__restrict__ active, double *__restrict__ part,
+                                    Direct dir) {
     __shared__ double sh[kDotGroup * 32];
+    pdl_enter();
     if (active && !active[blk_sys[blockIdx.x]]) return;   // a converged system: not needed
     const int k = *dk;
     const int nb = gridDim.x;
@@ -104,27 +124,27 @@ __global__ void dots_partial_kernel(int64_t n, const double *__restrict__ fn,
             acc[1] = fma(df, f, acc[1]);
         }
         const int o[2] = {k, k + 1};
-        block_reduce_write<2>(acc, sh, o, nb, part);
+        block_reduce_write<2>(acc, sh, o, nb, part, dir, k);
         return;
     }
     const int o0 = (int)(blockIdx.y - 1) * kDotGroup;
     if (o0 >= k) return;
     switch (k - o0 < kDotGroup ? k - o0 : kDotGroup) {
-        case 1: dots_group<1, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 2: dots_group<2, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 3: dots_group<3, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 4: dots_group<4, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 5: dots_group<5, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 6: dots_group<6, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        case 7: dots_group<7, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
-        default: dots_group<kDotGroup, H>(D, n, o0, fn, i0, i1, sh, nb, part); break;
+        case 1: dots_group<1, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 2: dots_group<2, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 3: dots_group<3, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 4: dots_group<4, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 5: dots_group<5, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 6: dots_group<6, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        case 7: dots_group<7, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
+        default: dots_group<kDotGroup, H>(D, n, o0, fn, i0, i1, sh, nb, part, dir, k); break;
     }
 }
 
 __global__ void dots_final_kernel(int n_sys, int max_out, const int *__restrict__ dk, int nblocks,
                                   const int *__restrict__ sys_blk, const double *__restrict__ part,
-                                  int sstride, double *__restrict__ out,
-                                  float *__restrict__ out32) {
+                                  Direct res) {
+    pdl_enter();
     // one warp per (system, output), lanes stride the system's partials, fixed-order tree
     const int64_t job = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -135,59 +155,62 @@ __global__ void dots_final_kernel(int n_sys, int max_out, const int *__restrict_
     for (int b = sys_blk[sy] + lane; b < sys_blk[sy + 1]; b += 32) s += part[(int64_t)o * nblocks + b];
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-    if (lane == 0) {
-        out[(int64_t)sy * sstride + o] = s;
-        if (out32) out32[(int64_t)sy * sstride + o] = (float)s;   // for the FP32 history sums
-        // |df|^2: also 1/|df| in slot k + 2 (free until the next iteration), so
-        // that the update multiplies instead of dividing in every entry
-        if (o == *dk) out[(int64_t)sy * sstride + o + 2] = s > 0.0 ? 1.0 / sqrt(s) : 0.0;
-    }
+    if (lane == 0) write_result(res, sy, o, *dk, s);
 }
 
 // g += sum_i c_i alpha_i; history pair k; w = g + c_k (df . fn)/|df|, with the
-// scalars of entry i's system; w = 0 in systems that have converged.
+// scalars of entry i's system; w = 0 in systems that have converged. The last
+// block to finish moves the device's k to the next history slot (flags[3] counts
+// the blocks and wraps to zero).
 template <typename H>
-__global__ void update_kernel(int64_t n, const int *__restrict__ dk,
+__global__ void update_kernel(int64_t n, int *__restrict__ dk,
                               const double *__restrict__ scal_all, const float *__restrict__ scal32,
                               int sstride, const int *__restrict__ sys_of,
                               const int *__restrict__ active, const double *__restrict__ fn,
                               const double *__restrict__ fk, double *__restrict__ g,
                               H *__restrict__ C, H *__restrict__ D, double *__restrict__ w,
                               int *__restrict__ flags) {
+    pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int sy = sys_of[i / 6];
     const int k = *dk;
-    if (!active[sy]) {
-        // a converged system takes no step and no history pair (zero rows, so
-        // that carried pairs hold nothing stale for it)
-        w[i] = 0.0;
-        C[(int64_t)k * n + i] = (H)0;
-        D[(int64_t)k * n + i] = (H)0;
-        return;
+    if (i < n) {
+        const int sy = sys_of[i / 6];
+        if (!active[sy]) {
+            // a converged system takes no step and no history pair (zero rows, so
+            // that carried pairs hold nothing stale for it)
+            w[i] = 0.0;
+            C[(int64_t)k * n + i] = (H)0;
+            D[(int64_t)k * n + i] = (H)0;
+        } else {
+            const double *scal = scal_all + (int64_t)sy * sstride;
+            const double ndf2 = scal[k];
+            if (!(ndf2 > 0.0)) flags[0] = 1;
+            double gi = g[i];
+            if (sizeof(H) == sizeof(double)) {
+                for (int l = 0; l < k; ++l) gi += (double)C[(int64_t)l * n + i] * scal[l];
+            } else {
+                // the history sum in FP32 (mixed mode), added to g once
+                const float *sc32 = scal32 + (int64_t)sy * sstride;
+                float h = 0.f;
+                for (int l = 0; l < k; ++l) h = fmaf((float)C[(int64_t)l * n + i], sc32[l], h);
+                gi += (double)h;
+            }
+            const double indf = scal[k + 2];            // 1/|df|
+            const double c = -gi * indf;
+            const double d = (fn[i] - fk[i]) * indf;
+            C[(int64_t)k * n + i] = (H)c;
+            D[(int64_t)k * n + i] = (H)d;
+            w[i] = gi + c * (scal[k + 1] * indf);
+        }
     }
-    const double *scal = scal_all + (int64_t)sy * sstride;
-    const double ndf2 = scal[k];
-    if (!(ndf2 > 0.0)) flags[0] = 1;
-    double gi = g[i];
-    if (sizeof(H) == sizeof(double)) {
-        for (int l = 0; l < k; ++l) gi += (double)C[(int64_t)l * n + i] * scal[l];
-    } else {
-        // the history sum in FP32 (mixed mode), added to g once
-        const float *sc32 = scal32 + (int64_t)sy * sstride;
-        float h = 0.f;
-        for (int l = 0; l < k; ++l) h = fmaf((float)C[(int64_t)l * n + i], sc32[l], h);
-        gi += (double)h;
+    __syncthreads();            // every thread of the block has read k
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicInc(reinterpret_cast<unsigned *>(flags + 3), gridDim.x - 1) == gridDim.x - 1)
+            *dk = k + 1;
     }
-    const double indf = scal[k + 2];            // 1/|df|
-    const double c = -gi * indf;
-    const double d = (fn[i] - fk[i]) * indf;
-    C[(int64_t)k * n + i] = (H)c;
-    D[(int64_t)k * n + i] = (H)d;
-    w[i] = gi + c * (scal[k + 1] * indf);
 }
 
-__global__ void k_advance_kernel(int *dk) { *dk += 1; }
 __global__ void k_set_kernel(int *dk, int k) { *dk = k; }
 
 // w += sum_{l<k} c_l alpha_l (alpha_l = d_l . f in the scalars of entry i's
@@ -237,39 +260,41 @@ cudaError_t broyden_axpy_step(fil_ctx *c) {
     return cudaGetLastError();
 }
 
-cudaError_t broyden_dots(fil_ctx *c) {
+// The dot products of f (and of f - fk) with the history into c->scal.
+static cudaError_t dots(fil_ctx *c, const double *f, const double *fk, const int *active) {
     const int64_t n = c->lay.nX;
-    if (c->C32)
-        dots_partial_kernel<float><<<dots_grid(c), kRedThreads, 0, c->stream>>>(
-            n, c->fn, c->fk, c->D32, c->d_k, c->blk_beg, c->blk_sys,
-            c->n_sys > 1 ? c->d_active : nullptr, c->red_part);
-    else
-        dots_partial_kernel<double><<<dots_grid(c), kRedThreads, 0, c->stream>>>(
-            n, c->fn, c->fk, c->D, c->d_k, c->blk_beg, c->blk_sys,
-            c->n_sys > 1 ? c->d_active : nullptr, c->red_part);
+    const Direct res{c->scal, c->C32 ? c->scal32 : nullptr, c->sstride};
+    // a system per block: the blocks' sums are the results
+    const bool one = c->red_blocks == c->n_sys;
+    const Direct dir = one ? res : Direct{nullptr, nullptr, 0};
+    cudaError_t e =
+        c->C32 ? launch_pdl(dots_partial_kernel<float>, dots_grid(c), kRedThreads, 0, c->stream, n, f,
+                            fk, c->D32, c->d_k, c->blk_beg, c->blk_sys, active, c->red_part, dir)
+               : launch_pdl(dots_partial_kernel<double>, dots_grid(c), kRedThreads, 0, c->stream, n,
+                            f, fk, c->D, c->d_k, c->blk_beg, c->blk_sys, active, c->red_part, dir);
+    c->n_launches += 1;
+    if (one || e != cudaSuccess) return e;
     const int max_out = c->hist_cap + 2;
     const int64_t jobs = (int64_t)c->n_sys * max_out;
-    dots_final_kernel<<<(unsigned)((jobs + 7) / 8), 256, 0, c->stream>>>(
-        c->n_sys, max_out, c->d_k, c->red_blocks, c->sys_blk_off, c->red_part, c->sstride, c->scal,
-        c->C32 ? c->scal32 : nullptr);
-    c->n_launches += 2;
-    return cudaGetLastError();
+    c->n_launches += 1;
+    return launch_pdl(dots_final_kernel, (unsigned)((jobs + 7) / 8), 256, 0, c->stream, c->n_sys,
+                      max_out, c->d_k, c->red_blocks, c->sys_blk_off, c->red_part, res);
+}
+
+cudaError_t broyden_dots(fil_ctx *c) {
+    return dots(c, c->fn, c->fk, c->n_sys > 1 ? c->d_active : nullptr);
 }
 
 cudaError_t broyden_update(fil_ctx *c) {
     const int64_t n = c->lay.nX;
     const unsigned grid = (unsigned)((n + 255) / 256);
-    if (c->C32)
-        update_kernel<float><<<grid, 256, 0, c->stream>>>(
-            n, c->d_k, c->scal, c->scal32, c->sstride, c->lay.sys_of, c->d_active, c->fn, c->fk,
-            c->g, c->C32, c->D32, c->w, c->d_flags);
-    else
-        update_kernel<double><<<grid, 256, 0, c->stream>>>(
-            n, c->d_k, c->scal, nullptr, c->sstride, c->lay.sys_of, c->d_active, c->fn, c->fk,
-            c->g, c->C, c->D, c->w, c->d_flags);
-    k_advance_kernel<<<1, 1, 0, c->stream>>>(c->d_k);     // the next history slot
-    c->n_launches += 2;
-    return cudaGetLastError();
+    c->n_launches += 1;
+    return c->C32 ? launch_pdl(update_kernel<float>, grid, 256, 0, c->stream, n, c->d_k, c->scal,
+                               c->scal32, c->sstride, c->lay.sys_of, c->d_active, c->fn, c->fk, c->g,
+                               c->C32, c->D32, c->w, c->d_flags)
+                  : launch_pdl(update_kernel<double>, grid, 256, 0, c->stream, n, c->d_k, c->scal,
+                               (const float *)nullptr, c->sstride, c->lay.sys_of, c->d_active, c->fn,
+                               c->fk, c->g, c->C, c->D, c->w, c->d_flags);
 }
 
 cudaError_t broyden_carry(fil_ctx *c, int from, int m, const double *f, double *w) {
@@ -289,17 +314,8 @@ cudaError_t broyden_carry(fil_ctx *c, int from, int m, const double *f, double *
     }
     k_set_kernel<<<1, 1, 0, c->stream>>>(c->d_k, m);
     // alpha_i = d_i . f (outputs k and k + 1 come out zero with fn = fk = f)
-    if (c->C32)
-        dots_partial_kernel<float><<<dots_grid(c), kRedThreads, 0, c->stream>>>(
-            n, f, f, c->D32, c->d_k, c->blk_beg, c->blk_sys, nullptr, c->red_part);
-    else
-        dots_partial_kernel<double><<<dots_grid(c), kRedThreads, 0, c->stream>>>(
-            n, f, f, c->D, c->d_k, c->blk_beg, c->blk_sys, nullptr, c->red_part);
-    const int max_out = c->hist_cap + 2;
-    const int64_t jobs = (int64_t)c->n_sys * max_out;
-    dots_final_kernel<<<(unsigned)((jobs + 7) / 8), 256, 0, c->stream>>>(
-        c->n_sys, max_out, c->d_k, c->red_blocks, c->sys_blk_off, c->red_part, c->sstride,
-        c->scal, c->C32 ? c->scal32 : nullptr);
+    const cudaError_t ed = dots(c, f, f, nullptr);
+    if (ed != cudaSuccess) return ed;
     const unsigned grid = (unsigned)((n + 255) / 256);
     if (c->C32)
         history_apply_kernel<float><<<grid, 256, 0, c->stream>>>(n, c->d_k, c->scal, c->sstride,
@@ -307,7 +323,7 @@ cudaError_t broyden_carry(fil_ctx *c, int from, int m, const double *f, double *
     else
         history_apply_kernel<double><<<grid, 256, 0, c->stream>>>(n, c->d_k, c->scal, c->sstride,
                                                                    c->lay.sys_of, c->C, w);
-    c->n_launches += 4;
+    c->n_launches += 2;
     return cudaGetLastError();
 }
 

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/fil.h"
@@ -161,6 +162,7 @@ struct fil_ctx {
     int64_t graph_launches[2], graph_applies[2];
     int in_step;           // a step was begun and not committed
     int iters_step;        // Broyden iterations of the current step
+    cudaEvent_t status_ev = nullptr;   // after the status copy of a Broyden iteration
     int conv;              // current iterate satisfies ||f||_inf <= tol * a
 
     // J0 factors: banded (drag mobility, App. B.2) or dense per filament
@@ -243,6 +245,34 @@ inline bool pair32_on(const fil_ctx *c) { return c->prec != FIL_FP64; }
 inline int rpy_tile(const fil_ctx *c) { return c->rpy_threads * c->rpy_tpt; }
 inline bool fast_mixed(const fil_ctx *c) { return c->prec == FIL_MIXED; }
 
+// Programmatic dependent launch through the chain of an iteration's kernels: a
+// kernel launched with launch_pdl may become resident while the kernel before it
+// in the stream still runs, and pdl_enter, its first statement, holds it until
+// that kernel is complete and its writes are visible (so every kernel given to
+// launch_pdl starts with pdl_enter). What overlaps is the launch itself: the
+// iterations of small systems are chains of a dozen kernels of 2-10 us, and each
+// boundary cost 1-2 us more.
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, Args &&...args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Launchers (all enqueue on c->stream and return a cudaError_t).
 cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
                       bool active_only = false);
@@ -255,7 +285,10 @@ cudaError_t rpy_set_schedule(fil_ctx *c, int tpt, int threads, int ctas, int spl
 cudaError_t rpy_upload_tables(fil_ctx *c);  // the layout tables, after the arena exists
 size_t rpy_partial_bytes(const fil_ctx *c);
 
-cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool active_only = false);
+// eval: first part of a residual evaluation (the norms of residual_rows restart);
+// step: first Xn = Xk - w, and X must be Xn
+cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool active_only = false,
+                          bool eval = false, bool step = false);
 // fprev non-null: systems that have converged copy their rows from fprev
 cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *fprev = nullptr);
 // adds the steric barrier forces of the positions Yc to FT (no-op when FS = 0);

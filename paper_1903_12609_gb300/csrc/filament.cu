@@ -51,8 +51,13 @@ __device__ __forceinline__ V3 robot_arm_pass(V3 t, bool active, int n, double dL
     return Yn;
 }
 
-// unpack (+ forces): one warp per filament.
-__global__ void unpack_forces_kernel(Layout lay, const double *__restrict__ X,
+// unpack (+ forces): one warp per filament. With kStep the warp first forms its
+// filament's entries of the new iterate, X = Xk - w (of every system, converged
+// or not), and goes on from them.
+template <bool kStep>
+__global__ void unpack_forces_kernel(Layout lay, double *X, const double *__restrict__ Xk,
+                                     const double *__restrict__ w, int n_sys,
+                                     unsigned long long *__restrict__ finf,
                                      const double *__restrict__ qj, ForceParams fp,
                                      const double *__restrict__ Fext,
                                      const double *__restrict__ Text,
@@ -60,12 +65,22 @@ __global__ void unpack_forces_kernel(Layout lay, const double *__restrict__ X,
                                      const int *__restrict__ active, double *__restrict__ qc,
                                      double *__restrict__ Yc, double *__restrict__ FT,
                                      double *__restrict__ Tint) {
+    pdl_enter();
     const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
+    if (finf) {      // ||f||_inf of every system restarts (n_sys <= M, so the grid covers them)
+        const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        if (i < n_sys) finf[i] = 0;
+    }
     if (warp >= lay.M) return;
     const int s0 = lay.off[warp];
-    if (active && !active[lay.sys_of[s0]]) return;   // a converged system keeps its unpack
     const int N = lay.off[warp + 1] - s0;
+    if constexpr (kStep) {
+        const int64_t x0 = 6 * (int64_t)s0;
+        for (int i = lane; i < 6 * N; i += 32) X[x0 + i] = Xk[x0 + i] - w[x0 + i];
+        __syncwarp();
+    }
+    if (active && !active[lay.sys_of[s0]]) return;   // a converged system keeps its unpack
     const double *Xf = X + 6 * (int64_t)s0;
 
     V3 carry_Y = ld3(Xf);
@@ -121,6 +136,8 @@ __global__ void unpack_forces_kernel(Layout lay, const double *__restrict__ X,
     }
 }
 
+constexpr int kRowThreads = 256;
+
 struct Scheme {
     double a1, a0, bdt, g;   // f = Y - a1 Y^j - a0 Y^{j-1} - bdt V ; u - g u^j - bdt dexpinv
 };
@@ -137,6 +154,7 @@ __global__ void residual_rows_kernel(Layout lay, const double *__restrict__ X,
                                      const int *__restrict__ active,
                                      const double *__restrict__ fprev, double *__restrict__ f,
                                      unsigned long long *__restrict__ finf_bits) {
+    pdl_enter();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double m = 0.0;
     bool eval = g < lay.S;
@@ -401,14 +419,18 @@ unsigned seg_grid(int64_t S, int threads) { return (unsigned)((S + threads - 1) 
 
 }  // namespace
 
-cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool active_only) {
+cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool active_only, bool eval,
+                          bool step) {
     ForceParams fp{c->dL, c->KB, c->KT, c->g0, c->kmu, c->knu};
-    unpack_forces_kernel<<<warp_grid(c->lay.M, 128), 128, 0, c->stream>>>(
-        c->lay, X, c->q, fp, c->has_Fext ? c->Fext : nullptr, c->has_Text ? c->Text : nullptr,
-        c->has_follower ? c->follower : nullptr, with_forces, active_only ? c->d_active : nullptr,
-        c->qc, c->Yc, c->FT, with_forces == 2 ? c->Tint : nullptr);
+    const auto kernel = step ? unpack_forces_kernel<true> : unpack_forces_kernel<false>;
     c->n_launches += 1;
-    return cudaGetLastError();
+    // (X is written only where step is set, and is then c->Xn)
+    return launch_pdl(kernel, warp_grid(c->lay.M, 128), 128, 0, c->stream, c->lay,
+                      const_cast<double *>(X), c->Xk, c->w, c->n_sys, eval ? c->d_finf : nullptr,
+                      c->q, fp, c->has_Fext ? c->Fext : nullptr, c->has_Text ? c->Text : nullptr,
+                      c->has_follower ? c->follower : nullptr, with_forces,
+                      active_only ? c->d_active : nullptr, c->qc, c->Yc, c->FT,
+                      with_forces == 2 ? c->Tint : nullptr);
 }
 
 cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *fprev) {
@@ -418,13 +440,10 @@ cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *
     } else {
         sc = {1.0, 0.0, c->dt, 0.0};
     }
-    cudaError_t e = cudaMemsetAsync(c->d_finf, 0, sizeof(unsigned long long) * c->n_sys, c->stream);
-    if (e != cudaSuccess) return e;
-    residual_rows_kernel<<<seg_grid(c->lay.S, 256), 256, 0, c->stream>>>(
-        c->lay, X, c->Yc, c->VW, c->Y, c->Yprev, c->uprev, sc, fprev ? c->d_active : nullptr,
-        fprev, f, c->d_finf);
     c->n_launches += 1;
-    return cudaGetLastError();
+    return launch_pdl(residual_rows_kernel, seg_grid(c->lay.S, kRowThreads), kRowThreads, 0, c->stream,
+                      c->lay, X, c->Yc, c->VW, c->Y, c->Yprev, c->uprev, sc,
+                      fprev ? c->d_active : nullptr, fprev, f, c->d_finf);
 }
 
 cudaError_t init_straight(fil_ctx *c, const double *base, const double *t, const double *mu,

@@ -247,6 +247,7 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
                                   const double *b, double *x, int zmax,
                                   const int *__restrict__ active, int fil_per_cta) {
     extern __shared__ __align__(16) unsigned char zraw[];
+    pdl_enter();
     const int slot = threadIdx.x / kSolveLanes;        // filament within the CTA
     const int lane = threadIdx.x % kSolveLanes;
     const int f = blockIdx.x * fil_per_cta + slot;
@@ -447,14 +448,12 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
     }
     const int threads = (kSolveLanes * fils + 31) / 32 * 32;
     const unsigned grid = (unsigned)((c->lay.M + fils - 1) / fils);
-    if (c->band32)
-        band_solve_kernel<float><<<grid, threads, smem, c->stream>>>(
-            c->lay, c->band32, c->piv, make_params(c).ct, b, x, zmax, active, fils);
-    else
-        band_solve_kernel<double><<<grid, threads, smem, c->stream>>>(
-            c->lay, c->band, c->piv, make_params(c).ct, b, x, zmax, active, fils);
     c->n_launches += 1;
-    return cudaGetLastError();
+    const double ct = make_params(c).ct;
+    return c->band32 ? launch_pdl(band_solve_kernel<float>, grid, threads, smem, c->stream, c->lay,
+                                  c->band32, c->piv, ct, b, x, zmax, active, fils)
+                     : launch_pdl(band_solve_kernel<double>, grid, threads, smem, c->stream, c->lay,
+                                  c->band, c->piv, ct, b, x, zmax, active, fils);
 }
 
 }  // namespace fil

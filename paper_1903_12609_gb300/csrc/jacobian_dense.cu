@@ -578,6 +578,7 @@ j0_apply_inverse_kernel(Layout lay, const int64_t *__restrict__ jofs,
                         const float *__restrict__ inv_all, const double *b, double *x,
                         const int *__restrict__ active) {
     __shared__ float rs[6 * kMaxDenseSeg], ys[6 * kMaxDenseSeg];
+    pdl_enter();
     const int f = blockIdx.x;
     const int s0 = lay.off[f];
     if (active && !active[lay.sys_of[s0]]) return;   // converged system: rows not needed
@@ -613,6 +614,7 @@ j0_solve_fused_kernel(Layout lay, const int64_t *__restrict__ jofs,
                       const double *b, double *x, const int *__restrict__ active,
                       int refine) {
     extern __shared__ __align__(16) unsigned char smraw[];
+    pdl_enter();
     const int f = blockIdx.x;
     const int s0 = lay.off[f];
     if (active && !active[lay.sys_of[s0]]) return;   // converged system: rows not needed
@@ -1031,10 +1033,9 @@ size_t j0_solve_smem(int maxN) {
 
 cudaError_t j0_dense_solve(fil_ctx *c, const double *b, double *x, const int *active) {
     if (fast_mixed(c)) {
-        j0_apply_inverse_kernel<<<c->lay.M, kApplyThreads, 0, c->stream>>>(c->lay, c->jofs,
-                                                                          c->jinv, b, x, active);
         c->n_launches += 1;
-        return cudaGetLastError();
+        return launch_pdl(j0_apply_inverse_kernel, c->lay.M, kApplyThreads, 0, c->stream, c->lay,
+                          c->jofs, c->jinv, b, x, active);
     }
     DenseParams dp;
     dp.jp = J0Params{c->dL, c->KB, c->KT, c->g0, c->kmu, c->knu, 0.0, 0.0};
@@ -1046,11 +1047,9 @@ cudaError_t j0_dense_solve(fil_ctx *c, const double *b, double *x, const int *ac
     cudaError_t e = cudaFuncSetAttribute(j0_solve_fused_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    j0_solve_fused_kernel<<<c->lay.M, kSolveThreads, smem, c->stream>>>(
-        c->lay, c->jofs, c->auxofs, dp, c->aux, c->jinv, b, x, active,
-        kJ0Refine);
     c->n_launches += 1;
-    return cudaGetLastError();
+    return launch_pdl(j0_solve_fused_kernel, c->lay.M, kSolveThreads, smem, c->stream, c->lay, c->jofs,
+                      c->auxofs, dp, c->aux, c->jinv, b, x, active, kJ0Refine);
 }
 
 }  // namespace fil

@@ -164,6 +164,20 @@ __device__ __forceinline__ int64_t segment_at(const SysMap &m, int64_t P, int64_
     return m.pad_map ? (int64_t)m.pad_map[P] : (P < S ? P : -1);
 }
 
+// Error-free transformation s + e = a + b (Knuth's TwoSum), with the adds
+// kept out of FMA contraction and reassociation.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// a b - c d to within 1.5 ulp of the exact value (Kahan).
+__device__ __forceinline__ float diff_of_products(float a, float b, float c, float d) {
+    const float w = __fmul_rn(c, d);
+    return __fadd_rn(__fmaf_rn(a, b, -w), __fmaf_rn(-c, d, w));
+}
+
 // ---------------------------------------------------------------------------
 // Pack: FP64 (Y, FT) -> FP32 source groups of kRpyComp = 32 padded positions.
 // A group is Rec::kGroupF4 float4: first its centre (c_x, c_y, c_z, 0), the mean of
@@ -193,9 +207,12 @@ struct Rec {
     static constexpr int kSums = kFrames ? 12 : 6;                // packed sums of the far loop
 };
 
+// (two warps per CTA: a small system's groups then spread over the SMs)
+constexpr int kPackThreads = 64;
 template <bool kFrames>
-__global__ void pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
+__global__ void __launch_bounds__(kPackThreads) pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
                               int64_t S, int64_t Spad, SysMap sm, float4 *__restrict__ src) {
+    pdl_enter();
     const int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (P >= Spad) return;             // Spad is a multiple of 32: whole warps leave
     const int64_t i = segment_at(sm, P, S);
@@ -218,10 +235,10 @@ __global__ void pack32_kernel(const double *__restrict__ Y, const double *__rest
     if constexpr (kFrames) {
         const unsigned live = __ballot_sync(0xffffffffu, i >= 0);
         const float inv = live ? 1.f / (float)__popc(live) : 0.f;
-        float cen[3], sp[3];
+        float cen[3], sp[3], yh[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            float m = __double2float_rn(y[c]);
+            float m = yh[c] = __double2float_rn(y[c]);
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) m += __shfl_xor_sync(0xffffffffu, m, d);
             cen[c] = m * inv;
@@ -229,19 +246,22 @@ __global__ void pack32_kernel(const double *__restrict__ Y, const double *__rest
         if (lane == 0) g[0] = make_float4(cen[0], cen[1], cen[2], 0.f);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double r = y[c] - (double)cen[c];
-            sp[c] = __double2float_rn(r);
+            // s' = y - c from the FP32 parts of y (the FP64 unit has 1/64 of the rate)
+            const float l = __double2float_rn(y[c] - (double)yh[c]);
+            float u, e;
+            two_sum(yh[c], -cen[c], u, e);
+            e = __fadd_rn(e, l);
+            two_sum(u, e, sp[c], e);
             v[c] = -sp[c];
-            v[15 + c] = -__double2float_rn(r - (double)sp[c]);
+            v[15 + c] = -e;
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            // -(T x s')_c and -(2/3)(F x s')_c of the rounded T, F, s'
+            // -(T x s')_c and -(2/3)(F x s')_c, the differences of products with the
+            // rounding of one product carried along (one FMA each)
             const int p = (c + 1) % 3, q = (c + 2) % 3;
-            const double t = (double)f[3 + p] * sp[q] - (double)f[3 + q] * sp[p];
-            const double w = (double)f[p] * sp[q] - (double)f[q] * sp[p];
-            v[9 + c] = -__double2float_rn(t);
-            v[12 + c] = -__double2float_rn(w * (2.0 / 3.0));
+            v[9 + c] = -diff_of_products(f[3 + p], sp[q], f[3 + q], sp[p]);
+            v[12 + c] = (-2.f / 3.f) * diff_of_products(f[p], sp[q], f[q], sp[p]);
         }
     } else {
 #pragma unroll
@@ -263,6 +283,7 @@ __global__ void pack32_kernel(const double *__restrict__ Y, const double *__rest
 // FP64 records: 9 doubles per segment (Y, F, T); padding far away, no load.
 __global__ void pack64_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
                               int64_t S, int64_t Spad, SysMap sm, double *__restrict__ src) {
+    pdl_enter();
     const int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (P >= Spad) return;
     const int64_t i = segment_at(sm, P, S);
@@ -276,14 +297,6 @@ __global__ void pack64_kernel(const double *__restrict__ Y, const double *__rest
         o[0] = o[1] = o[2] = (double)kFarPad;
         for (int k = 0; k < 6; ++k) o[3 + k] = 0.0;
     }
-}
-
-// Error-free transformation s + e = a + b (Knuth's TwoSum), with the adds
-// kept out of FMA contraction and reassociation.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
 // 1/sqrt(x): one MUFU operation (PTX rsqrt.approx.ftz.f32, max relative error
@@ -453,9 +466,10 @@ __device__ __forceinline__ void combine_group(const float2 *acc, const float2 *t
         for (int c = 0; c < 6; ++c) out[c] = __fadd_rn(acc[c].x, acc[c].y);
         return;
     }
+    constexpr int kSums = Rec<kFrames>::kSums;
     float s[12];
 #pragma unroll
-    for (int c = 0; c < 12; ++c) s[c] = __fadd_rn(acc[c].x, acc[c].y);
+    for (int c = 0; c < kSums; ++c) s[c] = __fadd_rn(acc[c].x, acc[c].y);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const int p = (c + 1) % 3, q = (c + 2) % 3;
@@ -776,6 +790,7 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
     // target slot, and which of the SPLIT sets of source groups the thread takes
     const int tid = SPLIT == 1 ? (int)threadIdx.x : (int)(threadIdx.x % kRpyThreads);
     const int set = SPLIT == 1 ? 0 : (int)(threadIdx.x / kRpyThreads);
+    pdl_enter();
     const int64_t b = blockIdx.x;
     resolve_dyn(smap, W);
     int64_t u = unit_start(b, W, G);
@@ -1092,6 +1107,9 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
     if (u < u_end) {
         tile = u / n_units;
         ubeg = tile * n_units;
+    }
+    pdl_enter();
+    if (u < u_end) {
         stage_group(buf, src + kGroupF4 * (u - ubeg), lane);
     }
     int cur = 0;
@@ -1227,6 +1245,7 @@ rpy_pair64_kernel(const double *__restrict__ src, SysMap smap, int64_t W, int G,
     constexpr int kTile = kRpyThreads * TPT;
     __shared__ double sm[2][kRec];
     const int tid = threadIdx.x;
+    pdl_enter();
     const int64_t b = blockIdx.x;
     resolve_dyn(smap, W);
     int64_t u = unit_start(b, W, G);
@@ -1405,6 +1424,7 @@ __device__ __forceinline__ void add64(const double *f, const double *d, const do
 __global__ void __launch_bounds__(32)
 rpy_direct64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, int S,
                     RpyConst64 k, double scale, double *__restrict__ VW) {
+    pdl_enter();
     const int n = blockIdx.x, lane = threadIdx.x;
     const double t0 = Y[3 * (int64_t)n], t1 = Y[3 * (int64_t)n + 1], t2 = Y[3 * (int64_t)n + 2];
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -1474,6 +1494,7 @@ rpy_sym64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, in
         while ((J + 1) * J / 2 <= (int)blockIdx.x) ++J;
         I = (int)blockIdx.x - J * (J - 1) / 2;
     }
+    pdl_enter();
     {
         const int side = threadIdx.x >> 6, l = threadIdx.x & 63;
         const int n = (side ? J : I) * kSymTile + l;
@@ -1552,6 +1573,7 @@ rpy_sym64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, in
 __global__ void __launch_bounds__(64)
 sum64_kernel(const double *__restrict__ slots, int S, int tiles, double scale,
              double *__restrict__ VW) {
+    pdl_enter();
     const int n = blockIdx.x * 64 + threadIdx.x, c = blockIdx.y;
     if (n >= S) return;
     const int64_t rows = (int64_t)tiles * kSymTile;
@@ -1814,14 +1836,15 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     // (and read the unit count from the device), so captured graphs stay valid
     if (pair32_on(c)) {
         const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
-        pack<<<pgrid, pb, 0, c->stream>>>(Y, FT, S, c->Spad, sm, c->src32);
+        launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
+                   c->Spad, sm, c->src32);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         const RpyConst32 k = make_const<float, RpyConst32>(c->a);
         if (c->rpy_auto) {
             const int G = warp_grid(W, c->num_sms);
-            rpy_pair32_warp_kernel<<<G, 32 * kWarpCta, kWarpSmem, c->stream>>>(
-                c->src32, sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
+            launch_pdl(rpy_pair32_warp_kernel, G, 32 * kWarpCta, kWarpSmem, c->stream, c->src32, sm,
+                       W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
         } else {
             const int G = (int)(active_only ? c->rpy_grid32 : std::min<int64_t>(c->rpy_grid32, W));
             const bool split = c->rpy_tpt == 1 && c->rpy_split == 2;
@@ -1832,8 +1855,8 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
                               : (split               ? rpy_pair32_kernel<false, 1, 2>
                                  : c->rpy_tpt == 1   ? rpy_pair32_kernel<false, 1>
                                                      : rpy_pair32_kernel<false, 2>);
-            pair<<<G, kRpyThreads * (split ? 2 : 1), 0, c->stream>>>(
-                c->src32, sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
+            launch_pdl(pair, G, kRpyThreads * (split ? 2 : 1), 0, c->stream, c->src32, sm, W, G, k,
+                       (float *)c->partials, c->tile_cnt, scale, VW);
         }
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
@@ -1846,14 +1869,15 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
             if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
             if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
             if (S <= kDirectMaxSeg) {
-                rpy_direct64_kernel<<<(unsigned)S, 32, 0, c->stream>>>(Y, FT, (int)S, k, scale, VW);
+                launch_pdl(rpy_direct64_kernel, (unsigned)S, 32, 0, c->stream, Y, FT, (int)S, k, scale,
+                           VW);
                 c->n_launches += 1;
             } else {
                 const int tiles = (int)((S + kSymTile - 1) / kSymTile);
-                rpy_sym64_kernel<<<(unsigned)(tiles * (tiles + 1) / 2), kSymThreads, 0, c->stream>>>(
-                    Y, FT, (int)S, tiles, k, (double *)c->partials);
-                sum64_kernel<<<dim3((unsigned)((S + 63) / 64), 6), 64, 0, c->stream>>>(
-                    (const double *)c->partials, (int)S, tiles, scale, VW);
+                launch_pdl(rpy_sym64_kernel, (unsigned)(tiles * (tiles + 1) / 2), kSymThreads, 0,
+                           c->stream, Y, FT, (int)S, tiles, k, (double *)c->partials);
+                launch_pdl(sum64_kernel, dim3((unsigned)((S + 63) / 64), 6), 64, 0, c->stream,
+                           (const double *)c->partials, (int)S, tiles, scale, VW);
                 c->n_launches += 2;
             }
             if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
@@ -1864,15 +1888,11 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
             return cudaGetLastError();
         }
         const int G = (int)(active_only ? c->rpy_grid64 : std::min<int64_t>(c->rpy_grid64, W));
-        pack64_kernel<<<pgrid, pb, 0, c->stream>>>(Y, FT, S, c->Spad, sm, c->src64);
+        launch_pdl(pack64_kernel, pgrid, pb, 0, c->stream, Y, FT, S, c->Spad, sm, c->src64);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
-        if (c->rpy_tpt == 1)
-            rpy_pair64_kernel<1><<<G, kRpyThreads, 0, c->stream>>>(
-                c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
-        else
-            rpy_pair64_kernel<2><<<G, kRpyThreads, 0, c->stream>>>(
-                c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
+        launch_pdl(c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G, kRpyThreads, 0,
+                   c->stream, c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
     }
@@ -2115,12 +2135,11 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     float *part = reinterpret_cast<float *>(base + kNoAllocSrcBytes);
     // every source record up to Spad and every partial slot a tile's sum reads
     // is written below; the tile counters are zero between launches
-    const int pb = 256;
     SysMap sm{};                       // one system, no tables
     sm.n_tiles = tiles;
     sm.n_units = n_units;
     sm.n_src = n_seg;
-    cudaError_t e = launch(pack32_kernel<true>, (unsigned)((Spad + pb - 1) / pb), pb, 0, st, Y, FT, n_seg,
+    cudaError_t e = launch(pack32_kernel<true>, (unsigned)(Spad / kPackThreads), kPackThreads, 0, st, Y, FT, n_seg,
                            Spad, sm, src);
     if (e == cudaSuccess)
         e = launch(rpy_pair32_warp_kernel, (unsigned)G, 32 * kWarpCta, kWarpSmem, st,

@@ -39,6 +39,7 @@ __global__ void steric_bin_kernel(int64_t S, const double *__restrict__ Y,
                                   uint32_t mask, int cap, int *__restrict__ count,
                                   int *__restrict__ bucket, int4 *__restrict__ cell,
                                   float4 *__restrict__ frac, int *__restrict__ flags) {
+    pdl_enter();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= S) return;
     const double x = Y[3 * g], y = Y[3 * g + 1], z = Y[3 * g + 2];
@@ -66,6 +67,7 @@ steric_force_kernel(Layout lay, const double *__restrict__ Y, float hf, uint32_t
                     const int4 *__restrict__ cell, const float4 *__restrict__ frac, double a,
                     double FS, double chi, const int *__restrict__ active,
                     double *__restrict__ FT, int *__restrict__ flags) {
+    pdl_enter();
     static_assert(kStericNbrMax <= 64, "two candidates per lane");
     __shared__ int s_cand[kStericWarps][kStericNbrMax];
     __shared__ int s_sorted[kStericWarps][kStericNbrMax];
@@ -151,16 +153,16 @@ cudaError_t steric_forces(fil_ctx *c, bool active_only) {
     const uint32_t mask = (uint32_t)(c->steric_buckets - 1);
     cudaError_t e = cudaMemsetAsync(c->steric_count, 0, sizeof(int) * c->steric_buckets, c->stream);
     if (e != cudaSuccess) return e;
-    steric_bin_kernel<<<(unsigned)((S + 255) / 256), 256, 0, c->stream>>>(
-        S, c->Yc, c->lay.sys_of, h, 1.0 / h, mask, kStericCap, c->steric_count, c->steric_bucket,
-        c->steric_cell, c->steric_frac, c->d_flags);
-    steric_force_kernel<<<(unsigned)((S + kStericWarps - 1) / kStericWarps), 32 * kStericWarps, 0,
-                          c->stream>>>(
-        c->lay, c->Yc, (float)h, mask, kStericCap, c->steric_count, c->steric_bucket,
-        c->steric_cell, c->steric_frac, c->a, c->steric_FS, c->steric_chi,
-        active_only ? c->d_active : nullptr, c->FT, c->d_flags);
+    e = launch_pdl(steric_bin_kernel, (unsigned)((S + 255) / 256), 256, 0, c->stream, S, c->Yc,
+                   c->lay.sys_of, h, 1.0 / h, mask, kStericCap, c->steric_count, c->steric_bucket,
+                   c->steric_cell, c->steric_frac, c->d_flags);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(steric_force_kernel, (unsigned)((S + kStericWarps - 1) / kStericWarps),
+                   32 * kStericWarps, 0, c->stream, c->lay, c->Yc, (float)h, mask, kStericCap,
+                   c->steric_count, c->steric_bucket, c->steric_cell, c->steric_frac, c->a,
+                   c->steric_FS, c->steric_chi, active_only ? c->d_active : nullptr, c->FT, c->d_flags);
     c->n_launches += 2;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace fil
