@@ -252,14 +252,20 @@ inline bool fast_mixed(const fil_ctx *c) { return c->prec == FIL_MIXED; }
 // launch_pdl starts with pdl_enter). What overlaps is the launch itself: the
 // iterations of small systems are chains of a dozen kernels of 2-10 us, and each
 // boundary cost 1-2 us more.
+//
+// launch_dep with early == false is the plain launch. CTAs that become resident
+// early go to whatever SMs have room at that moment, several to one SM while
+// others get none, and keep that placement. A kernel of one wave or less that
+// is bound by each SM's FP64 rate then waits for the fullest SM, so such kernels
+// start early only while they are small; the lines are measured at each launch.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t st, Args &&...args) {
+inline cudaError_t launch_dep(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                              size_t smem, cudaStream_t st, Args &&...args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
@@ -269,8 +275,14 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, Args &&...args) {
+    return launch_dep(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // Launchers (all enqueue on c->stream and return a cudaError_t).

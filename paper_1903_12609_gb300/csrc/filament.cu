@@ -414,6 +414,8 @@ __global__ void commit_kernel(Layout lay, const double *__restrict__ X,
     }
 }
 
+constexpr int kUnpackEarly = 6000, kRowsEarly = 512;   // segments of one system, see the launches
+
 unsigned warp_grid(int M, int threads) { return (unsigned)(((int64_t)M * 32 + threads - 1) / threads); }
 unsigned seg_grid(int64_t S, int threads) { return (unsigned)((S + threads - 1) / threads); }
 
@@ -424,8 +426,12 @@ cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool act
     ForceParams fp{c->dL, c->KB, c->KT, c->g0, c->kmu, c->knu};
     const auto kernel = step ? unpack_forces_kernel<true> : unpack_forces_kernel<false>;
     c->n_launches += 1;
+    // Early (launch_dep) up to kUnpackEarly segments: one time step of a 32-segment
+    // filament cloud took 3363 us with the early launch and 3401 us without at 4 000
+    // segments, 6192 and 6100 at 8 000, 16.44 and 16.29 ms at 16 000. Ensembles: 0.1%.
+    const bool early = c->n_sys > 1 || c->lay.S <= kUnpackEarly;
     // (X is written only where step is set, and is then c->Xn)
-    return launch_pdl(kernel, warp_grid(c->lay.M, 128), 128, 0, c->stream, c->lay,
+    return launch_dep(early, kernel, warp_grid(c->lay.M, 128), 128, 0, c->stream, c->lay,
                       const_cast<double *>(X), c->Xk, c->w, c->n_sys, eval ? c->d_finf : nullptr,
                       c->q, fp, c->has_Fext ? c->Fext : nullptr, c->has_Text ? c->Text : nullptr,
                       c->has_follower ? c->follower : nullptr, with_forces,
@@ -441,8 +447,13 @@ cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *
         sc = {1.0, 0.0, c->dt, 0.0};
     }
     c->n_launches += 1;
-    return launch_pdl(residual_rows_kernel, seg_grid(c->lay.S, kRowThreads), kRowThreads, 0, c->stream,
-                      c->lay, X, c->Yc, c->VW, c->Y, c->Yprev, c->uprev, sc,
+    // Early (launch_dep) behind the FP64 kernels, in ensembles and up to kRowsEarly
+    // segments. Behind the FP32 kernel of one system, whose CTAs all leave room, the rows
+    // crowd: a residual took 62.2 us early and 63.6 us plainly at 320 segments, 65.8 and
+    // 63.8 at 640, 87.3 and 77.9 at 2 560, 175 and 168 at 8 000.
+    const bool early = c->n_sys > 1 || !pair32_on(c) || c->lay.S <= kRowsEarly;
+    return launch_dep(early, residual_rows_kernel, seg_grid(c->lay.S, kRowThreads), kRowThreads, 0,
+                      c->stream, c->lay, X, c->Yc, c->VW, c->Y, c->Yprev, c->uprev, sc,
                       fprev ? c->d_active : nullptr, fprev, f, c->d_finf);
 }
 
