@@ -172,13 +172,16 @@ void carve(fil_ctx *c, Arena &ar, int red_blocks, size_t partial_bytes) {
     if (c->j0_model == FIL_J0_DRAG) {
         c->band = fast_mixed(c) ? nullptr : ar.take<double>((size_t)nband * kBandW);
         c->band32 = fast_mixed(c) ? ar.take<float>((size_t)nband * kBandW) : nullptr;
+        const bool blocked = block_solve_on(c);
+        c->bmaps = blocked ? ar.take<double>((size_t)c->bmaps_len) : nullptr;
         c->jinv = nullptr;
-        c->jofs = nullptr;
+        c->jofs = blocked ? ar.take<int64_t>(M + 1) : nullptr;
         c->aux = nullptr;
         c->auxofs = nullptr;
     } else {
         c->band = nullptr;
         c->band32 = nullptr;
+        c->bmaps = nullptr;
         c->jinv = ar.take<float>((size_t)c->jdense_len);
         c->jofs = ar.take<int64_t>(M + 1);
         c->aux = ar.take<double>((size_t)c->aux_len);
@@ -377,13 +380,15 @@ fil_status fil_create_ensemble(const fil_params *p, int32_t n_sys, const int32_t
     blk_beg.push_back(6 * S);
     std::vector<int64_t> sys_xoff(n_sys + 1);
     for (int s = 0; s <= n_sys; ++s) sys_xoff[s] = 6 * c->sys_seg_off_h[s];
-    std::vector<int64_t> jofs(p->n_fil + 1, 0), auxofs(p->n_fil + 1, 0);
+    std::vector<int64_t> jofs(p->n_fil + 1, 0), auxofs(p->n_fil + 1, 0), bofs(p->n_fil + 1, 0);
     for (int i = 0; i < p->n_fil; ++i) {
         const int64_t Ni = c->N_host[i];
         jofs[i + 1] = jofs[i] + 36 * Ni * Ni;
+        bofs[i + 1] = bofs[i] + (6 * Ni - 3 + kBlkRows - 1) / kBlkRows;
         auxofs[i + 1] = auxofs[i] + 60 * Ni + 5 * Ni * Ni;   // layout in jacobian_dense.cu
     }
     c->jdense_len = jofs[p->n_fil];
+    c->bmaps_len = bofs[p->n_fil] * kBlkDoubles;
     c->aux_len = auxofs[p->n_fil];
     c->stream = (cudaStream_t)p->stream;
     c->have_prev = 0; c->ylev = 0; c->hist = 0; c->steps = 0; c->k = 0; c->in_step = 0;
@@ -459,7 +464,8 @@ fil_status fil_create_ensemble(const fil_params *p, int32_t n_sys, const int32_t
         e = cudaMemcpyAsync(c->q, q0.data(), sizeof(double) * 4 * S, cudaMemcpyHostToDevice,
                             c->stream);
     if (e == cudaSuccess && c->jofs)
-        e = cudaMemcpyAsync(c->jofs, jofs.data(), sizeof(int64_t) * (p->n_fil + 1),
+        e = cudaMemcpyAsync(c->jofs, (c->bmaps ? bofs : jofs).data(),
+                            sizeof(int64_t) * (p->n_fil + 1),
                             cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess && c->auxofs)
         e = cudaMemcpyAsync(c->auxofs, auxofs.data(), sizeof(int64_t) * (p->n_fil + 1),

@@ -26,6 +26,8 @@ constexpr int kBandKL = 8;
 constexpr int kBandKU = 8;
 constexpr int kBandW = 2 * kBandKL + kBandKU + 1;   // row window: c - i in [-8, 16]
 constexpr size_t kSolveSmemMax = 200 * 1024;        // shared memory of one band-solve CTA
+constexpr int kBlkRows = 16, kBlkDoubles = 1088;     // a block of the blocked solve (jacobian.cu)
+constexpr int kBlkMaxSeg = 16384;
 constexpr int kMaxSegPerFil = (int)(kSolveSmemMax / (6 * sizeof(double)));
 // The filament-RPY J0 keeps a filament's block in shared memory for its
 // FP32 inverse: (6N)^2 floats <= 200 KB, i.e. N <= 38; refinement steps per solve.
@@ -170,10 +172,12 @@ struct fil_ctx {
     int j0_model;
     double *band;
     float *band32;         // the band in FP32, factored in place (mixed precision; band unused)
+    double *bmaps;         // the blocked solve's maps (jacobian.cu), or null
     int *piv;
     float *jinv;           // per filament: FP32 J0, then its inverse in place
-    int64_t *jofs;         // [M+1] offsets of the (6N)^2 blocks
+    int64_t *jofs;         // [M+1] offsets of the (6N)^2 blocks, or of bmaps in blocks
     int64_t jdense_len;
+    int64_t bmaps_len;
     double *aux;           // per-filament FP64 data of J0 (matrix-free residual)
     int64_t *auxofs;       // [M+1]
     int64_t aux_len;
@@ -319,6 +323,7 @@ cudaError_t init_straight(fil_ctx *c, const double *base, const double *t, const
 cudaError_t extrapolate_guess(fil_ctx *c, double *X0);
 cudaError_t commit_state(fil_ctx *c, const double *X);
 
+bool block_solve_on(const fil_ctx *c);      // drag model: the solve runs in blocks of rows
 cudaError_t j0_build_factor(fil_ctx *c, const double *X);
 // active non-null: filaments of converged systems are skipped (their rows of x
 // are left as they were)

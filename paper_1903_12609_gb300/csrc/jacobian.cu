@@ -224,12 +224,106 @@ band_lu_kernel(Layout lay, T *__restrict__ band_all, int *__restrict__ piv_all,
 #undef RB
 }
 
+// 1/x by Newton's iteration y += y (1 - x y) from the hardware's seed (about
+// 2^-20): two steps, each one fused residual and one fused update, leave an
+// error of rounding size. The seed flushes what 1/x or x would make subnormal,
+// so those, infinities and NaN divide.
+__device__ __forceinline__ double recip(double x) {
+    const int e = (__double2hiint(x) >> 20) & 0x7ff;
+    if (e < 2 || e > 2044) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
+constexpr int kLu64Threads = 128;
+
+// The same elimination in FP64 for one system: a CTA per filament. A column is
+// one chain (pivot search, reciprocal, multipliers, rank-1 update, next column)
+// and a warp instruction on FP64 takes 64 cycles of its quarter of the SM, so
+// what counts is the number of them in one warp's chain. Each of the 128
+// threads updates one element (8 rows x 16 columns, one warp instruction on
+// each quarter), the pivot search compares bit patterns as integers, the nine
+// candidates' reciprocals are formed beside it by recip above, and rows are
+// exchanged by reading from the other row. One 20-segment filament (117
+// columns): 168 us with one warp's work as in band_lu_kernel, 75 us here.
+// Ensembles keep band_lu_kernel: their iteration counts follow the last bit.
+__global__ void __launch_bounds__(kLu64Threads)
+band_lu64_kernel(Layout lay, double *__restrict__ band_all, int *__restrict__ piv_all,
+                 int *__restrict__ flags) {
+    static_assert(kLu64Threads == 16 * kBandKL && kBandKL + kBandKU == 16, "a thread per element");
+    __shared__ double R[kLuRing * kBandW];
+    const int f = blockIdx.x, t = threadIdx.x, lane = t & 31;
+    const int s0 = lay.off[f];
+    const int n = 6 * (lay.off[f + 1] - s0) - 3;
+    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)f;
+    double *G = band_all + row0 * kBandW;
+    int *piv = piv_all + row0;
+#define RB(i, c) R[((i) & (kLuRing - 1)) * kBandW + ((c) - (i) + kBandKL)]
+    for (int r = 0; r < kLuAhead && r < n; ++r)
+        if (t < kBandW) cp_async_elem(&R[r * kBandW + t], G + (int64_t)r * kBandW + t);
+    cp_async_commit();
+    cp_async_wait<0>();
+    for (int j = 0; j < n; ++j) {
+        {
+            const int r = j + kLuAhead;
+            if (r < n && t < kBandW)
+                cp_async_elem(&R[(r & (kLuRing - 1)) * kBandW + t], G + (int64_t)r * kBandW + t);
+            cp_async_commit();
+        }
+        // rows up to j + 8, requested at column j + 8 - kLuAhead or before, have landed
+        cp_async_wait<kLuAhead - kBandKL>();
+        __syncthreads();
+        const int last = min(n - 1, j + kBandKL);
+        // pivot: first row of maximal |A(i, j)|, i in [j, last] (every warp finds it)
+        const bool cand = lane <= kBandKL && j + lane <= last;
+        const double v = cand ? RB(j + lane, j) : 0.0;
+        const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu;
+        const unsigned lo = (unsigned)__double2loint(v);
+        const double rv = recip(cand && (hi | lo) ? v : 1.0);
+        const unsigned mhi = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
+        const int pl = __ffs(__ballot_sync(0xffffffffu, cand && hi == mhi && lo == mlo)) - 1;
+        const int p = j + pl;
+        const bool zero = (mhi | mlo) == 0;
+        const double inv = zero ? 0.0 : __shfl_sync(0xffffffffu, rv, pl);
+        const int cmax = min(n - 1, j + kBandKL + kBandKU);
+        // element (i, c) of the trailing window, from row j where the rows change places
+        const int i = j + 1 + (t >> 4), c = j + 1 + (t & 15);
+        const int src = i == p ? j : i;
+        const bool in = i <= last && c <= cmax;
+        double l = 0.0, a = 0.0;
+        if (i <= last) l = RB(src, j) * inv;
+        if (in) a = fma(-l, RB(p, c), RB(src, c));
+        // row j is final: the multipliers that lie in it, the reciprocal pivot, U
+        if (t < kBandW) {
+            const int cj = j + t - kBandKL;
+            G[(int64_t)j * kBandW + t] = t < kBandKL                 ? R[(j & (kLuRing - 1)) * kBandW + t]
+                                         : t == kBandKL ? inv
+                                         : cj <= cmax   ? RB(p, cj)
+                                                        : 0.0;
+        }
+        if (t == 0) {
+            piv[j] = p;
+            if (zero) atomicOr(flags + 1, 1);
+        }
+        __syncthreads();
+        if (!zero) {
+            if (in) RB(i, c) = a;
+            if ((t & 15) == 0 && i <= last) RB(i, j) = l;
+        }
+    }
+#undef RB
+}
+
 constexpr int kSolvePf = 8;     // rows of factors loaded ahead by the band solve
 constexpr int kSolveLanes = 16; // lanes per filament
 
-// x = J0^{-1} b for every filament (b and x in the X / f layout; may alias),
-// with the factors and the working vector in precision T, 16 lanes (half a
-// warp) per filament.
+// Forward and backward substitution in the banded factors for one right-hand
+// side z (n entries in shared memory, in band order, zero before row jf), by
+// 16 lanes, half a warp; the two halves of a warp run the longer one's n_both
+// steps together.
 //
 // A row step is a chain: the finished entry z_j, one multiply-add in each row
 // it reaches, the next finished entry. The window of rows it reaches (j + 1 ..
@@ -240,58 +334,21 @@ constexpr int kSolveLanes = 16; // lanes per filament
 // instructions of a whole warp. One 20-segment filament in FP64 41 -> 30 us,
 // where the FP64 unit takes 64 cycles per warp instruction; the steps of 256
 // ensemble systems in FP32 80.5 -> 77.7 ms. Same bits.)
-// The two halves of a warp run the longer one's steps together.
 template <typename T>
-__global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
-                                  const int *__restrict__ piv_all, double ct,
-                                  const double *b, double *x, int zmax,
-                                  const int *__restrict__ active, int fil_per_cta) {
-    extern __shared__ __align__(16) unsigned char zraw[];
-    pdl_enter();
-    const int slot = threadIdx.x / kSolveLanes;        // filament within the CTA
-    const int lane = threadIdx.x % kSolveLanes;
-    const int f = blockIdx.x * fil_per_cta + slot;
-    // (a half without a filament, or of a converged system, takes no rows)
-    bool live = slot < fil_per_cta && f < lay.M;
-    int s0 = 0, N = 0;
-    if (live) {
-        s0 = lay.off[f];
-        N = lay.off[f + 1] - s0;
-        if (active && !active[lay.sys_of[s0]]) live = false;
-    }
-    const int n = live ? 6 * N - 3 : 0;
-    const int n_both = max(n, __shfl_xor_sync(0xffffffffu, n, kSolveLanes));
-    if (n_both == 0) return;
-    T *z = reinterpret_cast<T *>(zraw) + (int64_t)(live ? slot : 0) * zmax;
-    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)(live ? f : 0);
-    const T *A = band_all + row0 * kBandW;
-    const int *piv = piv_all + row0;
-    const double *bf = b + 6 * (int64_t)s0;
-    double *xf = x + 6 * (int64_t)s0;
+__device__ __forceinline__ void band_substitute(const T *__restrict__ A,
+                                                const int *__restrict__ piv, T *z, int n,
+                                                int n_both, int lane, int jf) {
 #define BAND(i, c) A[(int64_t)(i) * kBandW + ((c) - (i) + kBandKL)]
-    // gather the right-hand side in band order
-    double b1x = 0.0, b1y = 0.0, b1z = 0.0;
-    if (live) {
-        for (int e = lane; e < 3 * N; e += kSolveLanes) {
-            const int s = e / 3, r = e % 3;
-            z[6 * s + r] = (T)bf[3 + 3 * s + r];   // rotation rows of segment s
-            if (s <= N - 2) {
-                const double b3n = bf[3 + 3 * N + 3 * s + r];                  // f3 of segment s+1
-                const double b3p = (s == 0) ? bf[r] : bf[3 + 3 * N + 3 * (s - 1) + r];
-                z[6 * s + 3 + r] = (T)(b3n - b3p);
-            }
-        }
-        b1x = bf[0];
-        b1y = bf[1];
-        b1z = bf[2];
-    }
-    __syncwarp();
     // The factors a row step needs do not depend on z, so each lane loads them
     // kSolvePf rows ahead into a register queue: the loads of the next block are
     // in flight while the current block's chain runs.
     // forward: L with row interchanges applied in elimination order; lane l holds
     // the row r in [j, j + 15] with r = l (mod 16)
-    T w = lane < n ? z[lane] : T(0);
+    T w;
+    {
+        const int r = jf + ((lane - jf) & (kSolveLanes - 1));
+        w = r < n ? z[r] : T(0);
+    }
     {
         T lq[kSolvePf];
         int pq[kSolvePf];
@@ -301,8 +358,8 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
             p = j < n ? piv[j] : j;
         };
 #pragma unroll
-        for (int u = 0; u < kSolvePf; ++u) fetch(u, lq[u], pq[u]);
-        for (int jb = 0; jb < n_both; jb += kSolvePf) {
+        for (int u = 0; u < kSolvePf; ++u) fetch(jf + u, lq[u], pq[u]);
+        for (int jb = jf; jb < n_both; jb += kSolvePf) {
             T ln[kSolvePf];
             int pn[kSolvePf];
 #pragma unroll
@@ -381,6 +438,57 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
         }
     }
     __syncwarp();
+#undef BAND
+}
+
+// x = J0^{-1} b for every filament (b and x in the X / f layout; may alias),
+// with the factors and the working vector in precision T, 16 lanes (half a
+// warp) per filament.
+template <typename T>
+__global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
+                                  const int *__restrict__ piv_all, double ct,
+                                  const double *b, double *x, int zmax,
+                                  const int *__restrict__ active, int fil_per_cta) {
+    extern __shared__ __align__(16) unsigned char zraw[];
+    pdl_enter();
+    const int slot = threadIdx.x / kSolveLanes;        // filament within the CTA
+    const int lane = threadIdx.x % kSolveLanes;
+    const int f = blockIdx.x * fil_per_cta + slot;
+    // (a half without a filament, or of a converged system, takes no rows)
+    bool live = slot < fil_per_cta && f < lay.M;
+    int s0 = 0, N = 0;
+    if (live) {
+        s0 = lay.off[f];
+        N = lay.off[f + 1] - s0;
+        if (active && !active[lay.sys_of[s0]]) live = false;
+    }
+    const int n = live ? 6 * N - 3 : 0;
+    const int n_both = max(n, __shfl_xor_sync(0xffffffffu, n, kSolveLanes));
+    if (n_both == 0) return;
+    T *z = reinterpret_cast<T *>(zraw) + (int64_t)(live ? slot : 0) * zmax;
+    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)(live ? f : 0);
+    const T *A = band_all + row0 * kBandW;
+    const int *piv = piv_all + row0;
+    const double *bf = b + 6 * (int64_t)s0;
+    double *xf = x + 6 * (int64_t)s0;
+    // gather the right-hand side in band order
+    double b1x = 0.0, b1y = 0.0, b1z = 0.0;
+    if (live) {
+        for (int e = lane; e < 3 * N; e += kSolveLanes) {
+            const int s = e / 3, r = e % 3;
+            z[6 * s + r] = (T)bf[3 + 3 * s + r];   // rotation rows of segment s
+            if (s <= N - 2) {
+                const double b3n = bf[3 + 3 * N + 3 * s + r];                  // f3 of segment s+1
+                const double b3p = (s == 0) ? bf[r] : bf[3 + 3 * N + 3 * (s - 1) + r];
+                z[6 * s + 3 + r] = (T)(b3n - b3p);
+            }
+        }
+        b1x = bf[0];
+        b1y = bf[1];
+        b1z = bf[2];
+    }
+    __syncwarp();
+    band_substitute(A, piv, z, n, n_both, lane, 0);
     if (!live) return;
     // scatter back: u_s, Lam_j, and Y_1 = b1 + c_t Lam_0
     for (int e = lane; e < 3 * N; e += kSolveLanes) {
@@ -395,9 +503,219 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
         xf[1] = b1y + ct * l1;
         xf[2] = b1z + ct * l2;
     }
+}
+
+// The solve of one FP64 system in blocks of kBlk rows. Substitution row by row is
+// a serial chain of 2 (6N - 3) steps, and a chain step on FP64 (a multiply-add or
+// two, each 64 cycles of a quarter of the SM, and the shuffle between) costs the
+// same whether one row or 32 take part. So each factorization also forms, for
+// every block of kBlk columns, what its steps do together to the rows they
+// reach: forward, interchanges included, one dense map of the kBlk + 8 rows
+// from the block's first on (F); backward one of the block's kBlk entries to
+// the solution there and to the updates of the 16 rows above (B). A solve is
+// then one small matrix-vector product per block and direction, whose columns
+// spread over the lanes of four warps.
+//
+// The maps are made of the same factors. Against extended arithmetic a solve is as
+// close as row by row: relative error 1.05e-15 and 1.23e-15 (rms, blocks and rows)
+// at 20 segments, 2.09e-15 and 2.12e-15 at 40, 5.07e-15 and 5.16e-15 for 4 x 64; the
+// full inverse of a filament's band, as quick to apply, was 1.3 to 2 times as far
+// off. Blocks of 16 rows fill four warps (F: 24 x 24, B: 32 x 16); larger ones do
+// more work per row (24: F 32 x 32, B 40 x 24).
+//
+// One 20-segment filament: a solve 33 -> 14.6 us, forming the maps 14.5 us once a
+// factorization. The rule (block_solve_on) is two filaments for each SM, as long as
+// the chains bound the solve and not the SMs' FP64 rate. Four time steps at drag
+// mobility, rows and blocks: 1 x 20 segments 5.20 and 3.35 ms, 1 x 100 30.9 and 15.9,
+// 20 x 32 14.9 and 11.4, 152 x 10 13.0 and 12.6, 304 x 10 43.2 and 42.4. Beyond, each
+// filament added costs a block's 4x as many multiply-adds. kBlkMaxSeg bounds the maps'
+// memory (3.3 KB a segment). Ensembles keep the rows: their iteration counts follow
+// the last bit.
+constexpr int kBlk = kBlkRows;
+constexpr int kFwd = kBlk + kBandKL;                       // rows (and columns) of F
+constexpr int kBwd = kBlk + kBandKL + kBandKU;             // rows of B
+constexpr int kBlkThreads = 128;                           // 8 rows x 4 column groups a warp
+constexpr int kFwdThreads = 4 * kFwd;
+static_assert(4 * kBwd == kBlkThreads && kBwd == 32 && kFwd == 24, "the lanes' share of F and B");
+static_assert(kFwd * kFwd + kBwd * kBlk == kBlkDoubles, "doubles of a block's maps");
+
+// Position of (row, column) of F or B in the order the solve's threads read them:
+// thread (row / 8) 32 + (column mod 4) 8 + row mod 8 takes columns 4 k + column mod 4.
+__device__ __forceinline__ int map_pos(int r, int c, int threads) {
+    return (c >> 2) * threads + (r >> 3) * 32 + (c & 3) * 8 + (r & 7);
+}
+
+// F (blockIdx.z = 0) and B (1) of one block, by one warp: the block's steps
+// applied to unit vectors, a lane per column (F) or two (B, half the rows each).
+__global__ void __launch_bounds__(32)
+band_block_kernel(Layout lay, const int64_t *__restrict__ bofs, const double *__restrict__ band_all,
+                  const int *__restrict__ piv_all, double *__restrict__ maps) {
+    __shared__ double rows[kBwd * kBandW];     // the band rows the block reaches
+    __shared__ double w[kBwd][32];             // the vectors: [row of the window][lane]
+    pdl_enter();
+    const int f = blockIdx.x, lane = threadIdx.x;
+    const int s0 = lay.off[f];
+    const int n = 6 * (lay.off[f + 1] - s0) - 3;
+    const int jb = kBlk * blockIdx.y;
+    if (jb >= n) return;
+    const int64_t row0 = 6 * (int64_t)s0 - 3 * (int64_t)f;
+    double *out = maps + (bofs[f] + blockIdx.y) * kBlkDoubles;
+    const int steps = min(kBlk, n - jb);
+    const bool forward = blockIdx.z == 0;
+    const int i0 = forward ? jb : jb - (kBandKL + kBandKU);     // first row of the window
+    const int ni = forward ? kFwd : kBwd;
+    for (int e = lane; e < ni * kBandW; e += 32) {
+        const int i = i0 + e / kBandW;
+        rows[e] = i >= 0 && i < n ? band_all[(row0 + i0) * kBandW + e] : 0.0;
+    }
+#define BAND(i, c) rows[((i) - i0) * kBandW + ((c) - (i) + kBandKL)]
+    if (forward) {
+        for (int r = 0; r < kFwd; ++r) w[r][lane] = r == lane ? 1.0 : 0.0;
+        int pv = lane < steps ? piv_all[row0 + jb + lane] - jb : 0;
+        __syncwarp();
+        for (int jj = 0; jj < steps; ++jj) {
+            const int p = __shfl_sync(0xffffffffu, pv, jj);
+            const double z = w[p][lane];
+            w[p][lane] = w[jj][lane];
+            w[jj][lane] = z;
+#pragma unroll
+            for (int d = 1; d <= kBandKL; ++d)       // (rows past the last hold zeros)
+                w[jj + d][lane] = fma(-BAND(jb + jj + d, jb + jj), z, w[jj + d][lane]);
+        }
+        if (lane < kFwd)
+            for (int r = 0; r < kFwd; ++r) out[map_pos(r, lane, kFwdThreads)] = w[r][lane];
+    } else {
+        const int c = lane & (kBlk - 1), half = lane / kBlk;
+        for (int r = half; r < kBwd; r += 2) w[r][c] = r == c + kBwd - kBlk ? 1.0 : 0.0;
+        __syncwarp();
+        for (int jj = steps - 1; jj >= 0; --jj) {
+            const int j = jb + jj, rj = jj + kBwd - kBlk;
+            const double z = w[rj][c] * BAND(j, j);
+            __syncwarp();
+            if (half == 0) w[rj][c] = z;
+#pragma unroll
+            for (int d = 0; d < (kBandKL + kBandKU) / 2; ++d) {
+                const int r = jj + half * (kBandKL + kBandKU) / 2 + d;      // row i0 + r
+                w[r][c] = fma(-BAND(i0 + r, j), z, w[r][c]);                // (zeros above row 0)
+            }
+            __syncwarp();
+        }
+        out += kFwd * kFwd;
+        for (int r = half; r < kBwd; r += 2) out[map_pos(r, c, kBlkThreads)] = w[r][c];
+    }
 #undef BAND
 }
 
+// x = J0^{-1} b with those maps, a CTA per filament (b and x may alias: b is read
+// before x is written). Each step reads the block's input from one of two small
+// buffers and leaves the next block's in the other, one barrier a step; the maps
+// of the next step are loaded during it.
+__global__ void __launch_bounds__(kBlkThreads)
+band_block_solve_kernel(Layout lay, const int64_t *__restrict__ bofs,
+                        const double *__restrict__ maps, double ct, int zmax, const double *b,
+                        double *x) {
+    extern __shared__ __align__(16) unsigned char zraw[];
+    __shared__ double next[2][kBlk];
+    pdl_enter();
+    const int f = blockIdx.x, t = threadIdx.x;
+    const int s0 = lay.off[f];
+    const int N = lay.off[f + 1] - s0;
+    const int n = 6 * N - 3;
+    const int nb = (n + kBlk - 1) / kBlk;
+    double *z = reinterpret_cast<double *>(zraw);     // the right-hand side, in band order
+    double *y = z + zmax;                             // after the forward pass, then x
+    const double *bf = b + 6 * (int64_t)s0;
+    double *xf = x + 6 * (int64_t)s0;
+    const double *mf = maps + bofs[f] * kBlkDoubles + t;
+    const int row = (t >> 5) * 8 + (t & 7), g = (t >> 3) & 3;     // row of the map, column group
+    constexpr int kF = kFwd / 4, kB = kBlk / 4;
+    double m[kF];
+    if (t < kFwdThreads) {
+#pragma unroll
+        for (int k = 0; k < kF; ++k) m[k] = mf[k * kFwdThreads];
+    }
+    for (int i = t; i < nb * kBlk + kBandKL; i += kBlkThreads) {
+        const int s = i / 6, q = i % 6;
+        double v = 0.0;                               // (rows past the last)
+        if (i < n) {
+            if (q < 3) {
+                v = bf[3 + 3 * s + q];                // rotation rows of segment s
+            } else {                                  // f3 of segment s + 1, less that of s
+                const int r = q - 3;
+                v = bf[3 + 3 * N + 3 * s + r] -
+                    (s == 0 ? bf[r] : bf[3 + 3 * N + 3 * (s - 1) + r]);
+            }
+        }
+        z[i] = v;
+        if (i < kBandKL) next[0][i] = v;
+    }
+    const double b1 = t < 3 ? bf[t] : 0.0;
+    __syncthreads();
+    for (int k0 = 0; k0 < nb; ++k0) {
+        const int jb = k0 * kBlk, now = k0 & 1;
+        double a = 0.0, mn[kF];
+        if (t < kFwdThreads) {
+            if (k0 + 1 < nb) {
+#pragma unroll
+                for (int k = 0; k < kF; ++k)
+                    mn[k] = mf[(int64_t)(k0 + 1) * kBlkDoubles + k * kFwdThreads];
+            }
+#pragma unroll
+            for (int k = 0; k < kF; ++k)
+                a = fma(m[k], 4 * k < kBandKL ? next[now][4 * k + g] : z[jb + 4 * k + g], a);
+            a += __shfl_xor_sync(0xffffffffu, a, 8);
+            a += __shfl_xor_sync(0xffffffffu, a, 16);
+            if (g == 0) {
+                if (row < kBlk)
+                    y[jb + row] = a;
+                else
+                    next[now ^ 1][row - kBlk] = a;
+            }
+#pragma unroll
+            for (int k = 0; k < kF; ++k) m[k] = mn[k];
+        }
+        if (k0 + 1 < nb) __syncthreads();
+    }
+    mf += kFwd * kFwd;
+#pragma unroll
+    for (int k = 0; k < kB; ++k) m[k] = mf[(int64_t)(nb - 1) * kBlkDoubles + k * kBlkThreads];
+    __syncthreads();
+    if (t < kBlk) next[0][t] = y[(nb - 1) * kBlk + t];
+    __syncthreads();
+    for (int k0 = nb - 1, now = 0; k0 >= 0; --k0, now ^= 1) {
+        const int jb = k0 * kBlk;
+        double mn[kB];
+        if (k0 > 0) {
+#pragma unroll
+            for (int k = 0; k < kB; ++k)
+                mn[k] = mf[(int64_t)(k0 - 1) * kBlkDoubles + k * kBlkThreads];
+        }
+        double a = 0.0;
+#pragma unroll
+        for (int k = 0; k < kB; ++k) a = fma(m[k], next[now][4 * k + g], a);
+        a += __shfl_xor_sync(0xffffffffu, a, 8);
+        a += __shfl_xor_sync(0xffffffffu, a, 16);
+        if (g == 0) {
+            if (row >= kBlk)
+                y[jb + row - kBlk] = a;
+            else if (k0 > 0)
+                next[now ^ 1][row] = y[jb - kBlk + row] + a;
+        }
+#pragma unroll
+        for (int k = 0; k < kB; ++k) m[k] = mn[k];
+        __syncthreads();
+    }
+    // scatter: u_s, Lam_j, and Y_1 = b1 + c_t Lam_0
+    for (int i = t; i < n; i += kBlkThreads) {
+        const int s = i / 6, q = i % 6;
+        xf[q < 3 ? 3 + 3 * s + q : 3 + 3 * N + 3 * s + q - 3] = y[i];
+    }
+    if (t < 3) xf[t] = b1 + ct * (N >= 2 ? y[3 + t] : 0.0);
+}
+
+size_t block_solve_smem(const fil_ctx *c) {
+    return 2 * sizeof(double) * (size_t)(6 * c->lay.maxN + 2 * kBlk);
+}
 
 J0Params make_params(const fil_ctx *c) {
     const double beta = c->have_prev ? 2.0 / 3.0 : 1.0;
@@ -407,6 +725,11 @@ J0Params make_params(const fil_ctx *c) {
 }
 
 }  // namespace
+
+bool block_solve_on(const fil_ctx *c) {
+    return c->n_sys == 1 && !fast_mixed(c) && c->lay.M <= 2 * c->num_sms && c->lay.S <= kBlkMaxSeg &&
+           block_solve_smem(c) <= kSolveSmemMax;
+}
 
 cudaError_t j0_build_factor(fil_ctx *c, const double *X) {
     const unsigned grid = (unsigned)(((int64_t)c->lay.M * 32 + kJ0Threads - 1) / kJ0Threads);
@@ -422,16 +745,39 @@ cudaError_t j0_build_factor(fil_ctx *c, const double *X) {
     } else {
         j0_build_kernel<double><<<grid, kJ0Threads, 0, c->stream>>>(c->lay, X, c->qc, c->Tint, p,
                                                                     c->band);
-        band_lu_kernel<double><<<grid, kJ0Threads, 0, c->stream>>>(c->lay, c->band, c->piv,
-                                                                   c->d_flags);
+        if (c->n_sys == 1)
+            band_lu64_kernel<<<c->lay.M, kLu64Threads, 0, c->stream>>>(c->lay, c->band, c->piv,
+                                                                       c->d_flags);
+        else
+            band_lu_kernel<double><<<grid, kJ0Threads, 0, c->stream>>>(c->lay, c->band, c->piv,
+                                                                       c->d_flags);
     }
     c->n_launches += 2;
+    if (c->bmaps) {
+        const unsigned blocks = (unsigned)((6 * c->lay.maxN - 3 + kBlk - 1) / kBlk);
+        c->n_launches += 1;
+        return launch_pdl(band_block_kernel, dim3((unsigned)c->lay.M, blocks, 2), 32, 0, c->stream,
+                          c->lay, c->jofs, c->band, c->piv, c->bmaps);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) {
-    // half a warp per filament; up to 4 warps per CTA, fewer for long filaments so
+    // in blocks of rows (one system, which no list of active ones narrows), else half a warp per filament; up to 4 warps per CTA, fewer for long filaments so
     // that each filament's right-hand side fits in shared memory
+    const double ct = make_params(c).ct;
+    if (c->bmaps) {
+        const size_t smem = block_solve_smem(c);
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(band_block_solve_kernel,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        c->n_launches += 1;
+        return launch_pdl(band_block_solve_kernel, c->lay.M, kBlkThreads, smem, c->stream, c->lay,
+                          c->jofs, c->bmaps, ct, 6 * c->lay.maxN + 2 * kBlk, b, x);
+    }
     const int zmax = 6 * c->lay.maxN;
     const size_t per = (size_t)zmax * sizeof(double);
     const int fils = (int)std::min<size_t>(8, kSolveSmemMax / per);
@@ -449,7 +795,6 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
     const int threads = (kSolveLanes * fils + 31) / 32 * 32;
     const unsigned grid = (unsigned)((c->lay.M + fils - 1) / fils);
     c->n_launches += 1;
-    const double ct = make_params(c).ct;
     return c->band32 ? launch_pdl(band_solve_kernel<float>, grid, threads, smem, c->stream, c->lay,
                                   c->band32, c->piv, ct, b, x, zmax, active, fils)
                      : launch_pdl(band_solve_kernel<double>, grid, threads, smem, c->stream, c->lay,
