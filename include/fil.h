@@ -434,8 +434,8 @@ fil_status fil_fma_peak(int32_t fp64, double *flops_per_s, double *sm_mhz);
  * inside another framework's memory pool or a host process whose device
  * allocations belong to someone else -- and so cannot hold a context.
  * It computes the same product as fil_mobility_apply of a FIL_MIXED context
- * (FP32 pair sums with compensated accumulation, FP64 results) for S =
- * n_seg segments with radius a and viscosity eta: Y (S x 3), FT (S x 6) and
+ * (FP32 pair sums with compensated accumulation, FP64 results; up to 160
+ * segments FP64 throughout) for S = n_seg segments with radius a and viscosity eta: Y (S x 3), FT (S x 6) and
  * VW (S x 6) must be DEVICE pointers of the current device (or managed
  * memory), owned by the caller. It allocates nothing: its scratch is a fixed
  * static device array of about 9.6 MB in the library (plus 512 per-tile

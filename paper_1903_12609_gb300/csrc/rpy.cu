@@ -1475,6 +1475,11 @@ constexpr int kSymTile = 64;
 constexpr int kSymThreads = 128;
 constexpr int64_t kSymMaxSeg = 8192;          // slots: (S / 64) x 6 S doubles
 constexpr int64_t kDirectMaxSeg = 1024;       // up to here a warp per target is faster
+// The FP32 modes take it too while it is faster than packing and the FP32 kernel,
+// whose chain of one unit alone is 10-13 us: at 32 segments 5.1 and 10.6 us, at 128
+// 9.7 and 13.8, at 192 13.7 and 12.7. (FP64 throughout, so closer than the FP32 sums.)
+constexpr int64_t kDirect32MaxSeg = 160;
+inline int64_t direct_max(bool pair32) { return pair32 ? kDirect32MaxSeg : kDirectMaxSeg; }
 
 __global__ void __launch_bounds__(kSymThreads)
 rpy_sym64_kernel(const double *__restrict__ Y, const double *__restrict__ FT, int S, int tiles,
@@ -1834,6 +1839,23 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     if (W == 0) return cudaSuccess;
     // the active-tile list changes between applies: its launches keep a fixed grid
     // (and read the unit count from the device), so captured graphs stay valid
+    if (c->rpy_auto && S <= direct_max(pair32_on(c)) && !overlaps(VW, 6 * S, Y, 3 * S) &&
+        !overlaps(VW, 6 * S, FT, 6 * S)) {
+        // Early (launch_dep) while each SM partition has at most one target's warp. One
+        // FP64 time step of a 32-segment filament cloud, early and plainly: 1.57 and 1.61
+        // ms at 320 segments, 2.40 and 2.40 at 640, 3.91 and 3.55 at 960.
+        if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
+        if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
+        launch_dep(S <= 4 * c->num_sms, rpy_direct64_kernel, (unsigned)S, 32, 0, c->stream, Y, FT,
+                   (int)S, make_const<double, RpyConst64>(c->a), scale, VW);
+        if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
+        if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
+        if (timed) c->prof_n += 1;
+        c->n_launches += 1;
+        c->n_applies += 1;
+        c->n_pairs += c->pairs_all;
+        return cudaGetLastError();
+    }
     if (pair32_on(c)) {
         const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
         launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
@@ -1868,22 +1890,14 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
             !overlaps(VW, 6 * S, FT, 6 * S)) {
             if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
             if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
-            // Early (launch_dep) while each SM partition has at most one target's warp, never
-            // for the pairs' tiles. One time step of a 32-segment filament cloud, early and
-            // plainly: 1.57 and 1.61 ms at 320 segments, 2.40 and 2.40 at 640, 3.91 and 3.55
-            // at 960, 10.7 and 9.5 at 1 920.
-            if (S <= kDirectMaxSeg) {
-                launch_dep(S <= 4 * c->num_sms, rpy_direct64_kernel, (unsigned)S, 32, 0, c->stream, Y,
-                           FT, (int)S, k, scale, VW);
-                c->n_launches += 1;
-            } else {
-                const int tiles = (int)((S + kSymTile - 1) / kSymTile);
-                launch_dep(false, rpy_sym64_kernel, (unsigned)(tiles * (tiles + 1) / 2), kSymThreads,
-                           0, c->stream, Y, FT, (int)S, tiles, k, (double *)c->partials);
-                launch_pdl(sum64_kernel, dim3((unsigned)((S + 63) / 64), 6), 64, 0, c->stream,
-                           (const double *)c->partials, (int)S, tiles, scale, VW);
-                c->n_launches += 2;
-            }
+            // (a plain launch: one FP64 time step of a 32-segment filament cloud took 10.7 ms
+            // with the early one and 9.5 without at 1 920 segments, see launch_dep)
+            const int tiles = (int)((S + kSymTile - 1) / kSymTile);
+            launch_dep(false, rpy_sym64_kernel, (unsigned)(tiles * (tiles + 1) / 2), kSymThreads, 0,
+                       c->stream, Y, FT, (int)S, tiles, k, (double *)c->partials);
+            launch_pdl(sum64_kernel, dim3((unsigned)((S + 63) / 64), 6), 64, 0, c->stream,
+                       (const double *)c->partials, (int)S, tiles, scale, VW);
+            c->n_launches += 2;
             if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
             if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
             if (timed) c->prof_n += 1;
@@ -2130,6 +2144,13 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     int grid_max = 1;
     if (noalloc_setup(dev, &base, &cnt, &grid_max) != cudaSuccess) return FIL_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
+    if (n_seg <= kDirect32MaxSeg && !overlaps(VW, 6 * n_seg, Y, 3 * n_seg) &&
+        !overlaps(VW, 6 * n_seg, FT, 6 * n_seg)) {       // as fil_mobility_apply
+        const cudaError_t e = launch(rpy_direct64_kernel, (unsigned)n_seg, 32, 0, st,
+                                     Y, FT, (int)n_seg, make_const<double, RpyConst64>(a),
+                                     1.0 / (8.0 * kPi * eta), VW);
+        return e == cudaSuccess ? FIL_OK : FIL_ECUDA;
+    }
     const int64_t tiles = (n_seg + kWarpTile - 1) / kWarpTile;
     const int64_t Spad = tiles * kWarpTile;
     const int64_t n_units = (n_seg + kRpyComp - 1) / kRpyComp;   // source groups per tile
