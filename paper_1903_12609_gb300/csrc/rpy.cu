@@ -207,16 +207,41 @@ struct Rec {
     static constexpr int kSums = kFrames ? 12 : 6;                // packed sums of the far loop
 };
 
+// Order of the n groups' records for the automatic schedule: 16 runs of neighbouring
+// groups dealt out in turn, so that the groups whose close pairs cost a tile up to
+// three times a far unit (its own and the next ones of its filaments) go to
+// different warps. spread_group: the group at place i; spread_place: its inverse.
+// spread_count: n where the order pays, else 0, the groups' own. Whole applies,
+// own order and spread: 960 segments 21.8 and 23.1 us (a unit per warp: nothing to
+// spread), 1 920 35.9 and 33.9, 3 200 46.3 and 43.0, 6 400 89.1 and 87.4, 9 651 in
+// ragged filaments 175.9 and 172.6, 16 000 400.7 and 401.8, 32 000 1483 and 1492.
+__host__ __device__ __forceinline__ int spread_count(int64_t n) {
+    return n >= 48 && n <= 384 ? (int)n : 0;
+}
+__device__ __forceinline__ int spread_group(int i, int n) {
+    const int r = i & 15, q = n >> 4, rem = n & 15;
+    return i < n ? r * q + min(r, rem) + (i >> 4) : i;
+}
+__device__ __forceinline__ int spread_place(int g, int n) {
+    const int q = n >> 4, head = (n & 15) * (q + 1);       // groups in the longer runs
+    if (g >= n) return g;
+    const int r = g < head ? g / (q + 1) : (n & 15) + (g - head) / q;
+    return 16 * (g < head ? g % (q + 1) : (g - head) % q) + r;
+}
+
 // (two warps per CTA: a small system's groups then spread over the SMs)
 constexpr int kPackThreads = 64;
 template <bool kFrames>
 __global__ void __launch_bounds__(kPackThreads) pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
-                              int64_t S, int64_t Spad, SysMap sm, float4 *__restrict__ src) {
+                              int64_t S, int64_t Spad, SysMap sm, int n_spread,
+                              float4 *__restrict__ src) {
     pdl_enter();
     const int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (P >= Spad) return;             // Spad is a multiple of 32: whole warps leave
-    const int64_t i = segment_at(sm, P, S);
     const int lane = threadIdx.x & 31;
+    // (the first n_spread groups in the order of spread_group, the rest in their own)
+    const int64_t i = segment_at(
+        sm, n_spread ? 32 * (int64_t)spread_group((int)(P >> 5), n_spread) + lane : P, S);
     double y[3] = {0.0, 0.0, 0.0};
     float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i >= 0) {
@@ -1086,6 +1111,7 @@ __device__ __noinline__ void finish_warp_tiles(const SysMap &smap, int64_t W, in
     }
 }
 
+template <bool kSpread>
 __global__ void __launch_bounds__(32 * kWarpCta, 1)
 rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int n_ctas,
                        RpyConst32 k, float *__restrict__ part, int *__restrict__ cnt,
@@ -1120,7 +1146,9 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
         float th[2][3], tl[2][3], hi[2][6], lo[2][6];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            load_target<true>(src, base + 32 * t + lane, th[t], tl[t]);
+            int64_t P = base + 32 * t;
+            if constexpr (kSpread) P = 32 * (int64_t)spread_place((int)(P >> 5), (int)n_units);
+            load_target<true>(src, P + lane, th[t], tl[t]);
 #pragma unroll
             for (int c = 0; c < 6; ++c) hi[t][c] = lo[t][c] = 0.f;
         }
@@ -1633,8 +1661,12 @@ int64_t count_tiles(const fil_ctx *c, int T) {
 }
 
 cudaError_t allow_warp_smem() {
-    return cudaFuncSetAttribute(rpy_pair32_warp_kernel,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmem);
+    for (const auto kernel : {rpy_pair32_warp_kernel<false>, rpy_pair32_warp_kernel<true>}) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Tiles of T targets of every system (only tiles that hold real targets),
@@ -1858,15 +1890,17 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     }
     if (pair32_on(c)) {
         const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
+        const int n_spread = c->rpy_auto ? spread_count((S + kRpyComp - 1) / kRpyComp) : 0;
         launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
-                   c->Spad, sm, c->src32);
+                   c->Spad, sm, n_spread, c->src32);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         const RpyConst32 k = make_const<float, RpyConst32>(c->a);
         if (c->rpy_auto) {
             const int G = warp_grid(W, c->num_sms);
-            launch_pdl(rpy_pair32_warp_kernel, G, 32 * kWarpCta, kWarpSmem, c->stream, c->src32, sm,
-                       W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
+            launch_pdl(n_spread ? rpy_pair32_warp_kernel<true> : rpy_pair32_warp_kernel<false>, G,
+                       32 * kWarpCta, kWarpSmem, c->stream, c->src32, sm, W, G, k,
+                       (float *)c->partials, c->tile_cnt, scale, VW);
         } else {
             const int G = (int)(active_only ? c->rpy_grid32 : std::min<int64_t>(c->rpy_grid32, W));
             const bool split = c->rpy_tpt == 1 && c->rpy_split == 2;
@@ -2164,11 +2198,12 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     sm.n_tiles = tiles;
     sm.n_units = n_units;
     sm.n_src = n_seg;
+    const int n_spread = spread_count(n_units);
     cudaError_t e = launch(pack32_kernel<true>, (unsigned)(Spad / kPackThreads), kPackThreads, 0, st, Y, FT, n_seg,
-                           Spad, sm, src);
+                           Spad, sm, n_spread, src);
     if (e == cudaSuccess)
-        e = launch(rpy_pair32_warp_kernel, (unsigned)G, 32 * kWarpCta, kWarpSmem, st,
-                   (const float4 *)src, sm, W, G, make_const<float, RpyConst32>(a), part, cnt,
-                   1.0 / (8.0 * kPi * eta), VW);
+        e = launch(n_spread ? rpy_pair32_warp_kernel<true> : rpy_pair32_warp_kernel<false>,
+                   (unsigned)G, 32 * kWarpCta, kWarpSmem, st, (const float4 *)src, sm, W, G,
+                   make_const<float, RpyConst32>(a), part, cnt, 1.0 / (8.0 * kPi * eta), VW);
     return e == cudaSuccess ? FIL_OK : FIL_ECUDA;
 }
