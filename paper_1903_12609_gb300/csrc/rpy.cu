@@ -1409,7 +1409,8 @@ __device__ __forceinline__ double rsqrt_iter(double x) {
 __device__ __forceinline__ void coef64(double r2, const RpyConst64 &k, double &A, double &B,
                                        double &C, double &D, double &G) {
     const long long bits = __double_as_longlong(r2);
-    const bool none = bits < __double_as_longlong(1e-290);    // r = 0: 1/r taken as 0
+    // 1/r taken as 0 where r = 0 and where r^2 overflows
+    const bool none = bits < __double_as_longlong(1e-290) || bits >= 0x7ff0000000000000ll;
     const double rinv = none ? 0.0 : rsqrt_iter(r2);
     const double rinv2 = rinv * rinv;
     G = rinv * rinv2;
