@@ -646,15 +646,20 @@ __device__ __forceinline__ void pair64(double tx, double ty, double tz, const do
     acc[5] = fma(C, Tz, fma(dT, dz, fma(Fx, ey, fma(-Fy, ex, acc[5]))));
 }
 
-// Asynchronous copy of a chunk of source records (n float4) from global to
-// shared memory, 16 bytes per cp.async, spread over the CTA's threads; the
-// copies land when cp_async_wait_all returns (plus a barrier for the others').
-template <int kThreads>
-__device__ __forceinline__ void stage_chunk(float4 *dst, const float4 *__restrict__ g, int n,
-                                            int tid) {
-    for (int i = tid; i < n; i += kThreads) {
-        const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + i);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g + i) : "memory");
+// One lane's share of the asynchronous copy of a group of sources from global to
+// shared memory (16 bytes per cp.async, one commit group): a warp streams its own
+// groups, and waits with cp.async.wait_group and __syncwarp alone.
+template <bool kFrames>
+__device__ __forceinline__ void stage_group(float4 *dst, const float4 *__restrict__ g, int lane) {
+    constexpr int kF4 = Rec<kFrames>::kGroupF4;
+#pragma unroll
+    for (int i = 0; i < (kF4 + 31) / 32; ++i) {
+        const int e = lane + 32 * i;
+        if (e < kF4) {
+            const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + e);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g + e)
+                         : "memory");
+        }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -787,11 +792,19 @@ __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, 
 //    differences in the far form, and exactly only when distinct segments
 //    overlap.
 // SPLIT = 2 (128-target tiles only) gives a CTA twice the warps on the same
-// targets: the two sets of four warps take alternate 32-source groups of every
-// chunk and their sums are added (float-float, in set order) before the
+// targets: the two sets of four warps take alternate 32-source groups
+// and their sums are added (float-float, in set order) before the
 // partial is written.
-// These kernels run for schedules set by hand or chosen by the autotuner; the
-// automatic schedule runs rpy_pair32_warp_kernel below.
+// Each warp streams its groups through two buffers of its own and meets the others
+// only at the tile's end, so that one that evaluates a close group again (its own
+// filaments': every few groups in a system of some hundred segments, where they
+// took a quarter of the apply) delays nobody. Measured, 256 systems of about 1000
+// segments, with chunks of four groups shared by the CTA between barriers: 965 us an
+// apply; close groups' loop unrolled by 4 942; streams of their own 930; an empty
+// second slot left out 910, all with the same bits. By 8 the loop spills: 1037.
+// These kernels run ensembles, and one system where its schedule is set by hand or
+// chosen by the autotuner; the automatic schedule of one system runs
+// rpy_pair32_warp_kernel below.
 // ---------------------------------------------------------------------------
 constexpr int min_blocks(bool frames, int tpt, int split) {
     return split == 2 ? kRpyMinBlocksSplit2
@@ -804,17 +817,18 @@ __global__ void __launch_bounds__(kRpyThreads * SPLIT, min_blocks(kFrames, TPT, 
 rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G, RpyConst32 k,
                   float *__restrict__ part, int *__restrict__ cnt, double scale,
                   double *__restrict__ VW) {
-    constexpr int kPer = kRpyChunk / kRpyComp;            // groups per staged chunk
     constexpr int kGroupF4 = Rec<kFrames>::kGroupF4, kPairF4 = Rec<kFrames>::kPairF4;
     constexpr int kUnitGroups = unit_sources(kFrames) / kRpyComp;   // groups per work unit
-    constexpr int kRec = kGroupF4 * kPer;
+    constexpr int kWarps = kRpyThreads * SPLIT / 32;
     constexpr int kT = TPT;                               // targets per thread
     constexpr int kTile = kRpyThreads * TPT;              // targets per tile
     static_assert(SPLIT == 1 || (SPLIT == 2 && TPT == 1), "source split: 128-target tiles only");
-    __shared__ float4 sm[2][kRec];
+    __shared__ float4 sm[kWarps][2][kGroupF4];            // two groups of each warp
     // target slot, and which of the SPLIT sets of source groups the thread takes
     const int tid = SPLIT == 1 ? (int)threadIdx.x : (int)(threadIdx.x % kRpyThreads);
     const int set = SPLIT == 1 ? 0 : (int)(threadIdx.x / kRpyThreads);
+    const int lane = tid & 31;
+    float4(*buf)[kGroupF4] = sm[threadIdx.x >> 5];
     pdl_enter();
     const int64_t b = blockIdx.x;
     resolve_dyn(smap, W);
@@ -832,131 +846,132 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
         const int64_t c_begin = (u - ubeg) * kUnitGroups;
         const int64_t c_end = min((u_last - ubeg) * kUnitGroups, (nsrc + kRpyComp - 1) / kRpyComp);
 
-        // first chunk -> buffer 0
-        int n_grp = (int)min((int64_t)kPer, c_end - c_begin);
-        stage_chunk<kRpyThreads * SPLIT>(sm[0], srcs + kGroupF4 * c_begin, kGroupF4 * n_grp,
-                                         threadIdx.x);
+        // first target of this warp (slot 0)
+        const int64_t wbase = ptile * kTile + (tid & ~31);
+        // a warp whose targets are all padding (in a system's last tile) computes
+        // nothing; the tile's sum never reads those rows
+        // ensembles: a warp whose second slot is all padding leaves that out too
+        const bool both = kFrames || kT == 1 || wbase + kRpyThreads - src0 < nsrc;
+        const int64_t g_end = wbase - src0 < nsrc ? c_end : c_begin;
+        int64_t grp = c_begin + set;
+        if (grp < g_end) stage_group<kFrames>(buf[0], srcs + kGroupF4 * grp, lane);
         float th[kT][3], tl[kT][3];
 #pragma unroll
         for (int t = 0; t < kT; ++t)
             load_target<kFrames>(src, ptile * kTile + t * kRpyThreads + tid, th[t], tl[t]);
-        [[maybe_unused]] const int lane = tid & 31;
-        // first target of this warp (slot 0), for the own-group test of 128-target tiles
-        [[maybe_unused]] const int64_t wbase = ptile * kTile + (tid & ~31);
-        // 128-target tiles (small systems): a warp whose targets are all padding (in a
-        // system's last tile) computes nothing; the tile's sum never reads those rows
-        bool idle = false;
-        if constexpr (TPT == 1) idle = wbase - src0 >= nsrc;
         float hi[kT][6], lo[kT][6];
 #pragma unroll
         for (int t = 0; t < kT; ++t)
 #pragma unroll
             for (int c = 0; c < 6; ++c) hi[t][c] = lo[t][c] = 0.f;
-        cp_async_wait_all();
-        __syncthreads();
 
-        int buf = 0;
-        for (int64_t ch = c_begin; ch < c_end; ch += kPer, buf ^= 1) {
-            // the next chunk streams into the other buffer while this one is computed
-            // (that buffer was last read before the barrier that ended the previous chunk)
-            const bool has_next = (ch + kPer < c_end);
-            const int n_next = has_next ? (int)min((int64_t)kPer, c_end - ch - kPer) : 0;
-            if (has_next)
-                stage_chunk<kRpyThreads * SPLIT>(sm[buf ^ 1], srcs + kGroupF4 * (ch + kPer),
-                                                 kGroupF4 * n_next, threadIdx.x);
-            const float4 *s = sm[buf];
 #pragma unroll 1
-            for (int grp = set; grp < (idle ? 0 : n_grp); grp += SPLIT) {
-                const float4 *qg = s + kGroupF4 * grp + Rec<kFrames>::kHead;
-                float out[kT][6];
-                // the group that holds this warp's own segments
-                const bool own =
-                    TPT == 1 && src0 + (ch + grp) * kRpyComp == wbase;
-                bool near = own;
-                if (!own) {
-                    float2 t2[kT][3], acc[kT][Rec<kFrames>::kSums];
+        for (int cur = 0; grp < g_end; grp += SPLIT, cur ^= 1) {
+            if (grp + SPLIT < g_end) {
+                stage_group<kFrames>(buf[cur ^ 1], srcs + kGroupF4 * (grp + SPLIT), lane);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                cp_async_wait_all();
+            }
+            __syncwarp();
+            const float4 *qg = buf[cur] + Rec<kFrames>::kHead;
+            float out[kT][6];
+            // the group that holds this warp's own segments
+            const bool own =
+                TPT == 1 && src0 + grp * kRpyComp == wbase;
+            bool near = own;
+            if (!own) {
+                float2 t2[kT][3], acc[kT][Rec<kFrames>::kSums];
 #pragma unroll
-                    for (int t = 0; t < kT; ++t) {
-                        to_frame<kFrames>(qg, th[t], tl[t], t2[t]);
+                for (int t = 0; t < kT; ++t) {
+                    to_frame<kFrames>(qg, th[t], tl[t], t2[t]);
 #pragma unroll
-                        for (int c = 0; c < Rec<kFrames>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
-                    }
-                    float rmin2 = k.close2;
+                    for (int c = 0; c < Rec<kFrames>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
+                }
+                float rmin2 = k.close2;
+                if (both) {
 #pragma unroll (kRpyUnroll / 2)
                     for (int jp = 0; jp < kRpyComp / 2; ++jp) {
 #pragma unroll
                         for (int t = 0; t < kT; ++t)
                             pair32_far<kFrames>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
                     }
-                    near = __any_sync(0xffffffffu, rmin2 < k.close2);
-#pragma unroll
-                    for (int t = 0; t < kT; ++t)
-                        combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
+                } else {
+#pragma unroll (kRpyUnroll / 2)
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                        pair32_far<kFrames>(t2[0], qg + kPairF4 * jp, k, acc[0], rmin2);
                 }
-                if (near) {
-                    // (one target at a time: fewer live registers)
-#pragma unroll
-                    for (int t = 0; t < kT; ++t) {
-                        float uh[3], ul[3];
-                        to_frame_hl<kFrames>(qg, th[t], tl[t], uh, ul);
-                        float2 acc[6];
-                        float rmin2 = k.close2;
-                        bool exact = TPT == 2;
-                        if constexpr (TPT == 1) {
-                            const int self_j = own ? lane : -1;
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
-#pragma unroll 1
-                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                                pair32_near<kFrames, kFarHiLo>(uh, ul, qg + kPairF4 * jp, k, acc,
-                                                               rmin2, self_j, 2 * jp);
-                            // overlapping distinct segments (r < 2a): the exact coefficients
-                            exact = __any_sync(0xffffffffu, rmin2 < k.near2);
-                        }
-                        if (exact) {
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
-#pragma unroll 1
-                            for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                                pair32_near<kFrames, kExact>(uh, ul, qg + kPairF4 * jp, k, acc, rmin2);
-                        }
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) out[t][c] = __fadd_rn(acc[c].x, acc[c].y);
-                        if (own && !exact) {
-                            // the self term, left out of the far-form pass above:
-                            // 4/(3a) F_n and T_n / a^3
-                            const float *f = reinterpret_cast<const float *>(
-                                                 qg + kPairF4 * (lane >> 1)) + (lane & 1);
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) {
-                                out[t][c] = fmaf(k.ov_A0, f[2 * (3 + c)], out[t][c]);
-                                out[t][3 + c] = fmaf(k.ov_C0, f[2 * (6 + c)], out[t][3 + c]);
-                            }
-                        }
-                    }
-                }
+                // (where slot 1 is left out: in a group with padding sources its padding
+                // targets would have met them at r = 0)
+                near = __any_sync(0xffffffffu, rmin2 < k.close2) ||
+                       (!both && (grp + 1) * kRpyComp > nsrc);
 #pragma unroll
                 for (int t = 0; t < kT; ++t)
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) {
-                        float sh, e;
-                        two_sum(hi[t][c], out[t][c], sh, e);
-                        hi[t][c] = sh;
-                        lo[t][c] = __fadd_rn(lo[t][c], e);
-                    }
+                    combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
             }
-            if (has_next) cp_async_wait_all();
-            n_grp = n_next;
-            __syncthreads();
+            if (near) {
+                // (one target at a time: fewer live registers)
+#pragma unroll
+                for (int t = 0; t < kT; ++t) {
+                    if (t == 1 && !both) continue;
+                    float uh[3], ul[3];
+                    to_frame_hl<kFrames>(qg, th[t], tl[t], uh, ul);
+                    float2 acc[6];
+                    float rmin2 = k.close2;
+                    bool exact = TPT == 2;
+                    if constexpr (TPT == 1) {
+                        const int self_j = own ? lane : -1;
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
+#pragma unroll 1
+                        for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                            pair32_near<kFrames, kFarHiLo>(uh, ul, qg + kPairF4 * jp, k, acc,
+                                                           rmin2, self_j, 2 * jp);
+                        // overlapping distinct segments (r < 2a): the exact coefficients
+                        exact = __any_sync(0xffffffffu, rmin2 < k.near2);
+                    }
+                    if (exact) {
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
+#pragma unroll (kFrames ? 1 : 4)
+                        for (int jp = 0; jp < kRpyComp / 2; ++jp)
+                            pair32_near<kFrames, kExact>(uh, ul, qg + kPairF4 * jp, k, acc, rmin2);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) out[t][c] = __fadd_rn(acc[c].x, acc[c].y);
+                    if (own && !exact) {
+                        // the self term, left out of the far-form pass above:
+                        // 4/(3a) F_n and T_n / a^3
+                        const float *f = reinterpret_cast<const float *>(
+                                             qg + kPairF4 * (lane >> 1)) + (lane & 1);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            out[t][c] = fmaf(k.ov_A0, f[2 * (3 + c)], out[t][c]);
+                            out[t][3 + c] = fmaf(k.ov_C0, f[2 * (6 + c)], out[t][3 + c]);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < kT; ++t)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    float sh, e;
+                    two_sum(hi[t][c], out[t][c], sh, e);
+                    hi[t][c] = sh;
+                    lo[t][c] = __fadd_rn(lo[t][c], e);
+                }
+            __syncwarp();     // every lane is done with this buffer before it is refilled
         }
 
         if constexpr (SPLIT > 1) {
             // the other sets' sums join the first's in set order (TwoSum of the hi
-            // parts, the lo parts into its error, renormalised), through the chunk
+            // parts, the lo parts into its error, renormalised), through the group
             // buffers, which are next written after the barrier in finish_tile
-            float *xs = reinterpret_cast<float *>(&sm[0][0]);
+            float *xs = reinterpret_cast<float *>(&sm[0][0][0]);
             static_assert((SPLIT - 1) * 12 * kRpyThreads * sizeof(float) <= sizeof(sm),
-                          "the sets' sums fit in the chunk buffers");
+                          "the sets' sums fit in the group buffers");
+            __syncthreads();          // every warp is done with its groups
             if (set > 0) {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
@@ -1029,20 +1044,6 @@ __host__ __device__ __forceinline__ int64_t warp_count(int64_t W, int64_t n_ctas
     const int64_t most = n_ctas * kWarpCta;
     const int64_t m = (W + most - 1) / most;
     return (W + m - 1) / m;
-}
-
-// One lane's share of the asynchronous copy of a group.
-__device__ __forceinline__ void stage_group(float4 *dst, const float4 *__restrict__ g, int lane) {
-#pragma unroll
-    for (int i = 0; i < (kGroupF4 + 31) / 32; ++i) {
-        const int e = lane + 32 * i;
-        if (e < kGroupF4) {
-            const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + e);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g + e)
-                         : "memory");
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // The tiles that the CTA's units (those of warps [w0, w1)) lie in, once its
@@ -1136,7 +1137,7 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
     }
     pdl_enter();
     if (u < u_end) {
-        stage_group(buf, src + kGroupF4 * (u - ubeg), lane);
+        stage_group<true>(buf, src + kGroupF4 * (u - ubeg), lane);
     }
     int cur = 0;
     while (u < u_end) {
@@ -1157,7 +1158,7 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
             if (u + 1 < u_end) {
                 // the next group, or the first one for the next tile
                 const int64_t gn = u + 1 < s_end ? u + 1 - ubeg : 0;
-                stage_group(buf + kGroupF4 * (cur ^ 1), src + kGroupF4 * gn, lane);
+                stage_group<true>(buf + kGroupF4 * (cur ^ 1), src + kGroupF4 * gn, lane);
                 asm volatile("cp.async.wait_group 1;" ::: "memory");
             } else {
                 cp_async_wait_all();
