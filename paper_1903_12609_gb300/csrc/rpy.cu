@@ -1705,11 +1705,6 @@ int occupancy(K kernel, int threads = kRpyThreads) {
     return std::max(1, occ);
 }
 
-void set_grids(fil_ctx *c) {
-    c->rpy_grid32 = c->rpy_ctas * c->num_sms;
-    c->rpy_grid64 = c->rpy_ctas * c->num_sms;
-}
-
 // Resident CTAs per SM of the pair kernel of a schedule (targets per thread,
 // source split; the split exists for the FP32 kernel with one target per thread).
 int pair_occupancy(const fil_ctx *c, int tpt, int split) {
@@ -1717,6 +1712,16 @@ int pair_occupancy(const fil_ctx *c, int tpt, int split) {
         return tpt == 1 ? occupancy(rpy_pair64_kernel<1>) : occupancy(rpy_pair64_kernel<2>);
     if (tpt == 2) return kRpyMaxCtasTpt2;
     return split == 2 ? kRpyMaxCtasSplit2 : kRpyMaxCtasTpt1;
+}
+
+// The grid of the current schedule, and whether it fills the SMs. One that does not
+// is launched plainly: an early launch (launch_dep) would put two CTAs on some SMs and
+// none on others (32 000 segments, 256-target tiles at one CTA per SM: 1786 us plainly,
+// 3091 early).
+void set_grids(fil_ctx *c) {
+    c->rpy_grid32 = c->rpy_ctas * c->num_sms;
+    c->rpy_grid64 = c->rpy_ctas * c->num_sms;
+    c->rpy_full = c->rpy_ctas >= pair_occupancy(c, c->rpy_tpt, c->rpy_split);
 }
 
 }  // namespace
@@ -1871,6 +1876,10 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     const SysMap sm = sys_map(c, active_only);
     const int64_t W = active_only ? c->act_units : c->rpy_units;
     if (W == 0) return cudaSuccess;
+    // the stream-K kernels start early where the grid is full, or too small to crowd (a
+    // 128-target schedule of 3 CTAs per SM: 320 segments, 30 units, 16.0 us early and
+    // 18.5 plainly; 960, 240 units, 27.9 and 26.7; 256 systems 1519 and 855)
+    const bool early = c->rpy_full || W <= c->num_sms;
     // the active-tile list changes between applies: its launches keep a fixed grid
     // (and read the unit count from the device), so captured graphs stay valid
     if (c->rpy_auto && S <= direct_max(pair32_on(c)) && !overlaps(VW, 6 * S, Y, 3 * S) &&
@@ -1913,8 +1922,8 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
                               : (split               ? rpy_pair32_kernel<false, 1, 2>
                                  : c->rpy_tpt == 1   ? rpy_pair32_kernel<false, 1>
                                                      : rpy_pair32_kernel<false, 2>);
-            launch_pdl(pair, G, kRpyThreads * (split ? 2 : 1), 0, c->stream, c->src32, sm, W, G, k,
-                       (float *)c->partials, c->tile_cnt, scale, VW);
+            launch_dep(early, pair, G, kRpyThreads * (split ? 2 : 1), 0, c->stream, c->src32,
+                       sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
         }
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
@@ -1945,8 +1954,8 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         launch_pdl(pack64_kernel, pgrid, pb, 0, c->stream, Y, FT, S, c->Spad, sm, c->src64);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
-        launch_pdl(c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G, kRpyThreads, 0,
-                   c->stream, c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
+        launch_dep(early, c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G,
+                   kRpyThreads, 0, c->stream, c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
     }
