@@ -479,6 +479,52 @@ __device__ __forceinline__ void pair32_far(const float2 *t, const float4 *q, con
     acc[11] = __ffma2_rn(G, Fz, acc[11]);
 }
 
+// The same sums of two targets, lane x and lane y of t, and source H (0 even, 1 odd)
+// of the record: a source's values are then single registers, the same for both
+// lanes, and a packed FMA reads one register fewer. Measured (same bits, whole applies,
+// the loop over the records unrolled in full): 32 000 segments 1477 us with pair32_far,
+// 1426 with this; 9 600 159 and 155; unrolled by 8 1484 and 161, as iterations of the
+// loop do not overlap. Up to 640 segments it costs 0.2 us of 14 to 19.
+template <int H>
+__device__ __forceinline__ float2 both(const float4 &v, int half) {
+    const float x = half ? (H ? v.w : v.z) : (H ? v.y : v.x);
+    return f2(x, x);
+}
+template <int H>
+__device__ __forceinline__ void pair32_far2(const float2 *t, const float4 *q, const RpyConst32 &k,
+                                            float2 *acc, float2 &rmin2) {
+    const float2 nk2 = f2(-k.k2a2, -k.k2a2);
+    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3], q4 = q[4], q5 = q[5], q6 = q[6];
+    const float q7 = reinterpret_cast<const float *>(q + 7)[H];
+    const float2 dx = __fadd2_rn(t[0], both<H>(q0, 0));
+    const float2 dy = __fadd2_rn(t[1], both<H>(q0, 1));
+    const float2 dz = __fadd2_rn(t[2], both<H>(q1, 0));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+    const float2 rinv = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+    rmin2 = f2(fminf(rmin2.x, r2.x), fminf(rmin2.y, r2.y));
+    const float2 rinv2 = __fmul2_rn(rinv, rinv);
+    const float2 G = __fmul2_rn(rinv, rinv2);
+    const float2 rinv5 = __fmul2_rn(G, rinv2);
+    const float2 B = __ffma2_rn(nk2, rinv5, G);
+    const float2 Fx = both<H>(q1, 1), Fy = both<H>(q2, 0), Fz = both<H>(q2, 1);
+    const float2 Tx = both<H>(q3, 0), Ty = both<H>(q3, 1), Tz = both<H>(q4, 0);
+    const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
+    const float2 dT =
+        __fmul2_rn(rinv5, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
+    acc[0] = __ffma2_rn(rinv, Fx, __ffma2_rn(G, both<H>(q4, 1), __ffma2_rn(bF, dx, acc[0])));
+    acc[1] = __ffma2_rn(rinv, Fy, __ffma2_rn(G, both<H>(q5, 0), __ffma2_rn(bF, dy, acc[1])));
+    acc[2] = __ffma2_rn(rinv, Fz, __ffma2_rn(G, both<H>(q5, 1), __ffma2_rn(bF, dz, acc[2])));
+    acc[3] = __ffma2_rn(G, both<H>(q6, 0), __ffma2_rn(dT, dx, acc[3]));
+    acc[4] = __ffma2_rn(G, both<H>(q6, 1), __ffma2_rn(dT, dy, acc[4]));
+    acc[5] = __ffma2_rn(G, f2(q7, q7), __ffma2_rn(dT, dz, acc[5]));
+    acc[6] = __ffma2_rn(G, Tx, acc[6]);
+    acc[7] = __ffma2_rn(G, Ty, acc[7]);
+    acc[8] = __ffma2_rn(G, Tz, acc[8]);
+    acc[9] = __ffma2_rn(G, Fx, acc[9]);
+    acc[10] = __ffma2_rn(G, Fy, acc[10]);
+    acc[11] = __ffma2_rn(G, Fz, acc[11]);
+}
+
 // The (V, Omega) terms of a group from the twelve sums of pair32_far: with
 // P = sum G T and Q = sum G F,
 //   V     = acc[0..2] + (2a^2/3) Q + P x t
@@ -502,6 +548,25 @@ __device__ __forceinline__ void combine_group(const float2 *acc, const float2 *t
                       fmaf(s[6 + p], t[q].x, fmaf(-s[6 + q], t[p].x, s[c])));
         out[3 + c] = fmaf(1.5f, s[3 + c],
                           fmaf(-0.5f, s[6 + c], fmaf(s[9 + p], t[q].x, -s[9 + q] * t[p].x)));
+    }
+}
+
+// The same for two targets, from the sums of pair32_far2 over the even and the odd
+// sources.
+__device__ __forceinline__ void combine_group2(const float2 (&acc)[2][Rec<true>::kSums],
+                                               const float2 *t, float k23, float2 *out) {
+    float2 s[Rec<true>::kSums];
+#pragma unroll
+    for (int c = 0; c < Rec<true>::kSums; ++c) s[c] = __fadd2_rn(acc[0][c], acc[1][c]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int p = (c + 1) % 3, q = (c + 2) % 3;
+        out[c] = __ffma2_rn(f2(k23, k23), s[9 + c],
+                            __ffma2_rn(s[6 + p], t[q], __ffma2_rn(neg2(s[6 + q]), t[p], s[c])));
+        out[3 + c] = __ffma2_rn(
+            f2(1.5f, 1.5f), s[3 + c],
+            __ffma2_rn(f2(-0.5f, -0.5f), s[6 + c],
+                       __ffma2_rn(s[9 + p], t[q], __fmul2_rn(neg2(s[9 + q]), t[p]))));
     }
 }
 
@@ -1027,7 +1092,10 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
 // Measured, whole applies, against 256-target tiles of four warps with a barrier
 // per 128 sources: 9 651 segments in ragged filaments 224 -> 181 us, 3200
 // segments 73 -> 50 us, 32 000 1504 -> 1491 us (at the close groups' loop
-// unrolled by 2; by 4 its registers cost the far loop 7%). One system only.
+// unrolled by 2; by 4 its registers cost the far loop 7%). One system only. With the
+// two targets of a lane packed (pair32_far2) and the spread order 9 651 take 160 us,
+// 3200 44 and 32 000 1426; of these 36 us are the compensated fold and 10 the close
+// groups, the rest the far loop and each group's start.
 // ---------------------------------------------------------------------------
 constexpr int kWarpTile = kRpyMinTile;          // targets per tile
 constexpr int kWarpPart = 12 * kWarpTile;       // floats of a partial
@@ -1144,15 +1212,16 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
         const int64_t base = tile * kWarpTile;              // the tile's first target
         const int64_t s_end = min(u_end, ubeg + n_units);  // this warp's units of the tile
         const bool whole = u == ubeg && s_end == ubeg + n_units;
-        float th[2][3], tl[2][3], hi[2][6], lo[2][6];
+        float th[2][3], tl[2][3];
+        float2 hi[6], lo[6];                               // lane x: slot 0, lane y: slot 1
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             int64_t P = base + 32 * t;
             if constexpr (kSpread) P = 32 * (int64_t)spread_place((int)(P >> 5), (int)n_units);
             load_target<true>(src, P + lane, th[t], tl[t]);
-#pragma unroll
-            for (int c = 0; c < 6; ++c) hi[t][c] = lo[t][c] = 0.f;
         }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) hi[c] = lo[c] = f2(0.f, 0.f);
 #pragma unroll 1
         for (; u < s_end; ++u, cur ^= 1) {
             if (u + 1 < u_end) {
@@ -1165,38 +1234,35 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
             }
             __syncwarp();
             const float4 *qg = buf + kGroupF4 * cur + Rec<true>::kHead;
-            float out[2][6];
-            float rmin2[2] = {k.close2, k.close2};
+            float2 out[6], rmin2 = f2(k.close2, k.close2);
             {
-                float2 t2[2][3], acc[2][Rec<true>::kSums];
+                const float4 ce = qg[-1];
+                const float cc[3] = {ce.x, ce.y, ce.z};
+                float2 t2[3], acc[2][Rec<true>::kSums];
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    to_frame<true>(qg, th[t], tl[t], t2[t]);
+                for (int x = 0; x < 3; ++x)
+                    t2[x] = f2(__fadd_rn(__fsub_rn(th[0][x], cc[x]), tl[0][x]),
+                               __fadd_rn(__fsub_rn(th[1][x], cc[x]), tl[1][x]));
 #pragma unroll
-                    for (int c = 0; c < Rec<true>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
-                }
-#pragma unroll (kRpyUnroll / 2)
+                for (int c = 0; c < Rec<true>::kSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
+#pragma unroll
                 for (int jp = 0; jp < kRpyComp / 2; ++jp) {
-#pragma unroll
-                    for (int t = 0; t < 2; ++t)
-                        pair32_far<true>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2[t]);
+                    pair32_far2<0>(t2, qg + kPairF4 * jp, k, acc[0], rmin2);
+                    pair32_far2<1>(t2, qg + kPairF4 * jp, k, acc[1], rmin2);
                 }
-#pragma unroll
-                for (int t = 0; t < 2; ++t)
-                    combine_group<true>(acc[t], t2[t], k.k23a2, out[t]);
+                combine_group2(acc, t2, k.k23a2, out);
             }
             // slots in which a pair came closer than R_c, one at a time through one copy of
             // the code: with hi/lo differences in the far form, or with the exact
             // coefficients where a pair overlaps (the group that holds the slot's own
             // segments counts as one: it has the self pairs)
             unsigned close = 0;
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-                if (__any_sync(0xffffffffu, rmin2[t] < k.close2)) close |= 1u << t;
+            if (__any_sync(0xffffffffu, rmin2.x < k.close2)) close |= 1u;
+            if (__any_sync(0xffffffffu, rmin2.y < k.close2)) close |= 2u;
             while (close) {
                 const bool t1 = close == 2u;
                 close &= 2u * (close == 3u);
-                const bool exact = __any_sync(0xffffffffu, (t1 ? rmin2[1] : rmin2[0]) < k.over2);
+                const bool exact = __any_sync(0xffffffffu, (t1 ? rmin2.y : rmin2.x) < k.over2);
                 float ph[3], pl[3], uh[3], ul[3];
 #pragma unroll
                 for (int x = 0; x < 3; ++x) {
@@ -1220,19 +1286,18 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
                     const float v = __fadd_rn(acc[c].x, acc[c].y);
-                    if (t1) out[1][c] = v;
-                    else out[0][c] = v;
+                    if (t1) out[c].y = v;
+                    else out[c].x = v;
                 }
             }
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    float sh, e;
-                    two_sum(hi[t][c], out[t][c], sh, e);
-                    hi[t][c] = sh;
-                    lo[t][c] = __fadd_rn(lo[t][c], e);
-                }
+            for (int c = 0; c < 6; ++c) {
+                float2 sh, e;
+                two_sum(hi[c].x, out[c].x, sh.x, e.x);
+                two_sum(hi[c].y, out[c].y, sh.y, e.y);
+                hi[c] = sh;
+                lo[c] = __fadd2_rn(lo[c], e);
+            }
             __syncwarp();     // every lane is done with this buffer before it is refilled
         }
         if (whole) {
@@ -1242,7 +1307,8 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
                 if (n >= 0) {
 #pragma unroll
                     for (int c = 0; c < 6; ++c)
-                        VW[6 * n + c] = ((double)hi[t][c] + (double)lo[t][c]) * scale;
+                        VW[6 * n + c] = (t ? (double)hi[c].y + (double)lo[c].y
+                                           : (double)hi[c].x + (double)lo[c].x) * scale;
                 }
             }
         } else {
@@ -1251,8 +1317,8 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
             for (int t = 0; t < 2; ++t)
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
-                    p[c * kWarpTile + 32 * t + lane] = hi[t][c];
-                    p[(6 + c) * kWarpTile + 32 * t + lane] = lo[t][c];
+                    p[c * kWarpTile + 32 * t + lane] = t ? hi[c].y : hi[c].x;
+                    p[(6 + c) * kWarpTile + 32 * t + lane] = t ? lo[c].y : lo[c].x;
                 }
         }
         tile += 1;
@@ -1704,6 +1770,7 @@ int occupancy(K kernel, int threads = kRpyThreads) {
         return 1;
     return std::max(1, occ);
 }
+
 
 // Resident CTAs per SM of the pair kernel of a schedule (targets per thread,
 // source split; the split exists for the FP32 kernel with one target per thread).
