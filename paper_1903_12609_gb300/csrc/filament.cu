@@ -414,7 +414,8 @@ __global__ void commit_kernel(Layout lay, const double *__restrict__ X,
     }
 }
 
-constexpr int kUnpackEarly = 6000, kRowsEarly = 512;   // segments of one system, see the launches
+// segments up to which the kernel starts early, see the launches
+constexpr int kUnpackEarly = 6000, kRowsEarly = 512, kEnsembleEarly = 4000;
 
 unsigned warp_grid(int M, int threads) { return (unsigned)(((int64_t)M * 32 + threads - 1) / threads); }
 unsigned seg_grid(int64_t S, int threads) { return (unsigned)((S + threads - 1) / threads); }
@@ -428,8 +429,10 @@ cudaError_t unpack_forces(fil_ctx *c, const double *X, int with_forces, bool act
     c->n_launches += 1;
     // Early (launch_dep) up to kUnpackEarly segments: one time step of a 32-segment
     // filament cloud took 3363 us with the early launch and 3401 us without at 4 000
-    // segments, 6192 and 6100 at 8 000, 16.44 and 16.29 ms at 16 000. Ensembles: 0.1%.
-    const bool early = c->n_sys > 1 || c->lay.S <= kUnpackEarly;
+    // segments, 6192 and 6100 at 8 000, 16.44 and 16.29 ms at 16 000. Ensembles, with the
+    // residual rows, two steps: 3.53 and 3.62 ms at 1 177 segments, 4.74 and 4.57 at 4 645,
+    // 6.41 and 6.28 at 12 417, 9.37 and 8.30 at 38 113, 74.7 and 74.6 at 277 000.
+    const bool early = c->lay.S <= (c->n_sys > 1 ? kEnsembleEarly : kUnpackEarly);
     // (X is written only where step is set, and is then c->Xn)
     return launch_dep(early, kernel, warp_grid(c->lay.M, 128), 128, 0, c->stream, c->lay,
                       const_cast<double *>(X), c->Xk, c->w, c->n_sys, eval ? c->d_finf : nullptr,
@@ -447,11 +450,12 @@ cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *
         sc = {1.0, 0.0, c->dt, 0.0};
     }
     c->n_launches += 1;
-    // Early (launch_dep) behind the FP64 kernels, in ensembles and up to kRowsEarly
-    // segments. Behind the FP32 kernel of one system, whose CTAs all leave room, the rows
-    // crowd: a residual took 62.2 us early and 63.6 us plainly at 320 segments, 65.8 and
+    // Early (launch_dep) behind the FP64 kernels of one system, in small ensembles (see
+    // unpack_forces) and up to kRowsEarly segments. Behind the FP32 kernel of one system,
+    // whose CTAs all leave room, the rows crowd: a residual took 62.2 us early and 63.6 us plainly at 320 segments, 65.8 and
     // 63.8 at 640, 87.3 and 77.9 at 2 560, 175 and 168 at 8 000.
-    const bool early = c->n_sys > 1 || !pair32_on(c) || c->lay.S <= kRowsEarly;
+    const bool early = c->n_sys > 1 ? c->lay.S <= kEnsembleEarly
+                                    : !pair32_on(c) || c->lay.S <= kRowsEarly;
     return launch_dep(early, residual_rows_kernel, seg_grid(c->lay.S, kRowThreads), kRowThreads, 0,
                       c->stream, c->lay, X, c->Yc, c->VW, c->Y, c->Yprev, c->uprev, sc,
                       fprev ? c->d_active : nullptr, fprev, f, c->d_finf);

@@ -795,10 +795,15 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
     const int threads = (kSolveLanes * fils + 31) / 32 * 32;
     const unsigned grid = (unsigned)((c->lay.M + fils - 1) / fils);
     c->n_launches += 1;
-    return c->band32 ? launch_pdl(band_solve_kernel<float>, grid, threads, smem, c->stream, c->lay,
-                                  c->band32, c->piv, ct, b, x, zmax, active, fils)
-                     : launch_pdl(band_solve_kernel<double>, grid, threads, smem, c->stream, c->lay,
-                                  c->band, c->piv, ct, b, x, zmax, active, fils);
+    // Early (launch_dep) up to one filament per SM: the kernel is one wave, each SM bound
+    // by its chains, and waits for the fullest SM. Two steps of ensembles, early and
+    // plainly: 3.46 and 3.53 ms with 51 filaments, 4.77 and 4.36 with 232, 6.42 and 5.47
+    // with 336, 10.40 and 9.37 with 1 460, 74.9 and 74.7 with 8 192.
+    const bool early = c->lay.M <= c->num_sms;
+    return c->band32 ? launch_dep(early, band_solve_kernel<float>, grid, threads, smem, c->stream,
+                                  c->lay, c->band32, c->piv, ct, b, x, zmax, active, fils)
+                     : launch_dep(early, band_solve_kernel<double>, grid, threads, smem, c->stream,
+                                  c->lay, c->band, c->piv, ct, b, x, zmax, active, fils);
 }
 
 }  // namespace fil
