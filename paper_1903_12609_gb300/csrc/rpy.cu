@@ -1943,10 +1943,14 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     const SysMap sm = sys_map(c, active_only);
     const int64_t W = active_only ? c->act_units : c->rpy_units;
     if (W == 0) return cudaSuccess;
-    // the stream-K kernels start early where the grid is full, or too small to crowd (a
-    // 128-target schedule of 3 CTAs per SM: 320 segments, 30 units, 16.0 us early and
-    // 18.5 plainly; 960, 240 units, 27.9 and 26.7; 256 systems 1519 and 855)
-    const bool early = c->rpy_full || W <= c->num_sms;
+    // The stream-K kernels start early (launch_dep) where the grid is full, and in ensembles
+    // has a unit for every CTA, or too small to crowd. Ensembles' applies, early and
+    // plainly: 25 systems of 6 780 segments (about 100 units) 86.2 and 45.5 us, 9 of 5 460
+    // 71.0 and 45.5, 64 small ones 66.3 and 55.5, 5 of 2 059 (40 units) 41.5 and 45.4. One
+    // system in 128-target tiles, 3 CTAs per SM: 320 segments, 30 units, 16.0 and 18.5; 960,
+    // 240 units, 27.9 and 26.7. 256 systems in such tiles 1519 and 855.
+    const bool early = (c->rpy_full && (c->n_sys == 1 || W >= c->rpy_grid32)) ||
+                       W <= (c->n_sys == 1 ? c->num_sms : c->num_sms / 3);
     // the active-tile list changes between applies: its launches keep a fixed grid
     // (and read the unit count from the device), so captured graphs stay valid
     if (c->rpy_auto && S <= direct_max(pair32_on(c)) && !overlaps(VW, 6 * S, Y, 3 * S) &&
