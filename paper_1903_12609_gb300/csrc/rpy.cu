@@ -180,7 +180,7 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 
 // ---------------------------------------------------------------------------
 // Pack: FP64 (Y, FT) -> FP32 source groups of kRpyComp = 32 padded positions.
-// A group is Rec::kGroupF4 float4: first its centre (c_x, c_y, c_z, 0), the mean of
+// A group is Rec::kGroupF4 float4: first its centre (c_x, c_y, c_z, w), the mean of
 // its real positions relative to the first segment of the apply (the apply is
 // translation invariant, and FP32 rounding then depends on the extent of the
 // suspension, not on where it sits), rounded to FP32; then 16 source pairs of
@@ -189,7 +189,8 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 // and value c of source h (0 even, 1 odd) of a pair sits at float 2c + h, so
 // that each float2 holds one component of both; the far-form loop reads the
 // first 15. One warp packs one group. Padding records sit far away with zero
-// load, so they add exactly zero.
+// load, so they add exactly zero. w is the squared radius within which targets take
+// the cross products per pair (wide_radius2; 0: none).
 // Ensembles keep records without a frame (kFrames false): 12 values per source
 //   -y(hi) 3 | F 3 | T 3 | -y(lo) 3,   y = Y - Y_0 = hi + lo.
 // Their systems with the drag J0 take tens of Broyden iterations whose path
@@ -229,12 +230,41 @@ __device__ __forceinline__ int spread_place(int g, int n) {
     return 16 * (g < head ? g % (q + 1) : (g - head) % q) + r;
 }
 
+// The squared radius around a group's centre within which its targets are summed
+// with the cross products formed per pair (w of the group), 0 for none. The sums in
+// the group's frame (pair32_far) leave a cross product as the difference of two sums,
+// (sum G F) x t - sum G (F x s), which cancel where |t| and |s| are large against the
+// distance: at the targets inside the ball a group spans when its segments are not
+// neighbours of one another. A group whose consecutive segments lie within R_c is a
+// piece of one filament and keeps the sums in its frame at any extent, as does one
+// within 16a. Error of Omega against 64 bits (2%, 32 000 segments), with the cross
+// products per pair everywhere, in the frames everywhere, and by this rule: single
+// segments 1.81e-7, 2.43e-7, 1.65e-7; filaments of 8 1.62, 1.77, 1.56; of 16 to 48
+// 1.63, 1.68, 1.60; of 32 1.63, 1.62, 1.60. Whole applies in the frames everywhere and
+// by the rule: 1515 and 1671 us, 1436 and 1592, 1421 and 1516, 1426 and 1435. (A ball of
+// half that squared radius would be 1-3% faster and no longer as close for filaments of 16.)
+constexpr float kCompact = 16.f, kChainGap = 4.f;
+__device__ __forceinline__ float wide_radius2(const float *sp, bool live, float a) {
+    const unsigned all = 0xffffffffu;
+    float gap2 = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float d = sp[c] - __shfl_up_sync(all, sp[c], 1);       // (lane 0: its own)
+        gap2 = fmaf(d, d, gap2);
+    }
+    float ext2 = live ? fmaf(sp[0], sp[0], fmaf(sp[1], sp[1], sp[2] * sp[2])) : 0.f;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) ext2 = fmaxf(ext2, __shfl_xor_sync(all, ext2, d));
+    const bool chain = !__any_sync(all, live && gap2 > kChainGap * kChainGap * a * a);
+    return chain || ext2 <= kCompact * kCompact * a * a ? 0.f : ext2;
+}
+
 // (two warps per CTA: a small system's groups then spread over the SMs)
 constexpr int kPackThreads = 64;
 template <bool kFrames>
-__global__ void __launch_bounds__(kPackThreads) pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT,
-                              int64_t S, int64_t Spad, SysMap sm, int n_spread,
-                              float4 *__restrict__ src) {
+__global__ void __launch_bounds__(kPackThreads)
+pack32_kernel(const double *__restrict__ Y, const double *__restrict__ FT, int64_t S, int64_t Spad,
+              SysMap sm, int n_spread, float a, float4 *__restrict__ src) {
     pdl_enter();
     const int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (P >= Spad) return;             // Spad is a multiple of 32: whole warps leave
@@ -268,7 +298,6 @@ __global__ void __launch_bounds__(kPackThreads) pack32_kernel(const double *__re
             for (int d = 16; d > 0; d >>= 1) m += __shfl_xor_sync(0xffffffffu, m, d);
             cen[c] = m * inv;
         }
-        if (lane == 0) g[0] = make_float4(cen[0], cen[1], cen[2], 0.f);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             // s' = y - c from the FP32 parts of y (the FP64 unit has 1/64 of the rate)
@@ -288,6 +317,8 @@ __global__ void __launch_bounds__(kPackThreads) pack32_kernel(const double *__re
             v[9 + c] = -diff_of_products(f[3 + p], sp[q], f[3 + q], sp[p]);
             v[12 + c] = (-2.f / 3.f) * diff_of_products(f[p], sp[q], f[q], sp[p]);
         }
+        const float w2 = wide_radius2(sp, i >= 0, a);
+        if (lane == 0) g[0] = make_float4(cen[0], cen[1], cen[2], w2);
     } else {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -351,20 +382,12 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Exact coefficients of one pair (one lane): the far form for r^2 >= (2a)^2,
 // the overlapping-sphere form below it and the self values at r = 0, chosen
 // without a branch (both are evaluated; this runs in recomputed groups only).
-template <bool kFrames>
 __device__ __forceinline__ void coef_exact(float r2, const RpyConst32 &k, float &A, float &B,
                                            float &C, float &D, float &G) {
     const bool ov = r2 < k.near2;
-    float rinv, r, ri;
-    if constexpr (kFrames) {
-        // one MUFU operation (r = 0, and what ftz would make of a tiny r, as 1/r = 0)
-        rinv = ri = r2 > 1e-30f ? rsqrt_approx(r2) : 0.f;
-        r = r2 * rinv;
-    } else {
-        rinv = rsqrt_approx(fmaxf(r2, k.near2));   // the far form's, finite everywhere
-        r = sqrt_approx(r2);
-        ri = r > 0.f ? rcp_approx(r) : 0.f;
-    }
+    const float rinv = rsqrt_approx(fmaxf(r2, k.near2));   // the far form's, finite everywhere
+    const float r = sqrt_approx(r2);
+    const float ri = r > 0.f ? rcp_approx(r) : 0.f;
     const float rinv2 = rinv * rinv;
     const float rinv3 = rinv * rinv2;
     const float rinv5 = rinv3 * rinv2;
@@ -378,12 +401,9 @@ __device__ __forceinline__ void coef_exact(float r2, const RpyConst32 &k, float 
 // (V, Omega) sums of a pair with the coefficients A..G and the difference d,
 // the cross products formed for the pair (negated operands fold into the
 // packed FMA).
-__device__ __forceinline__ void add_pair(const float4 *q, float2 dx, float2 dy, float2 dz, float2 A,
+__device__ __forceinline__ void add_pair(float2 dx, float2 dy, float2 dz, float2 Fx, float2 Fy,
+                                         float2 Fz, float2 Tx, float2 Ty, float2 Tz, float2 A,
                                          float2 B, float2 C, float2 D, float2 G, float2 *acc) {
-    const float4 q1 = q[1], q2 = q[2], q3 = q[3];
-    const float2 Tz = reinterpret_cast<const float2 *>(q + 4)[0];
-    const float2 Fx = f2(q1.z, q1.w), Fy = f2(q2.x, q2.y), Fz = f2(q2.z, q2.w);
-    const float2 Tx = f2(q3.x, q3.y), Ty = f2(q3.z, q3.w);
     const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
     const float2 dT = __fmul2_rn(D, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
     const float2 ex = __fmul2_rn(G, dx), ey = __fmul2_rn(G, dy), ez = __fmul2_rn(G, dz);
@@ -395,6 +415,15 @@ __device__ __forceinline__ void add_pair(const float4 *q, float2 dx, float2 dy, 
     acc[3] = __ffma2_rn(C, Tx, __ffma2_rn(dT, dx, __ffma2_rn(Fy, ez, __ffma2_rn(nFz, ey, acc[3]))));
     acc[4] = __ffma2_rn(C, Ty, __ffma2_rn(dT, dy, __ffma2_rn(Fz, ex, __ffma2_rn(nFx, ez, acc[4]))));
     acc[5] = __ffma2_rn(C, Tz, __ffma2_rn(dT, dz, __ffma2_rn(Fx, ey, __ffma2_rn(nFy, ex, acc[5]))));
+}
+
+// The loads of a record's two sources.
+__device__ __forceinline__ void add_pair(const float4 *q, float2 dx, float2 dy, float2 dz, float2 A,
+                                         float2 B, float2 C, float2 D, float2 G, float2 *acc) {
+    const float4 q1 = q[1], q2 = q[2], q3 = q[3];
+    const float2 Tz = reinterpret_cast<const float2 *>(q + 4)[0];
+    add_pair(dx, dy, dz, f2(q1.z, q1.w), f2(q2.x, q2.y), f2(q2.z, q2.w), f2(q3.x, q3.y),
+             f2(q3.z, q3.w), Tz, A, B, C, D, G, acc);
 }
 
 // Far-form coefficients.
@@ -421,15 +450,16 @@ __device__ __forceinline__ void far_coef(float2 rinv, const RpyConst32 &k, float
 // and likewise for F x d, so that a pair needs no G d: 12 sums take
 //   acc[0..2] += (1/r) F + B (d.F) d - G (T x s)   (V without its G F part)
 //   acc[3..5] += r^-5 (d.T) d - (2/3) G (F x s)    (2/3 of Omega's d-terms)
-//   acc[6..8] += G T,  acc[9..11] += G F           (see fold_group)
+//   acc[6..8] += G T,  acc[9..11] += G F           (see combine_group)
 // in 39 FP32 operations a pair, 9 fewer than with the cross products formed
 // for every pair. What bounds the loop is register operands: a packed FMA
 // with three distinct register operands issues every third cycle, one with
 // two every second, and this form drops 3-operand FMAs (24 -> 21 sums) as
 // well as multiplies.
-// Measured (32 000 segments, pair kernel): 1700 us with the cross products formed
-// per pair, 1491 us in this form, and the error against 64 bits 2.0e-7 -> 1.7e-7
-// (the frames make the differences finer).
+// Measured (32 000 segments in filaments of 32, pair kernel): 1700 us with the cross
+// products formed per pair, 1491 us in this form; error against 64 bits of V 1.85e-7
+// and 1.55e-7 (the frames make the differences finer), of Omega 1.63e-7 and 1.60e-7.
+// Omega gains nothing where a group spans more than its neighbourhood: see wide_radius2.
 // Without frames (ensembles): t relative to the first segment, 48 operations,
 //   acc[0..2] += V terms, acc[3..5] += Omega terms.
 template <bool kFrames>
@@ -525,6 +555,57 @@ __device__ __forceinline__ void pair32_far2(const float2 *t, const float4 *q, co
     acc[11] = __ffma2_rn(G, Fz, acc[11]);
 }
 
+// Two targets against source H, for the targets inside a wide group (wide_radius2): as
+// pair32_far2, but Omega's cross product formed for the pair,
+//   acc[0..2] += A F + B (d.F) d - G (T x s)   (V without P x t)
+//   acc[3..5] += D (d.T) d + G (F x d)         (Omega without -P/2)
+//   acc[6..8] += G T = P
+// V keeps its frame: dominated by A F, it is closer to 64 bits there. 44 operations a pair
+// (48 with V's cross product per pair too: 32 000 single segments 1741 us, 1673 in this
+// form). The loop is unrolled by 2 only: a warp changes between it and the far loop, and
+// both must fit in the instruction cache (9 651 segments in ragged filaments by 2 180 us,
+// by 4 185; with 48 operations by 8 205, by 16 236).
+constexpr int kCrossSums = 9;
+template <int H>
+__device__ __forceinline__ void pair32_cross2(const float2 *t, const float4 *q, const RpyConst32 &k,
+                                              float2 *acc, float2 &rmin2) {
+    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3], q4 = q[4], q5 = q[5];
+    const float2 dx = __fadd2_rn(t[0], both<H>(q0, 0));
+    const float2 dy = __fadd2_rn(t[1], both<H>(q0, 1));
+    const float2 dz = __fadd2_rn(t[2], both<H>(q1, 0));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+    rmin2 = f2(fminf(rmin2.x, r2.x), fminf(rmin2.y, r2.y));
+    float2 A, B, C, D, G;
+    far_coef(f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y)), k, A, B, C, D, G);
+    const float2 Fx = both<H>(q1, 1), Fy = both<H>(q2, 0), Fz = both<H>(q2, 1);
+    const float2 Tx = both<H>(q3, 0), Ty = both<H>(q3, 1), Tz = both<H>(q4, 0);
+    const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
+    const float2 dT = __fmul2_rn(D, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
+    const float2 ex = __fmul2_rn(G, dx), ey = __fmul2_rn(G, dy), ez = __fmul2_rn(G, dz);
+    acc[0] = __ffma2_rn(A, Fx, __ffma2_rn(G, both<H>(q4, 1), __ffma2_rn(bF, dx, acc[0])));
+    acc[1] = __ffma2_rn(A, Fy, __ffma2_rn(G, both<H>(q5, 0), __ffma2_rn(bF, dy, acc[1])));
+    acc[2] = __ffma2_rn(A, Fz, __ffma2_rn(G, both<H>(q5, 1), __ffma2_rn(bF, dz, acc[2])));
+    acc[3] = __ffma2_rn(dT, dx, __ffma2_rn(Fy, ez, __ffma2_rn(neg2(Fz), ey, acc[3])));
+    acc[4] = __ffma2_rn(dT, dy, __ffma2_rn(Fz, ex, __ffma2_rn(neg2(Fx), ez, acc[4])));
+    acc[5] = __ffma2_rn(dT, dz, __ffma2_rn(Fx, ey, __ffma2_rn(neg2(Fy), ex, acc[5])));
+    acc[6] = __ffma2_rn(G, Tx, acc[6]);
+    acc[7] = __ffma2_rn(G, Ty, acc[7]);
+    acc[8] = __ffma2_rn(G, Tz, acc[8]);
+}
+
+__device__ __forceinline__ void combine_cross2(const float2 (&acc)[2][kCrossSums], const float2 *t,
+                                               float2 *out) {
+    float2 s[kCrossSums];
+#pragma unroll
+    for (int c = 0; c < kCrossSums; ++c) s[c] = __fadd2_rn(acc[0][c], acc[1][c]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int p = (c + 1) % 3, q = (c + 2) % 3;
+        out[c] = __ffma2_rn(s[6 + p], t[q], __ffma2_rn(neg2(s[6 + q]), t[p], s[c]));
+        out[3 + c] = __ffma2_rn(f2(-0.5f, -0.5f), s[6 + c], s[3 + c]);
+    }
+}
+
 // The (V, Omega) terms of a group from the twelve sums of pair32_far: with
 // P = sum G T and Q = sum G F,
 //   V     = acc[0..2] + (2a^2/3) Q + P x t
@@ -605,8 +686,8 @@ __device__ __forceinline__ void pair32_near(const float *th, const float *tl, co
         rmin2 = fminf(rmin2, fminf(sx ? k.close2 : r2.x, sy ? k.close2 : r2.y));
         far_coef(rinv, k, A, B, C, D, G);
     } else {
-        coef_exact<kFrames>(r2.x, k, A.x, B.x, C.x, D.x, G.x);
-        coef_exact<kFrames>(r2.y, k, A.y, B.y, C.y, D.y, G.y);
+        coef_exact(r2.x, k, A.x, B.x, C.x, D.x, G.x);
+        coef_exact(r2.y, k, A.y, B.y, C.y, D.y, G.y);
     }
     add_pair(q, dx, dy, dz, A, B, C, D, G, acc);
 }
@@ -947,14 +1028,27 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
             bool near = own;
             if (!own) {
                 float2 t2[kT][3], acc[kT][Rec<kFrames>::kSums];
+                bool cross = false;          // a target inside a wide group
 #pragma unroll
                 for (int t = 0; t < kT; ++t) {
                     to_frame<kFrames>(qg, th[t], tl[t], t2[t]);
+                    if constexpr (kFrames)
+                        cross = cross || fmaf(t2[t][0].x, t2[t][0].x,
+                                              fmaf(t2[t][1].x, t2[t][1].x,
+                                                   t2[t][2].x * t2[t][2].x)) < qg[-1].w;
 #pragma unroll
                     for (int c = 0; c < Rec<kFrames>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
                 }
+                if constexpr (kFrames) cross = __any_sync(0xffffffffu, cross);
                 float rmin2 = k.close2;
-                if (both) {
+                if (kFrames && cross) {
+#pragma unroll 2
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp) {
+#pragma unroll
+                        for (int t = 0; t < kT; ++t)
+                            pair32_far<false>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
+                    }
+                } else if (both) {
 #pragma unroll (kRpyUnroll / 2)
                     for (int jp = 0; jp < kRpyComp / 2; ++jp) {
 #pragma unroll
@@ -971,8 +1065,10 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
                 near = __any_sync(0xffffffffu, rmin2 < k.close2) ||
                        (!both && (grp + 1) * kRpyComp > nsrc);
 #pragma unroll
-                for (int t = 0; t < kT; ++t)
-                    combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
+                for (int t = 0; t < kT; ++t) {
+                    if (kFrames && cross) combine_group<false>(acc[t], t2[t], k.k23a2, out[t]);
+                    else combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
+                }
             }
             if (near) {
                 // (one target at a time: fewer live registers)
@@ -1238,19 +1334,34 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
             {
                 const float4 ce = qg[-1];
                 const float cc[3] = {ce.x, ce.y, ce.z};
-                float2 t2[3], acc[2][Rec<true>::kSums];
+                float2 t2[3];
 #pragma unroll
                 for (int x = 0; x < 3; ++x)
                     t2[x] = f2(__fadd_rn(__fsub_rn(th[0][x], cc[x]), tl[0][x]),
                                __fadd_rn(__fsub_rn(th[1][x], cc[x]), tl[1][x]));
+                const float2 tt =
+                    __ffma2_rn(t2[0], t2[0], __ffma2_rn(t2[1], t2[1], __fmul2_rn(t2[2], t2[2])));
+                if (!__any_sync(0xffffffffu, fminf(tt.x, tt.y) < ce.w)) {
+                    float2 acc[2][Rec<true>::kSums];
 #pragma unroll
-                for (int c = 0; c < Rec<true>::kSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
+                    for (int c = 0; c < Rec<true>::kSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
 #pragma unroll
-                for (int jp = 0; jp < kRpyComp / 2; ++jp) {
-                    pair32_far2<0>(t2, qg + kPairF4 * jp, k, acc[0], rmin2);
-                    pair32_far2<1>(t2, qg + kPairF4 * jp, k, acc[1], rmin2);
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp) {
+                        pair32_far2<0>(t2, qg + kPairF4 * jp, k, acc[0], rmin2);
+                        pair32_far2<1>(t2, qg + kPairF4 * jp, k, acc[1], rmin2);
+                    }
+                    combine_group2(acc, t2, k.k23a2, out);
+                } else {
+                    float2 acc[2][kCrossSums];
+#pragma unroll
+                    for (int c = 0; c < kCrossSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
+#pragma unroll 2
+                    for (int jp = 0; jp < kRpyComp / 2; ++jp) {
+                        pair32_cross2<0>(t2, qg + kPairF4 * jp, k, acc[0], rmin2);
+                        pair32_cross2<1>(t2, qg + kPairF4 * jp, k, acc[1], rmin2);
+                    }
+                    combine_cross2(acc, t2, out);
                 }
-                combine_group2(acc, t2, k.k23a2, out);
             }
             // slots in which a pair came closer than R_c, one at a time through one copy of
             // the code: with hi/lo differences in the far form, or with the exact
@@ -1974,7 +2085,7 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
         const int n_spread = c->rpy_auto ? spread_count((S + kRpyComp - 1) / kRpyComp) : 0;
         launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
-                   c->Spad, sm, n_spread, c->src32);
+                   c->Spad, sm, n_spread, (float)c->a, c->src32);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         const RpyConst32 k = make_const<float, RpyConst32>(c->a);
@@ -2282,7 +2393,7 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     sm.n_src = n_seg;
     const int n_spread = spread_count(n_units);
     cudaError_t e = launch(pack32_kernel<true>, (unsigned)(Spad / kPackThreads), kPackThreads, 0, st, Y, FT, n_seg,
-                           Spad, sm, n_spread, src);
+                           Spad, sm, n_spread, (float)a, src);
     if (e == cudaSuccess)
         e = launch(n_spread ? rpy_pair32_warp_kernel<true> : rpy_pair32_warp_kernel<false>,
                    (unsigned)G, 32 * kWarpCta, kWarpSmem, st, (const float4 *)src, sm, W, G,
