@@ -128,8 +128,9 @@ input_kernel(const float *__restrict__ x, int64_t B, const float *__restrict__ m
              const float *__restrict__ stdv, bf16 *__restrict__ X, bf16 *__restrict__ Xt,
              int64_t ldt, int64_t Kb) {
     tc::pdl_launch_next();
-    const int c = blockIdx.x * kInThreads + threadIdx.x;
-    const int64_t b0 = (int64_t)blockIdx.y * kRows;
+    // (rows along x: the other dimensions end at 65 535 blocks, 2 097 120 rows)
+    const int c = blockIdx.y * kInThreads + threadIdx.x;
+    const int64_t b0 = (int64_t)blockIdx.x * kRows;
     const bool in = c < kIn;
     const float mu = in ? mean[c] : 0.f, sd = in ? stdv[c] : 1.f;
     float v[kRows];
@@ -383,7 +384,7 @@ cudaError_t one_product(fil_mlp *m, const tc::Problem &p) {
 // without it m->Y takes the normalised ones.
 cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train, float *y) {
     const int64_t Kb = round_up(B, tc::kTileK);
-    const dim3 grid(4, (unsigned)(((train ? Kb : B) + kRows - 1) / kRows));
+    const dim3 grid((unsigned)(((train ? Kb : B) + kRows - 1) / kRows), 4);
     input_kernel<<<grid, kInThreads, 0, m->stream>>>(x, B, m->in_mean, m->in_std, m->X,
                                                      train ? m->Xt : nullptr, m->ldt, Kb);
     cudaError_t e = cudaGetLastError();
