@@ -161,7 +161,10 @@ __global__ void output_kernel(const float *__restrict__ yhat, int64_t n, const f
 // dY = (y^ - t^) / B in BF16 (row-major, and transposed with columns B .. Kb - 1
 // zero), its FP32 column sums over each CTA's 32 rows, and each CTA's part of
 // the loss: squares and their sum in float-float (TwoSum), FP64 once per thread
-// (one CTA over the whole batch in FP64 took 234 us at 1024 rows).
+// (one CTA over the whole batch in FP64 took 234 us at 1024 rows). Where a square or
+// the sum would leave FP32's range (or is infinite or NaN), and where the squares'
+// rounding errors would, a thread sums its squares in FP64.
+constexpr float kSquareMax = 1e38f, kSquareMin = 1e-12f;
 constexpr int kLossThreads = kOut;
 __global__ void __launch_bounds__(kLossThreads)
 loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t B,
@@ -181,12 +184,13 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
         y[r] = in ? yhat[(b0 + r) * kOut + c] : 0.f;
         g[r] = in ? t[(b0 + r) * kOut + c] : mu;
     }
-    float hi = 0.f, lo = 0.f, sum = 0.f;
+    float hi = 0.f, lo = 0.f, sum = 0.f, most = 0.f;
     uint32_t h[kRows / 2];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
         const bool in = b0 + r < B;
         const float d = in ? y[r] - (g[r] - mu) / sd : 0.f;
+        most = fmaxf(most, fabsf(d));
         const float sq = __fmul_rn(d, d), se = __fmaf_rn(d, d, -sq);
         const float s = __fadd_rn(hi, sq), bb = __fsub_rn(s, hi);
         lo = __fadd_rn(lo, __fadd_rn(se, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(sq, bb))));
@@ -203,6 +207,14 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
     if ((int)blockIdx.x >= n_part) return;      // rows of the zero padding only
     col_sums[(int64_t)blockIdx.x * kOut + c] = sum;
     double acc = 0.5 * ((double)hi + (double)lo);
+    if (!(hi < kSquareMax && (most > kSquareMin || most == 0.f))) {
+        acc = 0.0;
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            const double d = b0 + r < B ? (double)(y[r] - (g[r] - mu) / sd) : 0.0;
+            acc = fma(0.5 * d, d, acc);
+        }
+    }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
     if ((c & 31) == 0) red[c >> 5] = acc;
