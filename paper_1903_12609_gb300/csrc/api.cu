@@ -917,7 +917,8 @@ fil_status fil_broyden_step(fil_ctx *c, int32_t *converged, double *finf) {
     // and the host waits for the copy alone, so that the GPU works while the host
     // decides. What the last iteration of a step enqueued in vain (it touches the step
     // w and history slots that no pair counts) is cheaper there than a round trip of
-    // ~20 us in every iteration; for large systems it is not.
+    // ~20 us in every iteration; for large systems it is not. (An evaluation that failed
+    // leaves them alone, see update_kernel.)
     const bool ahead = c->n_sys == 1 && c->lay.S <= kAheadMaxSeg;
     if (ahead) {
         if (!c->status_ev) CK(cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming));

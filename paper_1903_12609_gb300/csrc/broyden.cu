@@ -161,7 +161,9 @@ __global__ void dots_final_kernel(int n_sys, int max_out, const int *__restrict_
 // g += sum_i c_i alpha_i; history pair k; w = g + c_k (df . fn)/|df|, with the
 // scalars of entry i's system; w = 0 in systems that have converged. The last
 // block to finish moves the device's k to the next history slot (flags[3] counts
-// the blocks and wraps to zero).
+// the blocks and wraps to zero). With `finf` (one system, whose update may run before
+// the host has read the status) an evaluation that failed -- steric overflow, f not
+// finite -- leaves w, the history and k as they were, so that the step can be repeated.
 template <typename H>
 __global__ void update_kernel(int64_t n, int *__restrict__ dk,
                               const double *__restrict__ scal_all, const float *__restrict__ scal32,
@@ -169,8 +171,10 @@ __global__ void update_kernel(int64_t n, int *__restrict__ dk,
                               const int *__restrict__ active, const double *__restrict__ fn,
                               const double *__restrict__ fk, double *__restrict__ g,
                               H *__restrict__ C, H *__restrict__ D, double *__restrict__ w,
-                              int *__restrict__ flags) {
+                              int *__restrict__ flags,
+                              const unsigned long long *__restrict__ finf) {
     pdl_enter();
+    if (finf && (flags[2] || *finf >= 0x7ff0000000000000ull)) return;   // every block
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int k = *dk;
     if (i < n) {
@@ -288,13 +292,14 @@ cudaError_t broyden_dots(fil_ctx *c) {
 cudaError_t broyden_update(fil_ctx *c) {
     const int64_t n = c->lay.nX;
     const unsigned grid = (unsigned)((n + 255) / 256);
+    const unsigned long long *finf = c->n_sys == 1 ? c->d_finf : nullptr;
     c->n_launches += 1;
     return c->C32 ? launch_pdl(update_kernel<float>, grid, 256, 0, c->stream, n, c->d_k, c->scal,
                                c->scal32, c->sstride, c->lay.sys_of, c->d_active, c->fn, c->fk, c->g,
-                               c->C32, c->D32, c->w, c->d_flags)
+                               c->C32, c->D32, c->w, c->d_flags, finf)
                   : launch_pdl(update_kernel<double>, grid, 256, 0, c->stream, n, c->d_k, c->scal,
                                (const float *)nullptr, c->sstride, c->lay.sys_of, c->d_active, c->fn,
-                               c->fk, c->g, c->C, c->D, c->w, c->d_flags);
+                               c->fk, c->g, c->C, c->D, c->w, c->d_flags, finf);
 }
 
 cudaError_t broyden_carry(fil_ctx *c, int from, int m, const double *f, double *w) {
