@@ -132,20 +132,21 @@ fil_status fil_create_ensemble(const fil_params *p, int32_t n_sys, const int32_t
  * current / last step and the last ||f||_inf that was read. */
 fil_status fil_sys_stats(const fil_ctx *c, int32_t *iters, double *finf);
 
-/* Autotuner of the RPY pair kernel: times the pair kernel (which also sums
- * each tile's partials) of `reps` mobility applies of the current state's
- * loads (CUDA events around it, so host launch gaps do not count) for every
+/* Autotuner of the RPY pair kernel: times `reps` mobility applies of the current
+ * state's loads (CUDA events around each, so host launch gaps do not count) for every
  * candidate schedule -- tiles of 256 targets (2 per thread) or 128 targets
  * (1 per thread, with source split 1 or 2 on the FP32 path: see
- * fil_set_source_split), 1..occupancy resident CTAs per SM for the stream-K
- * split of the (tile, sources) work units, and the automatic schedule a new
- * context of one system starts with on the FP32 path -- and keeps the fastest for all
+ * fil_set_source_split), 1..the largest count of CTAs per SM fil_set_pair_schedule
+ * takes for the stream-K split of the (tile, sources) work units, and the automatic
+ * schedule a new context of one system starts with -- and keeps the fastest for all
  * later applies (if that is the automatic one it stays in use, and the outputs
- * name the 256-target tiles a new context reports). The applies first run for 50 ms of wall time (an idle GPU's
+ * name the 256-target tiles a new context reports). One system of at most 160 segments
+ * on the FP32 path keeps the automatic schedule, whose sums are FP64 there. The applies
+ * first run for 50 ms of wall time (an idle GPU's
  * clock is still rising then) and the candidates are swept twice, each
- * keeping its faster time. Reports the choice (nullable outputs) and its
- * pair-kernel time per apply in ms. Results change only in rounding (the
- * summation order of the pair terms). FIL_ESTATE inside a step. */
+ * keeping its faster time. Reports the choice (nullable outputs) and the time of its
+ * pair kernel (which also sums each tile's partials) per apply in ms. Results change
+ * only in rounding (the summation order of the pair terms). FIL_ESTATE inside a step. */
 fil_status fil_autotune(fil_ctx *c, int32_t reps, int32_t *tile, int32_t *ctas_per_sm,
                         double *ms);
 

@@ -241,6 +241,7 @@ struct fil_ctx {
     int prof_n;
     cudaEvent_t *prof_ev;  // 2 * kProfMax events, created on first use
     cudaEvent_t *tune_ev = nullptr;   // the autotuner's pair of events for the next apply
+    bool tune_pair = false;           // around its pair kernel only
 };
 
 namespace fil {

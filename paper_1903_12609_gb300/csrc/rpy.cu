@@ -2054,6 +2054,8 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     const SysMap sm = sys_map(c, active_only);
     const int64_t W = active_only ? c->act_units : c->rpy_units;
     if (W == 0) return cudaSuccess;
+    // (with tune_pair set the first event is recorded again after the packing)
+    if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
     // The stream-K kernels start early (launch_dep) where the grid is full, and in ensembles
     // has a unit for every CTA, or too small to crowd. Ensembles' applies, early and
     // plainly: 25 systems of 6 780 segments (about 100 units) 86.2 and 45.5 us, 9 of 5 460
@@ -2069,7 +2071,6 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         // Early (launch_dep) while each SM partition has at most one target's warp. One
         // FP64 time step of a 32-segment filament cloud, early and plainly: 1.57 and 1.61
         // ms at 320 segments, 2.40 and 2.40 at 640, 3.91 and 3.55 at 960.
-        if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         launch_dep(S <= 4 * c->num_sms, rpy_direct64_kernel, (unsigned)S, 32, 0, c->stream, Y, FT,
                    (int)S, make_const<double, RpyConst64>(c->a), scale, VW);
@@ -2086,7 +2087,7 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         const int n_spread = c->rpy_auto ? spread_count((S + kRpyComp - 1) / kRpyComp) : 0;
         launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
                    c->Spad, sm, n_spread, (float)c->a, c->src32);
-        if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
+        if (c->tune_ev && c->tune_pair) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         const RpyConst32 k = make_const<float, RpyConst32>(c->a);
         if (c->rpy_auto) {
@@ -2115,7 +2116,6 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         // the result overwrites them (or is too large for the slots)
         if (c->rpy_auto && S <= kSymMaxSeg && !overlaps(VW, 6 * S, Y, 3 * S) &&
             !overlaps(VW, 6 * S, FT, 6 * S)) {
-            if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
             if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
             // (a plain launch: one FP64 time step of a 32-segment filament cloud took 10.7 ms
             // with the early one and 9.5 without at 1 920 segments, see launch_dep)
@@ -2134,7 +2134,7 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         }
         const int G = (int)(active_only ? c->rpy_grid64 : std::min<int64_t>(c->rpy_grid64, W));
         launch_pdl(pack64_kernel, pgrid, pb, 0, c->stream, Y, FT, S, c->Spad, sm, c->src64);
-        if (c->tune_ev) cudaEventRecord(c->tune_ev[0], c->stream);
+        if (c->tune_ev && c->tune_pair) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         launch_dep(early, c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G,
                    kRpyThreads, 0, c->stream, c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
@@ -2150,7 +2150,12 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
 
 
 // Autotuner of the pair kernel: times every (targets per thread, resident CTAs
-// per SM) candidate on `reps` applies of (Y, FT) and keeps the fastest. An idle
+// per SM) candidate on `reps` applies of (Y, FT) and keeps the fastest. What is
+// compared are whole applies, as some schedules pack their sources in a launch of
+// their own, and an event between the two launches would keep the second from
+// starting early; the choice's pair kernel alone is timed at the end, for the
+// report. An FP32 system small enough for the direct FP64 sums has no other
+// candidate, so that tuning does not change its accuracy. An idle
 // GPU runs at a low clock for some tens of milliseconds after work arrives, so
 // the applies first run for kSpinUpMs of wall time, and the candidates are then
 // swept twice, each keeping the faster of its two times: a candidate measured
@@ -2169,7 +2174,8 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
     for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
     struct cand { int tpt, split, ctas, automatic; float ms; };
     std::vector<cand> cands;
-    for (int tpt = 1; tpt <= 2; ++tpt) {
+    const bool direct = c->n_sys == 1 && pair32_on(c) && c->lay.S <= kDirect32MaxSeg;
+    for (int tpt = 1; tpt <= 2 && !direct; ++tpt) {
         for (int split = 1; split <= (tpt == 1 && pair32_on(c) ? 2 : 1); ++split) {
             const int occ = pair_occupancy(c, tpt, split);
             for (int ctas = 1; ctas <= std::min(occ, c->rpy_ctas_max); ++ctas)
@@ -2184,59 +2190,59 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
         const std::chrono::duration<double, std::milli> dt = std::chrono::steady_clock::now() - t0;
         if (dt.count() >= kSpinUpMs) break;
     }
+    const auto use = [&](const cand &k) {
+        c->rpy_auto = k.automatic;
+        c->rpy_tpt = k.tpt;
+        c->rpy_split = k.split;
+        c->rpy_threads = kRpyThreads;
+        c->rpy_ctas = k.ctas;
+        set_grids(c);
+        build_tiles(c);
+        return upload_tiles(c);
+    };
+    // the time of `reps` applies, or of their pair kernels, in the schedule in use
+    const auto time = [&](bool pair, float &ms) {
+        cudaError_t er = rpy_apply(c, Y, FT, VW);       // warm-up
+        c->tune_pair = pair;
+        for (int r = 0; r < reps && er == cudaSuccess; ++r) {
+            c->tune_ev = &ev[2 * r];
+            er = rpy_apply(c, Y, FT, VW);
+            c->tune_ev = nullptr;
+        }
+        if (er == cudaSuccess) er = cudaStreamSynchronize(c->stream);
+        ms = 0.f;
+        for (int r = 0; r < reps && er == cudaSuccess; ++r) {
+            float one = 0.f;
+            er = cudaEventElapsedTime(&one, ev[2 * r], ev[2 * r + 1]);
+            ms += one;
+        }
+        return er;
+    };
+    cand best{c->rpy_tpt, c->rpy_split, c->rpy_ctas, c->rpy_auto, 1e30f};
     for (int sweep = 0; sweep < kSweeps && e == cudaSuccess; ++sweep) {
         for (cand &k : cands) {
-            if (e != cudaSuccess) break;
-            c->rpy_auto = k.automatic;
-            c->rpy_tpt = k.tpt;
-            c->rpy_split = k.split;
-            c->rpy_threads = kRpyThreads;
-            c->rpy_ctas = k.ctas;
-            set_grids(c);
-            build_tiles(c);
-            e = upload_tiles(c);
-            if (e == cudaSuccess) e = rpy_apply(c, Y, FT, VW);       // warm-up
-            for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-                c->tune_ev = &ev[2 * r];
-                e = rpy_apply(c, Y, FT, VW);
-                c->tune_ev = nullptr;
-            }
-            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             float ms = 0.f;
-            for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-                float one = 0.f;
-                e = cudaEventElapsedTime(&one, ev[2 * r], ev[2 * r + 1]);
-                ms += one;
-            }
-            if (e == cudaSuccess) k.ms = std::min(k.ms, ms);
+            e = use(k);
+            if (e == cudaSuccess) e = time(false, ms);
+            if (e != cudaSuccess) break;
+            k.ms = std::min(k.ms, ms);
         }
     }
-    c->tune_ev = nullptr;
+    for (const cand &k : cands)
+        if (k.ms < best.ms) best = k;
+    const cudaError_t eu = use(best);       // (a valid schedule also where a launch failed)
+    if (e == cudaSuccess) e = eu;
+    for (int sweep = 0; sweep < kSweeps && e == cudaSuccess; ++sweep) {
+        float ms = 0.f;
+        e = time(true, ms);
+        best.ms = sweep ? std::min(best.ms, ms) : ms;
+    }
     for (cudaEvent_t x : ev)
         if (x) cudaEventDestroy(x);
-    float best = 1e30f;
-    int best_tpt = c->rpy_tpt, best_split = c->rpy_split, best_ctas = c->rpy_ctas,
-        best_auto = c->rpy_auto;
-    for (const cand &k : cands)
-        if (k.ms < best) {
-            best = k.ms;
-            best_tpt = k.tpt;
-            best_split = k.split;
-            best_ctas = k.ctas;
-            best_auto = k.automatic;
-        }
-    c->rpy_auto = best_auto;
-    c->rpy_tpt = best_tpt;
-    c->rpy_split = best_split;
-    c->rpy_threads = kRpyThreads;
-    c->rpy_ctas = best_ctas;
-    set_grids(c);
-    build_tiles(c);
-    if (e == cudaSuccess) e = upload_tiles(c);
     c->n_applies = a0;
     c->n_launches = l0;
     c->n_pairs = p0;
-    if (best_ms) *best_ms = best / std::max(1, reps);
+    if (best_ms) *best_ms = best.ms / std::max(1, reps);
     return e;
 }
 
