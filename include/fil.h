@@ -150,14 +150,21 @@ fil_status fil_sys_stats(const fil_ctx *c, int32_t *iters, double *finf);
 fil_status fil_autotune(fil_ctx *c, int32_t reps, int32_t *tile, int32_t *ctas_per_sm,
                         double *ms);
 
-/* Set the pair schedule by hand (the autotuner's candidates): tile 256 with 2
- * targets per thread or tile 128 with 1, and ctas_per_sm from 1 to the
- * kernel's occupancy; the source split goes back to 1. FIL_EINVAL for another
- * combination, FIL_ESTATE inside a step. fil_pair_schedule reads the current
- * one (nullable outputs). On the FP32 path a context of one system whose
- * schedule was never set reports 256-target tiles at 4 CTAs per SM and runs the
- * automatic schedule: 64-target tiles per warp, the (tile, source group) units
- * split evenly over one CTA of 12 warps per SM. */
+/* Set the pair schedule (the autotuner's candidates): tile 256 with 2
+ * targets per thread or tile 128 with 1, and ctas_per_sm from 1 to 4 or 6 on the FP32
+ * path (2 with a source split; more than are resident at once run in waves) and to the
+ * kernel's occupancy on the FP64 path; the source split goes back to 1. FIL_EINVAL for
+ * another combination, FIL_ESTATE inside a step. fil_pair_schedule reads the current
+ * one (nullable outputs).
+ * A new context reports 256-target tiles at the largest ctas_per_sm. In a context of
+ * one system these values name the automatic schedule, whether reported, set or chosen
+ * by the autotuner: on the FP32 path up to 160 segments one warp per target, summed in
+ * FP64, and beyond that 64-target tiles per warp, the (tile, source group) units split
+ * evenly over one CTA of 12 warps per SM; on the FP64 path up to 1024 segments one warp
+ * per target, up to 8192 every unordered pair once, and the 256-target tiles beyond. An
+ * apply whose result overlaps its inputs runs as if larger (FP64: in the 256-target
+ * tiles). Another schedule therefore replaces the FP64 sums of a small FP32 system by
+ * FP32 ones; setting these values brings them back. */
 fil_status fil_set_pair_schedule(fil_ctx *c, int32_t tile, int32_t targets_per_thread,
                                  int32_t ctas_per_sm);
 fil_status fil_pair_schedule(const fil_ctx *c, int32_t *tile, int32_t *targets_per_thread,

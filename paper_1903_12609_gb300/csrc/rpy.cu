@@ -1904,6 +1904,13 @@ void set_grids(fil_ctx *c) {
 
 }  // namespace
 
+// The automatic schedule of one system goes by the values a new context reports, so that
+// a schedule that was read and is set again is the one that ran.
+static int automatic_schedule(const fil_ctx *c, int tpt, int ctas, int split) {
+    return c->n_sys == 1 && tpt == kRpyTargetsPerThread && split == 1 &&
+           ctas == pair_occupancy(c, kRpyTargetsPerThread, 1);
+}
+
 cudaError_t rpy_setup(fil_ctx *c) {
     c->rpy_tpt = kRpyTargetsPerThread;
     c->rpy_threads = kRpyThreads;
@@ -1932,7 +1939,7 @@ cudaError_t rpy_setup(fil_ctx *c) {
         }
     c->rpy_tiles_max = count_tiles(c, kWarpTile);
     c->rpy_frames = pair32_on(c) && ns == 1 ? 1 : 0;
-    c->rpy_auto = ns == 1 ? 1 : 0;
+    c->rpy_auto = automatic_schedule(c, c->rpy_tpt, c->rpy_ctas, c->rpy_split);
     if (c->rpy_frames) {
         const cudaError_t e = allow_warp_smem();
         if (e != cudaSuccess) return e;
@@ -2172,17 +2179,17 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
     std::vector<cudaEvent_t> ev(2 * (size_t)std::max(1, reps), nullptr);
     cudaError_t e = cudaSuccess;
     for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
-    struct cand { int tpt, split, ctas, automatic; float ms; };
+    struct cand { int tpt, split, ctas; float ms; };
     std::vector<cand> cands;
     const bool direct = c->n_sys == 1 && pair32_on(c) && c->lay.S <= kDirect32MaxSeg;
     for (int tpt = 1; tpt <= 2 && !direct; ++tpt) {
         for (int split = 1; split <= (tpt == 1 && pair32_on(c) ? 2 : 1); ++split) {
             const int occ = pair_occupancy(c, tpt, split);
             for (int ctas = 1; ctas <= std::min(occ, c->rpy_ctas_max); ++ctas)
-                cands.push_back({tpt, split, ctas, 0, 1e30f});
+                cands.push_back({tpt, split, ctas, 1e30f});
         }
     }
-    if (c->n_sys == 1) cands.push_back({2, 1, pair_occupancy(c, 2, 1), 1, 1e30f});
+    if (direct) cands.push_back({kRpyTargetsPerThread, 1, pair_occupancy(c, 2, 1), 1e30f});
     const auto t0 = std::chrono::steady_clock::now();
     while (e == cudaSuccess) {
         for (int r = 0; r < 4 && e == cudaSuccess; ++r) e = rpy_apply(c, Y, FT, VW);
@@ -2191,14 +2198,7 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
         if (dt.count() >= kSpinUpMs) break;
     }
     const auto use = [&](const cand &k) {
-        c->rpy_auto = k.automatic;
-        c->rpy_tpt = k.tpt;
-        c->rpy_split = k.split;
-        c->rpy_threads = kRpyThreads;
-        c->rpy_ctas = k.ctas;
-        set_grids(c);
-        build_tiles(c);
-        return upload_tiles(c);
+        return rpy_set_schedule(c, k.tpt, kRpyThreads, k.ctas, k.split);
     };
     // the time of `reps` applies, or of their pair kernels, in the schedule in use
     const auto time = [&](bool pair, float &ms) {
@@ -2218,7 +2218,7 @@ cudaError_t rpy_autotune(fil_ctx *c, const double *Y, const double *FT, double *
         }
         return er;
     };
-    cand best{c->rpy_tpt, c->rpy_split, c->rpy_ctas, c->rpy_auto, 1e30f};
+    cand best{c->rpy_tpt, c->rpy_split, c->rpy_ctas, 1e30f};
     for (int sweep = 0; sweep < kSweeps && e == cudaSuccess; ++sweep) {
         for (cand &k : cands) {
             float ms = 0.f;
@@ -2257,7 +2257,7 @@ bool rpy_schedule_valid(const fil_ctx *c, int tpt, int threads, int ctas, int sp
 }
 
 cudaError_t rpy_set_schedule(fil_ctx *c, int tpt, int threads, int ctas, int split) {
-    c->rpy_auto = 0;
+    c->rpy_auto = automatic_schedule(c, tpt, ctas, split);
     c->rpy_tpt = tpt;
     c->rpy_split = split;
     c->rpy_threads = threads;
