@@ -166,6 +166,14 @@ __global__ void output_kernel(const float *__restrict__ yhat, int64_t n, const f
 // rounding errors would, a thread sums its squares in FP64.
 constexpr float kSquareMax = 1e38f, kSquareMin = 1e-12f;
 constexpr int kLossThreads = kOut;
+
+// hi + lo += x, the error of the addition (TwoSum) into lo.
+__device__ __forceinline__ void add_two(float &hi, float &lo, float x) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
+}
+
 __global__ void __launch_bounds__(kLossThreads)
 loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t B,
             const float *__restrict__ mean, const float *__restrict__ stdv, bf16 *__restrict__ dY,
@@ -184,19 +192,18 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
         y[r] = in ? yhat[(b0 + r) * kOut + c] : 0.f;
         g[r] = in ? t[(b0 + r) * kOut + c] : mu;
     }
-    float hi = 0.f, lo = 0.f, sum = 0.f, most = 0.f;
+    float hi = 0.f, lo = 0.f, sum = 0.f, sum_lo = 0.f, most = 0.f;
     uint32_t h[kRows / 2];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
         const bool in = b0 + r < B;
         const float d = in ? y[r] - (g[r] - mu) / sd : 0.f;
         most = fmaxf(most, fabsf(d));
-        const float sq = __fmul_rn(d, d), se = __fmaf_rn(d, d, -sq);
-        const float s = __fadd_rn(hi, sq), bb = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(se, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(sq, bb))));
-        hi = s;
+        const float sq = __fmul_rn(d, d);
+        add_two(hi, lo, sq);
+        lo = __fadd_rn(lo, __fmaf_rn(d, d, -sq));
         const float gr = d * inv;
-        sum += gr;
+        add_two(sum, sum_lo, gr);
         const bf16 q = __float2bfloat16_rn(gr);
         const uint32_t bits = in ? *reinterpret_cast<const unsigned short *>(&q) : 0u;
         if (r & 1) h[r >> 1] |= bits << 16;
@@ -205,7 +212,7 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
     }
     store_column(dYt + (int64_t)c * ldt, b0, Kb, h);
     if ((int)blockIdx.x >= n_part) return;      // rows of the zero padding only
-    col_sums[(int64_t)blockIdx.x * kOut + c] = sum;
+    col_sums[(int64_t)blockIdx.x * kOut + c] = __fadd_rn(sum, sum_lo);
     double acc = 0.5 * ((double)hi + (double)lo);
     if (!(hi < kSquareMax && (most > kSquareMin || most == 0.f))) {
         acc = 0.0;
@@ -227,7 +234,7 @@ loss_kernel(const float *__restrict__ yhat, const float *__restrict__ t, int64_t
 
 // db_l[c] = sum of the column sums' parts (l < 3: one per row tile of the
 // product that formed dZ_l; l = 3: one per CTA of the loss kernel), and the
-// loss. Parts in order, eight loads in flight.
+// loss. Parts in order, compensated (TwoSum), eight loads in flight.
 struct BiasParts {
     const float *p[kLayers];
     int n[kLayers];
@@ -239,11 +246,11 @@ __global__ void finish_kernel(BiasParts bp, const double *__restrict__ part, int
     const int l = blockIdx.y, c = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = l < 3 ? kHid : kOut;
     if (c < N) {
-        float s = 0.f;
+        float s = 0.f, lo = 0.f;
         const float *p = bp.p[l] + c;
 #pragma unroll 8
-        for (int i = 0; i < bp.n[l]; ++i) s += p[(int64_t)i * N];
-        bp.db[l][c] = s;
+        for (int i = 0; i < bp.n[l]; ++i) add_two(s, lo, p[(int64_t)i * N]);
+        bp.db[l][c] = __fadd_rn(s, lo);
     }
     if (l == 0 && blockIdx.x == 0 && threadIdx.x < 32) {
         double a = 0.0;
