@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "approx64.cuh"
 #include "fil_internal.cuh"
 #include "j0_common.cuh"
 #include "quat.cuh"
@@ -222,19 +223,6 @@ band_lu_kernel(Layout lay, T *__restrict__ band_all, int *__restrict__ piv_all,
         }
     }
 #undef RB
-}
-
-// 1/x by Newton's iteration y += y (1 - x y) from the hardware's seed (about
-// 2^-20): two steps, each one fused residual and one fused update, leave an
-// error of rounding size. The seed flushes what 1/x or x would make subnormal,
-// so those, infinities and NaN divide.
-__device__ __forceinline__ double recip(double x) {
-    const int e = (__double2hiint(x) >> 20) & 0x7ff;
-    if (e < 2 || e > 2044) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
 }
 
 constexpr int kLu64Threads = 128;

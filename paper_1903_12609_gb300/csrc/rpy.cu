@@ -51,6 +51,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "approx64.cuh"
 #include "fil_internal.cuh"
 
 namespace fil {
@@ -1569,17 +1570,6 @@ rpy_pair64_kernel(const double *__restrict__ src, SysMap smap, int64_t W, int G,
 // shuffles, shared memory and integer work cost nothing beside it, and what
 // counts is the FP64 instructions per pair and how evenly they are spread.
 // ---------------------------------------------------------------------------
-
-// 1/sqrt(x) for normal x > 0: the hardware's approximation (PTX
-// rsqrt.approx.ftz.f64, ~20 bits) and one step of the third-order iteration
-//   y <- y + y e (1/2 + 3/8 e),  e = 1 - x y^2
-// (the series of (1 - e)^{-1/2}), whose next term, 5/16 e^3, is below 2^-57.
-__device__ __forceinline__ double rsqrt_iter(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(fma(0.375, e, 0.5), y * e, y);
-}
 
 // Coefficients of a pair at r^2. The comparisons are on the bits (r^2 >= 0), so
 // they take no FP64 instruction; the overlapping form runs only in warps that
