@@ -48,6 +48,7 @@ namespace {
 
 constexpr int kAsmThreads = 256;
 constexpr int kGemvRows = 4;   // rows per warp in flight in the streamed inverse apply
+constexpr int kGemvCols = 6;   // and columns per lane: n up to 192 in one round
 constexpr int kInvThreads = 512;
 constexpr int kMaxInvN = 6 * kMaxDenseSeg;   // rows of the largest inverted block
 
@@ -550,12 +551,20 @@ __device__ __forceinline__ void inv_gemv_cta(const float *Inv, const float *r, f
         float t[kGemvRows];
 #pragma unroll
         for (int u = 0; u < kGemvRows; ++u) t[u] = 0.f;
-#pragma unroll 6
-        for (int c = lane; c < n; c += 32) {
-            const float rc = r[c];
+        for (int c0 = lane; c0 < n; c0 += 32 * kGemvCols) {
+            float a[kGemvCols][kGemvRows];
 #pragma unroll
-            for (int u = 0; u < kGemvRows; ++u)
-                if (i0 + u < n) t[u] = fmaf(Inv[(int64_t)(i0 + u) * n + c], rc, t[u]);
+            for (int k = 0; k < kGemvCols; ++k)
+#pragma unroll
+                for (int u = 0; u < kGemvRows; ++u)
+                    a[k][u] = c0 + 32 * k < n && i0 + u < n
+                                  ? Inv[(int64_t)(i0 + u) * n + c0 + 32 * k] : 0.f;
+#pragma unroll
+            for (int k = 0; k < kGemvCols; ++k) {
+                const float rc = c0 + 32 * k < n ? r[c0 + 32 * k] : 0.f;
+#pragma unroll
+                for (int u = 0; u < kGemvRows; ++u) t[u] = fmaf(a[k][u], rc, t[u]);
+            }
         }
         const bool hi = lane & 16, odd = lane & 8;
         const float p = (hi ? t[2] : t[0]) + __shfl_xor_sync(all, hi ? t[0] : t[2], 16);
