@@ -763,8 +763,13 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
             if (e != cudaSuccess) return e;
         }
         c->n_launches += 1;
-        return launch_pdl(band_block_solve_kernel, c->lay.M, kBlkThreads, smem, c->stream, c->lay,
-                          c->jofs, c->bmaps, ct, 6 * c->lay.maxN + 2 * kBlk, b, x);
+        // Early (launch_dep) while its CTAs find SMs of their own. Three steps at drag
+        // mobility, early and plainly, FIL_FP64: 1.83 and 1.89 ms with 5 filaments, 3.23 and
+        // 3.41 with 20, 5.0 and 5.2 with 38, 10.9 and 11.0 with 76, 57.6 and 57.4 with 200;
+        // FIL_PAIR32: 4.39 and 4.35 with 38, 6.38 and 6.18 with 100, 19.7 and 17.7 with 300.
+        return launch_dep(c->lay.M <= c->num_sms / 3, band_block_solve_kernel, c->lay.M,
+                          kBlkThreads, smem, c->stream, c->lay, c->jofs, c->bmaps, ct,
+                          6 * c->lay.maxN + 2 * kBlk, b, x);
     }
     const int zmax = 6 * c->lay.maxN;
     const size_t per = (size_t)zmax * sizeof(double);

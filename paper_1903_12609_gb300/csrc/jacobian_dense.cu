@@ -1057,8 +1057,14 @@ cudaError_t j0_dense_solve(fil_ctx *c, const double *b, double *x, const int *ac
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     c->n_launches += 1;
-    return launch_pdl(j0_solve_fused_kernel, c->lay.M, kSolveThreads, smem, c->stream, c->lay, c->jofs,
-                      c->auxofs, dp, c->aux, c->jinv, b, x, active, kJ0Refine);
+    // Early (launch_dep) while its CTAs find SMs of their own, and where they fill all of
+    // them (4 CTAs each). One solve after another, early and plainly: 30.9 and 32.9 us with
+    // 20 filaments of 20 to 30 segments, 33 and 32.9 with 38, 34 and 32.9 with 60, 69 and
+    // 32.9 with 100, 62 and 53 with 300, 88 and 90 with 600, 134 and 136 with 1000; three
+    // steps 1.93 and 1.97 ms with 20, 2.92 and 2.72 with 152, 5.2 and 5.0 with 300.
+    const bool early = c->lay.M <= c->num_sms / 3 || c->lay.M >= 4 * c->num_sms;
+    return launch_dep(early, j0_solve_fused_kernel, c->lay.M, kSolveThreads, smem, c->stream, c->lay,
+                      c->jofs, c->auxofs, dp, c->aux, c->jinv, b, x, active, kJ0Refine);
 }
 
 }  // namespace fil
