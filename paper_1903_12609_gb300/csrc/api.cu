@@ -916,10 +916,17 @@ fil_status fil_broyden_step(fil_ctx *c, int32_t *converged, double *finf) {
     // One small system: the rest of the iteration is enqueued behind the status copy
     // and the host waits for the copy alone, so that the GPU works while the host
     // decides. What the last iteration of a step enqueued in vain (it touches the step
-    // w and history slots that no pair counts) is cheaper there than a round trip of
-    // ~20 us in every iteration; for large systems it is not. (An evaluation that failed
-    // leaves them alone, see update_kernel.)
-    const bool ahead = c->n_sys == 1 && c->lay.S <= kAheadMaxSeg;
+    // w and history slots that no pair counts) costs less there than a round trip of
+    // ~20 us in every iteration. (An evaluation that failed leaves them alone, see
+    // update_kernel.) Not with the FP64-refined filament-RPY solve, whose 30 us and more
+    // once a step are not made up by its few iterations. Three steps, ahead and not: drag
+    // J0, FIL_FP64, 1.50 and 1.57 ms at 160 segments, 4.64 and 4.71 at 1 000, 13.17 and
+    // 13.17 at 2 000, 31.31 and 31.35 at 3 000; FIL_PAIR32 2.63 and 2.78 at 240, 5.2 and
+    // 5.4 at 2 040; filament-RPY J0, FIL_MIXED 1.42 and 1.44 at 480, 1.69 and 1.65 at
+    // 2 040; FIL_PAIR32 (refined) 1.40 and 1.33 at 256, 1.81 and 1.72 at 1 024, 3.84 and
+    // 3.75 at 5 120.
+    const bool refined = c->j0_model == FIL_J0_FILAMENT_RPY && !fast_mixed(c);
+    const bool ahead = c->n_sys == 1 && c->lay.S <= kAheadMaxSeg && !refined;
     if (ahead) {
         if (!c->status_ev) CK(cudaEventCreateWithFlags(&c->status_ev, cudaEventDisableTiming));
         CK(copy_status(c));
