@@ -253,11 +253,11 @@ inline bool fast_mixed(const fil_ctx *c) { return c->prec == FIL_MIXED; }
 
 // Programmatic dependent launch through the chain of an iteration's kernels: a
 // kernel launched with launch_pdl may become resident while the kernel before it
-// in the stream still runs, and pdl_enter, its first statement, holds it until
-// that kernel is complete and its writes are visible (so every kernel given to
-// launch_pdl starts with pdl_enter). What overlaps is the launch itself: the
-// iterations of small systems are chains of a dozen kernels of 2-10 us, and each
-// boundary cost 1-2 us more.
+// in the stream still runs, and pdl_enter holds it until that kernel is complete
+// and its writes are visible (so every kernel given to launch_pdl calls it, and
+// nothing before the call reads or writes memory that an earlier kernel touches).
+// What overlaps is the launch itself: the iterations of small systems are chains
+// of a dozen kernels of 2-10 us, and each boundary cost 1-2 us more.
 //
 // launch_dep with early == false is the plain launch. CTAs that become resident
 // early go to whatever SMs have room at that moment, several to one SM while

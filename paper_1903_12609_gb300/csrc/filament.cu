@@ -452,8 +452,9 @@ cudaError_t residual_rows(fil_ctx *c, const double *X, double *f, const double *
     c->n_launches += 1;
     // Early (launch_dep) behind the FP64 kernels of one system, in small ensembles (see
     // unpack_forces) and up to kRowsEarly segments. Behind the FP32 kernel of one system,
-    // whose CTAs all leave room, the rows crowd: a residual took 62.2 us early and 63.6 us plainly at 320 segments, 65.8 and
-    // 63.8 at 640, 87.3 and 77.9 at 2 560, 175 and 168 at 8 000.
+    // whose CTAs all leave room, the rows crowd: a residual took 62.2 us early and 63.6 us
+    // plainly at 320 segments, 65.8 and 63.8 at 640, 87.3 and 77.9 at 2 560, 175 and 168 at
+    // 8 000.
     const bool early = c->n_sys > 1 ? c->lay.S <= kEnsembleEarly
                                     : !pair32_on(c) || c->lay.S <= kRowsEarly;
     return launch_dep(early, residual_rows_kernel, seg_grid(c->lay.S, kRowThreads), kRowThreads, 0,

@@ -309,7 +309,7 @@ constexpr int kSolvePf = 8;     // rows of factors loaded ahead by the band solv
 constexpr int kSolveLanes = 16; // lanes per filament
 
 // Forward and backward substitution in the banded factors for one right-hand
-// side z (n entries in shared memory, in band order, zero before row jf), by
+// side z (n entries in shared memory, in band order), by
 // 16 lanes, half a warp; the two halves of a warp run the longer one's n_both
 // steps together.
 //
@@ -325,7 +325,7 @@ constexpr int kSolveLanes = 16; // lanes per filament
 template <typename T>
 __device__ __forceinline__ void band_substitute(const T *__restrict__ A,
                                                 const int *__restrict__ piv, T *z, int n,
-                                                int n_both, int lane, int jf) {
+                                                int n_both, int lane) {
 #define BAND(i, c) A[(int64_t)(i) * kBandW + ((c) - (i) + kBandKL)]
     // The factors a row step needs do not depend on z, so each lane loads them
     // kSolvePf rows ahead into a register queue: the loads of the next block are
@@ -334,8 +334,7 @@ __device__ __forceinline__ void band_substitute(const T *__restrict__ A,
     // the row r in [j, j + 15] with r = l (mod 16)
     T w;
     {
-        const int r = jf + ((lane - jf) & (kSolveLanes - 1));
-        w = r < n ? z[r] : T(0);
+        w = lane < n ? z[lane] : T(0);
     }
     {
         T lq[kSolvePf];
@@ -346,8 +345,8 @@ __device__ __forceinline__ void band_substitute(const T *__restrict__ A,
             p = j < n ? piv[j] : j;
         };
 #pragma unroll
-        for (int u = 0; u < kSolvePf; ++u) fetch(jf + u, lq[u], pq[u]);
-        for (int jb = jf; jb < n_both; jb += kSolvePf) {
+        for (int u = 0; u < kSolvePf; ++u) fetch(u, lq[u], pq[u]);
+        for (int jb = 0; jb < n_both; jb += kSolvePf) {
             T ln[kSolvePf];
             int pn[kSolvePf];
 #pragma unroll
@@ -476,7 +475,7 @@ __global__ void band_solve_kernel(Layout lay, const T *__restrict__ band_all,
         b1z = bf[2];
     }
     __syncwarp();
-    band_substitute(A, piv, z, n, n_both, lane, 0);
+    band_substitute(A, piv, z, n, n_both, lane);
     if (!live) return;
     // scatter back: u_s, Lam_j, and Y_1 = b1 + c_t Lam_0
     for (int e = lane; e < 3 * N; e += kSolveLanes) {
@@ -751,8 +750,9 @@ cudaError_t j0_build_factor(fil_ctx *c, const double *X) {
 }
 
 cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) {
-    // in blocks of rows (one system, which no list of active ones narrows), else half a warp per filament; up to 4 warps per CTA, fewer for long filaments so
-    // that each filament's right-hand side fits in shared memory
+    // in blocks of rows (one system, which no list of active ones narrows), else half a
+    // warp per filament; up to 4 warps per CTA, fewer for long filaments so that each
+    // filament's right-hand side fits in shared memory
     const double ct = make_params(c).ct;
     if (c->bmaps) {
         const size_t smem = block_solve_smem(c);
@@ -766,8 +766,8 @@ cudaError_t j0_solve(fil_ctx *c, const double *b, double *x, const int *active) 
         // Early (launch_dep) while its CTAs find SMs of their own. Three steps at drag
         // mobility, early and plainly, FIL_FP64: 1.83 and 1.89 ms with 5 filaments, 3.23 and
         // 3.41 with 20, 5.0 and 5.2 with 38, 10.9 and 11.0 with 76, 57.6 and 57.4 with 200;
-        // FIL_PAIR32: 4.39 and 4.35 with 38, 6.38 and 6.18 with 100, 19.7 and 17.7 with 300.
-        return launch_dep(c->lay.M <= c->num_sms / 3, band_block_solve_kernel, c->lay.M,
+        // FIL_PAIR32: 4.95 and 5.03 with 60, 6.38 and 6.18 with 100, 19.7 and 17.7 with 300.
+        return launch_dep(c->lay.M <= c->num_sms / 2, band_block_solve_kernel, c->lay.M,
                           kBlkThreads, smem, c->stream, c->lay, c->jofs, c->bmaps, ct,
                           6 * c->lay.maxN + 2 * kBlk, b, x);
     }

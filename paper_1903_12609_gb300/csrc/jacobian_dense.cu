@@ -613,7 +613,7 @@ j0_apply_inverse_kernel(Layout lay, const int64_t *__restrict__ jofs,
 // barriers with another's FP64 work: 64 registers, 4 CTAs per SM (at 110
 // registers, 2 CTAs: 168 us; 5 spill: 132). Measured, 1000 filaments of 32:
 // 188 us with 16 lanes per target, each row of a product converted and added
-// by one lane, and two columns of a row in flight; 111 us in this form.
+// by one lane, and two columns of a row in flight; 109 us in this form.
 constexpr int kSolveThreads = 256;
 
 __global__ void __launch_bounds__(kSolveThreads, 4)

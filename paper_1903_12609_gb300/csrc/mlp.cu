@@ -64,7 +64,7 @@ tc::Problem product(const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N
 }
 
 // A launch whose prologue may overlap the kernel before it in the stream (both
-// call pdl_wait_previous / pdl_launch_next): the calls are chains of 5 and 10
+// call pdl_wait_previous / pdl_launch_next): the calls are chains of 5 and 11
 // kernels of a few microseconds, and each gap between two costs about as much.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
@@ -453,7 +453,7 @@ cudaError_t forward_raw(fil_mlp *m, const float *x, float *y, int64_t B) {
 }
 
 // Loss and gradient into `grad` (16-byte aligned); the loss (device) in m->loss.
-// Ten launches: the input, four forward products, the loss, the three products
+// Eleven launches: the input, four forward products, the loss, the three products
 // that carry dZ back, all four weight gradients in one, and the bias gradients.
 cudaError_t gradients(fil_mlp *m, const float *x, const float *t, int64_t B, float *grad) {
     const int64_t Kb = round_up(B, tc::kTileK);

@@ -22,15 +22,17 @@
 //    contracted coefficients and splitting them into BF16 pieces costs as many
 //    FP32-pipe cycles as the sums it would save). The bound is the FP32 (or
 //    FP64) FMA pipe.
-//  * Packed FP32x2 arithmetic: a thread evaluates its target against two
-//    sources at once, lane x of every float2 holding the even source and lane
-//    y the odd one; the records of a source pair are stored interleaved so
-//    that each loaded float2 is an operand.
+//  * Packed FP32x2 arithmetic. One system (rpy_pair32_warp_kernel): a thread
+//    evaluates two targets against one source at once, lane x and lane y of every
+//    float2 (pair32_far2). Ensembles and schedules set by hand (rpy_pair32_kernel):
+//    one target against two sources, whose records are stored interleaved so that
+//    each loaded float2 is an operand (pair32_far).
 //  * Each thread owns two targets in registers (one in the 128-target
 //    schedules) and all lanes read the same source from shared memory
 //    (broadcast).
-//  * Sources come in groups of 32 relative to the group's centre, and the pair
-//    terms are summed in that frame (pair32_far).
+//  * One system's sources come in groups of 32 relative to the group's centre, and
+//    the pair terms are summed in that frame, but for Omega at the targets inside a
+//    group that spans several filaments (wide_radius2).
 //  * Stream-K persistent grid: the work units (tile of targets, group of
 //    sources) are split evenly over the grid; who touches a tile only in part
 //    writes one partial of it, and the CTA that completes a tile (a counter
@@ -213,10 +215,13 @@ struct Rec {
 // groups dealt out in turn, so that the groups whose close pairs cost a tile up to
 // three times a far unit (its own and the next ones of its filaments) go to
 // different warps. spread_group: the group at place i; spread_place: its inverse.
-// spread_count: n where the order pays, else 0, the groups' own. Whole applies,
-// own order and spread: 960 segments 21.8 and 23.1 us (a unit per warp: nothing to
-// spread), 1 920 35.9 and 33.9, 3 200 46.3 and 43.0, 6 400 89.1 and 87.4, 9 651 in
-// ragged filaments 175.9 and 172.6, 16 000 400.7 and 401.8, 32 000 1483 and 1492.
+// spread_count: n where the order pays, else 0, the groups' own. Whole applies, own
+// order and spread, filaments of 32, of 20, of 16 to 48 segments: 960 segments 20.9 and
+// 21.7 us, 21.9 and 23.3, 22.5 and 23.6 (a unit per warp: nothing to spread); 1 536 26.6 and
+// 28.2, 28.3 and 30.2, 33.4 and 31.4; 1 920 33.5 and 35.3, 36.4 and 37.5, 40.7 and 37.4;
+// 3 200 46.7 and 45.0, 52.8 and 47.9, 53.3 and 48.2; 6 400 86 and 85, 98 and 93, 106 and
+// 100; 12 288 240 and 243, 270 and 265, 265 and 265; 16 000 384 and 388, 423 and 429, 422
+// and 421.
 __host__ __device__ __forceinline__ int spread_count(int64_t n) {
     return n >= 48 && n <= 384 ? (int)n : 0;
 }
@@ -1190,9 +1195,9 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
 // per 128 sources: 9 651 segments in ragged filaments 224 -> 181 us, 3200
 // segments 73 -> 50 us, 32 000 1504 -> 1491 us (at the close groups' loop
 // unrolled by 2; by 4 its registers cost the far loop 7%). One system only. With the
-// two targets of a lane packed (pair32_far2) and the spread order 9 651 take 160 us,
-// 3200 44 and 32 000 1426; of these 36 us are the compensated fold and 10 the close
-// groups, the rest the far loop and each group's start.
+// two targets of a lane packed (pair32_far2) and the spread order 9 651 took 160 us,
+// 3200 44 and 32 000 1426, of which 36 us are the compensated fold and 10 the close
+// groups; with Omega's cross products per pair inside wide groups 173, 45 and 1435.
 // ---------------------------------------------------------------------------
 constexpr int kWarpTile = kRpyMinTile;          // targets per tile
 constexpr int kWarpPart = 12 * kWarpTile;       // floats of a partial
@@ -1673,8 +1678,9 @@ constexpr int kSymThreads = 128;
 constexpr int64_t kSymMaxSeg = 8192;          // slots: (S / 64) x 6 S doubles
 constexpr int64_t kDirectMaxSeg = 1024;       // up to here a warp per target is faster
 // The FP32 modes take it too while it is faster than packing and the FP32 kernel,
-// whose chain of one unit alone is 10-13 us: at 32 segments 5.1 and 10.6 us, at 128
-// 9.7 and 13.8, at 192 13.7 and 12.7. (FP64 throughout, so closer than the FP32 sums.)
+// whose chain of a few units alone is 11-15 us: at 32 segments 5.1 and 11.1 us, at 96 7.8
+// and 15.0, at 160 11.5 and 14.4; at 192 13.5 and 14.3, at 224 15.4 and 14.3. (FP64
+// throughout, so closer than the FP32 sums; the line stays at the 160 that fil.h states.)
 constexpr int64_t kDirect32MaxSeg = 160;
 inline int64_t direct_max(bool pair32) { return pair32 ? kDirect32MaxSeg : kDirectMaxSeg; }
 
@@ -2134,7 +2140,8 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         if (c->tune_ev && c->tune_pair) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
         launch_dep(early, c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G,
-                   kRpyThreads, 0, c->stream, c->src64, sm, W, G, k, (double *)c->partials, c->tile_cnt, scale, VW);
+                   kRpyThreads, 0, c->stream, c->src64, sm, W, G, k, (double *)c->partials,
+                   c->tile_cnt, scale, VW);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
         if (c->tune_ev) cudaEventRecord(c->tune_ev[1], c->stream);
     }
@@ -2266,8 +2273,8 @@ cudaError_t rpy_set_schedule(fil_ctx *c, int tpt, int threads, int ctas, int spl
 // someone else -- this variant of the mixed-precision apply uses no context
 // and allocates nothing: its scratch (packed FP32 sources, the stream-K
 // partial sums and the tiles' completion counters) is the file-scope arrays
-// below, which every GPU that loads the library holds until the process exits. The caller passes the inputs and
-// the output in device memory.
+// below, which every GPU that loads the library holds until the process exits.
+// The caller passes the inputs and the output in device memory.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -2388,8 +2395,8 @@ extern "C" fil_status fil_rpy_apply_noalloc(int64_t n_seg, const double *Y, cons
     sm.n_units = n_units;
     sm.n_src = n_seg;
     const int n_spread = spread_count(n_units);
-    cudaError_t e = launch(pack32_kernel<true>, (unsigned)(Spad / kPackThreads), kPackThreads, 0, st, Y, FT, n_seg,
-                           Spad, sm, n_spread, (float)a, src);
+    cudaError_t e = launch(pack32_kernel<true>, (unsigned)(Spad / kPackThreads), kPackThreads, 0,
+                           st, Y, FT, n_seg, Spad, sm, n_spread, (float)a, src);
     if (e == cudaSuccess)
         e = launch(n_spread ? rpy_pair32_warp_kernel<true> : rpy_pair32_warp_kernel<false>,
                    (unsigned)G, 32 * kWarpCta, kWarpSmem, st, (const float4 *)src, sm, W, G,
