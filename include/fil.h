@@ -151,9 +151,9 @@ fil_status fil_autotune(fil_ctx *c, int32_t reps, int32_t *tile, int32_t *ctas_p
                         double *ms);
 
 /* Set the pair schedule (the autotuner's candidates): tile 256 with 2
- * targets per thread or tile 128 with 1, and ctas_per_sm from 1 to 4 or 6 on the FP32
- * path (2 with a source split; more than are resident at once run in waves) and to the
- * kernel's occupancy on the FP64 path; the source split goes back to 1. FIL_EINVAL for
+ * targets per thread or tile 128 with 1, and ctas_per_sm from 1 to the
+ * kernel's occupancy (FP32 path: 4 and 6, 2 with a source split); the source split goes
+ * back to 1. FIL_EINVAL for
  * another combination, FIL_ESTATE inside a step. fil_pair_schedule reads the current
  * one (nullable outputs).
  * A new context reports 256-target tiles at the largest ctas_per_sm. In a context of

@@ -113,8 +113,7 @@ struct fil_ctx {
                            // tile = rpy_threads x rpy_tpt targets
     int rpy_ctas;          // resident CTAs per SM of the stream-K grid
     bool rpy_full = true;  // as many as fit: the grid fills the SMs
-    int rpy_frames = 0;    // FP32 path: source groups in their own frames (one system; rpy.cu)
-    int rpy_auto = 0;      // one system, no schedule set by hand: the automatic kernels run (rpy.cu)
+    int rpy_auto = 0;      // one system in the automatic schedule (rpy.cu)
     int rpy_ctas_max;
     int64_t rpy_tiles_max; // listed tiles at the smallest tile size
     // the tiles of the systems still iterating (ensembles): applies inside a

@@ -24,7 +24,7 @@
 //    FP64) FMA pipe.
 //  * Packed FP32x2 arithmetic. One system (rpy_pair32_warp_kernel): a thread
 //    evaluates two targets against one source at once, lane x and lane y of every
-//    float2 (pair32_far2). Ensembles and schedules set by hand (rpy_pair32_kernel):
+//    float2 (pair32_far2). Ensembles and other schedules (rpy_pair32_kernel):
 //    one target against two sources, whose records are stored interleaved so that
 //    each loaded float2 is an operand (pair32_far).
 //  * Each thread owns two targets in registers (one in the 128-target
@@ -125,8 +125,8 @@ struct SysMap {
     const int64_t *dyn = nullptr;
 };
 
-// Sources of a work unit: one group where the sources are in frames (one system
-// on the FP32 path), else whole 128-source chunks.
+// Sources of a work unit: one group where the sources are in frames (the automatic
+// schedule of one FP32 system), else whole 128-source chunks.
 constexpr int unit_sources(bool frames) { return frames ? kRpyComp : kRpyChunk; }
 
 // The listed tiles and the unit count of a launch (from the device when dynamic).
@@ -194,9 +194,10 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 // first 15. One warp packs one group. Padding records sit far away with zero
 // load, so they add exactly zero. w is the squared radius within which targets take
 // the cross products per pair (wide_radius2; 0: none).
-// Ensembles keep records without a frame (kFrames false): 12 values per source
+// Ensembles, and one system in another schedule than the automatic one, have records
+// without a frame (kFrames false): 12 values per source
 //   -y(hi) 3 | F 3 | T 3 | -y(lo) 3,   y = Y - Y_0 = hi + lo.
-// Their systems with the drag J0 take tens of Broyden iterations whose path
+// The ensembles' systems with the drag J0 take tens of Broyden iterations whose path
 // follows the last bits of the pair sums (a system's count moves by one or two
 // with any other rounding, and its multipliers with it, by ~1e-3), so their
 // pair arithmetic, work units and order of sums stay those their trajectories
@@ -208,7 +209,6 @@ struct Rec {
     static constexpr int kLo = kFrames ? 7 : 4;                   // the lo parts: float4 kLo, half 1 on
     static constexpr int kHead = kFrames ? 1 : 0;                 // float4 before the pairs (centre)
     static constexpr int kGroupF4 = kHead + kPairF4 * kRpyComp / 2;
-    static constexpr int kSums = kFrames ? 12 : 6;                // packed sums of the far loop
 };
 
 // Order of the n groups' records for the automatic schedule: 16 runs of neighbouring
@@ -444,83 +444,48 @@ __device__ __forceinline__ void far_coef(float2 rinv, const RpyConst32 &k, float
     D = __fmul2_rn(f2(1.5f, 1.5f), rinv5);
 }
 
-// The inner loop: the pair terms of one target (position t, both lanes, in
-// the group's frame) and the two sources of a packed record q, lane x = even
-// source, lane y = odd source, in the far form, branch-free; whatever it
-// produces for close, overlapping or coincident pairs (Inf or NaN at r = 0)
-// is discarded by the caller, which evaluates such groups again. rmin2 tracks
-// the smallest r^2.
+// The inner loop without frames: the pair terms of one target (position t relative to
+// the apply's first segment, both lanes) and the two sources of a packed record q, lane
+// x = even source, lane y = odd source, in the far form, branch-free; whatever it
+// produces for close, overlapping or coincident pairs (Inf or NaN at r = 0) is
+// discarded by the caller, which evaluates such groups again. rmin2 tracks the
+// smallest r^2. 48 FP32 operations a pair, acc[0..2] += V terms, acc[3..5] += Omega
+// terms.
+__device__ __forceinline__ void pair32_far(const float2 *t, const float4 *q, const RpyConst32 &k,
+                                           float2 *acc, float &rmin2) {
+    const float4 q0 = q[0], q1 = q[1];
+    const float2 dx = __fadd2_rn(t[0], f2(q0.x, q0.y));
+    const float2 dy = __fadd2_rn(t[1], f2(q0.z, q0.w));
+    const float2 dz = __fadd2_rn(t[2], f2(q1.x, q1.y));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+    rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
+    float2 A, B, C, D, G;
+    far_coef(f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y)), k, A, B, C, D, G);
+    add_pair(q, dx, dy, dz, A, B, C, D, G, acc);
+}
+
+// The inner loop in the group's frame: the same for two targets, lane x and lane y of t,
+// and source H (0 even, 1 odd) of the record.
 //
 // With d = t - s in the group's frame the cross products split,
 //   sum G (T x d) = (sum G T) x t - sum G (T x s),
 // and likewise for F x d, so that a pair needs no G d: 12 sums take
 //   acc[0..2] += (1/r) F + B (d.F) d - G (T x s)   (V without its G F part)
 //   acc[3..5] += r^-5 (d.T) d - (2/3) G (F x s)    (2/3 of Omega's d-terms)
-//   acc[6..8] += G T,  acc[9..11] += G F           (see combine_group)
+//   acc[6..8] += G T,  acc[9..11] += G F           (see combine_group2)
 // in 39 FP32 operations a pair, 9 fewer than with the cross products formed
 // for every pair. What bounds the loop is register operands: a packed FMA
 // with three distinct register operands issues every third cycle, one with
 // two every second, and this form drops 3-operand FMAs (24 -> 21 sums) as
-// well as multiplies.
+// well as multiplies. Both targets take a source's values from single registers, so a
+// packed FMA reads one register fewer than with two sources in the lanes.
 // Measured (32 000 segments in filaments of 32, pair kernel): 1700 us with the cross
-// products formed per pair, 1491 us in this form; error against 64 bits of V 1.85e-7
-// and 1.55e-7 (the frames make the differences finer), of Omega 1.63e-7 and 1.60e-7.
-// Omega gains nothing where a group spans more than its neighbourhood: see wide_radius2.
-// Without frames (ensembles): t relative to the first segment, 48 operations,
-//   acc[0..2] += V terms, acc[3..5] += Omega terms.
-template <bool kFrames>
-__device__ __forceinline__ void pair32_far(const float2 *t, const float4 *q, const RpyConst32 &k,
-                                           float2 *acc, float &rmin2) {
-    if constexpr (!kFrames) {
-        const float4 q0 = q[0], q1 = q[1];
-        const float2 dx = __fadd2_rn(t[0], f2(q0.x, q0.y));
-        const float2 dy = __fadd2_rn(t[1], f2(q0.z, q0.w));
-        const float2 dz = __fadd2_rn(t[2], f2(q1.x, q1.y));
-        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-        rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
-        float2 A, B, C, D, G;
-        far_coef(f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y)), k, A, B, C, D, G);
-        add_pair(q, dx, dy, dz, A, B, C, D, G, acc);
-        return;
-    }
-    const float2 nk2 = f2(-k.k2a2, -k.k2a2);
-    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3], q4 = q[4], q5 = q[5], q6 = q[6];
-    const float2 q7 = reinterpret_cast<const float2 *>(q + 7)[0];
-    const float2 dx = __fadd2_rn(t[0], f2(q0.x, q0.y));
-    const float2 dy = __fadd2_rn(t[1], f2(q0.z, q0.w));
-    const float2 dz = __fadd2_rn(t[2], f2(q1.x, q1.y));
-    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-    const float2 rinv = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-    rmin2 = fminf(rmin2, fminf(r2.x, r2.y));
-    const float2 rinv2 = __fmul2_rn(rinv, rinv);
-    const float2 G = __fmul2_rn(rinv, rinv2);
-    const float2 rinv5 = __fmul2_rn(G, rinv2);
-    const float2 B = __ffma2_rn(nk2, rinv5, G);
-    const float2 Fx = f2(q1.z, q1.w), Fy = f2(q2.x, q2.y), Fz = f2(q2.z, q2.w);
-    const float2 Tx = f2(q3.x, q3.y), Ty = f2(q3.z, q3.w), Tz = f2(q4.x, q4.y);
-    const float2 bF = __fmul2_rn(B, __ffma2_rn(dx, Fx, __ffma2_rn(dy, Fy, __fmul2_rn(dz, Fz))));
-    const float2 dT =
-        __fmul2_rn(rinv5, __ffma2_rn(dx, Tx, __ffma2_rn(dy, Ty, __fmul2_rn(dz, Tz))));
-    acc[0] = __ffma2_rn(rinv, Fx, __ffma2_rn(G, f2(q4.z, q4.w), __ffma2_rn(bF, dx, acc[0])));
-    acc[1] = __ffma2_rn(rinv, Fy, __ffma2_rn(G, f2(q5.x, q5.y), __ffma2_rn(bF, dy, acc[1])));
-    acc[2] = __ffma2_rn(rinv, Fz, __ffma2_rn(G, f2(q5.z, q5.w), __ffma2_rn(bF, dz, acc[2])));
-    acc[3] = __ffma2_rn(G, f2(q6.x, q6.y), __ffma2_rn(dT, dx, acc[3]));
-    acc[4] = __ffma2_rn(G, f2(q6.z, q6.w), __ffma2_rn(dT, dy, acc[4]));
-    acc[5] = __ffma2_rn(G, q7, __ffma2_rn(dT, dz, acc[5]));
-    acc[6] = __ffma2_rn(G, Tx, acc[6]);
-    acc[7] = __ffma2_rn(G, Ty, acc[7]);
-    acc[8] = __ffma2_rn(G, Tz, acc[8]);
-    acc[9] = __ffma2_rn(G, Fx, acc[9]);
-    acc[10] = __ffma2_rn(G, Fy, acc[10]);
-    acc[11] = __ffma2_rn(G, Fz, acc[11]);
-}
-
-// The same sums of two targets, lane x and lane y of t, and source H (0 even, 1 odd)
-// of the record: a source's values are then single registers, the same for both
-// lanes, and a packed FMA reads one register fewer. Measured (same bits, whole applies,
-// the loop over the records unrolled in full): 32 000 segments 1477 us with pair32_far,
-// 1426 with this; 9 600 159 and 155; unrolled by 8 1484 and 161, as iterations of the
-// loop do not overlap. Up to 640 segments it costs 0.2 us of 14 to 19.
+// products formed per pair, 1491 us with two sources in the lanes (whole apply 1477),
+// 1426 (whole apply) in this form, unrolled in full; by 8 1484, as iterations of the loop
+// do not overlap. Error against 64 bits of V 1.85e-7 and 1.55e-7 (the frames make the
+// differences finer), of Omega 1.63e-7 and 1.60e-7: that gains nothing where a group spans
+// more than its neighbourhood, see wide_radius2.
+constexpr int kFarSums = 12;
 template <int H>
 __device__ __forceinline__ float2 both(const float4 &v, int half) {
     const float x = half ? (H ? v.w : v.z) : (H ? v.y : v.x);
@@ -612,39 +577,15 @@ __device__ __forceinline__ void combine_cross2(const float2 (&acc)[2][kCrossSums
     }
 }
 
-// The (V, Omega) terms of a group from the twelve sums of pair32_far: with
-// P = sum G T and Q = sum G F,
+// The (V, Omega) terms of a group for two targets, from the twelve sums of pair32_far2
+// over the even and the odd sources: with P = sum G T and Q = sum G F,
 //   V     = acc[0..2] + (2a^2/3) Q + P x t
 //   Omega = 3/2 acc[3..5] - P/2 + Q x t.
-template <bool kFrames>
-__device__ __forceinline__ void combine_group(const float2 *acc, const float2 *t, float k23,
-                                              float *out) {
-    if constexpr (!kFrames) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) out[c] = __fadd_rn(acc[c].x, acc[c].y);
-        return;
-    }
-    constexpr int kSums = Rec<kFrames>::kSums;
-    float s[12];
-#pragma unroll
-    for (int c = 0; c < kSums; ++c) s[c] = __fadd_rn(acc[c].x, acc[c].y);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int p = (c + 1) % 3, q = (c + 2) % 3;
-        out[c] = fmaf(k23, s[9 + c],
-                      fmaf(s[6 + p], t[q].x, fmaf(-s[6 + q], t[p].x, s[c])));
-        out[3 + c] = fmaf(1.5f, s[3 + c],
-                          fmaf(-0.5f, s[6 + c], fmaf(s[9 + p], t[q].x, -s[9 + q] * t[p].x)));
-    }
-}
-
-// The same for two targets, from the sums of pair32_far2 over the even and the odd
-// sources.
-__device__ __forceinline__ void combine_group2(const float2 (&acc)[2][Rec<true>::kSums],
+__device__ __forceinline__ void combine_group2(const float2 (&acc)[2][kFarSums],
                                                const float2 *t, float k23, float2 *out) {
-    float2 s[Rec<true>::kSums];
+    float2 s[kFarSums];
 #pragma unroll
-    for (int c = 0; c < Rec<true>::kSums; ++c) s[c] = __fadd2_rn(acc[0][c], acc[1][c]);
+    for (int c = 0; c < kFarSums; ++c) s[c] = __fadd2_rn(acc[0][c], acc[1][c]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const int p = (c + 1) % 3, q = (c + 2) % 3;
@@ -726,38 +667,16 @@ __device__ __forceinline__ void load_target(const float4 *src, int64_t P, float 
     }
 }
 
-// The target in the frame of the group with records q, for the far loop (t2,
-// both lanes) and as hi + lo parts.
-template <bool kFrames>
-__device__ __forceinline__ void to_frame(const float4 *q, const float *th, const float *tl,
-                                         float2 *t2) {
-    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-    if constexpr (kFrames) c = q[-1];
+// The target in the frame of the group with records q, as hi + lo parts.
+__device__ __forceinline__ void to_frame_hl(const float4 *q, const float *th, const float *tl,
+                                            float *uh, float *ul) {
+    const float4 c = q[-1];
     const float cc[3] = {c.x, c.y, c.z};
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-        const float v = kFrames ? __fadd_rn(__fsub_rn(th[x], cc[x]), tl[x]) : th[x];
-        t2[x] = f2(v, v);
-    }
-}
-template <bool kFrames>
-__device__ __forceinline__ void to_frame_hl(const float4 *q, const float *th, const float *tl,
-                                            float *uh, float *ul) {
-    if constexpr (kFrames) {
-        const float4 c = q[-1];
-        const float cc[3] = {c.x, c.y, c.z};
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            float e;
-            two_sum(th[x], -cc[x], uh[x], e);
-            ul[x] = __fadd_rn(e, tl[x]);
-        }
-    } else {
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            uh[x] = th[x];
-            ul[x] = tl[x];
-        }
+        float e;
+        two_sum(th[x], -cc[x], uh[x], e);
+        ul[x] = __fadd_rn(e, tl[x]);
     }
 }
 
@@ -931,10 +850,6 @@ __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, 
 // TPT per thread; their pair terms are summed in registers over groups of
 // kRpyComp sources with the branch-free far form (pair32_far) and the group
 // sums folded (TwoSum) into (hi, lo) accumulators.
-//  * The sources of a group are stored relative to the group's centre c and
-//    each target is taken into that frame once per group, t = (th - c) + tl:
-//    d = t - s then carries the rounding of coordinates of the size of the
-//    group and of the target's distance from it, not of the suspension.
 //  * A group in which the warp met a pair closer than R_c = 4a is evaluated
 //    again with hi/lo differences. TPT = 2, 256-target tiles (large systems):
 //    with the exact coefficients at once. TPT = 1, 128-target tiles (a warp's
@@ -954,23 +869,23 @@ __device__ __forceinline__ void finish_tile(const PT *part, const SysMap &smap, 
 // segments, with chunks of four groups shared by the CTA between barriers: 965 us an
 // apply; close groups' loop unrolled by 4 942; streams of their own 930; an empty
 // second slot left out 910, all with the same bits. By 8 the loop spills: 1037.
-// These kernels run ensembles, and one system where its schedule is set by hand or
-// chosen by the autotuner; the automatic schedule of one system runs
-// rpy_pair32_warp_kernel below.
+// These kernels run ensembles, and one system in another schedule than the automatic
+// one, which runs rpy_pair32_warp_kernel below. (One system in the groups' frames here
+// too was 5-8% faster at 32 000 segments in most of these schedules, 1541 and 1738 us
+// with 256-target tiles at 3 CTAs per SM, and slower with few warps: 3026 and 2538 with
+// 128-target tiles at one; the automatic schedule is faster than any, 1435.)
 // ---------------------------------------------------------------------------
-constexpr int min_blocks(bool frames, int tpt, int split) {
-    return split == 2 ? kRpyMinBlocksSplit2
-           : tpt == 2 ? (frames ? kRpyMinBlocksTpt2 : kRpyMaxCtasTpt2)
-                      : (frames ? kRpyMinBlocksTpt1 : kRpyMaxCtasTpt1);
+constexpr int min_blocks(int tpt, int split) {
+    return split == 2 ? kRpyMinBlocksSplit2 : tpt == 2 ? kRpyMinBlocksTpt2 : kRpyMinBlocksTpt1;
 }
 
-template <bool kFrames, int TPT, int SPLIT = 1>
-__global__ void __launch_bounds__(kRpyThreads * SPLIT, min_blocks(kFrames, TPT, SPLIT))
+template <int TPT, int SPLIT = 1>
+__global__ void __launch_bounds__(kRpyThreads * SPLIT, min_blocks(TPT, SPLIT))
 rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G, RpyConst32 k,
                   float *__restrict__ part, int *__restrict__ cnt, double scale,
                   double *__restrict__ VW) {
-    constexpr int kGroupF4 = Rec<kFrames>::kGroupF4, kPairF4 = Rec<kFrames>::kPairF4;
-    constexpr int kUnitGroups = unit_sources(kFrames) / kRpyComp;   // groups per work unit
+    constexpr int kGroupF4 = Rec<false>::kGroupF4, kPairF4 = Rec<false>::kPairF4;
+    constexpr int kUnitGroups = unit_sources(false) / kRpyComp;   // groups per work unit
     constexpr int kWarps = kRpyThreads * SPLIT / 32;
     constexpr int kT = TPT;                               // targets per thread
     constexpr int kTile = kRpyThreads * TPT;              // targets per tile
@@ -1002,15 +917,15 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
         const int64_t wbase = ptile * kTile + (tid & ~31);
         // a warp whose targets are all padding (in a system's last tile) computes
         // nothing; the tile's sum never reads those rows
-        // ensembles: a warp whose second slot is all padding leaves that out too
-        const bool both = kFrames || kT == 1 || wbase + kRpyThreads - src0 < nsrc;
+        // and one whose second slot is all padding leaves that out
+        const bool both = kT == 1 || wbase + kRpyThreads - src0 < nsrc;
         const int64_t g_end = wbase - src0 < nsrc ? c_end : c_begin;
         int64_t grp = c_begin + set;
-        if (grp < g_end) stage_group<kFrames>(buf[0], srcs + kGroupF4 * grp, lane);
+        if (grp < g_end) stage_group<false>(buf[0], srcs + kGroupF4 * grp, lane);
         float th[kT][3], tl[kT][3];
 #pragma unroll
         for (int t = 0; t < kT; ++t)
-            load_target<kFrames>(src, ptile * kTile + t * kRpyThreads + tid, th[t], tl[t]);
+            load_target<false>(src, ptile * kTile + t * kRpyThreads + tid, th[t], tl[t]);
         float hi[kT][6], lo[kT][6];
 #pragma unroll
         for (int t = 0; t < kT; ++t)
@@ -1020,69 +935,54 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
 #pragma unroll 1
         for (int cur = 0; grp < g_end; grp += SPLIT, cur ^= 1) {
             if (grp + SPLIT < g_end) {
-                stage_group<kFrames>(buf[cur ^ 1], srcs + kGroupF4 * (grp + SPLIT), lane);
+                stage_group<false>(buf[cur ^ 1], srcs + kGroupF4 * (grp + SPLIT), lane);
                 asm volatile("cp.async.wait_group 1;" ::: "memory");
             } else {
                 cp_async_wait_all();
             }
             __syncwarp();
-            const float4 *qg = buf[cur] + Rec<kFrames>::kHead;
+            const float4 *qg = buf[cur];
             float out[kT][6];
             // the group that holds this warp's own segments
             const bool own =
                 TPT == 1 && src0 + grp * kRpyComp == wbase;
             bool near = own;
             if (!own) {
-                float2 t2[kT][3], acc[kT][Rec<kFrames>::kSums];
-                bool cross = false;          // a target inside a wide group
+                float2 t2[kT][3], acc[kT][6];
 #pragma unroll
                 for (int t = 0; t < kT; ++t) {
-                    to_frame<kFrames>(qg, th[t], tl[t], t2[t]);
-                    if constexpr (kFrames)
-                        cross = cross || fmaf(t2[t][0].x, t2[t][0].x,
-                                              fmaf(t2[t][1].x, t2[t][1].x,
-                                                   t2[t][2].x * t2[t][2].x)) < qg[-1].w;
 #pragma unroll
-                    for (int c = 0; c < Rec<kFrames>::kSums; ++c) acc[t][c] = f2(0.f, 0.f);
+                    for (int x = 0; x < 3; ++x) t2[t][x] = f2(th[t][x], th[t][x]);
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) acc[t][c] = f2(0.f, 0.f);
                 }
-                if constexpr (kFrames) cross = __any_sync(0xffffffffu, cross);
                 float rmin2 = k.close2;
-                if (kFrames && cross) {
-#pragma unroll 2
-                    for (int jp = 0; jp < kRpyComp / 2; ++jp) {
-#pragma unroll
-                        for (int t = 0; t < kT; ++t)
-                            pair32_far<false>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
-                    }
-                } else if (both) {
+                if (both) {
 #pragma unroll (kRpyUnroll / 2)
                     for (int jp = 0; jp < kRpyComp / 2; ++jp) {
 #pragma unroll
                         for (int t = 0; t < kT; ++t)
-                            pair32_far<kFrames>(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
+                            pair32_far(t2[t], qg + kPairF4 * jp, k, acc[t], rmin2);
                     }
                 } else {
 #pragma unroll (kRpyUnroll / 2)
                     for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                        pair32_far<kFrames>(t2[0], qg + kPairF4 * jp, k, acc[0], rmin2);
+                        pair32_far(t2[0], qg + kPairF4 * jp, k, acc[0], rmin2);
                 }
                 // (where slot 1 is left out: in a group with padding sources its padding
                 // targets would have met them at r = 0)
                 near = __any_sync(0xffffffffu, rmin2 < k.close2) ||
                        (!both && (grp + 1) * kRpyComp > nsrc);
 #pragma unroll
-                for (int t = 0; t < kT; ++t) {
-                    if (kFrames && cross) combine_group<false>(acc[t], t2[t], k.k23a2, out[t]);
-                    else combine_group<kFrames>(acc[t], t2[t], k.k23a2, out[t]);
-                }
+                for (int t = 0; t < kT; ++t)
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) out[t][c] = __fadd_rn(acc[t][c].x, acc[t][c].y);
             }
             if (near) {
                 // (one target at a time: fewer live registers)
 #pragma unroll
                 for (int t = 0; t < kT; ++t) {
                     if (t == 1 && !both) continue;
-                    float uh[3], ul[3];
-                    to_frame_hl<kFrames>(qg, th[t], tl[t], uh, ul);
                     float2 acc[6];
                     float rmin2 = k.close2;
                     bool exact = TPT == 2;
@@ -1092,7 +992,7 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
                         for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
 #pragma unroll 1
                         for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                            pair32_near<kFrames, kFarHiLo>(uh, ul, qg + kPairF4 * jp, k, acc,
+                            pair32_near<false, kFarHiLo>(th[t], tl[t], qg + kPairF4 * jp, k, acc,
                                                            rmin2, self_j, 2 * jp);
                         // overlapping distinct segments (r < 2a): the exact coefficients
                         exact = __any_sync(0xffffffffu, rmin2 < k.near2);
@@ -1100,9 +1000,9 @@ rpy_pair32_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, int G,
                     if (exact) {
 #pragma unroll
                         for (int c = 0; c < 6; ++c) acc[c] = f2(0.f, 0.f);
-#pragma unroll (kFrames ? 1 : 4)
+#pragma unroll 4
                         for (int jp = 0; jp < kRpyComp / 2; ++jp)
-                            pair32_near<kFrames, kExact>(uh, ul, qg + kPairF4 * jp, k, acc, rmin2);
+                            pair32_near<false, kExact>(th[t], tl[t], qg + kPairF4 * jp, k, acc, rmin2);
                     }
 #pragma unroll
                     for (int c = 0; c < 6; ++c) out[t][c] = __fadd_rn(acc[c].x, acc[c].y);
@@ -1348,9 +1248,9 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
                 const float2 tt =
                     __ffma2_rn(t2[0], t2[0], __ffma2_rn(t2[1], t2[1], __fmul2_rn(t2[2], t2[2])));
                 if (!__any_sync(0xffffffffu, fminf(tt.x, tt.y) < ce.w)) {
-                    float2 acc[2][Rec<true>::kSums];
+                    float2 acc[2][kFarSums];
 #pragma unroll
-                    for (int c = 0; c < Rec<true>::kSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
+                    for (int c = 0; c < kFarSums; ++c) acc[0][c] = acc[1][c] = f2(0.f, 0.f);
 #pragma unroll
                     for (int jp = 0; jp < kRpyComp / 2; ++jp) {
                         pair32_far2<0>(t2, qg + kPairF4 * jp, k, acc[0], rmin2);
@@ -1386,7 +1286,7 @@ rpy_pair32_warp_kernel(const float4 *__restrict__ src, SysMap smap, int64_t W, i
                     ph[x] = t1 ? th[1][x] : th[0][x];
                     pl[x] = t1 ? tl[1][x] : tl[0][x];
                 }
-                to_frame_hl<true>(qg, ph, pl, uh, ul);
+                to_frame_hl(qg, ph, pl, uh, ul);
                 float2 acc[6];
                 float rm = 0.f;
 #pragma unroll
@@ -1798,13 +1698,16 @@ bool overlaps(const double *p, int64_t n, const double *q, int64_t m) {
     return a < b + 8 * (uintptr_t)m && b < a + 8 * (uintptr_t)n;
 }
 
+// Source groups in their own frames: the automatic schedule of one FP32 system.
+bool frames_on(const fil_ctx *c) { return pair32_on(c) && c->rpy_auto; }
+
 SysMap sys_map(const fil_ctx *c, bool active_only) {
     SysMap m{};
     m.n_src = c->lay.S;
     if (c->n_sys == 1 && !active_only) {
         // one system: tiles and groups in order, no table
         m.n_tiles = c->rpy_tiles;
-        const int per = unit_sources(c->rpy_frames != 0);
+        const int per = unit_sources(frames_on(c));
         m.n_units = (c->lay.S + per - 1) / per;
         return m;
     }
@@ -1847,8 +1750,8 @@ cudaError_t allow_warp_smem() {
 // Tiles of T targets of every system (only tiles that hold real targets),
 // each with ceil(S_s / unit) units.
 void build_tiles(fil_ctx *c) {
-    const int T = c->rpy_auto && c->rpy_frames ? kWarpTile : rpy_tile(c);
-    const int per = unit_sources(c->rpy_frames != 0);
+    const int T = frames_on(c) ? kWarpTile : rpy_tile(c);
+    const int per = unit_sources(frames_on(c));
     c->tile_unit_off_h.assign(1, 0);
     c->tile_src_h.clear();
     c->tile_nsrc_h.clear();
@@ -1884,8 +1787,7 @@ int occupancy(K kernel, int threads = kRpyThreads) {
 int pair_occupancy(const fil_ctx *c, int tpt, int split) {
     if (!pair32_on(c))
         return tpt == 1 ? occupancy(rpy_pair64_kernel<1>) : occupancy(rpy_pair64_kernel<2>);
-    if (tpt == 2) return kRpyMaxCtasTpt2;
-    return split == 2 ? kRpyMaxCtasSplit2 : kRpyMaxCtasTpt1;
+    return min_blocks(tpt, split);
 }
 
 // The grid of the current schedule, and whether it fills the SMs. One that does not
@@ -1913,7 +1815,7 @@ cudaError_t rpy_setup(fil_ctx *c) {
     const int occ = pair_occupancy(c, kRpyTargetsPerThread, 1);
     c->rpy_ctas = occ;
     c->rpy_split = 1;
-    c->rpy_ctas_max = std::max({occ, kRpyMaxCtasTpt1, kRpyMaxCtasTpt2,
+    c->rpy_ctas_max = std::max({occ, kRpyMinBlocksTpt1, kRpyMinBlocksTpt2,
                                 occupancy(rpy_pair64_kernel<1>), occupancy(rpy_pair64_kernel<2>)});
     set_grids(c);
     // padded layout: system s occupies [pad_off[s], pad_off[s+1]), a multiple of kRpyPad
@@ -1934,9 +1836,8 @@ cudaError_t rpy_setup(fil_ctx *c) {
             c->pad_map_h[P] = (int)g;
         }
     c->rpy_tiles_max = count_tiles(c, kWarpTile);
-    c->rpy_frames = pair32_on(c) && ns == 1 ? 1 : 0;
     c->rpy_auto = automatic_schedule(c, c->rpy_tpt, c->rpy_ctas, c->rpy_split);
-    if (c->rpy_frames) {
+    if (frames_on(c)) {
         const cudaError_t e = allow_warp_smem();
         if (e != cudaSuccess) return e;
     }
@@ -1981,7 +1882,7 @@ size_t rpy_partial_bytes(const fil_ctx *c) {
         const size_t b = (size_t)(G + count_tiles(c, T)) * T * 12 * sizeof(float);
         most = std::max(most, b);
     }
-    if (c->rpy_frames)
+    if (pair32_on(c) && c->n_sys == 1)
         most = std::max(most, (size_t)((int64_t)c->num_sms * kWarpCta + c->rpy_tiles_max) *
                                   kWarpPart * sizeof(float));
     else if (c->n_sys == 1 && c->lay.S > kDirectMaxSeg && c->lay.S <= kSymMaxSeg) {
@@ -2086,7 +1987,7 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         return cudaGetLastError();
     }
     if (pair32_on(c)) {
-        const auto pack = c->rpy_frames ? pack32_kernel<true> : pack32_kernel<false>;
+        const auto pack = c->rpy_auto ? pack32_kernel<true> : pack32_kernel<false>;
         const int n_spread = c->rpy_auto ? spread_count((S + kRpyComp - 1) / kRpyComp) : 0;
         launch_pdl(pack, (unsigned)(c->Spad / kPackThreads), kPackThreads, 0, c->stream, Y, FT, S,
                    c->Spad, sm, n_spread, (float)c->a, c->src32);
@@ -2101,13 +2002,9 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         } else {
             const int G = (int)(active_only ? c->rpy_grid32 : std::min<int64_t>(c->rpy_grid32, W));
             const bool split = c->rpy_tpt == 1 && c->rpy_split == 2;
-            const auto pair =
-                c->rpy_frames ? (split               ? rpy_pair32_kernel<true, 1, 2>
-                                 : c->rpy_tpt == 1   ? rpy_pair32_kernel<true, 1>
-                                                     : rpy_pair32_kernel<true, 2>)
-                              : (split               ? rpy_pair32_kernel<false, 1, 2>
-                                 : c->rpy_tpt == 1   ? rpy_pair32_kernel<false, 1>
-                                                     : rpy_pair32_kernel<false, 2>);
+            const auto pair = split             ? rpy_pair32_kernel<1, 2>
+                              : c->rpy_tpt == 1 ? rpy_pair32_kernel<1>
+                                                : rpy_pair32_kernel<2>;
             launch_dep(early, pair, G, kRpyThreads * (split ? 2 : 1), 0, c->stream, c->src32,
                        sm, W, G, k, (float *)c->partials, c->tile_cnt, scale, VW);
         }

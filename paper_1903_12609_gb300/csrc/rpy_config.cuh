@@ -15,16 +15,10 @@ constexpr int kRpyChunk = 128;                 // sources per shared-memory chun
 constexpr int kRpyComp = 32;                   // sources per compensated partial (FP32)
 // Resident CTAs per SM the FP32 pair kernels are compiled for, by targets per
 // thread and source split: caps the registers so that this many CTAs fit
-// (2 targets: 168 registers, 3 CTAs; 1 target: 96 registers, 5 CTAs; split in
-// two: 2 CTAs of 256 threads, 128 registers).
-constexpr int kRpyMinBlocksTpt2 = 3;
-constexpr int kRpyMinBlocksTpt1 = 5;
+// (2 targets: 128 registers; 1 target: 80; split in two, 256 threads: 128).
+constexpr int kRpyMinBlocksTpt2 = 4;
+constexpr int kRpyMinBlocksTpt1 = 6;
 constexpr int kRpyMinBlocksSplit2 = 2;
-// Most CTAs per SM a schedule of the FP32 kernels may ask for (grids larger
-// than the residency run in more than one wave).
-constexpr int kRpyMaxCtasTpt2 = 4;
-constexpr int kRpyMaxCtasTpt1 = 6;
-constexpr int kRpyMaxCtasSplit2 = 2;
 // float4 per two FP32 source records (the packed FP32x2 layout), and per group
 // of kRpyComp sources (its centre, then the records)
 constexpr int kRpyPairF4 = 9;
