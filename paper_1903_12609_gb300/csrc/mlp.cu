@@ -128,23 +128,28 @@ input_kernel(const float *__restrict__ x, int64_t B, const float *__restrict__ m
              const float *__restrict__ stdv, bf16 *__restrict__ X, bf16 *__restrict__ Xt,
              int64_t ldt, int64_t Kb) {
     tc::pdl_launch_next();
-    // (rows along x: the other dimensions end at 65 535 blocks, 2 097 120 rows)
-    const int c = blockIdx.y * kInThreads + threadIdx.x;
-    const int64_t b0 = (int64_t)blockIdx.x * kRows;
+    // (one dimension, the only one with more than 65 535 blocks. Addresses are a base a
+    // thread and small offsets: with the 64-bit row index in each of them the kernel took
+    // 100 registers and a forward pass of 100 000 rows 545 us; 55 and 483 in this form)
+    const int c = (int)(blockIdx.x % 4) * kInThreads + threadIdx.x;
+    const int64_t b0 = (int64_t)(blockIdx.x / 4) * kRows;
+    const int rows = (int)min((int64_t)kRows, B - b0);       // (0 or less: padding only)
+    const float *xp = x + b0 * kIn + c;
+    bf16 *Xp = X + b0 * kInP + c;
     const bool in = c < kIn;
     const float mu = in ? mean[c] : 0.f, sd = in ? stdv[c] : 1.f;
     float v[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r)
-        v[r] = in && b0 + r < B ? x[(b0 + r) * kIn + c] : mu;
+        v[r] = in && r < rows ? xp[r * kIn] : mu;
     uint32_t h[kRows / 2];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
         const bf16 q = __float2bfloat16_rn((v[r] - mu) / sd);
-        const uint32_t bits = b0 + r < B ? *reinterpret_cast<const unsigned short *>(&q) : 0u;
+        const uint32_t bits = r < rows ? *reinterpret_cast<const unsigned short *>(&q) : 0u;
         if (r & 1) h[r >> 1] |= bits << 16;
         else h[r >> 1] = bits;
-        if (b0 + r < B) X[(b0 + r) * kInP + c] = q;
+        if (r < rows) Xp[r * kInP] = q;
     }
     if (Xt) store_column(Xt + (int64_t)c * ldt, b0, Kb, h);
 }
@@ -403,7 +408,7 @@ cudaError_t one_product(fil_mlp *m, const tc::Problem &p) {
 // without it m->Y takes the normalised ones.
 cudaError_t forward(fil_mlp *m, const float *x, int64_t B, bool train, float *y) {
     const int64_t Kb = round_up(B, tc::kTileK);
-    const dim3 grid((unsigned)(((train ? Kb : B) + kRows - 1) / kRows), 4);
+    const dim3 grid(4 * (unsigned)(((train ? Kb : B) + kRows - 1) / kRows));
     input_kernel<<<grid, kInThreads, 0, m->stream>>>(x, B, m->in_mean, m->in_std, m->X,
                                                      train ? m->Xt : nullptr, m->ldt, Kb);
     cudaError_t e = cudaGetLastError();
