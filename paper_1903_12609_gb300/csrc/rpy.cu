@@ -1966,8 +1966,12 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
     // 71.0 and 45.5, 64 small ones 66.3 and 55.5, 5 of 2 059 (40 units) 41.5 and 45.4. One
     // system in 128-target tiles, 3 CTAs per SM: 320 segments, 30 units, 16.0 and 18.5; 960,
     // 240 units, 27.9 and 26.7. 256 systems in such tiles 1519 and 855.
-    const bool early = (c->rpy_full && (c->n_sys == 1 || W >= c->rpy_grid32)) ||
-                       W <= (c->n_sys == 1 ? c->num_sms : c->num_sms / 3);
+    // The FP64 kernel only where it is too small to crowd: its few units a CTA wait for the
+    // fullest SM, and early placement makes that a matter of luck (one system of 8 193
+    // segments 7.46 ms early and 7.16 plainly, 9 000 9.1 and 9.5, 10 000 10.7 and 11.3, 12 000
+    // 14.6 and 14.5; three systems in 8 193 3.2 and 2.9, in 16 000 9.1 and 8.9).
+    const bool small = W <= (c->n_sys == 1 ? c->num_sms : c->num_sms / 3);
+    const bool early = small || (c->rpy_full && (c->n_sys == 1 || W >= c->rpy_grid32));
     // the active-tile list changes between applies: its launches keep a fixed grid
     // (and read the unit count from the device), so captured graphs stay valid
     if (c->rpy_auto && S <= direct_max(pair32_on(c)) && !overlaps(VW, 6 * S, Y, 3 * S) &&
@@ -2036,7 +2040,7 @@ cudaError_t rpy_apply(fil_ctx *c, const double *Y, const double *FT, double *VW,
         launch_pdl(pack64_kernel, pgrid, pb, 0, c->stream, Y, FT, S, c->Spad, sm, c->src64);
         if (c->tune_ev && c->tune_pair) cudaEventRecord(c->tune_ev[0], c->stream);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n]);
-        launch_dep(early, c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G,
+        launch_dep(small, c->rpy_tpt == 1 ? rpy_pair64_kernel<1> : rpy_pair64_kernel<2>, G,
                    kRpyThreads, 0, c->stream, c->src64, sm, W, G, k, (double *)c->partials,
                    c->tile_cnt, scale, VW);
         if (timed) prof_record(c, c->prof_ev[2 * c->prof_n + 1]);
